@@ -508,10 +508,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     }
   } else if (warp == 17) {
     // ------------------------------------------------------------------ MMA issuer
-    // (whole warp runs the loop; only the tcgen05 instructions are predicated on lane 0)
+    // (one elected thread runs the loop)
     setmaxnreg_dec<40>();
-    {
-      const uint32_t leader = (lane == 0);
+    if (elect_one()) {
       constexpr uint32_t tmem = 0;   // checked above: TMEM operand addresses are immediates in this loop
       constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
       constexpr uint32_t idesc_acc = idesc_bf16_f32(128, D, 0, 1);
@@ -530,45 +529,45 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
 #pragma unroll
         for (int kk = 0; kk < kKSteps; ++kk) {
           const uint32_t c = ((kk >> 2) * kBoxBytes + (kk & 3) * 32) >> 4;
-          mma_ss(tmem + 256, dk + c, qd + c, idesc_s, kk > 0, leader);
+          mma_ss(tmem + 256, dk + c, qd + c, idesc_s, kk > 0);
         }
-        tc_commit(&bar->s_full, leader);
+        tc_commit(&bar->s_full);
       };
       auto issue_dP = [&](int ds) {   // dP^T = V dO^T into the U columns
         const uint64_t dod = ddo_base + ds * kStageStep;
 #pragma unroll
         for (int kk = 0; kk < kKSteps; ++kk) {
           const uint32_t c = ((kk >> 2) * kBoxBytes + (kk & 3) * 32) >> 4;
-          mma_ss(tmem + 384, dv + c, dod + c, idesc_s, kk > 0, leader);
+          mma_ss(tmem + 384, dv + c, dod + c, idesc_s, kk > 0);
         }
-        tc_commit(&bar->dp_full, leader);
+        tc_commit(&bar->dp_full);
       };
       auto issue_dQ = [&]() {         // dQ(i) = dS K into the U columns (a fresh accumulator for every item)
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
-          mma_ss(tmem + 384, dsm + ((kk * 2048) >> 4), dkm + ((kk * 2048) >> 4), idesc_dq, kk > 0, leader);
-        tc_commit(&bar->dq_full, leader);
+          mma_ss(tmem + 384, dsm + ((kk * 2048) >> 4), dkm + ((kk * 2048) >> 4), idesc_dq, kk > 0);
+        tc_commit(&bar->dq_full);
       };
       auto issue_dV = [&](int ds, bool first) {   // dV += P^T dO, P^T from the T columns
         const uint64_t dod = ddom_base + ds * kStageStep;
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
           mma_ts(tmem, tmem + 256 + (kk >> 1) * 32 + (kk & 1) * 8, dod + ((kk * 2048) >> 4), idesc_acc,
-                 (kk > 0 || !first) ? 1u : 0u, leader);
-        tc_commit(&bar->do_empty[ds], leader);
+                 (kk > 0 || !first) ? 1u : 0u);
+        tc_commit(&bar->do_empty[ds]);
       };
       auto issue_dK = [&](int qs, bool first) {   // dK += dS^T Q, dS^T from shared memory
         const uint64_t qd = dqm_base + qs * kStageStep;
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
           const uint32_t c = ((kk >> 2) * kBoxBytes + (kk & 3) * 32) >> 4;
-          mma_ss(tmem + D, dsk + c, qd + ((kk * 2048) >> 4), idesc_acc, (kk > 0 || !first) ? 1u : 0u, leader);
+          mma_ss(tmem + D, dsk + c, qd + ((kk * 2048) >> 4), idesc_acc, (kk > 0 || !first) ? 1u : 0u);
         }
-        tc_commit(&bar->q_empty[qs], leader);
-        tc_commit(&bar->ds_free, leader);
+        tc_commit(&bar->q_empty[qs]);
+        tc_commit(&bar->ds_free);
       };
-      bool ok = mbar_spin_warp(&bar->kv_full, 0, abort_flag) && mbar_spin_warp(&bar->q_full[0], 0, abort_flag) &&
-                mbar_spin_warp(&bar->do_full[0], 0, abort_flag);
+      bool ok = mbar_spin(&bar->kv_full, 0, abort_flag) && mbar_spin(&bar->q_full[0], 0, abort_flag) &&
+                mbar_spin(&bar->do_full[0], 0, abort_flag);
       if (ok) {
         tc_fence_after();
         issue_S(0);
@@ -576,17 +575,17 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       }
       for (int i = 0; ok && i < plan.total; ++i) {
         const bool more = i + 1 < plan.total;
-        if (!mbar_spin_warp(&bar->p_full, i & 1, abort_flag)) { ok = false; break; }
+        if (!mbar_spin(&bar->p_full, i & 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         issue_dV(i & 1, i == 0);
         if (more) {
           // S^T(i+1) overwrites P^T(i): dV(i) precedes it in issue order.  It does not depend on dS(i), so it goes
           // ahead of that wait: the compute warps find the next scores ready when they are done with dS(i)
-          if (!mbar_spin_warp(&bar->q_full[(i + 1) & 1], ((i + 1) >> 1) & 1, abort_flag)) { ok = false; break; }
+          if (!mbar_spin(&bar->q_full[(i + 1) & 1], ((i + 1) >> 1) & 1, abort_flag)) { ok = false; break; }
           tc_fence_after();
           issue_S((i + 1) & 1);
         }
-        if (!mbar_spin_warp(&bar->ds_full, i & 1, abort_flag)) { ok = false; break; }
+        if (!mbar_spin(&bar->ds_full, i & 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         issue_dQ();
         issue_dK(i & 1, i == 0);       // keeps the pipe busy while dQ(i) is read out
@@ -594,13 +593,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
           const int sn = (i + 1) & 1;
           const uint32_t phn = ((i + 1) >> 1) & 1;
           // dP^T(i+1) overwrites dQ(i): wait for its read-out
-          if (!mbar_spin_warp(&bar->u_free, i & 1, abort_flag) ||
-              !mbar_spin_warp(&bar->do_full[sn], phn, abort_flag)) { ok = false; break; }
+          if (!mbar_spin(&bar->u_free, i & 1, abort_flag) ||
+              !mbar_spin(&bar->do_full[sn], phn, abort_flag)) { ok = false; break; }
           tc_fence_after();
           issue_dP(sn);
         }
       }
-      if (ok) tc_commit(&bar->final_bar, leader);
+      if (ok) tc_commit(&bar->final_bar);
     }
     __syncwarp();
   } else {

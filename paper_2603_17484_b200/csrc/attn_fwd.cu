@@ -203,12 +203,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   } else if (warp == kMmaWarp) {
     // =========================================================================== MMA issuer
     setmaxnreg_dec<kOtherRegs>();
-    // The whole warp runs this loop (uniform control flow keeps the descriptor arithmetic in uniform registers);
-    // only the tcgen05 instructions themselves are predicated on lane 0.  Operand descriptors are built once per
-    // tile / stage and advanced by compile-time constants, so that issuing stays well under the 64 clocks one
-    // 128x128x16 MMA takes.
-    {
-      const uint32_t leader = (lane == 0);
+    // One elected thread runs this loop (see tc_commit): operand descriptors are built once per tile / stage and advanced
+    // by compile-time constants, so that issuing stays well under the 64 clocks one 128x128x16 MMA takes.
+    if (elect_one()) {
       constexpr uint32_t tmem = 0;   // checked above: TMEM operand addresses are immediates in this loop
       static_assert(kStages == 2 && kNumTiles == 2, "descriptor selects below assume two stages and two tiles");
       constexpr uint32_t idesc_qk = idesc_bf16_f32(kTileM, kTileN, 0, 0);
@@ -229,30 +226,30 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 #pragma unroll
         for (int kk = 0; kk < kKSteps; ++kk) {
           const uint32_t c = ((kk >> 2) * SM::kBoxBytes + (kk & 3) * 32) >> 4;
-          mma_ss(d, qd + c, kd + c, idesc_qk, kk > 0, leader);
+          mma_ss(d, qd + c, kd + c, idesc_qk, kk > 0);
         }
-        tc_commit(&bar->s_full[t], leader);
+        tc_commit(&bar->s_full[t]);
       };
       auto issue_pv = [&](int t, int s, uint32_t acc) {
         const uint64_t vd = s ? dv1 : dv0;
         const uint32_t d = tmem + kOCol0 + t * D, p = tmem + t * kTileN;
 #pragma unroll
         for (int kk = 0; kk < kTileN / 16; ++kk)
-          mma_ts(d, p + (kk >> 2) * 64 + (kk & 3) * 8, vd + ((kk * 2048) >> 4), idesc_pv, kk > 0 ? 1u : acc, leader);
+          mma_ts(d, p + (kk >> 2) * 64 + (kk & 3) * 8, vd + ((kk * 2048) >> 4), idesc_pv, kk > 0 ? 1u : acc);
       };
       auto in_range = [&](int t, int j) { return t ? (j >= lo1 && j <= hi1) : (j >= lo0 && j <= hi0); };
 
       if (jhi < jlo) ok = false;   // no key block at all (shared-window mode): nothing to issue, nobody waits
       // first key block: Q*K^T for both tiles
-      if (ok && !mbar_spin_warp(&bar->k_full[0], 0, abort_flag)) ok = false;
+      if (ok && !mbar_spin(&bar->k_full[0], 0, abort_flag)) ok = false;
 #pragma unroll
       for (int t = 0; t < kNumTiles; ++t) {
         if (ok && in_range(t, jlo)) {
-          if (!mbar_spin_warp(&bar->q_full[t], 0, abort_flag)) { ok = false; }
+          if (!mbar_spin(&bar->q_full[t], 0, abort_flag)) { ok = false; }
           else { tc_fence_after(); issue_qk(t, 0); }
         }
       }
-      if (ok) tc_commit(&bar->k_empty[0], leader);
+      if (ok) tc_commit(&bar->k_empty[0]);
 
       for (int j = jlo; ok && j <= jhi; ++j) {
         const int it = j - jlo, s = it & 1, sn = s ^ 1;
@@ -263,11 +260,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         for (int t = 0; t < kNumTiles; ++t) {
           if (ok && in_range(t, j)) {
             uint32_t& pc = t ? p_cnt1 : p_cnt0;
-            if (!mbar_spin_warp(&bar->p_full[t], pc & 1, abort_flag)) { ok = false; }
+            if (!mbar_spin(&bar->p_full[t], pc & 1, abort_flag)) { ok = false; }
             else {
               ++pc;
               if (!v_ready) {
-                if (!mbar_spin_warp(&bar->v_full[s], ph, abort_flag)) ok = false;
+                if (!mbar_spin(&bar->v_full[s], ph, abort_flag)) ok = false;
                 v_ready = true;
               }
               if (ok) {
@@ -278,10 +275,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
           }
           if (ok && j + 1 <= jhi && in_range(t, j + 1)) {
             if (!k_ready) {
-              if (!mbar_spin_warp(&bar->k_full[sn], phn, abort_flag)) ok = false;
+              if (!mbar_spin(&bar->k_full[sn], phn, abort_flag)) ok = false;
               k_ready = true;
             }
-            if (ok && j + 1 == (t ? lo1 : lo0) && !mbar_spin_warp(&bar->q_full[t], 0, abort_flag)) ok = false;
+            if (ok && j + 1 == (t ? lo1 : lo0) && !mbar_spin(&bar->q_full[t], 0, abort_flag)) ok = false;
             if (ok) {
               tc_fence_after();
               issue_qk(t, sn);
@@ -290,14 +287,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         }
         if (!ok) break;
         // V block j is released once both tiles' P*V have drained; K block j+1 once both Q*K^T have
-        if (!v_ready && !mbar_spin_warp(&bar->v_full[s], ph, abort_flag)) break;
-        tc_commit(&bar->v_empty[s], leader);
+        if (!v_ready && !mbar_spin(&bar->v_full[s], ph, abort_flag)) break;
+        tc_commit(&bar->v_empty[s]);
         if (j + 1 <= jhi) {
-          if (!k_ready && !mbar_spin_warp(&bar->k_full[sn], phn, abort_flag)) break;
-          tc_commit(&bar->k_empty[sn], leader);
+          if (!k_ready && !mbar_spin(&bar->k_full[sn], phn, abort_flag)) break;
+          tc_commit(&bar->k_empty[sn]);
         }
       }
-      if (ok) tc_commit(&bar->o_final, leader);
+      if (ok) tc_commit(&bar->o_final);
     }
     __syncwarp();
   } else if (warp > kMmaWarp) {

@@ -113,7 +113,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return true;
 }
 
-// Polling wait (mbarrier.test_wait never suspends the thread): lowest wake-up latency, for a single warp whose
+// Polling wait (mbarrier.test_wait never suspends the thread): lowest wake-up latency, for the single thread whose
 // reaction time is on the critical path.  Bounded like mbar_wait.
 __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
@@ -124,18 +124,16 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool mbar_spin_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  bool done = mbar_test_wait(bar, parity);
-  if (!__all_sync(0xffffffffu, done)) {
-    const uint64_t t0 = globaltimer_ns();
-    uint32_t spins = 0;
-    while (!__all_sync(0xffffffffu, done = mbar_test_wait(bar, parity))) {
-      if ((++spins & 0x3ffu) == 0) {
-        if (*abort_flag) return false;
-        if (globaltimer_ns() - t0 > kWaitLimitNs) {
-          *abort_flag = 1;
-          return false;
-        }
+__device__ __forceinline__ bool mbar_spin(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  if (mbar_test_wait(bar, parity)) return true;
+  const uint64_t t0 = globaltimer_ns();
+  uint32_t spins = 0;
+  while (!mbar_test_wait(bar, parity)) {
+    if ((++spins & 0x3ffu) == 0) {
+      if (*abort_flag) return false;
+      if (globaltimer_ns() - t0 > kWaitLimitNs) {
+        *abort_flag = 1;
+        return false;
       }
     }
   }
@@ -184,17 +182,15 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// The MMA-issuing warp runs its loop with all 32 lanes (uniform control flow, so that descriptor arithmetic
-// can stay in uniform registers) and only the tcgen05.mma / tcgen05.commit instruction itself is predicated on
-// one lane: every wrapper below takes `leader` (non-zero in exactly one lane of the warp).
+// The issuing loop runs in ONE thread, entered through `if (elect_one())`: the compiler then knows the branch to be
+// uniform and keeps the descriptors in uniform registers.  Issue takes about 25 clk per tcgen05.mma that way, against
+// 58 clk when all 32 lanes run the loop and every instruction is predicated on a lane -- close to the 64 clk a
+// 128x128x16 product takes, so that the pipe ran dry behind every wait.
 
 // mbarrier arrives once all tcgen05.mma previously issued by this thread have completed
-__device__ __forceinline__ void tc_commit(uint64_t* bar, uint32_t leader) {
-  asm volatile(
-      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
-      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}"
-      ::"r"(smem_u32(bar)), "r"(leader)
-      : "memory");
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+               : "memory");
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -226,22 +222,20 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn_maj
          (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]   (issued by the lane with leader != 0)
+// D[tmem] (+)= A[smem] * B[smem]
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate, uint32_t leader) {
+                                       uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem]
 __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate, uint32_t leader) {
+                                       uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
-      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 

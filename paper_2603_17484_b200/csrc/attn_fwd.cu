@@ -332,15 +332,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + c * 32, v[c]);
         tmem_ld_wait();
         if (partial) {
-          // edge block (causal diagonal, left window edge, ragged rows): masked scores become -inf, whose
-          // exponential is an exact zero below
+          // edge block (causal diagonal, left window edge, ragged rows): the row's visible keys are one range, hence one
+          // bit per column; masked scores become -inf, whose exponential is an exact zero below.  (Two comparisons of
+          // key positions per score instead cost 1100 to 2000 clk a block, next to 1800 for all of an interior one.)
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
+            const uint32_t visible = bit_range(pos_lo - k0 - c * 32, pos + 1 - k0 - c * 32);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              const int kp = k0 + c * 32 + e;
-              v[c][e] = (kp <= pos && kp >= pos_lo) ? v[c][e] : 0xff800000u;
-            }
+            for (int e = 0; e < 32; ++e) v[c][e] = (visible >> e) & 1u ? v[c][e] : 0xff800000u;
           }
         }
         float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;

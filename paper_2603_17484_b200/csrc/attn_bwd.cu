@@ -157,6 +157,7 @@ struct BwdArgs {
   float scale, scale_log2;
   int skip_local, skip_global;   // gradients of one module only (the other module has its own Q/K/V)
   int kb_begin, kb_count;        // key blocks [kb_begin, kb_begin + kb_count) of every KV head
+  int kb_outermost;              // launch order: key blocks outermost (1) or KV heads outermost (0)
   RowStrides dq_st, dk_st, dv_st;   // strides of the gradient tensors in elements
   float* dq_acc_loc;             // fp32 dQ accumulators (layout: see bwd_kernel), by row tile
   float* dq_acc_glb;             //                 and by compact tile; NULL when that module is skipped
@@ -202,6 +203,7 @@ struct ItemPlan {
   int glb_t0, glb_nt;   // first compact tile, number of compact tiles
   int per_head;         // loc_nt + glb_nt
   int total;            // per_head * G
+  int first, count;     // this CTA's share [first, first + count) of them
 };
 
 __device__ __forceinline__ ItemPlan make_plan(const BwdArgs& a, int b, int k0, int span = kTileN) {
@@ -239,7 +241,8 @@ __device__ __forceinline__ ItemPlan make_plan(const BwdArgs& a, int b, int k0, i
 struct ItemCursor {
   int h, r, per_head, loc_nt, loc_t0, glb_t0;
   __device__ __forceinline__ ItemCursor(const ItemPlan& p, int h0)
-      : h(h0), r(0), per_head(p.per_head), loc_nt(p.loc_nt), loc_t0(p.loc_t0), glb_t0(p.glb_t0) {}
+      : h(h0 + p.first / p.per_head), r(p.first % p.per_head), per_head(p.per_head), loc_nt(p.loc_nt), loc_t0(p.loc_t0),
+        glb_t0(p.glb_t0) {}
   __device__ __forceinline__ int glb() const { return r >= loc_nt; }
   __device__ __forceinline__ int tile() const { return r < loc_nt ? loc_t0 + r : glb_t0 + (r - loc_nt); }
   __device__ __forceinline__ void next() { if (++r == per_head) { r = 0; ++h; } }
@@ -334,22 +337,98 @@ __device__ __forceinline__ uint32_t visible_columns(const BwdArgs& a, int b, int
   return bit_range((int)first - col0, (last < row_end ? (int)last : row_end) - col0);
 }
 
-template <int D>
+// Byte offset in the rings of row kr of quarter q in slot `slot` of its owner; the 16-byte pieces of a row lie 128 rows
+// apart, so that a warp's accesses are contiguous.  kSplit - 1 slots of 4 / kSplit quarters of 128 x D / 2 floats.
+template <int D, int kSplit>
+__device__ __forceinline__ uint32_t dkv_slot_offset(int slot, int q, int kr) {
+  return (slot * (4 / kSplit) + q % (4 / kSplit)) * (128 * (D / 2) * 4) + kr * 16;
+}
+
+template <int D, int kSplit>
+__device__ __forceinline__ void send_dkv(uint32_t dst, uint32_t taddr, bool own) {
+#pragma unroll
+  for (int c = 0; c < D / 64; ++c) {
+    uint32_t v[32];
+    if (own) {
+      tmem_ld32(taddr + c * 32, v);
+      tmem_ld_wait();
+    } else {
+#pragma unroll
+      for (int e = 0; e < 32; ++e) v[e] = 0u;
+    }
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+      cluster_st128(dst + (c * 8 + x) * (128 * 16), v[4 * x], v[4 * x + 1], v[4 * x + 2], v[4 * x + 3]);
+  }
+}
+
+// One quarter of (dV | dK): accumulator (plus the other CTAs' shares of a cluster) to bf16.  own: this CTA had items.
+template <int D, int kSplit>
+__device__ __forceinline__ void store_dkv(const BwdArgs& a, const uint8_t* smem, uint32_t taddr, bool own, int b, int g,
+                                          int kp, int q, int kr) {
+  static_assert((kSplit - 1) * (4 / kSplit) * 128 * (D / 2) * 4 <= 4 * BwdSmem<D>::kTileBytes, "slots exceed the rings");
+  const bool valid = kp < a.Lk;
+  const int which = q >> 1, half = q & 1;
+  const RowStrides st = which == 0 ? a.dv_st : a.dk_st;
+  bf16* dst = (which == 0 ? a.dV : a.dK) + b * st.b + (valid ? kp : 0) * st.t + (int64_t)g * D + half * (D / 2);
+  const float mul = which == 0 ? 1.0f : a.scale;
+#pragma unroll
+  for (int c = 0; c < D / 64; ++c) {
+    uint32_t v[32];
+    if (own) {
+      tmem_ld32(taddr + c * 32, v);
+      tmem_ld_wait();
+    } else {
+#pragma unroll
+      for (int e = 0; e < 32; ++e) v[e] = 0u;
+    }
+#pragma unroll
+    for (int s = 0; s < kSplit - 1; ++s) {
+      const uint32_t src = smem_u32(smem + BwdSmem<D>::kQOff) + dkv_slot_offset<D, kSplit>(s, q, kr) + c * 8 * (128 * 16);
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const float4 f = lds128(src + x * (128 * 16));
+        v[4 * x] = __float_as_uint(__uint_as_float(v[4 * x]) + f.x);
+        v[4 * x + 1] = __float_as_uint(__uint_as_float(v[4 * x + 1]) + f.y);
+        v[4 * x + 2] = __float_as_uint(__uint_as_float(v[4 * x + 2]) + f.z);
+        v[4 * x + 3] = __float_as_uint(__uint_as_float(v[4 * x + 3]) + f.w);
+      }
+    }
+    if (valid) {
+      uint4* d4 = reinterpret_cast<uint4*>(dst + c * 32);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        float f[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * x + e]) * mul;
+        d4[x] = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+      }
+    }
+  }
+}
+
+// kSplit > 1: the kSplit CTAs of a cluster share one key block.  Each walks its part of the items, and at the end every
+// CTA sums one part of the columns of (dV | dK) over the cluster through distributed shared memory.
+template <int D, int kSplit>
 __global__ void __launch_bounds__(kDkvThreads, 1)
 bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapDO,
                const __grid_constant__ CUtensorMap mapQc, const __grid_constant__ CUtensorMap mapDOc,
                const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV, const BwdArgs a) {
   using SM = BwdSmem<D>;
   constexpr int kKSteps = D / 16;
-  // key blocks ascending (most work first) inside one KV head; KV heads outermost so that the CTAs
-  // running together share the same query tiles in L2
-  const int j = a.kb_begin + blockIdx.x % a.kb_count;
-  const int rest = blockIdx.x / a.kb_count;
+  // Key blocks ascending: most work first.  KV heads outermost lets the CTAs that run together share query tiles in L2;
+  // key blocks outermost starts the heaviest blocks of every head first, which a launch of few waves needs.
+  const int rank = kSplit > 1 ? (int)cluster_rank() : 0;
+  const int work = blockIdx.x / kSplit, heads = a.B * a.Hkv;
+  const int j = a.kb_begin + (a.kb_outermost ? work / heads : work % a.kb_count);
+  const int rest = a.kb_outermost ? work % heads : work / a.kb_count;
   const int b = rest % a.B;
   const int g = rest / a.B;
   const int G = a.Hq / a.Hkv;
   const int k0 = j * kTileN;
-  const ItemPlan plan = make_plan(a, b, k0);
+  ItemPlan plan = make_plan(a, b, k0);
+  plan.first = (int)((int64_t)plan.total * rank / kSplit);
+  plan.count = (int)((int64_t)plan.total * (rank + 1) / kSplit) - plan.first;
   const int n_c = a.skip_global ? 0 : a.n_routed[b];   // the routing arrays may be NULL when the global part is skipped
 
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -368,7 +447,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   }
   if (plan.total == 0) {
     // no query can see these keys: their gradients are zero
-    for (int i = tid; i < kTileN * (D / 8); i += blockDim.x) {
+    for (int i = tid; rank == 0 && i < kTileN * (D / 8); i += blockDim.x) {
       const int kr = i / (D / 8), c8 = i % (D / 8);
       if (k0 + kr < a.Lk) {
         const int64_t o = (int64_t)g * D + c8 * 8;
@@ -422,7 +501,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     const int n_tiles = (a.Lq + kTileM - 1) / kTileM;
     constexpr int kChunks = D / 32;     // 32-column TMEM loads of the whole tile; this warp takes half of them
     ItemCursor cur(plan, g * G);
-    for (int i = 0; i < plan.total; ++i) {
+    for (int i = 0; i < plan.count; ++i) {
       const int h = cur.h, glb = cur.glb(), tile = cur.tile();
       cur.next();
       float* acc = glb ? a.dq_acc_glb : a.dq_acc_loc;
@@ -451,13 +530,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   } else if (warp == 16) {
     // ------------------------------------------------------------------ TMA producer
     setmaxnreg_dec<40>();
-    if (lane == 0) {
+    if (lane == 0 && plan.count > 0) {
       tma_prefetch_desc(&mapQ); tma_prefetch_desc(&mapDO); tma_prefetch_desc(&mapQc); tma_prefetch_desc(&mapDOc);
       mbar_expect_tx(&bar->kv_full, 2 * SM::kTileBytes);
       tma_load_4d(sK, &mapK, &bar->kv_full, 0, k0, g * (D / 64), b);
       tma_load_4d(sV, &mapV, &bar->kv_full, 0, k0, g * (D / 64), b);
       ItemCursor cur(plan, g * G);
-      for (int i = 0; i < plan.total; ++i) {
+      for (int i = 0; i < plan.count; ++i) {
         const int glb = cur.glb(), row0 = cur.tile() * kTileM, hc = cur.h * (D / 64);
         cur.next();
         const int st = i & 1;
@@ -500,8 +579,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         r_lo[q] = (valid && a.seq_bounds != nullptr) ? __ldg(&a.seq_bounds[2 * token]) : -0x40000000;
       }
     };
-    load_item();
-    for (int i = 0; i < plan.total; ++i) {
+    if (plan.count > 0) load_item();
+    for (int i = 0; i < plan.count; ++i) {
       const int s = i & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(&bar->st_empty[s], ((i >> 1) & 1) ^ 1, abort_flag))) break;
       float* st_lse = reinterpret_cast<float*>(smem + SM::kStatOff + s * SM::kStatSlot);
@@ -521,7 +600,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       if (lane == 0) { st_flags[4] = r_glb; st_flags[5] = r_row0; st_flags[6] = r_h; }
       __syncwarp();
       mbar_arrive(&bar->st_full[s]);
-      if (i + 1 < plan.total) load_item();
+      if (i + 1 < plan.count) load_item();
     }
   } else if (warp == 17) {
     // ------------------------------------------------------------------ MMA issuer
@@ -583,15 +662,15 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         tc_commit(&bar->q_empty[qs]);
         tc_commit(&bar->ds_free);
       };
-      bool ok = mbar_spin(&bar->kv_full, 0, abort_flag) && mbar_spin(&bar->q_full[0], 0, abort_flag) &&
+      bool ok = plan.count > 0 && mbar_spin(&bar->kv_full, 0, abort_flag) && mbar_spin(&bar->q_full[0], 0, abort_flag) &&
                 mbar_spin(&bar->do_full[0], 0, abort_flag);
       if (ok) {
         tc_fence_after();
         issue_S(0);
         issue_dP(0);
       }
-      for (int i = 0; ok && i < plan.total; ++i) {
-        const bool more = i + 1 < plan.total;
+      for (int i = 0; ok && i < plan.count; ++i) {
+        const bool more = i + 1 < plan.count;
         if (!mbar_spin(&bar->p_full, i & 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         issue_dV(i & 1, i == 0);
@@ -629,7 +708,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     const uint32_t s_addr = tmem + lane_base + 256 + q * 32;
     const uint32_t dp_addr = tmem + lane_base + 384 + q * 32;
     bool ok = true;
-    for (int i = 0; i < plan.total; ++i) {
+    for (int i = 0; i < plan.count; ++i) {
       const int s = i & 1;
       // this item's row statistics go to registers before the scores are waited for
       if (!__all_sync(0xffffffffu, mbar_wait(&bar->st_full[s], (i >> 1) & 1, abort_flag))) { ok = false; break; }
@@ -726,32 +805,27 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       mbar_arrive(&bar->ds_full);
     }
     // epilogue: quarters 0,1 store the two column halves of dV, quarters 2,3 those of dK
-    if (ok && __all_sync(0xffffffffu, mbar_wait(&bar->final_bar, 0, abort_flag))) {
-      tc_fence_after();
-      const bool valid = kp < a.Lk;
-      const int which = q >> 1, half = q & 1;
-      const RowStrides st = which == 0 ? a.dv_st : a.dk_st;
-      const int64_t o = b * st.b + (valid ? kp : 0) * st.t + (int64_t)g * D + half * (D / 2);
-      bf16* dst = (which == 0 ? a.dV : a.dK) + o;
-      const float mul = which == 0 ? 1.0f : a.scale;
-#pragma unroll
-      for (int c = 0; c < D / 64; ++c) {
-        uint32_t v[32];
-        tmem_ld32(tmem + lane_base + which * D + half * (D / 2) + c * 32, v);
-        tmem_ld_wait();
-        if (valid) {
-          uint4* d4 = reinterpret_cast<uint4*>(dst + c * 32);
-#pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            float f[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[8 * x + e]) * mul;
-            d4[x] = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]),
-                               pack_bf16(f[6], f[7]));
-          }
-        }
-      }
+    const bool own = plan.count > 0;      // a CTA whose share is empty issued nothing and adds nothing
+    if (own && ok) ok = __all_sync(0xffffffffu, mbar_wait(&bar->final_bar, 0, abort_flag));
+    tc_fence_after();
+    if (kSplit > 1) {
+      // The accumulators of the cluster's CTAs: quarter q of (dV | dK) belongs to CTA q * kSplit / 4, every other CTA
+      // sends it its own into a slot of the Q / dO rings, which nobody reads once all products of the cluster are done.
+      const int owner = q * kSplit / 4, me = (int)cluster_rank();
+      cluster_sync();
+      if (owner != me)
+        send_dkv<D, kSplit>(cluster_map(smem_u32(smem + SM::kQOff), owner) +
+                            dkv_slot_offset<D, kSplit>((me - owner + kSplit) % kSplit - 1, q, kr),
+                            tmem + lane_base + q * (D / 2), own);
+      cluster_sync();
+      ok = ok && owner == me;
     }
+    if (ok) store_dkv<D, kSplit>(a, smem, tmem + lane_base + q * (D / 2), own, b, g, k0 + kr, q, kr);
+  }
+  if (kSplit > 1 && warp >= kComputeWarps) {   // the other warps' part in the two barriers
+    __syncwarp();
+    cluster_sync();
+    cluster_sync();
   }
   tc_fence_before();
   __syncthreads();
@@ -868,17 +942,50 @@ int dq_final_tiles(int split, int q_pos_offset, int n_tiles) {
   return t > n_tiles ? n_tiles : (int)t;
 }
 
+template <int D, int kSplit>
+cudaError_t launch_bwd_split(const BwdArgs& a, const CUtensorMap& mapQ, const CUtensorMap& mapDO, const CUtensorMap& mapQc,
+                             const CUtensorMap& mapDOc, const CUtensorMap& mapK, const CUtensorMap& mapV, cudaStream_t s) {
+  static PerDeviceOnce once;
+  cudaError_t e = once.run([] {
+    return cudaFuncSetAttribute(bwd_kernel<D, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::kTotal);
+  });
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kSplit; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)a.kb_count * a.B * a.Hkv * kSplit);
+  cfg.blockDim = dim3(kDkvThreads);
+  cfg.dynamicSmemBytes = BwdSmem<D>::kTotal;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = kSplit > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, bwd_kernel<D, kSplit>, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, a);
+}
+
+template <int D>
+cudaError_t launch_bwd_kernel(BwdArgs a, const CUtensorMap& mapQ, const CUtensorMap& mapDO, const CUtensorMap& mapQc,
+                              const CUtensorMap& mapDOc, const CUtensorMap& mapK, const CUtensorMap& mapV, int sms,
+                              cudaStream_t s) {
+  const int64_t blocks = (int64_t)a.kb_count * a.B * a.Hkv;
+  // A cluster per key block where one CTA per block leaves SMs idle or the heaviest block sets the time.  Measured, whole
+  // backward with 1 / 2 / 4 CTAs per block at 148 SMs: 32 blocks 224 / 153 / 110 us, 64 blocks 822 / 486 / 461, 128 blocks
+  // 750 / 478 / 527 and 272 / 206 / 238, 256 blocks 1435 / 1360 / 1467 and 381 / 399 / 454, 512 blocks 1481 / 1691 / 1907.
+  const int split = 2 * blocks < sms ? 4 : 2 * blocks < 3 * sms ? 2 : 1;
+  // Below eight waves the heaviest key blocks of every head go first (two sequences of 4096 tokens, 256 blocks: 1.20 ->
+  // 0.93 ms); with more waves the tail is short and either order measures the same, so the one with less L2 traffic stays.
+  a.kb_outermost = blocks < 8 * sms;
+  return split == 1   ? launch_bwd_split<D, 1>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, s)
+         : split == 2 ? launch_bwd_split<D, 2>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, s)
+                      : launch_bwd_split<D, 4>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, s);
+}
+
 template <int D>
 cudaError_t launch_bwd(const BwdArgs& base, const CUtensorMap& mapQ, const CUtensorMap& mapDO,
                        const CUtensorMap& mapQc, const CUtensorMap& mapDOc, const CUtensorMap& mapK,
                        const CUtensorMap& mapV, const uint8_t* d_mask, cudaStream_t s) {
   const DeviceInfo* dev = device_info();
   if (dev == nullptr) return cudaErrorUnknown;
-  static PerDeviceOnce once;
-  cudaError_t e = once.run([] {
-    return cudaFuncSetAttribute(bwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::kTotal);
-  });
-  if (e != cudaSuccess) return e;
   const int n_tiles = (base.Lq + kTileM - 1) / kTileM;
   dq_zero_kernel<<<dev->sms * 8, 256, 0, s>>>(base.dq_acc_loc, base.dq_acc_glb, base.n_routed, base.B, base.Hq, n_tiles,
                                               kTileM * D);
@@ -894,8 +1001,8 @@ cudaError_t launch_bwd(const BwdArgs& base, const CUtensorMap& mapQ, const CUten
     const int kb_end = part + 1 < n_ranges ? first[part + 1] : n_kblocks;
     a.kb_begin = first[part];
     a.kb_count = kb_end - first[part];
-    bwd_kernel<D><<<(unsigned)a.kb_count * base.B * base.Hkv, kDkvThreads, BwdSmem<D>::kTotal, s>>>(
-        mapQ, mapDO, mapQc, mapDOc, mapK, mapV, a);
+    const cudaError_t e = launch_bwd_kernel<D>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, dev->sms, s);
+    if (e != cudaSuccess) return e;
     phase_events().mark(s);
     const int t1 = part + 1 < n_ranges ? dq_final_tiles(kb_end, base.q_pos_offset, n_tiles) : n_tiles;
     if (t1 > t_done)

@@ -255,7 +255,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         const int it = j - jlo, s = it & 1, sn = s ^ 1;
         const uint32_t ph = (it >> 1) & 1;
         const uint32_t phn = ((it + 1) >> 1) & 1;
-        bool v_ready = false, k_ready = false;
+        // both operand blocks of this step are waited for ahead of the probabilities: they arrive long before, and
+        // a wait between P*V and the next Q*K^T, even one already satisfied, is part of a tile's serial chain
+        if (!mbar_spin(&bar->v_full[s], ph, abort_flag)) { ok = false; break; }
+        if (j + 1 <= jhi && !mbar_spin(&bar->k_full[sn], phn, abort_flag)) { ok = false; break; }
 #pragma unroll
         for (int t = 0; t < kNumTiles; ++t) {
           if (ok && in_range(t, j)) {
@@ -263,36 +266,19 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             if (!mbar_spin(&bar->p_full[t], pc & 1, abort_flag)) { ok = false; }
             else {
               ++pc;
-              if (!v_ready) {
-                if (!mbar_spin(&bar->v_full[s], ph, abort_flag)) ok = false;
-                v_ready = true;
-              }
-              if (ok) {
-                tc_fence_after();
-                issue_pv(t, s, j > (t ? lo1 : lo0) ? 1u : 0u);
-              }
+              tc_fence_after();
+              issue_pv(t, s, j > (t ? lo1 : lo0) ? 1u : 0u);
             }
           }
           if (ok && j + 1 <= jhi && in_range(t, j + 1)) {
-            if (!k_ready) {
-              if (!mbar_spin(&bar->k_full[sn], phn, abort_flag)) ok = false;
-              k_ready = true;
-            }
-            if (ok && j + 1 == (t ? lo1 : lo0) && !mbar_spin(&bar->q_full[t], 0, abort_flag)) ok = false;
-            if (ok) {
-              tc_fence_after();
-              issue_qk(t, sn);
-            }
+            if (j + 1 == (t ? lo1 : lo0) && !mbar_spin(&bar->q_full[t], 0, abort_flag)) ok = false;
+            if (ok) issue_qk(t, sn);
           }
         }
         if (!ok) break;
         // V block j is released once both tiles' P*V have drained; K block j+1 once both Q*K^T have
-        if (!v_ready && !mbar_spin(&bar->v_full[s], ph, abort_flag)) break;
         tc_commit(&bar->v_empty[s]);
-        if (j + 1 <= jhi) {
-          if (!k_ready && !mbar_spin(&bar->k_full[sn], phn, abort_flag)) break;
-          tc_commit(&bar->k_empty[sn]);
-        }
+        if (j + 1 <= jhi) tc_commit(&bar->k_empty[sn]);
       }
       if (ok) tc_commit(&bar->o_final);
     }

@@ -54,8 +54,8 @@ struct Barriers {
   uint64_t k_full[kStages], k_empty[kStages];
   uint64_t v_full[kStages], v_empty[kStages];
   uint64_t s_full[kNumTiles];
-  uint64_t p_full[kNumTiles];
-  uint64_t o_final;
+  uint64_t p_half[kNumTiles], p_full[kNumTiles];   // P of the first 64 keys of a block / of all
+  uint64_t o_final[kNumTiles];
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -147,7 +147,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     for (int t = 0; t < kNumTiles; ++t) {
       mbar_init(&bar->q_full[t], 1);
       mbar_init(&bar->s_full[t], 1);
+      mbar_init(&bar->p_half[t], kTileM);
       mbar_init(&bar->p_full[t], kTileM);
+      mbar_init(&bar->o_final[t], 1);
     }
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&bar->k_full[s], 1);
@@ -155,7 +157,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       mbar_init(&bar->v_full[s], 1);
       mbar_init(&bar->v_empty[s], 1);
     }
-    mbar_init(&bar->o_final, 1);
     bar->abort_flag = 0;
     fence_mbar_init();
   }
@@ -230,12 +231,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         }
         tc_commit(&bar->s_full[t]);
       };
-      auto issue_pv = [&](int t, int s, uint32_t acc) {
+      auto issue_pv = [&](int t, int s, int half, uint32_t acc) {   // P*V of 64 keys
         const uint64_t vd = s ? dv1 : dv0;
-        const uint32_t d = tmem + kOCol0 + t * D, p = tmem + t * kTileN;
+        const uint32_t d = tmem + kOCol0 + t * D, p = tmem + t * kTileN + half * 64;
 #pragma unroll
-        for (int kk = 0; kk < kTileN / 16; ++kk)
-          mma_ts(d, p + (kk >> 2) * 64 + (kk & 3) * 8, vd + ((kk * 2048) >> 4), idesc_pv, kk > 0 ? 1u : acc);
+        for (int kk = 0; kk < kTileN / 32; ++kk)
+          mma_ts(d, p + kk * 8, vd + (((half * 4 + kk) * 2048) >> 4), idesc_pv, kk > 0 ? 1u : acc);
       };
       auto in_range = [&](int t, int j) { return t ? (j >= lo1 && j <= hi1) : (j >= lo0 && j <= hi0); };
 
@@ -263,11 +264,19 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         for (int t = 0; t < kNumTiles; ++t) {
           if (ok && in_range(t, j)) {
             uint32_t& pc = t ? p_cnt1 : p_cnt0;
-            if (!mbar_spin(&bar->p_full[t], pc & 1, abort_flag)) { ok = false; }
-            else {
+            if (mbar_spin(&bar->p_half[t], pc & 1, abort_flag)) {
+              tc_fence_after();
+              issue_pv(t, s, 0, j > (t ? lo1 : lo0) ? 1u : 0u);
+            } else {
+              ok = false;
+            }
+            if (ok && mbar_spin(&bar->p_full[t], pc & 1, abort_flag)) {
               ++pc;
               tc_fence_after();
-              issue_pv(t, s, j > (t ? lo1 : lo0) ? 1u : 0u);
+              issue_pv(t, s, 1, 1u);
+              if (j == (t ? hi1 : hi0)) tc_commit(&bar->o_final[t]);
+            } else {
+              ok = false;
             }
           }
           if (ok && j + 1 <= jhi && in_range(t, j + 1)) {
@@ -280,7 +289,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         tc_commit(&bar->v_empty[s]);
         if (j + 1 <= jhi) tc_commit(&bar->k_empty[sn]);
       }
-      if (ok) tc_commit(&bar->o_final);
     }
     __syncwarp();
   } else if (warp > kMmaWarp) {
@@ -358,7 +366,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         }
         const float m_eff = (m_use == -INFINITY) ? 0.f : m_use;
         const float neg_m = -m_eff;
-        // probabilities; the bf16 P of keys 64h .. 64h+63 overwrites score columns 64h .. 64h+31
+        // probabilities; the bf16 P of keys 64h .. 64h+63 overwrites score columns 64h .. 64h+31.  A quarter of the
+        // exponentials runs on the FMA pipe: ex2 takes 8 clk a warp, 1024 of the 1430 clk this took with all on the
+        // special-function unit, and it is part of the tile's serial chain S -> P -> P*V -> next S (1200 clk now; three
+        // eighths and more are slower again).  The first half of P is handed over while the second is computed.
         float2 sum2 = make_float2(0.f, 0.f);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -367,11 +378,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
           for (int e = 0; e < 16; ++e) {
             const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[c][2 * e]), __uint_as_float(v[c][2 * e + 1])),
                                         make_float2(a.scale_log2, a.scale_log2), make_float2(neg_m, neg_m));
-            const float2 p = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+            const float2 p = e % 4 == 3 ? exp2_fma2(x) : make_float2(fast_exp2(x.x), fast_exp2(x.y));
             sum2 = __fadd2_rn(sum2, p);
             pk[e] = pack_bf16(p.x, p.y);
           }
           tmem_st16(s_addr + (c >> 1) * 64 + (c & 1) * 16, pk);
+          if (c == 1) {
+            tmem_st_wait();
+            tc_fence_before();
+            mbar_arrive(&bar->p_half[t]);
+          }
         }
         l += sum2.x + sum2.y;
         tmem_st_wait();
@@ -380,7 +396,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       }
 
       // ---- epilogue: O / l, log-sum-exp, store (local) or scatter + combine (global)
-      if (ok && (n_my == 0 || __all_sync(0xffffffffu, mbar_wait(&bar->o_final, 0, abort_flag)))) {
+      if (ok && (n_my == 0 || __all_sync(0xffffffffu, mbar_wait(&bar->o_final[t], 0, abort_flag)))) {
         tc_fence_after();
         float inv_l = (l > 0.f) ? 1.0f / l : 0.f;
         float lse2 = m_use + log2f(l);   // log-sum-exp in the exp2 domain

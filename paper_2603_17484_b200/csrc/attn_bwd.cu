@@ -201,10 +201,25 @@ __device__ __forceinline__ float bf16hi_to_f32(uint32_t packed) { return __uint_
 struct ItemPlan {
   int loc_t0, loc_nt;   // first local query tile, number of local tiles
   int glb_t0, glb_nt;   // first compact tile, number of compact tiles
-  int per_head;         // loc_nt + glb_nt
-  int total;            // per_head * G
-  int first, count;     // this CTA's share [first, first + count) of them
+  int total;            // items of the key block: (loc_nt + glb_nt) * G
 };
+
+// First tile at or after t0 that CTA `rank` of kSplit takes for head hg of the group: (tile + hg) % kSplit == rank.  By tile
+// and not by position in the item list, so that more query tiles behind a sequence (padding rows) leave the sums of dK
+// and dV as they are; shifted by the head, so that the shares are even.
+template <int kSplit>
+__device__ __forceinline__ int first_tile(int t0, int hg, int rank) {
+  return kSplit == 1 ? t0 : t0 + ((rank - t0 - hg) & (kSplit - 1));
+}
+template <int kSplit>
+__device__ __forceinline__ int share_count(const ItemPlan& p, int G, int rank) {
+  if (kSplit == 1) return p.total;
+  int n = 0;
+  for (int hg = 0; hg < G; ++hg)
+    n += (max(0, p.loc_t0 + p.loc_nt - first_tile<kSplit>(p.loc_t0, hg, rank)) + kSplit - 1) / kSplit +
+         (max(0, p.glb_t0 + p.glb_nt - first_tile<kSplit>(p.glb_t0, hg, rank)) + kSplit - 1) / kSplit;
+  return n;
+}
 
 __device__ __forceinline__ ItemPlan make_plan(const BwdArgs& a, int b, int k0, int span = kTileN) {
   ItemPlan p;
@@ -232,20 +247,40 @@ __device__ __forceinline__ ItemPlan make_plan(const BwdArgs& a, int b, int k0, i
     if (c_min >= c_end) { p.glb_t0 = 0; p.glb_nt = 0; }
     else { p.glb_t0 = c_min / kTileM; p.glb_nt = (c_end - 1) / kTileM - p.glb_t0 + 1; }
   }
-  p.per_head = p.loc_nt + p.glb_nt;
-  p.total = p.per_head * (a.Hq / a.Hkv);
+  p.total = (p.loc_nt + p.glb_nt) * (a.Hq / a.Hkv);
   return p;
 }
 
 // Walks the items of a CTA in order without divisions: (head, local/compact, tile).
+template <int kSplit>
 struct ItemCursor {
-  int h, r, per_head, loc_nt, loc_t0, glb_t0;
-  __device__ __forceinline__ ItemCursor(const ItemPlan& p, int h0)
-      : h(h0 + p.first / p.per_head), r(p.first % p.per_head), per_head(p.per_head), loc_nt(p.loc_nt), loc_t0(p.loc_t0),
-        glb_t0(p.glb_t0) {}
+  int hg, t, glb_part, loc_end, glb_end, loc_t0, glb_t0, h0, rank;
+  __device__ __forceinline__ ItemCursor(const ItemPlan& p, int h0_, int rank_)
+      : hg(-1), t(0), glb_part(1), loc_end(p.loc_t0 + p.loc_nt), glb_end(p.glb_nt > 0 ? p.glb_t0 + p.glb_nt : 0),
+        loc_t0(p.loc_t0), glb_t0(p.glb_t0), h0(h0_), rank(rank_) {
+    t = glb_end;
+    settle();
+  }
+  __device__ __forceinline__ int h() const { return h0 + hg; }
+  __device__ __forceinline__ int glb() const { return glb_part; }
+  __device__ __forceinline__ int tile() const { return t; }
+  __device__ __forceinline__ void settle() {    // to the next tile of the share: a head may hold none, kSplit heads do not
+    for (int n = 0; n <= kSplit && t >= (glb_part ? glb_end : loc_end);) {
+      if (glb_part) { glb_part = 0; ++hg; t = first_tile<kSplit>(loc_t0, hg, rank); ++n; }
+      else { glb_part = 1; t = first_tile<kSplit>(glb_t0, hg, rank); }
+    }
+  }
+  __device__ __forceinline__ void next() { t += kSplit; settle(); }
+};
+template <>
+struct ItemCursor<1> {
+  int head, r, per_head, loc_nt, loc_t0, glb_t0;
+  __device__ __forceinline__ ItemCursor(const ItemPlan& p, int h0, int)
+      : head(h0), r(0), per_head(p.loc_nt + p.glb_nt), loc_nt(p.loc_nt), loc_t0(p.loc_t0), glb_t0(p.glb_t0) {}
+  __device__ __forceinline__ int h() const { return head; }
   __device__ __forceinline__ int glb() const { return r >= loc_nt; }
   __device__ __forceinline__ int tile() const { return r < loc_nt ? loc_t0 + r : glb_t0 + (r - loc_nt); }
-  __device__ __forceinline__ void next() { if (++r == per_head) { r = 0; ++h; } }
+  __device__ __forceinline__ void next() { if (++r == per_head) { r = 0; ++head; } }
 };
 
 // ================================================================================================
@@ -426,9 +461,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   const int g = rest / a.B;
   const int G = a.Hq / a.Hkv;
   const int k0 = j * kTileN;
-  ItemPlan plan = make_plan(a, b, k0);
-  plan.first = (int)((int64_t)plan.total * rank / kSplit);
-  plan.count = (int)((int64_t)plan.total * (rank + 1) / kSplit) - plan.first;
+  const ItemPlan plan = make_plan(a, b, k0);
+  const int count = share_count<kSplit>(plan, G, rank);      // this CTA's items
   const int n_c = a.skip_global ? 0 : a.n_routed[b];   // the routing arrays may be NULL when the global part is skipped
 
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -500,9 +534,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     const uint32_t lane_base = static_cast<uint32_t>(grp * 32) << 16;
     const int n_tiles = (a.Lq + kTileM - 1) / kTileM;
     constexpr int kChunks = D / 32;     // 32-column TMEM loads of the whole tile; this warp takes half of them
-    ItemCursor cur(plan, g * G);
-    for (int i = 0; i < plan.count; ++i) {
-      const int h = cur.h, glb = cur.glb(), tile = cur.tile();
+    ItemCursor<kSplit> cur(plan, g * G, rank);
+    for (int i = 0; i < count; ++i) {
+      const int h = cur.h(), glb = cur.glb(), tile = cur.tile();
       cur.next();
       float* acc = glb ? a.dq_acc_glb : a.dq_acc_loc;
       const bool item_ok = dbg_in_range(tile >= 0 && tile < n_tiles && h >= 0 && h < a.Hq && acc != nullptr, a.status);
@@ -530,14 +564,14 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   } else if (warp == 16) {
     // ------------------------------------------------------------------ TMA producer
     setmaxnreg_dec<40>();
-    if (lane == 0 && plan.count > 0) {
+    if (lane == 0 && count > 0) {
       tma_prefetch_desc(&mapQ); tma_prefetch_desc(&mapDO); tma_prefetch_desc(&mapQc); tma_prefetch_desc(&mapDOc);
       mbar_expect_tx(&bar->kv_full, 2 * SM::kTileBytes);
       tma_load_4d(sK, &mapK, &bar->kv_full, 0, k0, g * (D / 64), b);
       tma_load_4d(sV, &mapV, &bar->kv_full, 0, k0, g * (D / 64), b);
-      ItemCursor cur(plan, g * G);
-      for (int i = 0; i < plan.count; ++i) {
-        const int glb = cur.glb(), row0 = cur.tile() * kTileM, hc = cur.h * (D / 64);
+      ItemCursor<kSplit> cur(plan, g * G, rank);
+      for (int i = 0; i < count; ++i) {
+        const int glb = cur.glb(), row0 = cur.tile() * kTileM, hc = cur.h() * (D / 64);
         cur.next();
         const int st = i & 1;
         const uint32_t ph = ((i >> 1) & 1) ^ 1;
@@ -557,9 +591,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     // The global loads of item i+1 are issued before waiting for its slot, so their latency is hidden.
     float r_lse[4], r_delta[4];
     int r_pos[4], r_lo[4], r_glb = 0, r_row0 = 0, r_h = 0;   // r_lo: first token of the row's sequence (packed batches)
-    ItemCursor cur(plan, g * G);
+    ItemCursor<kSplit> cur(plan, g * G, rank);
     auto load_item = [&]() {
-      const int h = cur.h, glb = cur.glb(), row0 = cur.tile() * kTileM;
+      const int h = cur.h(), glb = cur.glb(), row0 = cur.tile() * kTileM;
       cur.next();
       const int n_rows = glb ? n_c : a.Lq;
       const float* lse = glb ? a.lse_glb : a.lse_loc;
@@ -579,8 +613,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         r_lo[q] = (valid && a.seq_bounds != nullptr) ? __ldg(&a.seq_bounds[2 * token]) : -0x40000000;
       }
     };
-    if (plan.count > 0) load_item();
-    for (int i = 0; i < plan.count; ++i) {
+    if (count > 0) load_item();
+    for (int i = 0; i < count; ++i) {
       const int s = i & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(&bar->st_empty[s], ((i >> 1) & 1) ^ 1, abort_flag))) break;
       float* st_lse = reinterpret_cast<float*>(smem + SM::kStatOff + s * SM::kStatSlot);
@@ -600,7 +634,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       if (lane == 0) { st_flags[4] = r_glb; st_flags[5] = r_row0; st_flags[6] = r_h; }
       __syncwarp();
       mbar_arrive(&bar->st_full[s]);
-      if (i + 1 < plan.count) load_item();
+      if (i + 1 < count) load_item();
     }
   } else if (warp == 17) {
     // ------------------------------------------------------------------ MMA issuer
@@ -662,15 +696,15 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         tc_commit(&bar->q_empty[qs]);
         tc_commit(&bar->ds_free);
       };
-      bool ok = plan.count > 0 && mbar_spin(&bar->kv_full, 0, abort_flag) && mbar_spin(&bar->q_full[0], 0, abort_flag) &&
+      bool ok = count > 0 && mbar_spin(&bar->kv_full, 0, abort_flag) && mbar_spin(&bar->q_full[0], 0, abort_flag) &&
                 mbar_spin(&bar->do_full[0], 0, abort_flag);
       if (ok) {
         tc_fence_after();
         issue_S(0);
         issue_dP(0);
       }
-      for (int i = 0; ok && i < plan.count; ++i) {
-        const bool more = i + 1 < plan.count;
+      for (int i = 0; ok && i < count; ++i) {
+        const bool more = i + 1 < count;
         if (!mbar_spin(&bar->p_full, i & 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         issue_dV(i & 1, i == 0);
@@ -708,7 +742,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     const uint32_t s_addr = tmem + lane_base + 256 + q * 32;
     const uint32_t dp_addr = tmem + lane_base + 384 + q * 32;
     bool ok = true;
-    for (int i = 0; i < plan.count; ++i) {
+    for (int i = 0; i < count; ++i) {
       const int s = i & 1;
       // this item's row statistics go to registers before the scores are waited for
       if (!__all_sync(0xffffffffu, mbar_wait(&bar->st_full[s], (i >> 1) & 1, abort_flag))) { ok = false; break; }
@@ -805,7 +839,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       mbar_arrive(&bar->ds_full);
     }
     // epilogue: quarters 0,1 store the two column halves of dV, quarters 2,3 those of dK
-    const bool own = plan.count > 0;      // a CTA whose share is empty issued nothing and adds nothing
+    const bool own = count > 0;      // a CTA whose share is empty issued nothing and adds nothing
     if (own && ok) ok = __all_sync(0xffffffffu, mbar_wait(&bar->final_bar, 0, abort_flag));
     tc_fence_after();
     if (kSplit > 1) {
@@ -967,7 +1001,8 @@ template <int D>
 cudaError_t launch_bwd_kernel(BwdArgs a, const CUtensorMap& mapQ, const CUtensorMap& mapDO, const CUtensorMap& mapQc,
                               const CUtensorMap& mapDOc, const CUtensorMap& mapK, const CUtensorMap& mapV, int sms,
                               cudaStream_t s) {
-  const int64_t blocks = (int64_t)a.kb_count * a.B * a.Hkv;
+  // (of the whole sequence, also when the launch is one of several key-block ranges: the results stay the same)
+  const int64_t blocks = (int64_t)((a.Lk + kTileN - 1) / kTileN) * a.B * a.Hkv;
   // A cluster per key block where one CTA per block leaves SMs idle or the heaviest block sets the time.  Measured, whole
   // backward with 1 / 2 / 4 CTAs per block at 148 SMs: 32 blocks 224 / 153 / 110 us, 64 blocks 822 / 486 / 461, 128 blocks
   // 750 / 478 / 527 and 272 / 206 / 238, 256 blocks 1435 / 1360 / 1467 and 381 / 399 / 454, 512 blocks 1481 / 1691 / 1907.

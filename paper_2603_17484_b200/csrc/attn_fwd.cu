@@ -56,6 +56,7 @@ struct Barriers {
   uint64_t s_full[kNumTiles];
   uint64_t p_half[kNumTiles], p_full[kNumTiles];   // P of the first 64 keys of a block / of all
   uint64_t o_final[kNumTiles];
+  uint64_t staged[kNumTiles];     // the tile's output rows are in shared memory
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -70,7 +71,8 @@ struct TileRange {
 template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-                const __grid_constant__ CUtensorMap mapV, const FwdArgs a) {
+                const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapOut,
+                const __grid_constant__ CUtensorMap mapOut2, const FwdArgs a) {
   using SM = FwdSmem<D>;
   constexpr int kKSteps = D / 16;      // MMA k-steps of Q*K^T
   constexpr int kOCol0 = 2 * kTileN;   // first TMEM column of the O accumulators
@@ -150,6 +152,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       mbar_init(&bar->p_half[t], kTileM);
       mbar_init(&bar->p_full[t], kTileM);
       mbar_init(&bar->o_final[t], 1);
+      mbar_init(&bar->staged[t], kTileM);
     }
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&bar->k_full[s], 1);
@@ -417,62 +420,92 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
           const float lse = lse2 * 0.6931471805599453f;
           a.lse[((int64_t)b * a.Hq + h) * a.Lq + row] = lse;
         }
-        bf16* dst1 = nullptr;   // row-indexed destination (s rows, or compact a rows)
-        bf16* dst2 = nullptr;   // position-indexed destination
-        if (valid && dbg_in_range(row >= 0 && row < a.Lq && seq_row >= 0 && seq_row < a.Lq, a.status)) {
-          if (a.out) dst1 = a.out + b * a.out_st.b + row * a.out_st.t + (int64_t)h * D;
-          if (a.out2 && (a.combine_mask == nullptr || a.combine_mask[(int64_t)b * a.Lq + seq_row]))
-            dst2 = a.out2 + b * a.out2_st.b + seq_row * a.out2_st.t + (int64_t)h * D;
-        }
-        const bool accumulate = a.global_mode && a.accumulate_into_out2;
+        if (!a.global_mode) {
+          // A tile of consecutive rows leaves through its Q buffer (free once its last product is done) with one TMA store
+          // per destination.  A store per thread and row, 32 lines an instruction, took 4900 clk a tile, of 108000 for
+          // all of a CTA at W = 4096; rows gathered from shared memory by plain stores took as long.
 #pragma unroll 1
-        for (int c = 0; c < D / 32; ++c) {
-          uint32_t o[32];
-          if (n_my > 0) {
+          for (int c = 0; c < D / 32; ++c) {
+            uint32_t o[32];
             tmem_ld32(o_addr + c * 32, o);
             tmem_ld_wait();
-          } else {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] = 0u;    // no key before the window: the accumulator was never written
-          }
-          float f[32];
-#pragma unroll
-          for (int e = 0; e < 32; ++e) f[e] = __uint_as_float(o[e]) * inv_l;
-          if (shared && dst2) {
-            const uint4* s4 = reinterpret_cast<const uint4*>(dst2 + c * 32);   // s_t, written by the local pass
+            const uint32_t dst = smem_u32(sQ + t * SM::kQTileBytes) + (c >> 1) * SM::kBoxBytes + r * 128;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-              const uint4 old = s4[q];
-              const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
+              uint32_t w[4];
 #pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                f[8 * q + 2 * k] = fmaf(c_loc, __uint_as_float(ow[k] << 16), f[8 * q + 2 * k]);
-                f[8 * q + 2 * k + 1] = fmaf(c_loc, __uint_as_float(ow[k] & 0xffff0000u), f[8 * q + 2 * k + 1]);
-              }
+              for (int k = 0; k < 4; ++k)
+                w[k] = pack_bf16(__uint_as_float(o[8 * q + 2 * k]) * inv_l, __uint_as_float(o[8 * q + 2 * k + 1]) * inv_l);
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + ((((c & 1) * 4 + q) ^ (r & 7)) << 4)),
+                           "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
             }
           }
-          if (dst1) {
-            uint4* d4 = reinterpret_cast<uint4*>(dst1 + c * 32);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              d4[q] = make_uint4(pack_bf16(f[8 * q], f[8 * q + 1]), pack_bf16(f[8 * q + 2], f[8 * q + 3]),
-                                 pack_bf16(f[8 * q + 4], f[8 * q + 5]), pack_bf16(f[8 * q + 6], f[8 * q + 7]));
+          fence_async_smem();
+          mbar_arrive(&bar->staged[t]);
+          if (r == 0 && mbar_wait(&bar->staged[t], 0, abort_flag)) {
+            tma_store_4d(&mapOut, sQ + t * SM::kQTileBytes, 0, row0 + t * kTileM, h * (D / 64), b);
+            if (a.out2) tma_store_4d(&mapOut2, sQ + t * SM::kQTileBytes, 0, row0 + t * kTileM, h * (D / 64), b);
+            tma_store_commit();
+            tma_store_wait_read();
           }
-          if (dst2) {
-            uint4* d4 = reinterpret_cast<uint4*>(dst2 + c * 32);
+        } else {
+          bf16* dst1 = nullptr;   // row-indexed destination (s rows, or compact a rows)
+          bf16* dst2 = nullptr;   // position-indexed destination
+          if (valid && dbg_in_range(row >= 0 && row < a.Lq && seq_row >= 0 && seq_row < a.Lq, a.status)) {
+            if (a.out) dst1 = a.out + b * a.out_st.b + row * a.out_st.t + (int64_t)h * D;
+            if (a.out2 && (a.combine_mask == nullptr || a.combine_mask[(int64_t)b * a.Lq + seq_row]))
+              dst2 = a.out2 + b * a.out2_st.b + seq_row * a.out2_st.t + (int64_t)h * D;
+          }
+          const bool accumulate = a.global_mode && a.accumulate_into_out2;
+#pragma unroll 1
+          for (int c = 0; c < D / 32; ++c) {
+            uint32_t o[32];
+            if (n_my > 0) {
+              tmem_ld32(o_addr + c * 32, o);
+              tmem_ld_wait();
+            } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              if (accumulate) {
-                const uint4 old = d4[q];
+              for (int e = 0; e < 32; ++e) o[e] = 0u;    // no key before the window: the accumulator was never written
+            }
+            float f[32];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) f[e] = __uint_as_float(o[e]) * inv_l;
+            if (shared && dst2) {
+              const uint4* s4 = reinterpret_cast<const uint4*>(dst2 + c * 32);   // s_t, written by the local pass
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const uint4 old = s4[q];
                 const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                  f[8 * q + 2 * k] += __uint_as_float(ow[k] << 16);
-                  f[8 * q + 2 * k + 1] += __uint_as_float(ow[k] & 0xffff0000u);
+                  f[8 * q + 2 * k] = fmaf(c_loc, __uint_as_float(ow[k] << 16), f[8 * q + 2 * k]);
+                  f[8 * q + 2 * k + 1] = fmaf(c_loc, __uint_as_float(ow[k] & 0xffff0000u), f[8 * q + 2 * k + 1]);
                 }
               }
-              d4[q] = make_uint4(pack_bf16(f[8 * q], f[8 * q + 1]), pack_bf16(f[8 * q + 2], f[8 * q + 3]),
-                                 pack_bf16(f[8 * q + 4], f[8 * q + 5]), pack_bf16(f[8 * q + 6], f[8 * q + 7]));
+            }
+            if (dst1) {
+              uint4* d4 = reinterpret_cast<uint4*>(dst1 + c * 32);
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                d4[q] = make_uint4(pack_bf16(f[8 * q], f[8 * q + 1]), pack_bf16(f[8 * q + 2], f[8 * q + 3]),
+                                   pack_bf16(f[8 * q + 4], f[8 * q + 5]), pack_bf16(f[8 * q + 6], f[8 * q + 7]));
+            }
+            if (dst2) {
+              uint4* d4 = reinterpret_cast<uint4*>(dst2 + c * 32);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                if (accumulate) {
+                  const uint4 old = d4[q];
+                  const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
+#pragma unroll
+                  for (int k = 0; k < 4; ++k) {
+                    f[8 * q + 2 * k] += __uint_as_float(ow[k] << 16);
+                    f[8 * q + 2 * k + 1] += __uint_as_float(ow[k] & 0xffff0000u);
+                  }
+                }
+                d4[q] = make_uint4(pack_bf16(f[8 * q], f[8 * q + 1]), pack_bf16(f[8 * q + 2], f[8 * q + 3]),
+                                   pack_bf16(f[8 * q + 4], f[8 * q + 5]), pack_bf16(f[8 * q + 6], f[8 * q + 7]));
+              }
             }
           }
         }
@@ -496,7 +529,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 }  // namespace
 
 cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUtensorMap& mapK,
-                            const CUtensorMap& mapV, cudaStream_t stream) {
+                            const CUtensorMap& mapV, const CUtensorMap& mapOut, const CUtensorMap& mapOut2,
+                            cudaStream_t stream) {
   const unsigned grid = (unsigned)(a.pair_end - a.pair_begin) * a.Hq * a.B;
   if (a.pair_end <= a.pair_begin) return cudaSuccess;
   cudaError_t e;
@@ -506,14 +540,14 @@ cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUt
       return cudaFuncSetAttribute(attn_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::kTotal);
     });
     if (e != cudaSuccess) return e;
-    attn_fwd_kernel<128><<<grid, kFwdThreads, FwdSmem<128>::kTotal, stream>>>(mapQ, mapK, mapV, a);
+    attn_fwd_kernel<128><<<grid, kFwdThreads, FwdSmem<128>::kTotal, stream>>>(mapQ, mapK, mapV, mapOut, mapOut2, a);
   } else {
     static PerDeviceOnce once;
     e = once.run([] {
       return cudaFuncSetAttribute(attn_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::kTotal);
     });
     if (e != cudaSuccess) return e;
-    attn_fwd_kernel<64><<<grid, kFwdThreads, FwdSmem<64>::kTotal, stream>>>(mapQ, mapK, mapV, a);
+    attn_fwd_kernel<64><<<grid, kFwdThreads, FwdSmem<64>::kTotal, stream>>>(mapQ, mapK, mapV, mapOut, mapOut2, a);
   }
   return cudaGetLastError();
 }

@@ -345,7 +345,12 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
     a.lse = lse_loc;
     a.pair_begin = pair_begin;
     a.pair_end = pair_end;
-    if (launch_attn_fwd(a, mapQ, mapK, mapV, s) != cudaSuccess) return L2A_ERR_CUDA;
+    CUtensorMap mapOut, mapOut2;
+    if (!encode_rows_map(&mapOut, a.out, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, a.out_st.b, a.out_st.t)) return L2A_ERR_CUDA;
+    mapOut2 = mapOut;
+    if (a.out2 && !encode_rows_map(&mapOut2, a.out2, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, os.b, os.t))
+      return L2A_ERR_CUDA;
+    if (launch_attn_fwd(a, mapQ, mapK, mapV, mapOut, mapOut2, s) != cudaSuccess) return L2A_ERR_CUDA;
     a.pair_begin = 0;
     a.pair_end = n_pairs;
   } else if (skip_local) {
@@ -372,7 +377,7 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
       a.all_rows = 1;
       a.combine_mask = d_mask;
     }
-    if (launch_attn_fwd(a, force_all ? mapQ : mapQc, mapK, mapV, s) != cudaSuccess) return L2A_ERR_CUDA;
+    if (launch_attn_fwd(a, force_all ? mapQ : mapQc, mapK, mapV, mapK, mapK, s) != cudaSuccess) return L2A_ERR_CUDA;
   }
   pe.mark(s);
   return L2A_OK;

@@ -165,7 +165,8 @@ struct PhaseEvents {
 };
 PhaseEvents& phase_events();  // defined with the backward
 
-cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUtensorMap& mapK,
-                            const CUtensorMap& mapV, cudaStream_t stream);
+// mapOut / mapOut2: out and out2 as store targets in 128-row tiles; used by the local mode only
+cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUtensorMap& mapK, const CUtensorMap& mapV,
+                            const CUtensorMap& mapOut, const CUtensorMap& mapOut2, cudaStream_t stream);
 
 }  // namespace l2a

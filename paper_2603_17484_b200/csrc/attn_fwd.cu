@@ -19,6 +19,8 @@
 // While one tile's soft-max runs on the CUDA cores, the tensor core works on the other tile.
 // The online soft-max follows Algorithm 1 (running max m, running sum l, rescaled accumulator),
 // in the exp2 domain, with the rescale skipped while the maximum grows by less than 2^8.
+#include <algorithm>
+
 #include "l2a_common.cuh"
 #include "sm100_prims.cuh"
 
@@ -59,6 +61,7 @@ struct Barriers {
   uint64_t staged[kNumTiles];     // the tile's output rows are in shared memory
   uint32_t tmem_base;
   int abort_flag;
+  int last;       // this CTA finished last of its group's key splits
 };
 
 struct TileRange {
@@ -78,15 +81,29 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   constexpr int kOCol0 = 2 * kTileN;   // first TMEM column of the O accumulators
 
   // ---- work item: heaviest first (largest row index first), heads fastest for K/V reuse in L2
-  const int h = blockIdx.x % a.Hq;
-  const int rest = blockIdx.x / a.Hq;
-  const int b = rest % a.B;
-  const int pi = a.pair_end - 1 - rest / a.B;
-  const int g = h / (a.Hq / a.Hkv);
   const bool compact = a.global_mode && !a.all_rows;           // rows are compact indices into q_idx
+  int item = blockIdx.x, split = 0, n_split = 1, pi;
+  if (!a.global_mode) dependents_release();                    // the global pass may fill SMs as this one drains
+  if (compact) {
+    // the launch covers every row that could be routed; the groups that exist come first
+    int most = 0;
+    for (int i = threadIdx.x & 31; i < a.B; i += 32) most = max(most, a.n_routed[i]);
+    most = __reduce_max_sync(0xffffffffu, most);
+    const int64_t groups = (int64_t)((most + kRowsPerCta - 1) / kRowsPerCta) * a.Hq * a.B;
+    if (a.part != nullptr && groups > 0 && groups < kSplitGroups) n_split = min(kMaxKeySplit, kSplitItems / (int)groups);
+    if (item >= groups * n_split) { dependency_wait(); return; }
+    split = item % n_split;
+    item /= n_split;
+  }
+  const int group = item;
+  const int h = item % a.Hq;
+  const int rest = item / a.Hq;
+  const int b = rest % a.B;
+  const int g = h / (a.Hq / a.Hkv);
   const int n_rows = compact ? a.n_routed[b] : a.Lq;           // valid (compact) rows of this batch entry
+  pi = (compact ? (n_rows + kRowsPerCta - 1) / kRowsPerCta : a.pair_end) - 1 - rest / a.B;
   const int row0 = pi * kRowsPerCta;
-  if (row0 >= n_rows) return;
+  if (pi < 0 || row0 >= n_rows) { dependency_wait(); return; }
 
   const int32_t* q_idx_b = a.q_idx + (int64_t)b * a.Lq;
   const int w_eff = a.global_mode ? 0x3fffffff : a.window;
@@ -98,7 +115,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     // launches restricted to a row range take the groups whose last row falls into it: every group exactly once
     const int c_last = min(row0 + kRowsPerCta, n_rows) - 1;
     const int t_last = compact ? q_idx_b[c_last] : c_last;
-    if (t_last < a.row_begin || t_last >= a.row_end) return;
+    if (t_last < a.row_begin || t_last >= a.row_end) { dependency_wait(); return; }
   }
 
   TileRange tr[kNumTiles];
@@ -132,6 +149,20 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     } else {
       tr[t].min_pos = tr[t].max_pos = tr[t].max_lo = 0;
       tr[t].lo = 1; tr[t].hi = 0;
+    }
+  }
+
+  // this item's part of the group's key blocks
+  n_split = max(1, min(n_split, (jhi - jlo + 1) / kMinSplitBlocks));
+  if (split >= n_split) { dependency_wait(); return; }
+  if (n_split > 1) {
+    const int n = jhi - jlo + 1, first = jlo;
+    jlo = first + n * split / n_split;
+    jhi = first + n * (split + 1) / n_split - 1;
+#pragma unroll
+    for (int t = 0; t < kNumTiles; ++t) {
+      tr[t].lo = max(tr[t].lo, jlo);
+      tr[t].hi = min(tr[t].hi, jhi);
     }
   }
 
@@ -172,6 +203,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem = bar->tmem_base;
   if (tmem != 0) {
+    dependency_wait();
     // all 512 columns were requested, so the allocation must start at column 0; the MMA warp relies on it to
     // keep its TMEM operand addresses compile-time constants
     __syncthreads();
@@ -305,6 +337,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     const uint32_t s_addr = tmem + lane_base + t * kTileN;        // this row's 128 score columns
     const uint32_t o_addr = tmem + lane_base + kOCol0 + t * D;    // its D accumulator columns
     const TileRange my = t ? tr[1] : tr[0];
+    float m_use = -INFINITY;   // reference maximum, exp2 domain
+    float l = 0.f;             // row sum
+    bool ok = true;
+    const int n_my = my.active ? my.hi - my.lo + 1 : 0;
     if (my.active) {
       const int row = row0 + t * kTileM + r;           // sequence row (local) or compact row (global)
       const bool valid = row < n_rows;
@@ -312,10 +348,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       const int pos = valid ? seq_row + a.q_pos_offset - vis_shift : -1;   // largest visible key position
       int pos_lo = valid ? (pos - w_eff) : 0x7fffffff;                     // smallest visible key position
       if (valid && a.seq_bounds != nullptr) pos_lo = max(pos_lo, a.seq_bounds[2 * seq_row]);
-      float m_use = -INFINITY;   // reference maximum, exp2 domain
-      float l = 0.f;             // row sum
-      bool ok = true;
-      const int n_my = my.hi - my.lo + 1;
 
       for (int i = 0; i < n_my; ++i) {
         const int j = my.lo + i;
@@ -398,9 +430,54 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         mbar_arrive(&bar->p_full[t]);
       }
 
+      if (ok && n_my > 0) ok = __all_sync(0xffffffffu, mbar_wait(&bar->o_final[t], 0, abort_flag));
+      tc_fence_after();
+    }
+    const float* parts = nullptr;      // this row's slots, set in the CTA that combines them
+    if (n_split > 1) {
+      // Split key range: the rows go to this item's slot unnormalised, 16-byte pieces 128 rows apart; the CTA that
+      // finishes last combines the slots of the group.
+      constexpr size_t kSlot = kRowsPerCta * (D + 2);
+      float* slot = a.part + (size_t)blockIdx.x * kSlot + t * kTileM * (D + 2);
+      if (my.active) {
+#pragma unroll 1
+        for (int c = 0; n_my > 0 && c < D / 32; ++c) {
+          uint32_t o[32];
+          tmem_ld32(o_addr + c * 32, o);
+          tmem_ld_wait();
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+            *reinterpret_cast<uint4*>(slot + ((c * 8 + x) * kTileM + r) * 4) =
+                make_uint4(o[4 * x], o[4 * x + 1], o[4 * x + 2], o[4 * x + 3]);
+        }
+        slot[kTileM * D + r] = m_use;
+        slot[kTileM * (D + 1) + r] = n_my > 0 ? l : 0.f;
+      }
+      __threadfence();
+      named_barrier(1, kSoftmaxWarps * 32);      // (reached by every soft-max warp, also after a wait that ran out)
+      if (tid == 0) bar->last = atomicAdd(&a.part_count[group], 1) == n_split - 1;
+      named_barrier(1, kSoftmaxWarps * 32);
+      ok = ok && bar->last;
+      __threadfence();
+      if (ok && my.active) {
+        parts = a.part + (size_t)(blockIdx.x - split) * kSlot + t * kTileM * (D + 2) + r;
+        m_use = -INFINITY;
+        for (int s = 0; s < n_split; ++s)
+          if (__ldcg(parts + s * kSlot + kTileM * (D + 1)) != 0.f) m_use = fmaxf(m_use, __ldcg(parts + s * kSlot + kTileM * D));
+        l = 0.f;
+        for (int s = 0; s < n_split; ++s) {
+          const float ls = __ldcg(parts + s * kSlot + kTileM * (D + 1));
+          if (ls != 0.f) l += ls * fast_exp2(__ldcg(parts + s * kSlot + kTileM * D) - m_use);
+        }
+      }
+    }
+    if (my.active) {
       // ---- epilogue: O / l, log-sum-exp, store (local) or scatter + combine (global)
-      if (ok && (n_my == 0 || __all_sync(0xffffffffu, mbar_wait(&bar->o_final[t], 0, abort_flag)))) {
-        tc_fence_after();
+      if (a.global_mode) dependency_wait();      // out2 and lse_loc are the local pass's results
+      const int row = row0 + t * kTileM + r;
+      const bool valid = row < n_rows;
+      const int seq_row = valid ? (compact ? q_idx_b[row] : row) : -1;
+      if (ok) {
         float inv_l = (l > 0.f) ? 1.0f / l : 0.f;
         float lse2 = m_use + log2f(l);   // log-sum-exp in the exp2 domain
         float c_loc = 0.f;               // shared-window mode: weight of the local result s_t in a_t
@@ -460,12 +537,28 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 #pragma unroll 1
           for (int c = 0; c < D / 32; ++c) {
             uint32_t o[32];
-            if (n_my > 0) {
+            if (n_my > 0 && parts == nullptr) {
               tmem_ld32(o_addr + c * 32, o);
               tmem_ld_wait();
             } else {
 #pragma unroll
               for (int e = 0; e < 32; ++e) o[e] = 0u;    // no key before the window: the accumulator was never written
+            }
+            if (parts != nullptr) {
+              constexpr size_t kSlot = kRowsPerCta * (D + 2);
+              for (int s = 0; s < n_split; ++s) {
+                const float* p = parts + s * kSlot;
+                if (__ldcg(p + kTileM * (D + 1)) == 0.f) continue;      // no visible key in that part: nothing was written
+                const float w = fast_exp2(__ldcg(p + kTileM * D) - m_use);
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                  const float4 v = __ldcg(reinterpret_cast<const float4*>(p - r + ((c * 8 + x) * kTileM + r) * 4));
+                  o[4 * x] = __float_as_uint(fmaf(w, v.x, __uint_as_float(o[4 * x])));
+                  o[4 * x + 1] = __float_as_uint(fmaf(w, v.y, __uint_as_float(o[4 * x + 1])));
+                  o[4 * x + 2] = __float_as_uint(fmaf(w, v.z, __uint_as_float(o[4 * x + 2])));
+                  o[4 * x + 3] = __float_as_uint(fmaf(w, v.w, __uint_as_float(o[4 * x + 3])));
+                }
+              }
             }
             float f[32];
 #pragma unroll
@@ -515,6 +608,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 
   // ---- teardown
   tc_fence_before();
+  dependency_wait();       // this grid must not count as finished before the one it overlaps with
   __syncthreads();
   if (bar->abort_flag) {
     // a bounded wait ran out: give copies still in flight time to land before shared memory is released
@@ -531,8 +625,18 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUtensorMap& mapK,
                             const CUtensorMap& mapV, const CUtensorMap& mapOut, const CUtensorMap& mapOut2,
                             cudaStream_t stream) {
-  const unsigned grid = (unsigned)(a.pair_end - a.pair_begin) * a.Hq * a.B;
   if (a.pair_end <= a.pair_begin) return cudaSuccess;
+  int64_t grid = (int64_t)(a.pair_end - a.pair_begin) * a.Hq * a.B;
+  if (a.part != nullptr && grid < kSplitItems) grid = std::min<int64_t>(grid * kMaxKeySplit, kSplitItems);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kFwdThreads);
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = a.overlap ? 1 : 0;
   cudaError_t e;
   if (a.D == 128) {
     static PerDeviceOnce once;
@@ -540,16 +644,17 @@ cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUt
       return cudaFuncSetAttribute(attn_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::kTotal);
     });
     if (e != cudaSuccess) return e;
-    attn_fwd_kernel<128><<<grid, kFwdThreads, FwdSmem<128>::kTotal, stream>>>(mapQ, mapK, mapV, mapOut, mapOut2, a);
+    cfg.dynamicSmemBytes = FwdSmem<128>::kTotal;
+    return cudaLaunchKernelEx(&cfg, attn_fwd_kernel<128>, mapQ, mapK, mapV, mapOut, mapOut2, a);
   } else {
     static PerDeviceOnce once;
     e = once.run([] {
       return cudaFuncSetAttribute(attn_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::kTotal);
     });
     if (e != cudaSuccess) return e;
-    attn_fwd_kernel<64><<<grid, kFwdThreads, FwdSmem<64>::kTotal, stream>>>(mapQ, mapK, mapV, mapOut, mapOut2, a);
+    cfg.dynamicSmemBytes = FwdSmem<64>::kTotal;
+    return cudaLaunchKernelEx(&cfg, attn_fwd_kernel<64>, mapQ, mapK, mapV, mapOut, mapOut2, a);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace l2a

@@ -53,7 +53,17 @@ size_t route_ws_size(const l2a_params* p) {
   return kWsHeaderBytes + align_up((size_t)p->B * nblocks * sizeof(int32_t), 256);
 }
 size_t qrows_bytes(const l2a_params* p) { return align_up((size_t)p->B * p->Lq * p->Hq * p->D * sizeof(bf16), 256); }
-size_t fwd_ws_size(const l2a_params* p) { return kWsHeaderBytes + qrows_bytes(p); }
+// forward workspace: header, compacted queries, then the slots and counters of split key ranges
+int group_count(const l2a_params* p) {
+  const int64_t n = (int64_t)ceil_div(p->Lq, kRowsPerCta) * p->Hq * p->B;
+  return n < kSplitGroups ? (int)n : kSplitGroups;     // launches with more groups are not split
+}
+size_t part_bytes(const l2a_params* p) {
+  return align_up(split_slots(group_count(p)) * split_slot_floats(p->D) * sizeof(float), 256);
+}
+size_t fwd_ws_size(const l2a_params* p) {
+  return kWsHeaderBytes + qrows_bytes(p) + part_bytes(p) + align_up(kSplitGroups * sizeof(int32_t), 256);
+}
 
 bool ws_ok(const void* ws, size_t have, size_t need) { return ws && aligned(ws, 256) && have >= need; }
 
@@ -324,6 +334,13 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   a.shared_window = 0;
   a.lse_loc = nullptr;
   a.seq_bounds = p->seq_bounds;
+  a.part = nullptr;
+  a.part_count = nullptr;
+  a.overlap = 0;
+  // split key ranges: launches over the compacted rows (those of a row range too, so that their results stay the same)
+  const bool split = !skip_global && !force_all;
+  float* part = reinterpret_cast<float*>(ws + kWsHeaderBytes + qrows_bytes(p));
+  int32_t* part_count = reinterpret_cast<int32_t*>(ws + kWsHeaderBytes + qrows_bytes(p) + part_bytes(p));
 
   PhaseEvents& pe = phase_events();
   struct ClearOnExit { PhaseEvents& p; ~ClearOnExit() { p.clear(); } } clear_on_exit{pe};
@@ -331,7 +348,8 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   if (!skip_global && !force_all) {
     // consolidate routed query rows (Algorithm 1, step 1); independent of the local pass
     if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s,
-                           row_range ? prefix : nullptr, row_begin, row_end, qs, status) != cudaSuccess)
+                           row_range ? prefix : nullptr, row_begin, row_end, qs, status, split ? part_count : nullptr,
+                           split ? kSplitGroups : 0) != cudaSuccess)
       return L2A_ERR_CUDA;
   }
   pe.mark(s);
@@ -371,6 +389,12 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
     a.lse = lse_glb;
     a.shared_window = shared ? 1 : 0;
     a.lse_loc = lse_loc;
+    if (split) {
+      a.part = part;
+      a.part_count = part_count;
+    }
+    // (events between the launches ask for times of the passes one after the other)
+    a.overlap = !skip_local && !global_phase && pe.n == 0;
     if (force_all) {
       // Global Attention for every token (Section 3.3): same kernel over all rows in place; a_t is stored for
       // every row, and still only enters O where d_t = 1

@@ -82,7 +82,8 @@ cudaError_t launch_pack_sequences(const int32_t* cu_seqlens, int n_seq, int L, i
 cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx, const int32_t* n_routed,
                                int B, int L, int row_elems, cudaStream_t stream, const int32_t* prefix = nullptr,
                                int row_begin = 0, int row_end = 0, RowStrides src_strides = RowStrides{0, 0},
-                               int* status = nullptr);   // status: workspace status word (debug-build index checks)
+                               int* status = nullptr,    // status: workspace status word (debug-build index checks)
+                               int32_t* zero = nullptr, int n_zero = 0);   // n_zero words to clear on the way
 
 // z[b,t] = w . S[b,t,:] + bias (fp32 accumulation); optional sum over t of sigmoid(z)^2 per batch entry
 cudaError_t launch_router_logits(const bf16* S, const float* w, float bias, float* logits, float* sum_sq, int B,
@@ -118,7 +119,27 @@ struct FwdArgs {
   const float* lse_loc;      // [B,Hq,Lq] by row; read only when shared_window is set
   // Packed variable-length batch (B == 1): per token {first token of its sequence, one past the last}; NULL otherwise
   const int32_t* seq_bounds;
+  // Key-range splits of the compact groups (global mode; NULL: none): a slot of unnormalised rows with their maxima and
+  // sums for every work item of a split launch, and a zeroed counter per group, whose last CTA to finish combines them.
+  float* part;
+  int32_t* part_count;
+  int overlap;               // launched behind the local pass of the same call: may start before that has finished
 };
+// A global launch of so few groups (256 compact rows of a head) that they leave SMs idle splits their key ranges until it
+// has about two work items for each of the 148 SMs, at most kMaxKeySplit per group and not below kMinSplitBlocks key
+// blocks an item: an item's rows cost 3 us to store in fp32 and its group's last CTA reads them all back, about three key
+// blocks' time.  Measured, whole forward without / with: 2000 new tokens on 34K keys (64 groups) 525 / 369 us, 300 on 60K
+// (28 groups) 734 / 213, 4001 tokens (112 groups, 32 blocks at most) 178 / 169; but with 128 groups (8000 on 100K) 1686 /
+// 1707, and three items per SM there 1800, 196 groups (16K tokens) 901 / 945: no split from kSplitGroups on.
+constexpr int kSplitItems = 2 * 148;
+constexpr int kSplitGroups = 128;
+constexpr int kMaxKeySplit = 8;
+constexpr int kMinSplitBlocks = 16;
+inline int split_slots(int n_groups) {       // slots a shape with that many groups (all rows routed) can need
+  const int64_t n = (int64_t)n_groups * kMaxKeySplit;
+  return n < kSplitItems ? (int)n : kSplitItems;
+}
+inline size_t split_slot_floats(int D) { return (size_t)kRowsPerCta * (D + 2); }
 size_t bwd_ws_size(const l2a_params* p);
 // Key-block ranges of the backward when the caller registered phase events for them (11 events: four ranges, 7: two,
 // fewer: one launch).  Writes the first key block of ranges 1.. into `first` and returns the number of ranges; ranges

@@ -194,6 +194,17 @@ __device__ __forceinline__ void cluster_st128(uint32_t addr, uint32_t a, uint32_
                : "memory");
 }
 
+// barrier of `threads` threads of the CTA (id 1 .. 15)
+__device__ __forceinline__ void named_barrier(int id, int threads) {
+  asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Programmatic dependent launch: a grid launched with that attribute may start once every CTA of the grid before it has
+// started (and called release); wait returns when that grid has completed and its writes are visible.  Without the
+// attribute both are no-ops.
+__device__ __forceinline__ void dependents_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ----------------------------------------------------------------------------------------------
 // TMA (tiled, no cluster features): global -> shared, completion counted on an mbarrier
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {

@@ -1,9 +1,11 @@
 // Decode step of the layer (Section 3.4): one new query token per sequence attends to the last W+1 keys of the
 // cache (Local Attention) and, only if its routing decision d = 1, to the whole cache (Global Attention);
-// o = s + d * a.  The work is one pass over the K/V cache: HBM-bound.  The cache of every KV head is split into
-// chunks processed by independent CTAs (partial soft-max per chunk), merged by a second small kernel.
+// o = s + d * a.  The work is one pass over the K/V cache: HBM-bound.  The cache of every KV head is cut at the window's
+// first key and split into chunks processed by independent CTAs; a chunk's partial soft-max (acc, max, sum) inside the
+// window serves both modules, those before it exist for routed tokens only.  The CTA of a (sequence, KV head) that
+// finishes last combines the chunks: o is one weighted sum of their accumulators.
 //
-// Split kernel, one CTA = one chunk of keys of one (batch entry, KV head), for all G query heads of the group:
+// One CTA = one chunk of keys of one (batch entry, KV head), for all G query heads of the group:
 //   producer warp : streams 64-key K and V tiles through a ring of shared-memory stages with TMA (one 4-D copy
 //                   per tile, 128-byte swizzle), so tens of KB per SM are in flight whatever the compute warps do.
 //   compute warps : each takes 16 keys of every stage.  The G query heads are the rows of a 16-row MMA A operand
@@ -12,6 +14,8 @@
 //                   the V rows.  The tensor cores are used only to keep the instruction count per key low enough
 //                   that the copy engine, not instruction issue, sets the pace.
 #include <math.h>
+
+#include <algorithm>
 
 #include "l2a_common.cuh"
 #include "sm100_prims.cuh"
@@ -30,10 +34,11 @@ struct DecodeArgs {
   int B, Lk, Hq, Hkv, G;
   int window, q_pos;       // the new token sits at position q_pos (normally Lk - 1)
   float scale_log2;
-  int n_loc, n_glb;        // chunks of the local / global key range
+  int n_win, n_out;        // chunks of the window / of the keys before it
   const bf16* q;           // [B, Hq, D]
   const uint8_t* d;        // [B] routing decision of the new token (NULL = never routed)
-  float* part;             // [B, Hq, n_loc + n_glb, D + 2]  (acc[D], m, l)
+  float* part;             // [B, Hkv, n_win + n_out, G, D + 4]  (acc[D], m, l, 2 unused)
+  int* done;               // [B, Hkv] chunks finished so far; cleared by the caller
   bf16* O;                 // [B, Hq, D]
   int* status;             // workspace status word
 };
@@ -41,12 +46,15 @@ struct DecodeArgs {
 struct DecodeBars {
   uint64_t full[kDecStages], empty[kDecStages];
   int abort_flag;
+  int last;                // this CTA finished last of its (batch entry, KV head)
 };
 
+constexpr int kMaxWin = 64, kMaxOut = 512;   // chunks at most
 template <int D>
 constexpr size_t decode_smem_bytes() {
   return (size_t)kDecStages * 2 * kDecKeys * D * 2 + sizeof(DecodeBars);
 }
+static_assert(kMaxGroup * (kMaxWin + kMaxOut) * sizeof(float2) <= kDecStages * 2 * kDecKeys * 64 * 2, "weights exceed the stages");
 
 __device__ __forceinline__ void chunk_range(int lo, int hi, int n, int i, int& c_lo, int& c_hi) {
   const int len = hi - lo + 1;
@@ -86,11 +94,13 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   constexpr int kTileBytes = kDecKeys * D * 2;
   constexpr int kStageBytes = 2 * kTileBytes;       // K tile, then V tile
   const int item = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
-  const bool glb = item >= a.n_loc;
-  if (glb && (a.d == nullptr || a.d[b] == 0)) return;          // Global Attention is skipped when d = 0
-  const int lo = glb ? 0 : max(0, a.q_pos - a.window);
+  const bool outside = item >= a.n_win;
+  const bool routed = a.d != nullptr && a.d[b] != 0;
+  if (outside && !routed) return;                              // Global Attention is skipped when d = 0
+  const int win_lo = max(0, a.q_pos - a.window);
   int c_lo, c_hi;
-  chunk_range(lo, a.q_pos, glb ? a.n_glb : a.n_loc, glb ? item - a.n_loc : item, c_lo, c_hi);
+  if (outside) chunk_range(0, win_lo - 1, a.n_out, item - a.n_win, c_lo, c_hi);
+  else chunk_range(win_lo, a.q_pos, a.n_win, item, c_lo, c_hi);
   const int n_tiles = c_hi >= c_lo ? (c_hi - c_lo) / kDecKeys + 1 : 0;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -222,7 +232,9 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
       *reinterpret_cast<float2*>(&red_acc[(warp * G + hr) * D + j * 8 + 2 * t4]) = make_float2(acc[j][0], acc[j][1]);
   }
   __syncthreads();
-  const int n_items = a.n_loc + a.n_glb;
+  const int n_items = a.n_win + a.n_out;
+  constexpr int kRow = D + 4;
+  float* base = a.part + ((int64_t)b * a.Hkv + g) * n_items * (G * kRow);
   for (int i = tid; i < G * D; i += kDecThreads) {
     const int h = i / D, col = i % D;
     float M = -INFINITY;
@@ -234,9 +246,81 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
       L += red_l[w * G + h] * f;
       A += red_acc[(w * G + h) * D + col] * f;
     }
-    float* dst = a.part + (((int64_t)b * a.Hq + g * G + h) * n_items + item) * (D + 2);
+    float* dst = base + (item * G + h) * kRow;
     dst[col] = A;
     if (col == 0) { dst[D] = M; dst[D + 1] = L; }
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) bar->last = atomicAdd(&a.done[b * a.Hkv + g], 1) == (routed ? n_items : a.n_win) - 1;
+  __syncthreads();
+  if (bar->last) {
+    // ---- the last CTA of the (batch entry, KV head): weight of chunk i in head h's result,
+    //   o = sum_win acc_i 2^(m_i - M_win) / L_win + d * sum_all acc_i 2^(m_i - M_all) / L_all
+    __threadfence();
+    const int n = routed ? n_items : a.n_win;
+    float2* ml = reinterpret_cast<float2*>(smem);            // [n][G] (m, l), then (weight, -)
+    for (int i = tid; i < n * G; i += kDecThreads)
+      ml[i] = __ldcg(reinterpret_cast<const float2*>(base + (int64_t)i * kRow + D));
+    __syncthreads();
+    for (int h = warp; h < G; h += kDecComputeWarps + 1) {
+      float M[2] = {-INFINITY, -INFINITY}, L[2] = {0.f, 0.f};   // window, everything
+      for (int i = lane; i < n; i += 32) {
+        const float m = ml[i * G + h].x;
+        M[1] = fmaxf(M[1], m);
+        if (i < a.n_win) M[0] = fmaxf(M[0], m);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        M[0] = fmaxf(M[0], __shfl_xor_sync(0xffffffffu, M[0], o));
+        M[1] = fmaxf(M[1], __shfl_xor_sync(0xffffffffu, M[1], o));
+      }
+      for (int i = lane; i < n; i += 32) {
+        const float2 v = ml[i * G + h];
+        if (v.x != -INFINITY) {                                 // (a chunk without keys wrote no maximum)
+          L[1] += v.y * exp2f(v.x - M[1]);
+          if (i < a.n_win) L[0] += v.y * exp2f(v.x - M[0]);
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        L[0] += __shfl_xor_sync(0xffffffffu, L[0], o);
+        L[1] += __shfl_xor_sync(0xffffffffu, L[1], o);
+      }
+      for (int i = lane; i < n; i += 32) {
+        const float m = ml[i * G + h].x;
+        float w = 0.f;
+        if (m != -INFINITY) {
+          if (i < a.n_win) w = exp2f(m - M[0]) / L[0];
+          if (routed) w += exp2f(m - M[1]) / L[1];
+        }
+        ml[i * G + h].x = w;
+      }
+    }
+    __syncthreads();
+    // four columns a thread, sixteen chunks in flight: what counts here is the latency of the rounds
+    for (int x = tid; x < G * (D / 4); x += kDecThreads) {
+      const int h = x / (D / 4), c4 = x % (D / 4);
+      const float* src = base + h * kRow + c4 * 4;
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k0 = 0; k0 < n; k0 += 16) {
+        float4 v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          v[k] = k0 + k < n ? __ldcg(reinterpret_cast<const float4*>(src + (int64_t)(k0 + k) * (G * kRow)))
+                            : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          const float w = k0 + k < n ? ml[(k0 + k) * G + h].x : 0.f;
+          o.x = fmaf(w, v[k].x, o.x);
+          o.y = fmaf(w, v[k].y, o.y);
+          o.z = fmaf(w, v[k].z, o.z);
+          o.w = fmaf(w, v[k].w, o.w);
+        }
+      }
+      reinterpret_cast<uint2*>(a.O + ((int64_t)b * a.Hq + g * G + h) * D)[c4] =
+          make_uint2(pack_bf16(o.x, o.y), pack_bf16(o.z, o.w));
+    }
   }
   if (bar->abort_flag) {
     // a bounded wait ran out: give copies still in flight time to land before shared memory is released
@@ -247,53 +331,31 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   }
 }
 
-// Merges the chunk partials of one (batch entry, query head): s over the local chunks, a over the global ones.
-template <int D>
-__global__ void __launch_bounds__(D) decode_merge_kernel(const DecodeArgs a) {
-  const int h = blockIdx.x, b = blockIdx.y, col = threadIdx.x;
-  const int n_items = a.n_loc + a.n_glb;
-  const float* base = a.part + (((int64_t)b * a.Hq + h) * n_items) * (D + 2);
-  const bool routed = a.d != nullptr && a.d[b] != 0;
-  float out = 0.f;
-  for (int pass = 0; pass < (routed ? 2 : 1); ++pass) {
-    const int i0 = pass == 0 ? 0 : a.n_loc, i1 = pass == 0 ? a.n_loc : n_items;
-    float M = -INFINITY;
-    for (int i = i0; i < i1; ++i) M = fmaxf(M, base[i * (D + 2) + D]);
-    float L = 0.f, A = 0.f;
-    for (int i = i0; i < i1; ++i) {
-      const float mi = base[i * (D + 2) + D];
-      const float f = (mi == -INFINITY) ? 0.f : exp2f(mi - M);
-      L += base[i * (D + 2) + D + 1] * f;
-      A += base[i * (D + 2) + col] * f;
-    }
-    out += A / L;
-  }
-  a.O[((int64_t)b * a.Hq + h) * D + col] = __float2bfloat16(out);
-}
-
-void plan_chunks(const l2a_params* p, int* n_loc, int* n_glb) {
-  // Cache chunks of at most 2048 keys, shrunk (down to 512) when few (sequence, KV head) pairs exist so that the
-  // grid still covers the SMs a few times over; CTAs of non-routed sequences exit at once.  Local chunks of 256
-  // keys.  The merge reads at most 512 + 64 partials per head.
+// Chunks as long as one resident wave of CTAs (two per SM, 148 SMs) allows, between 256 and 4096 keys: every chunk costs
+// its launch and a row per head that the last CTA reads back.  Measured against four times as many: one sequence of 128K
+// keys (28/4 heads) 64 / 87 us, two of 40K 27 / 36, six of 100K with one KV head 63 / 84, 16 of 128K with four routed 342
+// (2048 keys at most: 353), 32 of 8000 not routed 90 / 92, one of 9001 16.4 with either.
+constexpr int kChunkTarget = 2 * 148, kChunkMin = 256, kChunkMax = 4096;
+void plan_chunks(const l2a_params* p, int* n_win, int* n_out) {
   const int pos = p->q_pos_offset;
-  const int local_len = (pos < p->window ? pos : p->window) + 1;
+  const int win = (pos < p->window ? pos : p->window) + 1, out = pos + 1 - win;
   const int64_t pairs = (int64_t)p->B * p->Hkv;
-  int64_t per = ((int64_t)(pos + 1) * pairs + 1183) / 1184;
-  per = per < 512 ? 512 : (per > 2048 ? 2048 : per);
-  int ng = ceil_div(pos + 1, (int)per);
-  if (ng > 512) ng = 512;
-  int nl = ceil_div(local_len, 256);
-  if (nl > 64) nl = 64;
-  *n_loc = nl < 1 ? 1 : nl;
-  *n_glb = ng < 1 ? 1 : ng;
+  auto chunk = [&](int64_t keys) {
+    const int64_t per = (keys * pairs + kChunkTarget - 1) / kChunkTarget;
+    return (int)(per < kChunkMin ? kChunkMin : (per > kChunkMax ? kChunkMax : (per + kDecKeys - 1) / kDecKeys * kDecKeys));
+  };
+  *n_win = std::min(ceil_div(win, chunk(win)), kMaxWin);
+  *n_out = std::min(ceil_div(out, chunk(pos + 1)), kMaxOut);
 }
 
 template <int D, int G>
 cudaError_t launch_split(const DecodeArgs& a, const CUtensorMap& mapK, const CUtensorMap& mapV, dim3 grid,
                          cudaStream_t s) {
   constexpr size_t smem = decode_smem_bytes<D>();
-  cudaError_t e = cudaFuncSetAttribute(decode_split_kernel<D, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  static PerDeviceOnce once;
+  const cudaError_t e = once.run([] {
+    return cudaFuncSetAttribute(decode_split_kernel<D, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  });
   if (e != cudaSuccess) return e;
   decode_split_kernel<D, G><<<grid, kDecThreads, smem, s>>>(a, mapK, mapV);
   return cudaGetLastError();
@@ -320,14 +382,16 @@ cudaError_t launch_split_d(const DecodeArgs& a, const CUtensorMap& mapK, const C
 
 using namespace l2a;
 
+static size_t done_bytes(const l2a_params* p) { return align_up((size_t)p->B * p->Hkv * sizeof(int), 256); }
+
 extern "C" l2a_status l2a_decode_workspace_bytes(const l2a_params* p, size_t* ws_bytes) {
   size_t unused = 0;
   l2a_status st = l2a_workspace_bytes(p, &unused, nullptr, nullptr);
   if (st != L2A_OK) return st;
   if (!ws_bytes || p->Lq != 1) return L2A_ERR_INVALID_ARG;
-  int nl, ng;
-  plan_chunks(p, &nl, &ng);
-  *ws_bytes = kWsHeaderBytes + align_up((size_t)p->B * p->Hq * (nl + ng) * (p->D + 2) * sizeof(float), 256);
+  int nw, no;
+  plan_chunks(p, &nw, &no);
+  *ws_bytes = kWsHeaderBytes + done_bytes(p) + align_up((size_t)p->B * p->Hq * (nw + no) * (p->D + 4) * sizeof(float), 256);
   return L2A_OK;
 }
 
@@ -345,7 +409,7 @@ extern "C" l2a_status l2a_decode(const l2a_params* p, const void* q, const void*
   if (p->q_pos_offset >= p->Lk) return L2A_ERR_INVALID_ARG;     // the new token's own key must be in the cache
   if (!ws || (reinterpret_cast<uintptr_t>(ws) % 256) != 0 || ws_bytes < need) return L2A_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
+  if (cudaMemsetAsync(ws, 0, kWsHeaderBytes + done_bytes(p), s) != cudaSuccess) return L2A_ERR_CUDA;   // status, counters
   CUtensorMap mapK, mapV;
   if (!is_dense(p->q_stride, p->Lq, p->Hq * p->D) || !is_dense(p->o_stride, p->Lq, p->Hq * p->D)) return L2A_ERR_UNSUPPORTED;
   const RowStrides ks = resolve_strides(p->k_stride, p->Lk, p->Hkv * p->D);
@@ -358,22 +422,14 @@ extern "C" l2a_status l2a_decode(const l2a_params* p, const void* q, const void*
   a.window = p->window;
   a.q_pos = p->q_pos_offset;
   a.scale_log2 = (p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)p->D)) * 1.4426950408889634f;
-  plan_chunks(p, &a.n_loc, &a.n_glb);
+  plan_chunks(p, &a.n_win, &a.n_out);
   a.q = static_cast<const bf16*>(q);
   a.d = d;
   a.status = static_cast<int*>(ws);
-  a.part = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + kWsHeaderBytes);
+  a.done = reinterpret_cast<int*>(static_cast<uint8_t*>(ws) + kWsHeaderBytes);
+  a.part = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + kWsHeaderBytes + done_bytes(p));
   a.O = static_cast<bf16*>(O);
-  dim3 grid(a.n_loc + a.n_glb, p->Hkv, p->B);
-  dim3 mgrid(p->Hq, p->B);
-  cudaError_t e;
-  if (p->D == 128) {
-    e = launch_split_d<128>(a, mapK, mapV, grid, s);
-    if (e == cudaSuccess) decode_merge_kernel<128><<<mgrid, 128, 0, s>>>(a);
-  } else {
-    e = launch_split_d<64>(a, mapK, mapV, grid, s);
-    if (e == cudaSuccess) decode_merge_kernel<64><<<mgrid, 64, 0, s>>>(a);
-  }
-  if (e != cudaSuccess) return L2A_ERR_CUDA;
-  return cudaGetLastError() == cudaSuccess ? L2A_OK : L2A_ERR_CUDA;
+  const dim3 grid(a.n_win + a.n_out, p->Hkv, p->B);
+  const cudaError_t e = p->D == 128 ? launch_split_d<128>(a, mapK, mapV, grid, s) : launch_split_d<64>(a, mapK, mapV, grid, s);
+  return e == cudaSuccess ? L2A_OK : L2A_ERR_CUDA;
 }

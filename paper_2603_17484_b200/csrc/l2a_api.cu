@@ -53,7 +53,8 @@ size_t route_ws_size(const l2a_params* p) {
   return kWsHeaderBytes + align_up((size_t)p->B * nblocks * sizeof(int32_t), 256);
 }
 size_t qrows_bytes(const l2a_params* p) { return align_up((size_t)p->B * p->Lq * p->Hq * p->D * sizeof(bf16), 256); }
-// forward workspace: header, compacted queries, then the slots and counters of split key ranges
+// forward workspace: header, counters of split key ranges, compacted queries, slots of split key ranges
+constexpr size_t kPartCountBytes = (kSplitGroups * sizeof(int32_t) + 255) / 256 * 256;
 int group_count(const l2a_params* p) {
   const int64_t n = (int64_t)ceil_div(p->Lq, kRowsPerCta) * p->Hq * p->B;
   return n < kSplitGroups ? (int)n : kSplitGroups;     // launches with more groups are not split
@@ -62,7 +63,7 @@ size_t part_bytes(const l2a_params* p) {
   return align_up(split_slots(group_count(p)) * split_slot_floats(p->D) * sizeof(float), 256);
 }
 size_t fwd_ws_size(const l2a_params* p) {
-  return kWsHeaderBytes + qrows_bytes(p) + part_bytes(p) + align_up(kSplitGroups * sizeof(int32_t), 256);
+  return kWsHeaderBytes + kPartCountBytes + qrows_bytes(p) + part_bytes(p);
 }
 
 bool ws_ok(const void* ws, size_t have, size_t need) { return ws && aligned(ws, 256) && have >= need; }
@@ -209,8 +210,8 @@ l2a_status l2a_route_compact(const l2a_params* p, const void* router, int router
   if (router_kind == L2A_ROUTER_LOGITS_BF16 && !aligned(router, 2)) return L2A_ERR_INVALID_ARG;
   if (!ws_ok(route_ws, route_ws_bytes, route_ws_size(p))) return L2A_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(route_ws, 0, kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
   RouteArgs a;
+  a.header = static_cast<int32_t*>(route_ws);
   a.router = router;
   a.router_kind = router_kind;
   a.threshold = logit_threshold;
@@ -294,7 +295,9 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint8_t* ws = static_cast<uint8_t*>(fwd_ws);
   int* status = reinterpret_cast<int*>(ws);
-  bf16* Qc = reinterpret_cast<bf16*>(ws + kWsHeaderBytes);
+  int32_t* part_count = reinterpret_cast<int32_t*>(ws + kWsHeaderBytes);
+  bf16* Qc = reinterpret_cast<bf16*>(ws + kWsHeaderBytes + kPartCountBytes);
+  float* part = reinterpret_cast<float*>(ws + kWsHeaderBytes + kPartCountBytes + qrows_bytes(p));
   const int n_pairs = ceil_div(p->Lq, kRowsPerCta);
   const bool whole = pair_end < 0 || (pair_begin == 0 && pair_end == n_pairs);
   if (pair_end < 0) pair_end = n_pairs;
@@ -303,7 +306,14 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   const bool row_range = row_begin > 0 || row_end < p->Lq;
   if (row_range && (!global_phase || row_begin < 0 || row_begin > row_end)) return L2A_ERR_INVALID_ARG;
   if (row_end > p->Lq) row_end = p->Lq;
-  if (clear_status && cudaMemsetAsync(ws, 0, kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
+  // the gather of the routed rows, first on the stream where there is one, clears the header and the counters behind it
+  // (not in the debug build, whose index checks in the same kernel report through the header)
+#ifdef L2A_DEBUG
+  const bool gather_clears = false;
+#else
+  const bool gather_clears = clear_status && !skip_global && !force_all;
+#endif
+  if (clear_status && !gather_clears && cudaMemsetAsync(ws, 0, kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
 
   CUtensorMap mapQ, mapK, mapV, mapQc;
   const RowStrides qs = resolve_strides(p->q_stride, p->Lq, p->Hq * p->D);
@@ -339,8 +349,6 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   a.overlap = 0;
   // split key ranges: launches over the compacted rows (those of a row range too, so that their results stay the same)
   const bool split = !skip_global && !force_all;
-  float* part = reinterpret_cast<float*>(ws + kWsHeaderBytes + qrows_bytes(p));
-  int32_t* part_count = reinterpret_cast<int32_t*>(ws + kWsHeaderBytes + qrows_bytes(p) + part_bytes(p));
 
   PhaseEvents& pe = phase_events();
   struct ClearOnExit { PhaseEvents& p; ~ClearOnExit() { p.clear(); } } clear_on_exit{pe};
@@ -348,8 +356,9 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   if (!skip_global && !force_all) {
     // consolidate routed query rows (Algorithm 1, step 1); independent of the local pass
     if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s,
-                           row_range ? prefix : nullptr, row_begin, row_end, qs, status, split ? part_count : nullptr,
-                           split ? kSplitGroups : 0) != cudaSuccess)
+                           row_range ? prefix : nullptr, row_begin, row_end, qs, status,
+                           gather_clears ? status : part_count,
+                           (int)((gather_clears ? kWsHeaderBytes + kPartCountBytes : kPartCountBytes) / 4)) != cudaSuccess)
       return L2A_ERR_CUDA;
   }
   pe.mark(s);

@@ -71,6 +71,7 @@ struct RouteArgs {
   int32_t* prefix;
   int32_t* block_sums;  // workspace: [B, nblocks]
   int nblocks;
+  int32_t* header = nullptr;   // workspace header to clear, NULL: none
 };
 constexpr int kRouteBlockElems = 4096;  // positions per CTA of the route/compact kernels
 cudaError_t launch_route_compact(const RouteArgs& a, cudaStream_t stream);

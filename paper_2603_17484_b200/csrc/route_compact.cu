@@ -1,11 +1,13 @@
 // Routing decision + query compaction (Eq. 3; Section 3.2; Algorithm 1 step 1), and the row gather
 // that consolidates routed rows into a contiguous buffer.
 //
-// Two small launches, both HBM/latency bound:
-//   route_count : each CTA thresholds 4096 positions and counts its routed ones (ballot + popc)
-//   route_scan  : each CTA sums the counts of the CTAs before it, rescans its own 4096 positions
-//                 (per-thread popcount of a 16-bit flag word, warp shuffle scan, cross-warp scan)
-//                 and writes d_mask, prefix, q_idx (ascending = stable) and the -1 tail.
+// One or two small launches, latency bound:
+//   route_count : each CTA thresholds 4096 positions and counts its routed ones (ballot + popc); skipped for short
+//                 sequences, whose CTAs count all positions themselves
+//   route_scan  : each CTA sums the counts of the CTAs before it and writes d_mask, prefix, q_idx (ascending = stable) and
+//                 the -1 tail of its own 4096 positions: a warp takes 512 consecutive ones, 32 at a time (one ballot),
+//                 so that every store is contiguous (a thread with 16 consecutive positions of its own, storing with a
+//                 stride of 64 bytes, took 9.8 us for a block, this 4).
 // Nothing is read back by the host: the routed count stays on the device.
 #include "l2a_common.cuh"
 
@@ -14,103 +16,96 @@ namespace l2a {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kPerThread = kRouteBlockElems / kThreads;  // 16
+constexpr int kWarps = kThreads / 32;
+constexpr int kRounds = kRouteBlockElems / kThreads;     // 32-position rounds of a warp
+// Blocks of a sequence up to which every CTA counts them all itself (16384 positions: 64 loads a thread, less than the
+// second launch costs).
+constexpr int kCountAllBlocks = 4;
 
-__device__ __forceinline__ uint32_t load_flags(const void* router, int kind, float thr, int64_t row_base, int t0,
-                                               int L) {
-  uint32_t flags = 0;
-  if (kind == L2A_ROUTER_MASK_U8) {
-    const uint8_t* m = static_cast<const uint8_t*>(router) + row_base;
-    if (t0 + kPerThread <= L && ((reinterpret_cast<uintptr_t>(m + t0) & 15) == 0)) {
-      const uint4 v = *reinterpret_cast<const uint4*>(m + t0);
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+__device__ __forceinline__ bool routed_at(const RouteArgs& a, int64_t i) {
+  if (a.router_kind == L2A_ROUTER_MASK_U8) return static_cast<const uint8_t*>(a.router)[i] != 0;
+  const float z = a.router_kind == L2A_ROUTER_LOGITS_BF16 ? __bfloat162float(static_cast<const bf16*>(a.router)[i])
+                                                          : static_cast<const float*>(a.router)[i];   // the upcast is exact
+  return z >= a.threshold;             // NaN compares false; -0.0 >= 0.0 is true
+}
+
+// routed positions among those of block blk this thread looks at
+__device__ __forceinline__ int count_block(const RouteArgs& a, int64_t row_base, int blk) {
+  int cnt = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if ((w[i] >> (8 * k)) & 0xffu) flags |= 1u << (4 * i + k);
-    } else {
-      for (int i = 0; i < kPerThread; ++i)
-        if (t0 + i < L && m[t0 + i]) flags |= 1u << i;
-    }
-  } else if (kind == L2A_ROUTER_LOGITS_BF16) {
-    const bf16* z = static_cast<const bf16*>(router) + row_base;
-    for (int i = 0; i < kPerThread; ++i)
-      if (t0 + i < L && __bfloat162float(z[t0 + i]) >= thr) flags |= 1u << i;   // the upcast is exact
-  } else {
-    const float* z = static_cast<const float*>(router) + row_base;
-    for (int i = 0; i < kPerThread; ++i)
-      if (t0 + i < L && z[t0 + i] >= thr) flags |= 1u << i;  // NaN compares false; -0.0 >= 0.0 is true
+  for (int i = 0; i < kRounds; ++i) {
+    const int t = blk * kRouteBlockElems + i * kThreads + threadIdx.x;
+    if (t < a.L && routed_at(a, row_base + t)) ++cnt;
   }
-  return flags;
+  return cnt;
 }
 
 __global__ void __launch_bounds__(kThreads) route_count_kernel(RouteArgs a) {
   const int b = blockIdx.y, blk = blockIdx.x;
-  const int t0 = blk * kRouteBlockElems + threadIdx.x * kPerThread;
-  const uint32_t flags = load_flags(a.router, a.router_kind, a.threshold, (int64_t)b * a.L, t0, a.L);
-  int cnt = __popc(flags);
-  __shared__ int warp_cnt[kThreads / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+  const int cnt = __reduce_add_sync(0xffffffffu, count_block(a, (int64_t)b * a.L, blk));
+  __shared__ int warp_cnt[kWarps];
   if ((threadIdx.x & 31) == 0) warp_cnt[threadIdx.x >> 5] = cnt;
   __syncthreads();
   if (threadIdx.x == 0) {
     int s = 0;
-    for (int w = 0; w < kThreads / 32; ++w) s += warp_cnt[w];
+    for (int w = 0; w < kWarps; ++w) s += warp_cnt[w];
     a.block_sums[b * a.nblocks + blk] = s;
   }
 }
 
+template <bool kCountAll>
 __global__ void __launch_bounds__(kThreads) route_scan_kernel(RouteArgs a) {
   const int b = blockIdx.y, blk = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ int red_before[kThreads / 32], red_total[kThreads / 32], warp_off[kThreads / 32];
+  const int64_t row_base = (int64_t)b * a.L;
+  __shared__ int red_before[kWarps], red_total[kWarps], warp_cnt[kWarps];
+  if (a.header != nullptr && blk == 0 && b == 0 && threadIdx.x < kWsHeaderBytes / 4) a.header[threadIdx.x] = 0;
 
-  // counts of the CTAs before this one, and the row total
+  // counts of the other CTAs' positions, and of those before this one's
   int before = 0, total = 0;
-  for (int i = threadIdx.x; i < a.nblocks; i += kThreads) {
-    const int v = a.block_sums[b * a.nblocks + i];
+  for (int i = kCountAll ? 0 : threadIdx.x; i < a.nblocks; i += kCountAll ? 1 : kThreads) {
+    if (i == blk) continue;
+    const int v = kCountAll ? count_block(a, row_base, i) : a.block_sums[b * a.nblocks + i];
     total += v;
     if (i < blk) before += v;
   }
+  before = __reduce_add_sync(0xffffffffu, before);
+  total = __reduce_add_sync(0xffffffffu, total);
+  // this warp's 512 positions
+  const int t0 = blk * kRouteBlockElems + warp * (32 * kRounds);
+  uint32_t words[kRounds];
+  int cnt = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    before += __shfl_xor_sync(0xffffffffu, before, o);
-    total += __shfl_xor_sync(0xffffffffu, total, o);
+  for (int i = 0; i < kRounds; ++i) {
+    const int t = t0 + i * 32 + lane;
+    words[i] = __ballot_sync(0xffffffffu, t < a.L && routed_at(a, row_base + t));
+    cnt += __popc(words[i]);
   }
-  if (lane == 0) { red_before[warp] = before; red_total[warp] = total; }
+  if (lane == 0) { red_before[warp] = before; red_total[warp] = total; warp_cnt[warp] = cnt; }
   __syncthreads();
-  before = 0; total = 0;
-  for (int w = 0; w < kThreads / 32; ++w) { before += red_before[w]; total += red_total[w]; }
-
-  const int t0 = blk * kRouteBlockElems + threadIdx.x * kPerThread;
-  const uint32_t flags = load_flags(a.router, a.router_kind, a.threshold, (int64_t)b * a.L, t0, a.L);
-  const int cnt = __popc(flags);
-  int incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
+  int c = 0;
+  total = 0;
+  for (int w = 0; w < kWarps; ++w) {
+    c += red_before[w];
+    total += red_total[w] + warp_cnt[w];
+    if (w < warp) c += warp_cnt[w];
   }
-  if (lane == 31) warp_off[warp] = incl;
-  __syncthreads();
-  int c = before + incl - cnt;
-  for (int w = 0; w < warp; ++w) c += warp_off[w];
 
-  uint8_t* dm = a.d_mask + (int64_t)b * a.L;
-  int32_t* qi = a.q_idx + (int64_t)b * a.L;
+  uint8_t* dm = a.d_mask + row_base;
+  int32_t* qi = a.q_idx + row_base;
   int32_t* pf = a.prefix + (int64_t)b * (a.L + 1);
 #pragma unroll
-  for (int i = 0; i < kPerThread; ++i) {
-    const int t = t0 + i;
+  for (int i = 0; i < kRounds; ++i) {
+    const int t = t0 + i * 32 + lane;
+    const int on = (words[i] >> lane) & 1;
+    const int ci = c + __popc(words[i] & ((1u << lane) - 1u));
     if (t < a.L) {
-      const int on = (flags >> i) & 1;
       dm[t] = (uint8_t)on;
-      pf[t] = c;
-      if (on) qi[c++] = t;
+      pf[t] = ci;
+      if (on) qi[ci] = t;
       if (t >= total) qi[t] = -1;  // compact slots past the routed count
     }
+    c += __popc(words[i]);
   }
   if (blk == 0 && threadIdx.x == 0) {
     a.n_routed[b] = total;
@@ -268,8 +263,12 @@ cudaError_t launch_pack_sequences(const int32_t* cu_seqlens, int n_seq, int L, i
 
 cudaError_t launch_route_compact(const RouteArgs& a, cudaStream_t stream) {
   dim3 grid(a.nblocks, a.B);
-  route_count_kernel<<<grid, kThreads, 0, stream>>>(a);
-  route_scan_kernel<<<grid, kThreads, 0, stream>>>(a);
+  if (a.nblocks <= kCountAllBlocks) {
+    route_scan_kernel<true><<<grid, kThreads, 0, stream>>>(a);
+  } else {
+    route_count_kernel<<<grid, kThreads, 0, stream>>>(a);
+    route_scan_kernel<false><<<grid, kThreads, 0, stream>>>(a);
+  }
   return cudaGetLastError();
 }
 

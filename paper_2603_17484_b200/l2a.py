@@ -53,6 +53,21 @@ class L2AError(RuntimeError):
         super().__init__(f"{where}: {status_string(code)} ({code})")
 
 
+# argument types of the calls made once per layer or token: p address, i int, f float, z size_t
+_CTYPES = {"p": ctypes.c_void_p, "i": ctypes.c_int, "f": ctypes.c_float, "z": ctypes.c_size_t}
+_SIGNATURES = {
+    "l2a_route_compact": "ppif" + "pppp" + "pzp",
+    "l2a_pack_sequences": "piipp",
+    "l2a_decode": "pppppppzp",
+    "l2a_router_logits": "pppf" + "ppp",
+    "l2a_forward": "pppp" + "pppp" + "ppppp" + "pzp",
+    "l2a_backward": "pppp" + "pppp" + "ppppp" + "pppp" + "pzp",
+    "l2a_backward_split": "pppp" + "pppp" + "pppppp" + "pppp" + "pzp",
+    "l2a_forward_sets": "ppppppp" + "pppp" + "ppppp" + "pzp",
+    "l2a_backward_sets": "ppppppp" + "pppp" + "ppppp" + "ppppppp" + "pzp",
+    "l2a_router_backward": "ppppp" + "f" + "pppppp",
+}
+
 _lib = None
 
 
@@ -68,6 +83,10 @@ def lib() -> ctypes.CDLL:
         L.l2a_status_string.argtypes = [ctypes.c_int]
         for name in EXPORTS[2:]:
             getattr(L, name).restype = ctypes.c_int
+        # with declared argument types plain Python numbers and addresses are converted in C: a call of l2a_forward took
+        # 9 us of ctypes objects before, half of a small launch
+        for name, kinds in _SIGNATURES.items():
+            getattr(L, name).argtypes = [_CTYPES[k] for k in kinds]
         _lib = L
     return _lib
 
@@ -91,19 +110,26 @@ def params(B, Lq, Lk, Hq, Hkv, D, window, q_pos_offset=None, softmax_scale=0.0, 
                      softmax_scale, flags, *st, None if seq_bounds is None else seq_bounds.data_ptr())
 
 
-def _ptr(t):
-    if t is None:
-        return ctypes.c_void_p(0)
-    if isinstance(t, torch.Tensor):
-        # strided views (slices of a fused buffer) are described by the strides in L2AParams; only the base
-        # address is passed
-        return ctypes.c_void_p(t.data_ptr())
-    return ctypes.c_void_p(int(t))
+def _addr(t):
+    """Address as a plain number (None: NULL).  Strided views (slices of a fused buffer) are described by the strides in
+    L2AParams; only the base address is passed."""
+    return None if t is None else t.data_ptr() if isinstance(t, torch.Tensor) else int(t)
+
+
+def _raw_stream(stream=None):
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
+
+
+def _bytes(t):
+    return 0 if t is None else t.numel() * t.element_size()
+
+
+def _ptr(t):       # for calls without a declared signature
+    return ctypes.c_void_p(_addr(t))
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return ctypes.c_void_p(_raw_stream(stream))
 
 
 def _check(code: int, where: str):
@@ -132,11 +158,9 @@ def l2a_selftest_wait_timeout(ws: torch.Tensor, limit_us: int, stream=None, chec
 
 def l2a_route_compact(p, router, router_kind, logit_threshold, d_mask, q_idx, n_routed, prefix, route_ws,
                       stream=None, check=True) -> int:
-    code = lib().l2a_route_compact(ctypes.byref(p), _ptr(router), ctypes.c_int(router_kind),
-                                   ctypes.c_float(logit_threshold), _ptr(d_mask), _ptr(q_idx), _ptr(n_routed),
-                                   _ptr(prefix), _ptr(route_ws),
-                                   ctypes.c_size_t(route_ws.numel() * route_ws.element_size() if route_ws is not None else 0),
-                                   _stream(stream))
+    code = lib().l2a_route_compact(ctypes.byref(p), _addr(router), router_kind,
+                                   logit_threshold, _addr(d_mask), _addr(q_idx), _addr(n_routed),
+                                   _addr(prefix), _addr(route_ws), _bytes(route_ws), _raw_stream(stream))
     if check:
         _check(code, "l2a_route_compact")
     return code
@@ -146,8 +170,8 @@ def l2a_pack_sequences(cu_seqlens, Lq, seq_bounds=None, stream=None):
     """cu_seqlens: int32 device tensor [n_seq + 1]; returns the int32 [Lq, 2] table for `params(seq_bounds=...)`."""
     if seq_bounds is None:
         seq_bounds = torch.empty((Lq, 2), dtype=torch.int32, device=cu_seqlens.device)
-    _check(lib().l2a_pack_sequences(_ptr(cu_seqlens), ctypes.c_int(cu_seqlens.numel() - 1), ctypes.c_int(Lq),
-                                    _ptr(seq_bounds), _stream(stream)), "l2a_pack_sequences")
+    _check(lib().l2a_pack_sequences(_addr(cu_seqlens), cu_seqlens.numel() - 1, Lq,
+                                    _addr(seq_bounds), _raw_stream(stream)), "l2a_pack_sequences")
     return seq_bounds
 
 
@@ -171,8 +195,8 @@ def l2a_decode_workspace_bytes(p) -> int:
 
 def l2a_decode(p, q, K, V, d, O, ws, stream=None, check=True) -> int:
     """Decode step: one new token per sequence against the K/V cache (local window always, whole cache if d = 1)."""
-    code = lib().l2a_decode(ctypes.byref(p), _ptr(q), _ptr(K), _ptr(V), _ptr(d), _ptr(O), _ptr(ws),
-                            ctypes.c_size_t(ws.numel() if ws is not None else 0), _stream(stream))
+    code = lib().l2a_decode(ctypes.byref(p), _addr(q), _addr(K), _addr(V), _addr(d), _addr(O), _addr(ws),
+                            _bytes(ws), _raw_stream(stream))
     if check:
         _check(code, "l2a_decode")
     return code
@@ -180,8 +204,8 @@ def l2a_decode(p, q, K, V, d, O, ws, stream=None, check=True) -> int:
 
 def l2a_router_logits(p, S, w, bias, logits, sum_sq=None, stream=None, check=True) -> int:
     """Router logits z_t = w . s_t + bias from the local output (Eq. 3); optional sum of sigmoid(z)^2 per batch entry."""
-    code = lib().l2a_router_logits(ctypes.byref(p), _ptr(S), _ptr(w), ctypes.c_float(bias), _ptr(logits), _ptr(sum_sq),
-                                   _stream(stream))
+    code = lib().l2a_router_logits(ctypes.byref(p), _addr(S), _addr(w), bias, _addr(logits), _addr(sum_sq),
+                                   _raw_stream(stream))
     if check:
         _check(code, "l2a_router_logits")
     return code
@@ -189,11 +213,9 @@ def l2a_router_logits(p, S, w, bias, logits, sum_sq=None, stream=None, check=Tru
 
 def l2a_forward(p, Q, K, V, d_mask, q_idx, n_routed, prefix, O, S_save, A_c, lse_loc, lse_glb, fwd_ws,
                 stream=None, check=True) -> int:
-    code = lib().l2a_forward(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(d_mask), _ptr(q_idx), _ptr(n_routed),
-                             _ptr(prefix), _ptr(O), _ptr(S_save), _ptr(A_c), _ptr(lse_loc), _ptr(lse_glb),
-                             _ptr(fwd_ws),
-                             ctypes.c_size_t(fwd_ws.numel() * fwd_ws.element_size() if fwd_ws is not None else 0),
-                             _stream(stream))
+    code = lib().l2a_forward(ctypes.byref(p), _addr(Q), _addr(K), _addr(V), _addr(d_mask), _addr(q_idx), _addr(n_routed),
+                             _addr(prefix), _addr(O), _addr(S_save), _addr(A_c), _addr(lse_loc), _addr(lse_glb),
+                             _addr(fwd_ws), _bytes(fwd_ws), _raw_stream(stream))
     if check:
         _check(code, "l2a_forward")
     return code
@@ -201,26 +223,20 @@ def l2a_forward(p, Q, K, V, d_mask, q_idx, n_routed, prefix, O, S_save, A_c, lse
 
 def l2a_backward(p, Q, K, V, d_mask, q_idx, n_routed, prefix, dO, S_save, A_c, lse_loc, lse_glb, dQ, dK, dV,
                  dgate, bwd_ws, stream=None, check=True) -> int:
-    code = lib().l2a_backward(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(d_mask), _ptr(q_idx),
-                              _ptr(n_routed), _ptr(prefix), _ptr(dO), _ptr(S_save), _ptr(A_c), _ptr(lse_loc),
-                              _ptr(lse_glb), _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(dgate), _ptr(bwd_ws),
-                              ctypes.c_size_t(bwd_ws.numel() * bwd_ws.element_size() if bwd_ws is not None else 0),
-                              _stream(stream))
+    code = lib().l2a_backward(ctypes.byref(p), _addr(Q), _addr(K), _addr(V), _addr(d_mask), _addr(q_idx),
+                              _addr(n_routed), _addr(prefix), _addr(dO), _addr(S_save), _addr(A_c), _addr(lse_loc),
+                              _addr(lse_glb), _addr(dQ), _addr(dK), _addr(dV), _addr(dgate), _addr(bwd_ws), _bytes(bwd_ws), _raw_stream(stream))
     if check:
         _check(code, "l2a_backward")
     return code
 
 
-def _nbytes(t):
-    return ctypes.c_size_t(t.numel() * t.element_size() if t is not None else 0)
-
-
 def l2a_forward_sets(p, Q, K, V, Qg, Kg, Vg, d_mask, q_idx, n_routed, prefix, O, S_save, A_c, lse_loc, lse_glb, fwd_ws,
                      stream=None, check=True) -> int:
     """l2a_forward with a second Q/K/V set for the Global Attention module (None, None, None = one set)."""
-    code = lib().l2a_forward_sets(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(Qg), _ptr(Kg), _ptr(Vg), _ptr(d_mask),
-                                  _ptr(q_idx), _ptr(n_routed), _ptr(prefix), _ptr(O), _ptr(S_save), _ptr(A_c),
-                                  _ptr(lse_loc), _ptr(lse_glb), _ptr(fwd_ws), _nbytes(fwd_ws), _stream(stream))
+    code = lib().l2a_forward_sets(ctypes.byref(p), _addr(Q), _addr(K), _addr(V), _addr(Qg), _addr(Kg), _addr(Vg), _addr(d_mask),
+                                  _addr(q_idx), _addr(n_routed), _addr(prefix), _addr(O), _addr(S_save), _addr(A_c),
+                                  _addr(lse_loc), _addr(lse_glb), _addr(fwd_ws), _bytes(fwd_ws), _raw_stream(stream))
     if check:
         _check(code, "l2a_forward_sets")
     return code
@@ -229,10 +245,10 @@ def l2a_forward_sets(p, Q, K, V, Qg, Kg, Vg, d_mask, q_idx, n_routed, prefix, O,
 def l2a_backward_sets(p, Q, K, V, Qg, Kg, Vg, d_mask, q_idx, n_routed, prefix, dO, S_save, A_c, lse_loc, lse_glb, dQ, dK,
                       dV, dQg, dKg, dVg, dgate, bwd_ws, stream=None, check=True) -> int:
     """l2a_backward with a second Q/K/V set: gradients of the local module's set and of the global module's set."""
-    code = lib().l2a_backward_sets(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(Qg), _ptr(Kg), _ptr(Vg),
-                                   _ptr(d_mask), _ptr(q_idx), _ptr(n_routed), _ptr(prefix), _ptr(dO), _ptr(S_save),
-                                   _ptr(A_c), _ptr(lse_loc), _ptr(lse_glb), _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(dQg),
-                                   _ptr(dKg), _ptr(dVg), _ptr(dgate), _ptr(bwd_ws), _nbytes(bwd_ws), _stream(stream))
+    code = lib().l2a_backward_sets(ctypes.byref(p), _addr(Q), _addr(K), _addr(V), _addr(Qg), _addr(Kg), _addr(Vg),
+                                   _addr(d_mask), _addr(q_idx), _addr(n_routed), _addr(prefix), _addr(dO), _addr(S_save),
+                                   _addr(A_c), _addr(lse_loc), _addr(lse_glb), _addr(dQ), _addr(dK), _addr(dV), _addr(dQg),
+                                   _addr(dKg), _addr(dVg), _addr(dgate), _addr(bwd_ws), _bytes(bwd_ws), _raw_stream(stream))
     if check:
         _check(code, "l2a_backward_sets")
     return code
@@ -241,12 +257,10 @@ def l2a_backward_sets(p, Q, K, V, Qg, Kg, Vg, d_mask, q_idx, n_routed, prefix, d
 def l2a_backward_split(p, Q, K, V, d_mask, q_idx, n_routed, prefix, dO, dS_loc, S_save, A_c, lse_loc, lse_glb, dQ,
                        dK, dV, dgate, bwd_ws, stream=None, check=True) -> int:
     """l2a_backward with a separate gradient dS_loc for the local output (dO + the router path)."""
-    code = lib().l2a_backward_split(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(d_mask), _ptr(q_idx),
-                                    _ptr(n_routed), _ptr(prefix), _ptr(dO), _ptr(dS_loc), _ptr(S_save), _ptr(A_c),
-                                    _ptr(lse_loc), _ptr(lse_glb), _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(dgate),
-                                    _ptr(bwd_ws),
-                                    ctypes.c_size_t(bwd_ws.numel() * bwd_ws.element_size() if bwd_ws is not None else 0),
-                                    _stream(stream))
+    code = lib().l2a_backward_split(ctypes.byref(p), _addr(Q), _addr(K), _addr(V), _addr(d_mask), _addr(q_idx),
+                                    _addr(n_routed), _addr(prefix), _addr(dO), _addr(dS_loc), _addr(S_save), _addr(A_c),
+                                    _addr(lse_loc), _addr(lse_glb), _addr(dQ), _addr(dK), _addr(dV), _addr(dgate),
+                                    _addr(bwd_ws), _bytes(bwd_ws), _raw_stream(stream))
     if check:
         _check(code, "l2a_backward_split")
     return code
@@ -255,9 +269,9 @@ def l2a_backward_split(p, Q, K, V, d_mask, q_idx, n_routed, prefix, dO, dS_loc, 
 def l2a_router_backward(p, S, w, logits, dgate, reg_coeff, dO=None, dz=None, dw=None, dbias=None, dS_loc=None,
                         stream=None, check=True) -> int:
     """Router backward (Eq. 7 + regulariser gradient): dz, dw, dbias and dS_loc = dO + dz * w."""
-    code = lib().l2a_router_backward(ctypes.byref(p), _ptr(S), _ptr(w), _ptr(logits), _ptr(dgate),
-                                     ctypes.c_float(reg_coeff), _ptr(dO), _ptr(dz), _ptr(dw), _ptr(dbias),
-                                     _ptr(dS_loc), _stream(stream))
+    code = lib().l2a_router_backward(ctypes.byref(p), _addr(S), _addr(w), _addr(logits), _addr(dgate),
+                                     reg_coeff, _addr(dO), _addr(dz), _addr(dw), _addr(dbias),
+                                     _addr(dS_loc), _raw_stream(stream))
     if check:
         _check(code, "l2a_router_backward")
     return code
@@ -287,10 +301,6 @@ class DeviceIO(ctypes.Structure):
         ("route_ws", ctypes.c_void_p), ("route_ws_bytes", ctypes.c_size_t),
         ("fwd_ws", ctypes.c_void_p), ("fwd_ws_bytes", ctypes.c_size_t),
         ("bwd_ws", ctypes.c_void_p), ("bwd_ws_bytes", ctypes.c_size_t)]
-
-
-def _addr(t):
-    return None if t is None else (t.data_ptr() if isinstance(t, torch.Tensor) else int(t))
 
 
 def l2a_step_host(p, host: dict, bufs: "Buffers", router_kind=ROUTER_MASK_U8, logit_threshold=0.0, stream=None,

@@ -60,6 +60,8 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(const bf16* __restrict__
   const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const bool split = dO_loc != dO;                     // separate gradient for the local output
+  dependency_wait();
+  dependents_release();
   const int sub = lane / kLanesPerHead;                // head inside the pass
   const int n_pass = (Hq + kHeadsPerPass - 1) / kHeadsPerPass;
   for (int64_t token = gw; token < n_tokens; token += n_warps) {
@@ -144,6 +146,8 @@ __global__ void __launch_bounds__(256) compact_stat_kernel(const float* __restri
                                                            const int32_t* __restrict__ n_routed, int L, int Hq) {
   const int b = blockIdx.z, h = blockIdx.y;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  dependency_wait();
+  dependents_release();
   if (c < n_routed[b]) {
     const int64_t base = ((int64_t)b * Hq + h) * L;
     by_c[base + c] = by_row[base + q_idx[(int64_t)b * L + c]];
@@ -453,6 +457,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   constexpr int kKSteps = D / 16;
   // Key blocks ascending: most work first.  KV heads outermost lets the CTAs that run together share query tiles in L2;
   // key blocks outermost starts the heaviest blocks of every head first, which a launch of few waves needs.
+  dependency_wait();
+  dependents_release();
   const int rank = kSplit > 1 ? (int)cluster_rank() : 0;
   const int work = blockIdx.x / kSplit, heads = a.B * a.Hkv;
   const int j = a.kb_begin + (a.kb_outermost ? work / heads : work % a.kb_count);
@@ -877,6 +883,8 @@ __global__ void __launch_bounds__(256) dq_zero_kernel(float* __restrict__ acc_lo
                                                       const int32_t* __restrict__ n_routed, int B, int Hq, int n_tiles,
                                                       int tile_floats) {
   const int per = B * Hq * n_tiles;
+  dependency_wait();
+  dependents_release();
   for (int item = blockIdx.x; item < 2 * per; item += gridDim.x) {
     const int which = item >= per, rem = which ? item - per : item;
     float* base = which ? acc_glb : acc_loc;
@@ -899,6 +907,7 @@ __global__ void __launch_bounds__(256) dq_merge_kernel(const float* __restrict__
   constexpr int kChunks = D / 8;             // 16-byte chunks per bf16 row
   constexpr int kRowBytes = D * 2 + 16;      // padded: conflict-free 16-byte accesses down a column
   __shared__ __align__(16) uint8_t tile_s[kTileM * kRowBytes];
+  dependency_wait();
   const int n_tiles = (L + kTileM - 1) / kTileM;
   const int h = blockIdx.x % Hq;
   const int tile = tile_begin + (blockIdx.x / Hq) % tile_count;
@@ -978,29 +987,35 @@ int dq_final_tiles(int split, int q_pos_offset, int n_tiles) {
 
 template <int D, int kSplit>
 cudaError_t launch_bwd_split(const BwdArgs& a, const CUtensorMap& mapQ, const CUtensorMap& mapDO, const CUtensorMap& mapQc,
-                             const CUtensorMap& mapDOc, const CUtensorMap& mapK, const CUtensorMap& mapV, cudaStream_t s) {
+                             const CUtensorMap& mapDOc, const CUtensorMap& mapK, const CUtensorMap& mapV, bool overlap,
+                             cudaStream_t s) {
   static PerDeviceOnce once;
   cudaError_t e = once.run([] {
     return cudaFuncSetAttribute(bwd_kernel<D, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<D>::kTotal);
   });
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = kSplit; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  if (kSplit == 1)
+    return launch_dependent(bwd_kernel<D, kSplit>, dim3((unsigned)a.kb_count * a.B * a.Hkv), kDkvThreads, BwdSmem<D>::kTotal, s,
+                            overlap, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, a);
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kSplit; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)a.kb_count * a.B * a.Hkv * kSplit);
   cfg.blockDim = dim3(kDkvThreads);
   cfg.dynamicSmemBytes = BwdSmem<D>::kTotal;
   cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = kSplit > 1 ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = overlap ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, bwd_kernel<D, kSplit>, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, a);
 }
 
 template <int D>
 cudaError_t launch_bwd_kernel(BwdArgs a, const CUtensorMap& mapQ, const CUtensorMap& mapDO, const CUtensorMap& mapQc,
                               const CUtensorMap& mapDOc, const CUtensorMap& mapK, const CUtensorMap& mapV, int sms,
-                              cudaStream_t s) {
+                              bool overlap, cudaStream_t s) {
   // (of the whole sequence, also when the launch is one of several key-block ranges: the results stay the same)
   const int64_t blocks = (int64_t)((a.Lk + kTileN - 1) / kTileN) * a.B * a.Hkv;
   // A cluster per key block where one CTA per block leaves SMs idle or the heaviest block sets the time.  Measured, whole
@@ -1010,9 +1025,9 @@ cudaError_t launch_bwd_kernel(BwdArgs a, const CUtensorMap& mapQ, const CUtensor
   // Below eight waves the heaviest key blocks of every head go first (two sequences of 4096 tokens, 256 blocks: 1.20 ->
   // 0.93 ms); with more waves the tail is short and either order measures the same, so the one with less L2 traffic stays.
   a.kb_outermost = blocks < 8 * sms;
-  return split == 1   ? launch_bwd_split<D, 1>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, s)
-         : split == 2 ? launch_bwd_split<D, 2>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, s)
-                      : launch_bwd_split<D, 4>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, s);
+  return split == 1   ? launch_bwd_split<D, 1>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, overlap, s)
+         : split == 2 ? launch_bwd_split<D, 2>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, overlap, s)
+                      : launch_bwd_split<D, 4>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, overlap, s);
 }
 
 template <int D>
@@ -1022,8 +1037,10 @@ cudaError_t launch_bwd(const BwdArgs& base, const CUtensorMap& mapQ, const CUten
   const DeviceInfo* dev = device_info();
   if (dev == nullptr) return cudaErrorUnknown;
   const int n_tiles = (base.Lq + kTileM - 1) / kTileM;
-  dq_zero_kernel<<<dev->sms * 8, 256, 0, s>>>(base.dq_acc_loc, base.dq_acc_glb, base.n_routed, base.B, base.Hq, n_tiles,
-                                              kTileM * D);
+  const bool overlap = phase_events().n == 0;    // (events between the launches ask for their times one after the other)
+  cudaError_t err = launch_dependent(dq_zero_kernel, dim3(dev->sms * 8), 256, 0, s, overlap, base.dq_acc_loc, base.dq_acc_glb,
+                                     base.n_routed, base.B, base.Hq, n_tiles, kTileM * D);
+  if (err != cudaSuccess) return err;
   phase_events().mark(s);
   const int n_kblocks = (base.Lk + kTileN - 1) / kTileN;
   // A caller that registered phase events for key-block ranges wants the gradients of the early rows while the rest is
@@ -1036,14 +1053,15 @@ cudaError_t launch_bwd(const BwdArgs& base, const CUtensorMap& mapQ, const CUten
     const int kb_end = part + 1 < n_ranges ? first[part + 1] : n_kblocks;
     a.kb_begin = first[part];
     a.kb_count = kb_end - first[part];
-    const cudaError_t e = launch_bwd_kernel<D>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, dev->sms, s);
+    const cudaError_t e = launch_bwd_kernel<D>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, dev->sms, overlap, s);
     if (e != cudaSuccess) return e;
     phase_events().mark(s);
     const int t1 = part + 1 < n_ranges ? dq_final_tiles(kb_end, base.q_pos_offset, n_tiles) : n_tiles;
-    if (t1 > t_done)
-      dq_merge_kernel<D><<<(unsigned)((t1 - t_done) * base.B * base.Hq), 256, 0, s>>>(
-          base.dq_acc_loc, base.dq_acc_glb, d_mask, base.prefix, base.dQ, base.B, base.Lq, base.Hq, base.scale,
-          base.dq_st.b, base.dq_st.t, t_done, t1 - t_done, base.status);
+    if (t1 > t_done &&
+        (err = launch_dependent(dq_merge_kernel<D>, dim3((unsigned)((t1 - t_done) * base.B * base.Hq)), 256, 0, s, overlap,
+                                base.dq_acc_loc, base.dq_acc_glb, d_mask, base.prefix, base.dQ, base.B, base.Lq, base.Hq,
+                                base.scale, base.dq_st.b, base.dq_st.t, t_done, t1 - t_done, base.status)) != cudaSuccess)
+      return err;
     if (t1 > t_done) t_done = t1;
     phase_events().mark(s);
   }
@@ -1162,13 +1180,14 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
 
   PhaseEvents& pe = phase_events();
   struct ClearOnExit { PhaseEvents& p; ~ClearOnExit() { p.clear(); } } clear_on_exit{pe};
+  const bool overlap = pe.n == 0;
   pe.mark(s);
   if (!skip_global) {
     if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s, nullptr, 0,
                            0, qs, reinterpret_cast<int*>(ws)) != cudaSuccess)
       return L2A_ERR_CUDA;
     if (launch_gather_rows(static_cast<const bf16*>(dO), dOc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s, nullptr,
-                           0, 0, os, reinterpret_cast<int*>(ws)) != cudaSuccess)
+                           0, 0, os, reinterpret_cast<int*>(ws), nullptr, 0, overlap) != cudaSuccess)
       return L2A_ERR_CUDA;
   }
   pe.mark(s);
@@ -1180,16 +1199,17 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
     int64_t blocks = (int64_t)dev->sms * (p->D == 128 ? dev->delta_ctas_128 : dev->delta_ctas_64);
     const int64_t max_blocks = ((int64_t)p->B * p->Lq + 7) / 8;
     if (blocks > max_blocks) blocks = max_blocks;
-    kern<<<(unsigned)blocks, 256, 0, s>>>(static_cast<const bf16*>(dO), static_cast<const bf16*>(dS_loc),
-                                          static_cast<const bf16*>(skip_local ? nullptr : S_save),
-                                          static_cast<const bf16*>(A_c), skip_global ? nullptr : d_mask, prefix,
-                                          delta_loc, delta_glb, dgate, p->B, p->Lq, p->Hq,
-                                          force_all ? 1 : 0, os.b, os.t, lse_loc, lse_glb, share ? lse_c : nullptr);
-    if (cudaGetLastError() != cudaSuccess) return L2A_ERR_CUDA;
+    if (launch_dependent(kern, dim3((unsigned)blocks), 256, 0, s, overlap && !skip_global, static_cast<const bf16*>(dO),
+                         static_cast<const bf16*>(dS_loc), static_cast<const bf16*>(skip_local ? nullptr : S_save),
+                         static_cast<const bf16*>(A_c), skip_global ? nullptr : d_mask, prefix, delta_loc, delta_glb, dgate,
+                         p->B, p->Lq, p->Hq, force_all ? 1 : 0, os.b, os.t, lse_loc, lse_glb, share ? lse_c : nullptr) !=
+        cudaSuccess)
+      return L2A_ERR_CUDA;
     if (force_all) {
       dim3 grid((p->Lq + 255) / 256, p->Hq, p->B);
-      compact_stat_kernel<<<grid, 256, 0, s>>>(lse_glb, lse_c, q_idx, n_routed, p->Lq, p->Hq);
-      if (cudaGetLastError() != cudaSuccess) return L2A_ERR_CUDA;
+      if (launch_dependent(compact_stat_kernel, grid, 256, 0, s, overlap, lse_glb, lse_c, q_idx, n_routed, p->Lq, p->Hq) !=
+          cudaSuccess)
+        return L2A_ERR_CUDA;
     }
   }
   BwdArgs a;

@@ -83,6 +83,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   // ---- work item: heaviest first (largest row index first), heads fastest for K/V reuse in L2
   const bool compact = a.global_mode && !a.all_rows;           // rows are compact indices into q_idx
   int item = blockIdx.x, split = 0, n_split = 1, pi;
+  if (a.overlap != 2) dependency_wait();
   if (!a.global_mode) dependents_release();                    // the global pass may fill SMs as this one drains
   if (compact) {
     // the launch covers every row that could be routed; the groups that exist come first
@@ -628,15 +629,6 @@ cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUt
   if (a.pair_end <= a.pair_begin) return cudaSuccess;
   int64_t grid = (int64_t)(a.pair_end - a.pair_begin) * a.Hq * a.B;
   if (a.part != nullptr && grid < kSplitItems) grid = std::min<int64_t>(grid * kMaxKeySplit, kSplitItems);
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kFwdThreads);
-  cfg.stream = stream;
-  cfg.attrs = &attr;
-  cfg.numAttrs = a.overlap ? 1 : 0;
   cudaError_t e;
   if (a.D == 128) {
     static PerDeviceOnce once;
@@ -644,16 +636,16 @@ cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUt
       return cudaFuncSetAttribute(attn_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::kTotal);
     });
     if (e != cudaSuccess) return e;
-    cfg.dynamicSmemBytes = FwdSmem<128>::kTotal;
-    return cudaLaunchKernelEx(&cfg, attn_fwd_kernel<128>, mapQ, mapK, mapV, mapOut, mapOut2, a);
+    return launch_dependent(attn_fwd_kernel<128>, dim3((unsigned)grid), kFwdThreads, FwdSmem<128>::kTotal, stream, a.overlap != 0,
+                            mapQ, mapK, mapV, mapOut, mapOut2, a);
   } else {
     static PerDeviceOnce once;
     e = once.run([] {
       return cudaFuncSetAttribute(attn_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::kTotal);
     });
     if (e != cudaSuccess) return e;
-    cfg.dynamicSmemBytes = FwdSmem<64>::kTotal;
-    return cudaLaunchKernelEx(&cfg, attn_fwd_kernel<64>, mapQ, mapK, mapV, mapOut, mapOut2, a);
+    return launch_dependent(attn_fwd_kernel<64>, dim3((unsigned)grid), kFwdThreads, FwdSmem<64>::kTotal, stream, a.overlap != 0,
+                            mapQ, mapK, mapV, mapOut, mapOut2, a);
   }
 }
 

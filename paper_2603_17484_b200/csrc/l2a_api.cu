@@ -352,13 +352,16 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
 
   PhaseEvents& pe = phase_events();
   struct ClearOnExit { PhaseEvents& p; ~ClearOnExit() { p.clear(); } } clear_on_exit{pe};
+  // (events between the launches ask for times of the passes one after the other)
+  const bool overlap = pe.n == 0;
   pe.mark(s);
   if (!skip_global && !force_all) {
     // consolidate routed query rows (Algorithm 1, step 1); independent of the local pass
     if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s,
                            row_range ? prefix : nullptr, row_begin, row_end, qs, status,
                            gather_clears ? status : part_count,
-                           (int)((gather_clears ? kWsHeaderBytes + kPartCountBytes : kPartCountBytes) / 4)) != cudaSuccess)
+                           (int)((gather_clears ? kWsHeaderBytes + kPartCountBytes : kPartCountBytes) / 4), overlap) !=
+        cudaSuccess)
       return L2A_ERR_CUDA;
   }
   pe.mark(s);
@@ -372,6 +375,7 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
     a.lse = lse_loc;
     a.pair_begin = pair_begin;
     a.pair_end = pair_end;
+    a.overlap = overlap ? 1 : 0;
     CUtensorMap mapOut, mapOut2;
     if (!encode_rows_map(&mapOut, a.out, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, a.out_st.b, a.out_st.t)) return L2A_ERR_CUDA;
     mapOut2 = mapOut;
@@ -402,8 +406,9 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
       a.part = part;
       a.part_count = part_count;
     }
-    // (events between the launches ask for times of the passes one after the other)
-    a.overlap = !skip_local && !global_phase && pe.n == 0;
+    // Behind the local pass the kernel waits only before it combines.  Its other inputs are complete by then: it starts
+    // after every local CTA has, and those wait for the gather and all before it.
+    a.overlap = !overlap ? 0 : !skip_local && !global_phase ? 2 : 1;
     if (force_all) {
       // Global Attention for every token (Section 3.3): same kernel over all rows in place; a_t is stored for
       // every row, and still only enters O where d_t = 1

@@ -30,6 +30,24 @@ __device__ __forceinline__ bool dbg_in_range(bool ok, int* status) {
 __device__ __forceinline__ bool dbg_in_range(bool, int*) { return true; }
 #endif
 
+// Launch that may overlap with the end of the kernel before it on the stream (programmatic dependent launch): for kernels
+// that call dependency_wait() before they touch memory.  overlap = false: a plain launch.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, bool overlap,
+                             A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -84,7 +102,8 @@ cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx,
                                int B, int L, int row_elems, cudaStream_t stream, const int32_t* prefix = nullptr,
                                int row_begin = 0, int row_end = 0, RowStrides src_strides = RowStrides{0, 0},
                                int* status = nullptr,    // status: workspace status word (debug-build index checks)
-                               int32_t* zero = nullptr, int n_zero = 0);   // n_zero words to clear on the way
+                               int32_t* zero = nullptr, int n_zero = 0,    // n_zero words to clear on the way
+                               bool overlap = false);    // may start under the end of the kernel before it
 
 // z[b,t] = w . S[b,t,:] + bias (fp32 accumulation); optional sum over t of sigmoid(z)^2 per batch entry
 cudaError_t launch_router_logits(const bf16* S, const float* w, float bias, float* logits, float* sum_sq, int B,
@@ -124,7 +143,8 @@ struct FwdArgs {
   // sums for every work item of a split launch, and a zeroed counter per group, whose last CTA to finish combines them.
   float* part;
   int32_t* part_count;
-  int overlap;               // launched behind the local pass of the same call: may start before that has finished
+  int overlap;               // programmatic dependent launch; 1: the kernel waits for the one before it at its start, 2 (the
+                             // global pass behind the local one of the same call): only before it combines
 };
 // A global launch of so few groups (256 compact rows of a head) that they leave SMs idle splits their key ranges until it
 // has about two work items for each of the 148 SMs, at most kMaxKeySplit per group and not below kMinSplitBlocks key

@@ -10,6 +10,7 @@
 //                 stride of 64 bytes, took 9.8 us for a block, this 4).
 // Nothing is read back by the host: the routed count stays on the device.
 #include "l2a_common.cuh"
+#include "sm100_prims.cuh"
 
 namespace l2a {
 
@@ -42,6 +43,7 @@ __device__ __forceinline__ int count_block(const RouteArgs& a, int64_t row_base,
 
 __global__ void __launch_bounds__(kThreads) route_count_kernel(RouteArgs a) {
   const int b = blockIdx.y, blk = blockIdx.x;
+  dependents_release();
   const int cnt = __reduce_add_sync(0xffffffffu, count_block(a, (int64_t)b * a.L, blk));
   __shared__ int warp_cnt[kWarps];
   if ((threadIdx.x & 31) == 0) warp_cnt[threadIdx.x >> 5] = cnt;
@@ -58,6 +60,8 @@ __global__ void __launch_bounds__(kThreads) route_scan_kernel(RouteArgs a) {
   const int b = blockIdx.y, blk = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t row_base = (int64_t)b * a.L;
+  if (!kCountAll) dependency_wait();
+  dependents_release();
   __shared__ int red_before[kWarps], red_total[kWarps], warp_cnt[kWarps];
   if (a.header != nullptr && blk == 0 && b == 0 && threadIdx.x < kWsHeaderBytes / 4) a.header[threadIdx.x] = 0;
 
@@ -123,6 +127,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* __restrict
                                                           int64_t src_row_chunks, int* status, int32_t* zero,
                                                           int n_zero) {
   const int b = blockIdx.y;
+  dependency_wait();
+  dependents_release();
   if (blockIdx.x == 0 && b == 0)
     for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0;
   const int n_c = n_routed[b];
@@ -267,22 +273,22 @@ cudaError_t launch_route_compact(const RouteArgs& a, cudaStream_t stream) {
     route_scan_kernel<true><<<grid, kThreads, 0, stream>>>(a);
   } else {
     route_count_kernel<<<grid, kThreads, 0, stream>>>(a);
-    route_scan_kernel<false><<<grid, kThreads, 0, stream>>>(a);
+    const cudaError_t e = launch_dependent(route_scan_kernel<false>, grid, kThreads, 0, stream, true, a);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx, const int32_t* n_routed, int B,
                                int L, int row_elems, cudaStream_t stream, const int32_t* prefix, int row_begin,
-                               int row_end, RowStrides src_strides, int* status, int32_t* zero, int n_zero) {
+                               int row_end, RowStrides src_strides, int* status, int32_t* zero, int n_zero, bool overlap) {
   const int row_chunks = row_elems * 2 / 16;
   const int64_t ts = src_strides.t > 0 ? src_strides.t : row_elems;
   const int64_t bs = src_strides.b > 0 ? src_strides.b : (int64_t)L * ts;
   int gx = L < 148 * 16 ? L : 148 * 16;
   dim3 grid(gx, B);
-  gather_rows_kernel<<<grid, 256, 0, stream>>>(src, dst, q_idx, n_routed, L, row_chunks, prefix, row_begin, row_end,
-                                               bs / 8, ts / 8, status, zero, n_zero);
-  return cudaGetLastError();
+  return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, overlap, src, dst, q_idx, n_routed, L, row_chunks, prefix,
+                          row_begin, row_end, bs / 8, ts / 8, status, zero, n_zero);
 }
 
 }  // namespace l2a

@@ -261,7 +261,8 @@ def run_decode(args):
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / args.steps
     row = cfg.Hkv * cfg.D * 2 * 2                                   # K and V bytes of one cached position
-    alg_bytes = float(B * (cfg.W + 1) * row + int(d_host.sum()) * Lk * row)
+    n_routed = int(d_host.sum())        # a routed sequence's window is part of its cache
+    alg_bytes = float((B - n_routed) * (cfg.W + 1) * row + n_routed * Lk * row)
     peaks = measured_peaks()
     gbs = alg_bytes / ms / 1e6
     print(json.dumps({
@@ -275,7 +276,7 @@ def run_decode(args):
                      # ncu capture of a 4-sequence case: DRAM read + write = 0.9975 x algorithmic bytes; scaled
                      "traffic": 0.9975 * alg_bytes, "traffic_source": "scaled from the 4-sequence ncu capture",
                      "algorithmic_bytes_per_launch": alg_bytes},
-        "gpu_launches": 2 * args.steps}), flush=True)
+        "gpu_launches": args.steps}), flush=True)
 
 
 def run_router(args):

@@ -612,8 +612,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         const int row = row0 + q * 32 + lane;
         const bool valid = row < n_rows;
         const int64_t si = ((int64_t)b * a.Hq + h) * a.Lq + (valid ? row : 0);
-        r_lse[q] = valid ? __ldg(&lse[si]) * kLog2e : 0.f;
-        r_delta[q] = valid ? __ldg(&dl[si]) : 0.f;
+        // (written by launches of this call that this one may overlap with: not through the read-only path)
+        r_lse[q] = valid ? __ldcg(&lse[si]) * kLog2e : 0.f;
+        r_delta[q] = valid ? __ldcg(&dl[si]) : 0.f;
         const int token = valid ? (glb ? __ldg(&a.q_idx[(int64_t)b * a.Lq + row]) : row) : 0;
         r_pos[q] = valid ? token - (glb ? a.vis_shift : 0) + a.q_pos_offset : -1;
         r_lo[q] = (valid && a.seq_bounds != nullptr) ? __ldg(&a.seq_bounds[2 * token]) : -0x40000000;
@@ -897,9 +898,10 @@ __global__ void __launch_bounds__(256) dq_zero_kernel(float* __restrict__ acc_lo
 
 // fp32 dQ accumulators -> bf16 dQ: dQ_t = scale * (local(t) + d_t * global(prefix[t])), for the row tiles
 // [tile_begin, tile_begin + tile_count).  One CTA per (batch, row tile, head); the accumulator blocks are read in their own order (512 contiguous bytes per warp), the bf16 rows leave
-// through shared memory as whole 2 D-byte segments.
+// through shared memory as whole 2 D-byte segments.  (The accumulators are neither __restrict__ nor read with __ldg: the
+// kernel may start while the one before it still adds to them.)
 template <int D>
-__global__ void __launch_bounds__(256) dq_merge_kernel(const float* __restrict__ acc_loc, const float* __restrict__ acc_glb,
+__global__ void __launch_bounds__(256) dq_merge_kernel(const float* acc_loc, const float* acc_glb,
                                                        const uint8_t* __restrict__ d_mask,
                                                        const int32_t* __restrict__ prefix, bf16* __restrict__ dQ, int B,
                                                        int L, int Hq, float scale, int64_t bs, int64_t ts,
@@ -922,7 +924,7 @@ __global__ void __launch_bounds__(256) dq_merge_kernel(const float* __restrict__
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
     if (loc) {
       const float4* p = reinterpret_cast<const float4*>(loc + (q * 4 + rq) * (8 * D) + c * 128 + lane * 4);
-      x = __ldg(p); y = __ldg(p + 32);
+      x = __ldcg(p); y = __ldcg(p + 32);
     }
     if (acc_glb && d_mask[(int64_t)b * L + t]) {
       const int cr = prefix[(int64_t)b * (L + 1) + t];
@@ -930,7 +932,7 @@ __global__ void __launch_bounds__(256) dq_merge_kernel(const float* __restrict__
       const float4* p = reinterpret_cast<const float4*>(
           acc_glb + (((int64_t)b * Hq + h) * n_tiles + (cr >> 7)) * tile_floats + (q * 4 + ((cr & 127) >> 5)) * (8 * D) +
           c * 128 + (cr & 31) * 4);
-      const float4 gx = __ldg(p), gy = __ldg(p + 32);
+      const float4 gx = __ldcg(p), gy = __ldcg(p + 32);
       x.x += gx.x; x.y += gx.y; x.z += gx.z; x.w += gx.w;
       y.x += gy.x; y.y += gy.y; y.z += gy.z; y.w += gy.w;
     }

@@ -117,12 +117,12 @@ __global__ void __launch_bounds__(kThreads) route_scan_kernel(RouteArgs a) {
   }
 }
 
-// One CTA per compact row (grid-stride); 16-byte chunks.
-__global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst,
-                                                          const int32_t* __restrict__ q_idx,
-                                                          const int32_t* __restrict__ n_routed, int L,
+// One CTA per compact row (grid-stride); 16-byte chunks.  No input is __restrict__ or read with __ldg: the kernel may start
+// while the one before it (the routing, or whatever produced the queries) still writes them.
+__global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16* dst, const int32_t* q_idx,
+                                                          const int32_t* n_routed, int L,
                                                           int row_chunks /* 16-byte chunks per row */,
-                                                          const int32_t* __restrict__ prefix, int row_begin,
+                                                          const int32_t* prefix, int row_begin,
                                                           int row_end, int64_t src_batch_chunks,
                                                           int64_t src_row_chunks, int* status, int32_t* zero,
                                                           int n_zero) {
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* __restrict
       const int t = q_idx[(int64_t)b * L + c];
       if (!dbg_in_range(t >= 0 && t < L, status)) continue;
       for (int i = threadIdx.x; i < row_chunks; i += blockDim.x)
-        d[(int64_t)c * row_chunks + i] = __ldg(&s[t * src_row_chunks + i]);
+        d[(int64_t)c * row_chunks + i] = __ldcg(&s[t * src_row_chunks + i]);
     } else {
       for (int i = threadIdx.x; i < row_chunks; i += blockDim.x)
         d[(int64_t)c * row_chunks + i] = make_uint4(0, 0, 0, 0);

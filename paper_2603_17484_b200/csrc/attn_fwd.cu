@@ -83,6 +83,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   // ---- work item: heaviest first (largest row index first), heads fastest for K/V reuse in L2
   const bool compact = a.global_mode && !a.all_rows;           // rows are compact indices into q_idx
   int item = blockIdx.x, split = 0, n_split = 1, pi;
+  // (2: what is read up to the combination was complete before the local pass, a plain launch, started)
   if (a.overlap != 2) dependency_wait();
   if (!a.global_mode) dependents_release();                    // the global pass may fill SMs as this one drains
   if (compact) {

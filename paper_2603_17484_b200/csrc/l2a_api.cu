@@ -375,7 +375,9 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
     a.lse = lse_loc;
     a.pair_begin = pair_begin;
     a.pair_end = pair_end;
-    a.overlap = overlap ? 1 : 0;
+    // Ahead of a global pass that starts under it the local pass is a plain launch: what the global pass reads before its
+    // own wait (routing, compacted queries) is then complete and visible before any kernel it can overlap with starts.
+    a.overlap = overlap && skip_global ? 1 : 0;
     CUtensorMap mapOut, mapOut2;
     if (!encode_rows_map(&mapOut, a.out, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, a.out_st.b, a.out_st.t)) return L2A_ERR_CUDA;
     mapOut2 = mapOut;
@@ -406,8 +408,8 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
       a.part = part;
       a.part_count = part_count;
     }
-    // Behind the local pass the kernel waits only before it combines.  Its other inputs are complete by then: it starts
-    // after every local CTA has, and those wait for the gather and all before it.
+    // Behind the local pass the kernel waits only before it combines.  The local pass is the one kernel it can overlap
+    // with, and a plain launch: the gather and all before it are complete, and visible, before that starts.
     a.overlap = !overlap ? 0 : !skip_local && !global_phase ? 2 : 1;
     if (force_all) {
       // Global Attention for every token (Section 3.3): same kernel over all rows in place; a_t is stored for

@@ -144,7 +144,7 @@ struct FwdArgs {
   float* part;
   int32_t* part_count;
   int overlap;               // programmatic dependent launch; 1: the kernel waits for the one before it at its start, 2 (the
-                             // global pass behind the local one of the same call): only before it combines
+                             // global pass behind the plainly launched local one of the same call): only before it combines
 };
 // A global launch of so few groups (256 compact rows of a head) that they leave SMs idle splits their key ranges until it
 // has about two work items for each of the 148 SMs, at most kMaxKeySplit per group and not below kMinSplitBlocks key

@@ -1,6 +1,7 @@
 """The launches of a step overlap (programmatic dependent launches): captured into a CUDA graph, on a stream of their own,
 and repeated without a synchronisation in between, they give the bits of single calls."""
-import numpy as np
+import ctypes
+
 import pytest
 import torch
 
@@ -54,3 +55,24 @@ def test_captured_step_equals_single_calls(L, Hq, Hkv, flags):
     torch.cuda.synchronize()
     assert l2a.l2a_workspace_status(b.fwd_ws) == 0 and l2a.l2a_workspace_status(b.bwd_ws) == 0
     assert b.check_guards()
+
+
+def test_global_pass_overlaps_only_a_plainly_launched_local_pass():
+    """The global pass reads the routing and the compacted queries before it waits for the local pass.  So the local pass,
+    the only kernel it may overlap with, has to be behind the gather by a full dependency (captured, not run)."""
+    cuda = ctypes.CDLL("libcuda.so.1")
+    c = Case(1, 300, 2, 1, 128, 64, synth.mask_bernoulli(1, 300, 0.3, seed=1), seed=2)
+    stream = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, stream=stream):
+        c.buf.forward()
+    graph = ctypes.c_void_p(g.raw_cuda_graph())
+    n = ctypes.c_size_t(0)
+    assert cuda.cuGraphGetEdges_v2(graph, None, None, None, ctypes.byref(n)) == 0
+    assert n.value == 2                                   # gather -> local -> global
+    src, dst, data = (ctypes.c_void_p * 2)(), (ctypes.c_void_p * 2)(), (ctypes.c_uint8 * 16)()    # 8 bytes an edge
+    assert cuda.cuGraphGetEdges_v2(graph, src, dst, data, ctypes.byref(n)) == 0
+    first = 0 if dst[0] == src[1] else 1
+    assert dst[first] == src[1 - first]
+    assert data[8 * first] == 0                           # from_port: full completion of the gather
+    assert data[8 * (1 - first)] == 1                     # programmatic: the global pass starts under the local one

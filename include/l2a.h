@@ -25,8 +25,10 @@
  *   - Routing is per token and shared by all heads (the router projection has one output, Eq. 3).
  *   - Each call validates its arguments on the host and returns L2A_ERR_* before launching
  *     anything; work is enqueued on `stream` (a cudaStream_t passed as void*; NULL = default).
- *   - Device-side waits are bounded; a wait that runs out is recorded in the workspace's status
- *     word and the kernels finish without writing further results (see l2a_workspace_status).
+ *   - Device-side waits are bounded (the hardware barriers between the CTAs of a cluster are reached behind
+ *     bounded waits only).  A wait that runs out is recorded in the workspace's status word; neither its CTA
+ *     nor another CTA of the launch that needs its part writes results from then on.  The call's later launches
+ *     still run, so that its outputs are not to be used (see l2a_workspace_status).
  */
 #ifndef L2A_H_
 #define L2A_H_
@@ -145,7 +147,10 @@ l2a_status l2a_workspace_bytes(const l2a_params* p, size_t* route_ws_bytes, size
  * never comes, while the other warps wait for something else: the first wait runs out, raises the CTA's abort flag,
  * the other warps leave their waits on seeing it, and the CTA writes the status word of workspace `ws` (any 256-byte
  * aligned device buffer of at least 256 bytes) -- the path every kernel of this library takes when a wait runs
- * out.  Afterwards l2a_workspace_status(ws) returns L2A_ERR_DEVICE_TIMEOUT and the context stays usable.  Nothing
+ * out.  Afterwards l2a_workspace_status(ws) returns L2A_ERR_DEVICE_TIMEOUT and the context stays usable.  The kernel runs
+ * as two clusters of two CTAs with that wait in the first CTA only, and leaves int32 words behind the status word:
+ * [1], [2] CTAs of each cluster that counted their part as done (1, 2), [3], [4] whether one of them would have combined
+ * the parts (0, 1), [5] .. [8] whether each CTA would have stored results behind the exchange (0, 0, 1, 1).  Nothing
  * traps, faults or spins without a limit.  Returns L2A_ERR_INVALID_ARG for a limit outside the range.
  */
 l2a_status l2a_selftest_wait_timeout(void* ws, unsigned limit_us, void* stream);

@@ -526,7 +526,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     // keep its TMEM operand addresses compile-time constants
     __syncthreads();
     if (warp == 17) tmem_dealloc(tmem, 512);
-    if (tid == 0) atomicExch(a.status, 3);
+    if (tid == 0) { atomicExch(a.status, 3); *abort_flag = 1; }
+    if (kSplit > 1) {       // the cluster's other CTAs store into this one's shared memory between the two barriers
+      __syncwarp();
+      cluster_sync();
+      if (tid == 0) share_abort<kSplit>(abort_flag);
+      cluster_sync();
+    }
     return;
   }
 
@@ -854,12 +860,14 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       // sends it its own into a slot of the Q / dO rings, which nobody reads once all products of the cluster are done.
       const int owner = q * kSplit / 4, me = (int)cluster_rank();
       cluster_sync();
+      if (tid == 0) share_abort<kSplit>(abort_flag);
+      __syncwarp();
       if (owner != me)
         send_dkv<D, kSplit>(cluster_map(smem_u32(smem + SM::kQOff), owner) +
                             dkv_slot_offset<D, kSplit>((me - owner + kSplit) % kSplit - 1, q, kr),
                             tmem + lane_base + q * (D / 2), own);
       cluster_sync();
-      ok = ok && owner == me;
+      ok = ok && owner == me && *abort_flag == 0;      // (all CTAs have left their waits: the flag is final)
     }
     if (ok) store_dkv<D, kSplit>(a, smem, tmem + lane_base + q * (D / 2), own, b, g, k0 + kr, q, kr);
   }

@@ -457,7 +457,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       }
       __threadfence();
       named_barrier(1, kSoftmaxWarps * 32);      // (reached by every soft-max warp, also after a wait that ran out)
-      if (tid == 0) bar->last = atomicAdd(&a.part_count[group], 1) == n_split - 1;
+      if (tid == 0) bar->last = arrive_last(&a.part_count[group], n_split, abort_flag);
       named_barrier(1, kSoftmaxWarps * 32);
       ok = ok && bar->last;
       __threadfence();

@@ -252,7 +252,7 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   }
   __threadfence();
   __syncthreads();
-  if (tid == 0) bar->last = atomicAdd(&a.done[b * a.Hkv + g], 1) == (routed ? n_items : a.n_win) - 1;
+  if (tid == 0) bar->last = arrive_last(&a.done[b * a.Hkv + g], routed ? n_items : a.n_win, abort_flag);
   __syncthreads();
   if (bar->last) {
     // ---- the last CTA of the (batch entry, KV head): weight of chunk i in head h's result,

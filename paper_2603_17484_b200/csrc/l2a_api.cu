@@ -150,11 +150,14 @@ namespace l2a {
 namespace {
 // The path a kernel takes when one of its waits runs out, on its own: one warp waits (bounded) for an mbarrier
 // arrival that never comes, the other warps wait for the first one's outcome through the same abort flag, and the
-// CTA records the failure in the status word -- what every kernel of this library does at its end.
-__global__ void __launch_bounds__(128) wait_timeout_selftest_kernel(int* status, uint64_t limit_ns) {
+// CTA records the failure in the status word -- what every kernel of this library does at its end.  Two clusters of two
+// CTAs: in the first CTA of the first one the wait runs out, the second cluster has no such wait.  The words behind the
+// status tell who counted and who went on to store results: see l2a_selftest_wait_timeout in l2a.h.
+__global__ void __cluster_dims__(2) __launch_bounds__(128) wait_timeout_selftest_kernel(int* words, uint64_t limit_ns) {
   __shared__ uint64_t never_arrives;
   __shared__ uint64_t second;
   __shared__ int abort_flag;
+  const int pair = blockIdx.x >> 1;
   if (threadIdx.x == 0) {
     mbar_init(&never_arrives, 1);
     mbar_init(&second, 1);
@@ -164,10 +167,21 @@ __global__ void __launch_bounds__(128) wait_timeout_selftest_kernel(int* status,
   __syncthreads();
   volatile int* af = &abort_flag;
   const uint64_t second_limit = 1000 * limit_ns < kWaitLimitNs ? 1000 * limit_ns : kWaitLimitNs;
-  if (threadIdx.x < 32) mbar_wait(&never_arrives, 0, af, limit_ns);   // gives up after limit_ns, raises the flag
-  else mbar_wait(&second, 0, af, second_limit);                        // leaves as soon as the flag is up
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < 32) mbar_wait(&never_arrives, 0, af, limit_ns);   // gives up after limit_ns, raises the flag
+    else mbar_wait(&second, 0, af, second_limit);                        // leaves as soon as the flag is up
+  }
   __syncthreads();
-  if (threadIdx.x == 0 && abort_flag) atomicExch(status, 1);
+  if (threadIdx.x == 0 && arrive_last(&words[1 + pair], 2, af)) words[3 + pair] = 1;
+  __syncthreads();
+  cluster_sync();
+  if (threadIdx.x == 0) share_abort<2>(af);
+  __syncwarp();
+  cluster_sync();
+  if (threadIdx.x == 0) {
+    if (*af) atomicExch(&words[0], 1);
+    else words[5 + blockIdx.x] = 1;
+  }
 }
 }  // namespace
 }  // namespace l2a
@@ -177,7 +191,7 @@ l2a_status l2a_selftest_wait_timeout(void* ws, unsigned limit_us, void* stream) 
   if (limit_us == 0 || limit_us > 1000000u) return L2A_ERR_INVALID_ARG;   // at most one second
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(ws, 0, l2a::kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
-  l2a::wait_timeout_selftest_kernel<<<1, 128, 0, s>>>(static_cast<int*>(ws), (uint64_t)limit_us * 1000ull);
+  l2a::wait_timeout_selftest_kernel<<<4, 128, 0, s>>>(static_cast<int*>(ws), (uint64_t)limit_us * 1000ull);
   return cudaGetLastError() == cudaSuccess ? L2A_OK : L2A_ERR_CUDA;
 }
 

@@ -194,6 +194,22 @@ __device__ __forceinline__ void cluster_st128(uint32_t addr, uint32_t a, uint32_
                : "memory");
 }
 
+// A wait that ran out in one CTA of a cluster of kCtas concerns all of them: between two cluster barriers that follow every
+// wait, one thread of each CTA passes its CTA's flag on, so that behind the second barrier none stores a result.
+template <int kCtas>
+__device__ __forceinline__ void share_abort(volatile int* abort_flag) {
+  if (*abort_flag == 0) return;
+#pragma unroll
+  for (uint32_t r = 0; r < kCtas; ++r)
+    asm volatile("st.shared::cluster.u32 [%0], 1;" ::"r"(cluster_map(smem_u32(const_cast<int*>(abort_flag)), r)) : "memory");
+}
+
+// Counted arrival of one thread per CTA whose part of a result is in memory: true for the last of n, which combines them.
+// A CTA whose wait ran out does not count, so that nobody combines its part.
+__device__ __forceinline__ bool arrive_last(int* counter, int n, const volatile int* abort_flag) {
+  return *abort_flag == 0 && atomicAdd(counter, 1) == n - 1;
+}
+
 // barrier of `threads` threads of the CTA (id 1 .. 15)
 __device__ __forceinline__ void named_barrier(int id, int threads) {
   asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");

@@ -32,3 +32,12 @@ def test_selftest_argument_checks():
     assert l2a.l2a_selftest_wait_timeout(ws, 0, check=False) == -1
     assert l2a.l2a_selftest_wait_timeout(ws, 2_000_000, check=False) == -1
     assert l2a.l2a_selftest_wait_timeout(None, 10, check=False) == -3
+
+
+def test_nothing_is_stored_from_the_parts_of_a_cta_whose_wait_ran_out():
+    """Neither the CTA that would combine counted parts nor the other CTAs of a cluster go on to store results (the path of
+    the split key ranges, the decode chunks and the backward clusters); a cluster without such a wait does."""
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    l2a.l2a_selftest_wait_timeout(ws, 1000)
+    assert l2a.l2a_workspace_status(ws) == -5
+    assert ws.view(torch.int32)[:9].tolist() == [1, 1, 2, 0, 1, 0, 0, 1, 1]

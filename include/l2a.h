@@ -360,7 +360,9 @@ l2a_status l2a_forward_routed(const l2a_params* p, const void* Q, const void* K,
  *   d           in : uint8 [B] routing decision of the new token (NULL = not routed); device memory.
  *   O           out: bf16 [B, 1, Hq, D].
  *   ws             : device workspace of l2a_decode_workspace_bytes, 256-byte aligned: a status header (read it
- *                    with l2a_workspace_status) and the partial soft-max results of the key chunks.
+ *                    with l2a_workspace_status) and the partial soft-max results of the key chunks.  The size
+ *                    returned for p is enough for every step at p's or a smaller position and batch (other
+ *                    fields alike): a decode loop allocates once, for its full cache.
  * Keys after q_pos_offset are never used, whatever they hold.  A layer whose Global Attention was pruned keeps
  * only its last window + 1 keys: call with d = NULL, Lk = window + 1 slots (q_pos_offset = Lk - 1); the result
  * does not depend on the order of the slots, so the cache may be a ring buffer.  HBM-bound: reads the local window once and, for

@@ -336,16 +336,33 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
 // keys (28/4 heads) 64 / 87 us, two of 40K 27 / 36, six of 100K with one KV head 63 / 84, 16 of 128K with four routed 342
 // (2048 keys at most: 353), 32 of 8000 not routed 90 / 92, one of 9001 16.4 with either.
 constexpr int kChunkTarget = 2 * 148, kChunkMin = 256, kChunkMax = 4096;
+void window_and_rest(const l2a_params* p, int* win, int* out) {
+  *win = std::min(p->q_pos_offset, p->window) + 1;
+  *out = p->q_pos_offset + 1 - *win;
+}
 void plan_chunks(const l2a_params* p, int* n_win, int* n_out) {
-  const int pos = p->q_pos_offset;
-  const int win = (pos < p->window ? pos : p->window) + 1, out = pos + 1 - win;
+  int win, out;
+  window_and_rest(p, &win, &out);
   const int64_t pairs = (int64_t)p->B * p->Hkv;
   auto chunk = [&](int64_t keys) {
     const int64_t per = (keys * pairs + kChunkTarget - 1) / kChunkTarget;
     return (int)(per < kChunkMin ? kChunkMin : (per > kChunkMax ? kChunkMax : (per + kDecKeys - 1) / kDecKeys * kDecKeys));
   };
   *n_win = std::min(ceil_div(win, chunk(win)), kMaxWin);
-  *n_out = std::min(ceil_div(out, chunk(pos + 1)), kMaxOut);
+  *n_out = std::min(ceil_div(out, chunk(win + out)), kMaxOut);
+}
+// Chunks of all (sequence, KV head) pairs at any position up to p's and any batch up to p's: a caller sizes the workspace
+// once, for the full cache, while the plan of a shorter one can have more chunks (its length is rounded to whole tiles).  A
+// chunk has at least kChunkMin keys and at least the share of keys * pairs / kChunkTarget, or kChunkMax.
+int64_t chunks_bound(const l2a_params* p) {
+  int win, out;
+  window_and_rest(p, &win, &out);
+  const int64_t pairs = (int64_t)p->B * p->Hkv;
+  auto bound = [&](int64_t keys, int cap) {
+    const int64_t by_share = std::min(pairs * ((keys + kChunkMin - 1) / kChunkMin), kChunkTarget + pairs);
+    return std::min(std::max(by_share, pairs * ((keys + kChunkMax - 1) / kChunkMax)), pairs * cap);
+  };
+  return bound(win, kMaxWin) + bound(out, kMaxOut);
 }
 
 template <int D, int G>
@@ -384,21 +401,27 @@ using namespace l2a;
 
 static size_t done_bytes(const l2a_params* p) { return align_up((size_t)p->B * p->Hkv * sizeof(int), 256); }
 
-extern "C" l2a_status l2a_decode_workspace_bytes(const l2a_params* p, size_t* ws_bytes) {
+static size_t decode_ws_size(const l2a_params* p, int64_t chunks) {
+  return kWsHeaderBytes + done_bytes(p) + align_up((size_t)chunks * (p->Hq / p->Hkv) * (p->D + 4) * sizeof(float), 256);
+}
+
+static l2a_status check_decode(const l2a_params* p) {
   size_t unused = 0;
-  l2a_status st = l2a_workspace_bytes(p, &unused, nullptr, nullptr);
+  const l2a_status st = l2a_workspace_bytes(p, &unused, nullptr, nullptr);
+  return st != L2A_OK ? st : p->Lq != 1 ? L2A_ERR_INVALID_ARG : L2A_OK;
+}
+
+extern "C" l2a_status l2a_decode_workspace_bytes(const l2a_params* p, size_t* ws_bytes) {
+  const l2a_status st = check_decode(p);
   if (st != L2A_OK) return st;
-  if (!ws_bytes || p->Lq != 1) return L2A_ERR_INVALID_ARG;
-  int nw, no;
-  plan_chunks(p, &nw, &no);
-  *ws_bytes = kWsHeaderBytes + done_bytes(p) + align_up((size_t)p->B * p->Hq * (nw + no) * (p->D + 4) * sizeof(float), 256);
+  if (!ws_bytes) return L2A_ERR_INVALID_ARG;
+  *ws_bytes = decode_ws_size(p, chunks_bound(p));
   return L2A_OK;
 }
 
 extern "C" l2a_status l2a_decode(const l2a_params* p, const void* q, const void* K, const void* V, const uint8_t* d,
                                  void* O, void* ws, size_t ws_bytes, void* stream) {
-  size_t need = 0;
-  l2a_status st = l2a_decode_workspace_bytes(p, &need);
+  const l2a_status st = check_decode(p);
   if (st != L2A_OK) return st;
   if (!q || !K || !V || !O) return L2A_ERR_INVALID_ARG;
   if ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(K) | reinterpret_cast<uintptr_t>(V) |
@@ -407,7 +430,11 @@ extern "C" l2a_status l2a_decode(const l2a_params* p, const void* q, const void*
   if (p->Hq / p->Hkv > kMaxGroup) return L2A_ERR_UNSUPPORTED;
   if (p->seq_bounds) return L2A_ERR_UNSUPPORTED;   // a decode step has one cache per batch entry
   if (p->q_pos_offset >= p->Lk) return L2A_ERR_INVALID_ARG;     // the new token's own key must be in the cache
-  if (!ws || (reinterpret_cast<uintptr_t>(ws) % 256) != 0 || ws_bytes < need) return L2A_ERR_WORKSPACE;
+  DecodeArgs a;
+  plan_chunks(p, &a.n_win, &a.n_out);
+  if (!ws || (reinterpret_cast<uintptr_t>(ws) % 256) != 0 ||
+      ws_bytes < decode_ws_size(p, (int64_t)p->B * p->Hkv * (a.n_win + a.n_out)))
+    return L2A_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(ws, 0, kWsHeaderBytes + done_bytes(p), s) != cudaSuccess) return L2A_ERR_CUDA;   // status, counters
   CUtensorMap mapK, mapV;
@@ -417,12 +444,10 @@ extern "C" l2a_status l2a_decode(const l2a_params* p, const void* q, const void*
   if (!encode_rows_map(&mapK, K, p->B, p->Lk, p->Hkv * p->D, kDecKeys, p->D, ks.b, ks.t) ||
       !encode_rows_map(&mapV, V, p->B, p->Lk, p->Hkv * p->D, kDecKeys, p->D, vs.b, vs.t))
     return L2A_ERR_CUDA;
-  DecodeArgs a;
   a.B = p->B; a.Lk = p->Lk; a.Hq = p->Hq; a.Hkv = p->Hkv; a.G = p->Hq / p->Hkv;
   a.window = p->window;
   a.q_pos = p->q_pos_offset;
   a.scale_log2 = (p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)p->D)) * 1.4426950408889634f;
-  plan_chunks(p, &a.n_win, &a.n_out);
   a.q = static_cast<const bf16*>(q);
   a.d = d;
   a.status = static_cast<int*>(ws);

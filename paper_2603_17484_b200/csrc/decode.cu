@@ -335,7 +335,13 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
 // its launch and a row per head that the last CTA reads back.  Measured against four times as many: one sequence of 128K
 // keys (28/4 heads) 64 / 87 us, two of 40K 27 / 36, six of 100K with one KV head 63 / 84, 16 of 128K with four routed 342
 // (2048 keys at most: 353), 32 of 8000 not routed 90 / 92, one of 9001 16.4 with either.
+// Before the window only routed sequences have work, and the host does not know which are.  Chunks there are no longer than
+// lets ONE routed sequence fill every SM once, but have 1536 keys: the CTAs of the others cost their launch.  Microseconds
+// without this limit / with it (/ with 1024 / 2048 keys): one routed of 16 sequences of 32K (28/4 heads) 68 / 49 (47 / 52),
+// of 32 of 60K (8/1) 59 / 39 (37 / 43), of 16 of 128K (8/1) 50 / 37 (35 / 38); none of 32 of 8000 (32/8) 89 / 91 (102 / 90),
+// none of 16 of 128K (8/1) 18.7 / 21.6 (22.8 / 20.9); all of 16 of 128K (8/1) 170 / 179 (184 / 176).
 constexpr int kChunkTarget = 2 * 148, kChunkMin = 256, kChunkMax = 4096;
+constexpr int kSoloTarget = 148, kSoloMin = 1536;
 void window_and_rest(const l2a_params* p, int* win, int* out) {
   *win = std::min(p->q_pos_offset, p->window) + 1;
   *out = p->q_pos_offset + 1 - *win;
@@ -344,25 +350,28 @@ void plan_chunks(const l2a_params* p, int* n_win, int* n_out) {
   int win, out;
   window_and_rest(p, &win, &out);
   const int64_t pairs = (int64_t)p->B * p->Hkv;
-  auto chunk = [&](int64_t keys) {
-    const int64_t per = (keys * pairs + kChunkTarget - 1) / kChunkTarget;
-    return (int)(per < kChunkMin ? kChunkMin : (per > kChunkMax ? kChunkMax : (per + kDecKeys - 1) / kDecKeys * kDecKeys));
+  auto chunk = [](int64_t keys, int target, int least) {     // keys over `target` chunks
+    const int64_t per = (keys + target - 1) / target;
+    return (int)(per < least ? least : (per > kChunkMax ? kChunkMax : (per + kDecKeys - 1) / kDecKeys * kDecKeys));
   };
-  *n_win = std::min(ceil_div(win, chunk(win)), kMaxWin);
-  *n_out = std::min(ceil_div(out, chunk(win + out)), kMaxOut);
+  *n_win = std::min(ceil_div(win, chunk(win * pairs, kChunkTarget, kChunkMin)), kMaxWin);
+  const int solo = chunk((int64_t)(win + out) * p->Hkv, kSoloTarget, kSoloMin);
+  *n_out = std::min(ceil_div(out, std::min(solo, chunk((win + out) * pairs, kChunkTarget, kChunkMin))), kMaxOut);
 }
 // Chunks of all (sequence, KV head) pairs at any position up to p's and any batch up to p's: a caller sizes the workspace
 // once, for the full cache, while the plan of a shorter one can have more chunks (its length is rounded to whole tiles).  A
-// chunk has at least kChunkMin keys and at least the share of keys * pairs / kChunkTarget, or kChunkMax.
+// chunk has at least kChunkMin keys and at least the share of keys * pairs / kChunkTarget, or kChunkMax; before the window
+// it may also have kSoloMin keys, and at least the share of keys * Hkv / kSoloTarget.
 int64_t chunks_bound(const l2a_params* p) {
   int win, out;
   window_and_rest(p, &win, &out);
   const int64_t pairs = (int64_t)p->B * p->Hkv;
-  auto bound = [&](int64_t keys, int cap) {
-    const int64_t by_share = std::min(pairs * ((keys + kChunkMin - 1) / kChunkMin), kChunkTarget + pairs);
-    return std::min(std::max(by_share, pairs * ((keys + kChunkMax - 1) / kChunkMax)), pairs * cap);
+  auto chunks = [&](int64_t keys, int length) { return pairs * ((keys + length - 1) / length); };
+  auto bound = [&](int64_t keys) {
+    return std::max(std::min(chunks(keys, kChunkMin), kChunkTarget + pairs), chunks(keys, kChunkMax));
   };
-  return bound(win, kMaxWin) + bound(out, kMaxOut);
+  const int64_t solo = std::min(chunks(out, kSoloMin), (int64_t)p->B * (kSoloTarget + p->Hkv));
+  return std::min(bound(win), pairs * kMaxWin) + std::min(std::max(bound(out), solo), pairs * kMaxOut);
 }
 
 template <int D, int G>

@@ -3,7 +3,8 @@
 // o = s + d * a.  The work is one pass over the K/V cache: HBM-bound.  The cache of every KV head is cut at the window's
 // first key and split into chunks processed by independent CTAs; a chunk's partial soft-max (acc, max, sum) inside the
 // window serves both modules, those before it exist for routed tokens only.  The CTA of a (sequence, KV head) that
-// finishes last combines the chunks: o is one weighted sum of their accumulators.
+// finishes last combines the chunks: o is one weighted sum of their accumulators.  A single chunk stores its result itself
+// (a window of 129 keys, 28/4 heads, not routed, calls back to back: 12.3 us through the combination, 8.3 without).
 //
 // One CTA = one chunk of keys of one (batch entry, KV head), for all G query heads of the group:
 //   producer warp : streams 64-key K and V tiles through a ring of shared-memory stages with TMA (one 4-D copy
@@ -233,6 +234,7 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   }
   __syncthreads();
   const int n_items = a.n_win + a.n_out;
+  const bool single = (routed ? n_items : a.n_win) == 1;       // nothing to combine: the result goes straight out
   constexpr int kRow = D + 4;
   float* base = a.part + ((int64_t)b * a.Hkv + g) * n_items * (G * kRow);
   for (int i = tid; i < G * D; i += kDecThreads) {
@@ -246,15 +248,23 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
       L += red_l[w * G + h] * f;
       A += red_acc[(w * G + h) * D + col] * f;
     }
+    if (single) {
+      float w = 1.f / L;
+      if (routed) w += 1.f / L;        // window and whole cache are the same keys
+      if (bar->abort_flag == 0) a.O[((int64_t)b * a.Hq + g * G + h) * D + col] = __float2bfloat16(w * A);
+      continue;
+    }
     float* dst = base + (item * G + h) * kRow;
     dst[col] = A;
     if (col == 0) { dst[D] = M; dst[D + 1] = L; }
   }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) bar->last = arrive_last(&a.done[b * a.Hkv + g], routed ? n_items : a.n_win, abort_flag);
-  __syncthreads();
-  if (bar->last) {
+  if (!single) {
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) bar->last = arrive_last(&a.done[b * a.Hkv + g], routed ? n_items : a.n_win, abort_flag);
+    __syncthreads();
+  }
+  if (!single && bar->last) {
     // ---- the last CTA of the (batch entry, KV head): weight of chunk i in head h's result,
     //   o = sum_win acc_i 2^(m_i - M_win) / L_win + d * sum_all acc_i 2^(m_i - M_all) / L_all
     __threadfence();

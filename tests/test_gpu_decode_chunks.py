@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
     (3, 1281, 8, 2, 64, 255),        # whole chunks of 256 on both sides
     (5, 1300, 16, 4, 128, 300),      # ragged last chunks
     (1, 5000, 3, 3, 64, 4096),
+    (3, 256, 14, 2, 128, 4096),      # a single chunk, routed or not
+    (2, 400, 8, 1, 64, 128),         # a single chunk when not routed, two when routed
 ])
 def test_chunks_around_the_window(B, Lk, Hq, Hkv, D, W):
     t = synth.qkv(B, 1, Hq, Hkv, D, seed=Lk + W, Lk=Lk)

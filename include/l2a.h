@@ -233,7 +233,10 @@ l2a_status l2a_router_logits(const l2a_params* p, const void* S, const float* w,
  *                    Both lse outputs may be NULL unless L2A_FLAG_SAVE_FOR_BWD is set.
  *   fwd_ws         : workspace of at least fwd_ws_bytes (holds the compact query buffer Q_c).
  * Scores and soft-max run in fp32, probabilities are rounded to bf16 for the second contraction,
- * accumulation is fp32.  Returns L2A_ERR_UNSUPPORTED for D not in {64, 128}.
+ * accumulation is fp32.  Results are bit-reproducible; with few routed rows in the call the keys of a routed row
+ * are split into parts (a function of Lq, Hq, B and the largest n_routed), each of which rounds its probabilities
+ * against its own running maximum, so that the routed rows of the same sequence in another batch can differ by
+ * that rounding.  Returns L2A_ERR_UNSUPPORTED for D not in {64, 128}.
  */
 l2a_status l2a_forward(const l2a_params* p, const void* Q, const void* K, const void* V,
                        const uint8_t* d_mask, const int32_t* q_idx, const int32_t* n_routed,
@@ -261,7 +264,9 @@ l2a_status l2a_forward(const l2a_params* p, const void* Q, const void* K, const 
  *   dQ          out: bf16 [B, Lq, Hq, D].  The contributions of the key blocks meet in fp32 accumulators in the
  *                    workspace through atomic additions, in no fixed order: two runs agree to fp32 rounding of
  *                    the sums (and almost always bit for bit after the bf16 rounding), not by construction.
- *   dK, dV      out: bf16 [B, Lk, Hkv, D].  Accumulated on chip in a fixed order: bit-reproducible.
+ *   dK, dV      out: bf16 [B, Lk, Hkv, D].  Accumulated on chip in a fixed order: bit-reproducible.  (The order
+ *                    follows from B * Hkv * ceil(Lk / 128): the same sequence in another batch, or its heads in
+ *                    several calls, can differ by the rounding of fp32 sums.)
  *   dgate       out: optional fp32 [B, Lq] (may be NULL): sum over heads of dO_t . a_t -- the
  *                    loss-dependent term of the straight-through router gradient (Eq. 7) -- for
  *                    the rows whose global output was computed: routed rows (0 elsewhere), or

@@ -178,3 +178,14 @@ def check_same_or_rounding(a: torch.Tensor, b: torch.Tensor, what: str):
     assert bool((diff <= step).all()), (what, float((diff / step).max()))
     frac = float((diff > 0).float().mean())
     assert frac <= 1e-2, (what, "fraction of differing elements", frac)
+
+
+def check_same_split(a: torch.Tensor, b: torch.Tensor, V: torch.Tensor, what: str):
+    """Attention outputs of two calls that split the key range differently: a part rounds its probabilities to bf16 against
+    its own running maximum, so each side is off by at most 2^-9 sum_j p_j |v_j| <= 2^-9 max|v| from that and by 2^-9 |o|
+    from the rounding of the result (twice where a is added to s), the two sides by twice that.  In the 2-norm the
+    roundings, independent and of relative size 2^-9 at most, stay below 2^-8."""
+    x, y = a.double(), b.double()
+    bound = 2.0 ** -8 * float(V.float().abs().max()) + 2.0 ** -7 * torch.maximum(x.abs(), y.abs())
+    assert bool(((x - y).abs() <= bound).all()), (what, float(((x - y).abs() / bound).max()))
+    assert float((x - y).norm()) <= 2.0 ** -8 * float(y.norm()), (what, float((x - y).norm() / y.norm()))

@@ -1,20 +1,33 @@
 """Head-parallel sharding needs no exchange on the attention path: a rank that owns the KV heads [g0, g1) and their
 query heads calls the same entry points on slices of the tensors (the head stride stays D, the token stride is the
-full row), and gets exactly the columns the whole call writes.  Run here as two shards on one GPU."""
+full row), and gets the columns the whole call writes: exactly where both calls share key blocks among as many CTAs and
+split key ranges alike (which follows from their numbers of key blocks and of groups of routed rows, so from the heads),
+up to rounding elsewhere.  Run here as two shards on one GPU."""
 import numpy as np
 import pytest
 import torch
 
 from paper_2603_17484_b200 import l2a, synth
-from tests.gpu_util import check_same_or_rounding, Case, run_backward
+from tests.gpu_util import check_same_or_rounding, check_same_split, Case, run_backward
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("extra", [0, l2a.FLAG_SHARED_WINDOW], ids=["plain", "shared_window"])
 def test_two_head_shards_equal_the_whole_layer(extra):
-    B, L, Hq, Hkv, D, W = 2, 900, 8, 4, 128, 160
-    d = synth.mask_bernoulli(B, L, 0.3, seed=11)
+    _two_shards(2, 900, 8, 4, 128, 160, 0.3, extra, "nothing")
+
+
+@pytest.mark.parametrize("B,L,Hq,Hkv,D,rho,differs", [
+    (1, 1500, 8, 8, 64, 0.3, "backward"),     # 96 key blocks: two CTAs each; 48 in a shard: four
+    (1, 4500, 32, 2, 64, 0.2, "forward"),     # 128 groups of routed rows: no split; 64 in a shard: two parts from 32 key blocks on
+])
+def test_two_head_shards_across_the_lines_of_the_plan(B, L, Hq, Hkv, D, rho, differs):
+    _two_shards(B, L, Hq, Hkv, D, 160, rho, 0, differs)
+
+
+def _two_shards(B, L, Hq, Hkv, D, W, rho, extra, differs):
+    d = synth.mask_bernoulli(B, L, rho, seed=11)
     c = Case(B, L, Hq, Hkv, D, W, d, seed=13, backward=True, flags=extra)
     c.run_forward()
     run_backward(c, with_dgate=True)
@@ -45,8 +58,11 @@ def test_two_head_shards_equal_the_whole_layer(extra):
         torch.cuda.synchronize()
         assert l2a.l2a_workspace_status(fwd_ws) == 0 and l2a.l2a_workspace_status(bwd_ws) == 0
         dgate += part      # the gate gradient sums over heads: the one value ranks would have to add up
+    if differs == "forward":
+        check_same_split(out["O"], whole["O"], b.V, "O")     # (the gradients then see another A_c)
+        return
     for k in out:
-        if k == "dQ":      # summed over the key blocks with fp32 atomics: order not fixed
+        if k == "dQ" or (differs == "backward" and k != "O"):   # dQ: summed over the key blocks with fp32 atomics: order not fixed
             check_same_or_rounding(out[k], whole[k], k)
         else:
             assert torch.equal(out[k].view(torch.int16), whole[k].view(torch.int16)), k

@@ -30,9 +30,10 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 // 2^x for two values on the FMA pipe, for x <= 127: x = n + f with n the nearest whole number (adding 1.5 * 2^23 + 127
-// leaves n + 127 in the low bits) and |f| <= 1/2; 2^f by a polynomial of degree 5 fitted for the least relative error, 2^n
-// from the exponent bits.  Relative error at most 2.2e-7, below the 2^-22 that ex2.approx is specified to; results under
-// 2^-126 are zero, as there, and NaN stays NaN.
+// leaves n + 127 in the low bits) and |f| <= 1/2; 2^f by the polynomial of degree 5 of the least relative error (Remez
+// exchange, rounded to fp32), 2^n from the exponent bits.  Relative error at most 2.2e-7, below the 2^-22 that ex2.approx is
+// specified to (tests/test_exp2_fma.py).  Results up to 2^-126.5 are zero, between that and 2^-126 subnormal
+// (ex2.approx.ftz gives zero there); NaN stays NaN.
 __device__ __forceinline__ float max_nan(float a, float b) {
   float d;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));

@@ -602,7 +602,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     // lse * log2(e) and Delta of the item's 128 query rows, plus per-quarter mask flags, go to shared memory.
     // The global loads of item i+1 are issued before waiting for its slot, so their latency is hidden.
     float r_lse[4], r_delta[4];
-    int r_pos[4], r_lo[4], r_glb = 0, r_row0 = 0, r_h = 0;   // r_lo: first token of the row's sequence (packed batches)
+    int r_pos[4], r_lo[4], r_glb = 0, r_row0 = 0;   // r_lo: first token of the row's sequence (packed batches)
     ItemCursor<kSplit> cur(plan, g * G, rank);
     auto load_item = [&]() {
       const int h = cur.h(), glb = cur.glb(), row0 = cur.tile() * kTileM;
@@ -612,7 +612,6 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       const float* dl = glb ? a.delta_glb : a.delta_loc;
       r_glb = glb;
       r_row0 = row0;
-      r_h = h;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int row = row0 + q * 32 + lane;
@@ -644,7 +643,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         const bool interior = __all_sync(0xffffffffu, lane_ok);
         if (lane == 0) st_flags[q] = interior ? 0 : 1;
       }
-      if (lane == 0) { st_flags[4] = r_glb; st_flags[5] = r_row0; st_flags[6] = r_h; }
+      if (lane == 0) { st_flags[4] = r_glb; st_flags[5] = r_row0; }
       __syncwarp();
       mbar_arrive(&bar->st_full[s]);
       if (i + 1 < count) load_item();

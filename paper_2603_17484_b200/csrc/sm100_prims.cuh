@@ -84,14 +84,6 @@ __device__ __forceinline__ float4 lds128(uint32_t saddr) {
   return v;
 }
 
-// Packs two fp32 values to bf16x2 with integer arithmetic (add half an ulp, keep the upper halves): round to
-// nearest with ties away from zero.  Used for the MMA operands P and dS, so that these conversions run on the
-// integer pipe instead of competing with ex2 for the special-function unit (where cvt executes).  Results
-// that go to memory use pack_bf16 (round to nearest even).
-__device__ __forceinline__ uint32_t pack_bf16_fast(float lo, float hi) {
-  return __byte_perm(__float_as_uint(lo) + 0x8000u, __float_as_uint(hi) + 0x8000u, 0x7632);
-}
-
 // ----------------------------------------------------------------------------------------------
 // mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -227,14 +219,6 @@ __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
-__device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int c0,
-                                            int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-      ::"r"(smem_u32(smem_dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
-      : "memory");
-}
-
 __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int c0,
                                             int c1, int c2, int c3) {
   asm volatile(
@@ -269,7 +253,7 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // The issuing loop runs in ONE thread, entered through `if (elect_one())`: the compiler then knows the branch to be
-// uniform and keeps the descriptors in uniform registers.  Issue takes about 25 clk per tcgen05.mma that way, against
+// uniform and keeps the descriptors in uniform registers.  Issue takes 27 clk per tcgen05.mma that way, against
 // 58 clk when all 32 lanes run the loop and every instruction is predicated on a lane -- close to the 64 clk a
 // 128x128x16 product takes, so that the pipe ran dry behind every wait.
 

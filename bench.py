@@ -9,7 +9,7 @@ through the host-buffer C-ABI calls with every step's transfers inside the timed
 alternating device tensors, l2a_step_host_async; ``e2e.blocking_step_ms`` is one synchronous l2a_step_host call); ``roofline`` describes the dominant kernel
 (timed with CUDA events at the phase boundaries the library records on its own stream; ``achieved`` counts the useful
 pairs of the metric, ``achieved_visited`` the pairs the launch really processes; ``traffic`` scales the DRAM bytes of
-the ncu capture of the same kernel on the 32K case); ``cpu_baseline`` times the fp64 oracle on a bounded sample of the
+the ncu capture of the same kernel on a slice of the headline workload with two KV heads); ``cpu_baseline`` times the fp64 oracle on a bounded sample of the
 workload at its full length and extrapolates the layer.  On the default workload three labelled secondary figures
 follow: ``shared_window_fusion`` (valid only because one Q/K/V set feeds both modules here), ``density_0.5`` and
 ``dense_reference`` (every token routed: the build's own dense path).  With N > 1 every rank runs an independent replica
@@ -37,8 +37,11 @@ METRIC = "L2A fwd+bwd useful TFLOP/s at 128K (one layer, one GPU)"
 KERNELS_PER_STEP = 11  # route: count, scan | fwd: gather, local, global | bwd: gather x2, delta, zero, five-GEMM kernel, merge
 FWD_PHASES = ("gather_q", "attn_fwd_local", "attn_fwd_global")
 BWD_PHASES = ("gather_q_dO", "bwd_delta_zero", "bwd", "bwd_dq_merge")
-# DRAM read + write over algorithmic bytes of a launch, from the ncu captures of the 32K case (profiles/)
-TRAFFIC_RATIO = {"bwd": 1.15, "attn_fwd_local": 0.94, "attn_fwd_global": 1.17}
+# DRAM read + write over algorithmic bytes of a launch, from the ncu capture of the 128K workload cut to two KV heads
+# (profiles/bwd_kernel_l2_traffic_128k_one_kv_head.md): the launch order of the whole workload, small enough for counters
+TRAFFIC_RATIO = {"bwd": 1.55, "attn_fwd_local": 0.95, "attn_fwd_global": 1.73}
+# the same of a decode launch with every sequence routed (profiles/decode_split_kernel_decode_128k.md)
+DECODE_TRAFFIC_RATIO = 1.004
 
 
 def measured_peaks():
@@ -273,8 +276,7 @@ def run_decode(args):
                    "l2_policy": "K/V cache of %.1f GB exceeds L2" % (2 * K.numel() * 2 / 1e9)},
         "roofline": {"bound": "hbm", "kernel": "decode_split_kernel", "achieved": gbs, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"],
-                     # ncu capture of a 4-sequence case: DRAM read + write = 0.9975 x algorithmic bytes; scaled
-                     "traffic": 0.9975 * alg_bytes, "traffic_source": "scaled from the 4-sequence ncu capture",
+                     "traffic": DECODE_TRAFFIC_RATIO * alg_bytes, "traffic_source": "scaled from the 4-sequence ncu capture",
                      "algorithmic_bytes_per_launch": alg_bytes},
         "gpu_launches": args.steps}), flush=True)
 
@@ -575,8 +577,8 @@ def main():
     achieved = per * HD * credited / phase_ms[dom] / 1e9
     achieved_visited = per * HD * visited / phase_ms[dom] / 1e9
     # DRAM traffic of the dominant kernel: not captured on this workload (a counter capture of a 12 GB, 100 ms launch is
-    # out of bounds for ncu here).  Taken from the capture of the same kernel on the 32K case (profiles/), where DRAM
-    # read + write was TRAFFIC_RATIO x the launch's algorithmic bytes, and scaled by this launch's algorithmic bytes.
+    # out of bounds for ncu here).  Taken from the capture of the same kernel on a slice with two KV heads (profiles/), where
+    # DRAM read + write was TRAFFIC_RATIO x the launch's algorithmic bytes, and scaled by this launch's algorithmic bytes.
     qb = cfg.B * cfg.L * cfg.Hq * cfg.D * 2
     kb = cfg.B * cfg.L * cfg.Hkv * cfg.D * 2
     rho_real = float(d.mean())
@@ -586,8 +588,9 @@ def main():
     ratio = TRAFFIC_RATIO.get(dom)
     roofline = {"bound": "tensor", "kernel": dom, "achieved": achieved, "peak": peaks["sustained"], "unit": "TFLOP/s",
                 "frac": achieved / peaks["sustained"], "traffic": ratio * alg_bytes if ratio else None,
-                "traffic_source": (f"{ratio} x algorithmic bytes: ratio of the ncu capture of this kernel on the 32K case "
-                                   f"(profiles/attention_kernels_qwen25_7b_32k.md), scaled to this launch") if ratio else None,
+                "traffic_source": (f"{ratio} x algorithmic bytes: ratio of the ncu capture of this kernel on two KV heads of "
+                                   f"the 128K workload (profiles/bwd_kernel_l2_traffic_128k_one_kv_head.md), scaled to this "
+                                   f"launch") if ratio else None,
                 "algorithmic_bytes_per_launch": alg_bytes,
                 "peak_kind": f"sustained bf16 GEMM, {peaks['source']}", "launch_ms": phase_ms[dom],
                 "algorithmic_flops_per_launch": per * HD * credited, "pairs_credited": int(credited),

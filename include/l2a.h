@@ -231,7 +231,8 @@ l2a_status l2a_router_logits(const l2a_params* p, const void* S, const float* w,
  *   lse_glb     out: fp32 [B, Hq, Lq], first n_routed[b] entries of each (b, h) row: natural-log
  *                    log-sum-exp of the global scores of compact row c (Algorithm 1's L_c).
  *                    Both lse outputs may be NULL unless L2A_FLAG_SAVE_FOR_BWD is set.
- *   fwd_ws         : workspace of at least fwd_ws_bytes (holds the compact query buffer Q_c).
+ *   fwd_ws         : workspace of at least fwd_ws_bytes (holds the compact query buffer Q_c, and the counters and
+ *                    fp32 partial rows of split key ranges).
  * Scores and soft-max run in fp32, probabilities are rounded to bf16 for the second contraction,
  * accumulation is fp32.  Results are bit-reproducible; with few routed rows in the call the keys of a routed row
  * are split into parts (a function of Lq, Hq, B and the largest n_routed), each of which rounds its probabilities

@@ -7,7 +7,7 @@
 //   route_scan  : each CTA sums the counts of the CTAs before it and writes d_mask, prefix, q_idx (ascending = stable) and
 //                 the -1 tail of its own 4096 positions: a warp takes 512 consecutive ones, 32 at a time (one ballot),
 //                 so that every store is contiguous (a thread with 16 consecutive positions of its own, storing with a
-//                 stride of 64 bytes, took 9.8 us for a block, this 4).
+//                 stride of 64 bytes, took 9.8 us for a block, this 5 to 8).
 // Nothing is read back by the host: the routed count stays on the device.
 #include "l2a_common.cuh"
 #include "sm100_prims.cuh"

@@ -12,7 +12,8 @@
 //   compute warps : each takes 16 keys of every stage.  The G query heads are the rows of a 16-row MMA A operand
 //                   (mma.sync m16n8k16, bf16 in, fp32 accumulate): S = Q K^T from ldmatrix'd K rows, running
 //                   soft-max in the exp2 domain on the accumulator fragment, O += P V from transposed ldmatrix of
-//                   the V rows.  The tensor cores are used only to keep the instruction count per key low enough
+//                   the V rows.  The rows of A that the heads leave free (8..15) take what the rounding of P to bf16 cuts
+//                   off: a window key's rounding enters s and a alike, and adds up there.  The tensor cores are used only to keep the instruction count per key low enough
 //                   that the copy engine, not instruction issue, sets the pace.
 #include <math.h>
 
@@ -73,13 +74,14 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t saddr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(saddr));
 }
-// D += A * B, A 16x16 (row), B 16x8 (col), bf16 operands, fp32 accumulators.  Rows 8..15 of A are zero here.
-__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
+// D += A * B, A 16x16 (row), B 16x8 (col), bf16 operands, fp32 accumulators; a0, a2: rows 0..7 of A, a1, a3: rows 8..15.
+__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                          uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
       "{%0, %1, %2, %3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
 // Address of the 16-byte chunk `chunk` (8 columns) of key row `row` inside a 64-key tile stored as D/64
@@ -175,8 +177,8 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
         for (int ks = 0; ks < D / 16; ++ks) {
           uint32_t kb[4];
           ldsm_x4(tile_addr(tK, k_row, ks * 2 + (lm & 1)), kb);
-          mma_16816(s0, qa[ks][0], qa[ks][1], kb[0], kb[1]);
-          mma_16816(s1, qa[ks][0], qa[ks][1], kb[2], kb[3]);
+          mma_16816(s0, qa[ks][0], 0u, qa[ks][1], 0u, kb[0], kb[1]);
+          mma_16816(s1, qa[ks][0], 0u, qa[ks][1], 0u, kb[2], kb[3]);
         }
         // this thread: head hr, keys key0 + 2*t4 + {0, 1} (s0) and key0 + 8 + 2*t4 + {0, 1} (s1)
         float sc[4] = {s0[0] * a.scale_log2, s0[1] * a.scale_log2, s1[0] * a.scale_log2, s1[1] * a.scale_log2};
@@ -199,17 +201,19 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
         m_run = m_new;
         if (__any_sync(0xffffffffu, alpha != 1.f)) {
 #pragma unroll
-          for (int j = 0; j < D / 8; ++j) { acc[j][0] *= alpha; acc[j][1] *= alpha; }
+          for (int j = 0; j < D / 8; ++j) { acc[j][0] *= alpha; acc[j][1] *= alpha; acc[j][2] *= alpha; acc[j][3] *= alpha; }
         }
         const uint32_t pa0 = pack_bf16(p0, p1), pa2 = pack_bf16(p2, p3);
+        const uint32_t pa1 = pack_bf16(p0 - __uint_as_float(pa0 << 16), p1 - __uint_as_float(pa0 & 0xffff0000u));
+        const uint32_t pa3 = pack_bf16(p2 - __uint_as_float(pa2 << 16), p3 - __uint_as_float(pa2 & 0xffff0000u));
         // ---- O += P V: B fragments are the transposed 8x8 blocks of the V rows
 #pragma unroll
         for (int jj = 0; jj < D / 16; ++jj) {
           uint32_t vb[4];
           ldsm_x4_t(tile_addr(tV, v_row, jj * 2 + (lm >> 1)), vb);
           if (tail) { vb[0] &= vm0; vb[1] &= vm1; vb[2] &= vm0; vb[3] &= vm1; }   // rows past the chunk may hold anything
-          mma_16816(acc[2 * jj], pa0, pa2, vb[0], vb[1]);
-          mma_16816(acc[2 * jj + 1], pa0, pa2, vb[2], vb[3]);
+          mma_16816(acc[2 * jj], pa0, pa1, pa2, pa3, vb[0], vb[1]);
+          mma_16816(acc[2 * jj + 1], pa0, pa1, pa2, pa3, vb[2], vb[3]);
         }
       }
       __syncwarp();
@@ -230,7 +234,9 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
     if (t4 == 0) { red_m[warp * G + hr] = m_run; red_l[warp * G + hr] = ls; }
 #pragma unroll
     for (int j = 0; j < D / 8; ++j)
-      *reinterpret_cast<float2*>(&red_acc[(warp * G + hr) * D + j * 8 + 2 * t4]) = make_float2(acc[j][0], acc[j][1]);
+      // (an infinite value stays what it is: the part cut off may have the other sign or be zero)
+      *reinterpret_cast<float2*>(&red_acc[(warp * G + hr) * D + j * 8 + 2 * t4]) =
+          make_float2(acc[j][0] + (isfinite(acc[j][0]) ? acc[j][2] : 0.f), acc[j][1] + (isfinite(acc[j][1]) ? acc[j][3] : 0.f));
   }
   __syncthreads();
   const int n_items = a.n_win + a.n_out;

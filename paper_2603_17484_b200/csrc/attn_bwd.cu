@@ -297,13 +297,18 @@ struct ItemCursor<1> {
 // All key blocks meet in those accumulators in no fixed order: dQ is not bit-reproducible from run to run
 // (dK, dV are).
 //   TMEM: dV [0,D) | dK [D,2D) | T [256,384): S^T(i), then P^T(i) (bf16, quarter-local) | U [384,512): dP^T(i),
-//         then dQ(i).
+//         then dS^T(i) (bf16, quarter-local), then dQ(i).
 //   Shared memory: K, V resident; Q and dO in two-stage rings; dS(i) (bf16, [key][query], swizzled like a TMA
-//   tile) -- the A operand of both dK += dS^T Q (read K-major) and dQ = dS K (read MN-major).
-//   MMA order per item i:  dV(i) | S^T(i+1) | dQ(i) | dK(i) | dP^T(i+1).  S^T(i+1) does not depend on dS(i), so it is
+//   tile) -- the A operand of dQ = dS K (read MN-major).
+//   MMA order per item i:  dV(i) | S^T(i+1) | dK(i) | dQ(i) | dP^T(i+1).  S^T(i+1) does not depend on dS(i), so it is
 //   issued ahead of the wait for it: the compute warps find the next scores ready when they are done with dS(i).
-//   Two loops run through the order: T: S^T -> P -> dV -> S^T and U: dP^T -> dS -> dQ -> read-out -> dP^T; dK(i) keeps the
-//   pipe busy while the read-out warps take dQ(i) out of TMEM, which frees U well before their reductions are issued.
+//   Two loops run through the order: T: S^T -> P -> dV -> S^T and U: dP^T -> dS -> dQ -> read-out -> dP^T.  What bounds an
+//   item is the traffic of shared memory (operands 2048 clk, TMA 512, dS, statistics and the reductions' data 1000 at 128
+//   bytes a clock), not the tensor pipe: so dK(i) takes dS^T from U, where it lies between dP^T(i) and dQ(i), and not from
+//   shared memory as before, although nothing then covers the read-out of dQ(i) that dP^T(i+1) waits for.  It also returns
+//   the Q stage to the TMA warp 500 clk earlier, whose load was late under the reductions.  Backward launch of 2 x 4096
+//   tokens (28/4 heads) 794 -> 758 us, of the local module at 8155 tokens 1037 -> 978; without the writes of dS it would
+//   take 685, without the TMA writes 694, without the statistics 732, without any of them and the reductions 560.
 
 // The reductions of one read-out warp: piece I of its 32 x D/2 share (4 columns each) goes to a byte offset from the
 // warp's base address that is a compile-time constant, so that all of them share one address register pair.
@@ -508,8 +513,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     mbar_init(&bar->s_full, 1);
     mbar_init(&bar->dp_full, 1);
     mbar_init(&bar->p_full, kComputeWarps * 32);     // P^T(i) is in TMEM
-    mbar_init(&bar->ds_full, kComputeWarps * 32);    // dS(i) is in shared memory and dP^T(i) has been read
-    mbar_init(&bar->ds_free, 1);                     // dQ(i) and dK(i) have consumed dS(i)
+    mbar_init(&bar->ds_full, kComputeWarps * 32);    // dS(i) is in shared memory and in TMEM
+    mbar_init(&bar->ds_free, 1);                     // dQ(i) has consumed dS(i)
     mbar_init(&bar->dq_full, 1);                     // dQ(i) is in TMEM
     mbar_init(&bar->u_free, 8 * 32);     // dQ(i) has been read out: the columns may take dP^T(i+1)
     mbar_init(&bar->final_bar, 1);
@@ -661,7 +666,6 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       const uint64_t dk = smem_desc_sw128(smem_u32(sK), 16, 1024), dv = smem_desc_sw128(smem_u32(sV), 16, 1024);
       const uint64_t dkm = smem_desc_sw128(smem_u32(sK), kBoxBytes, 1024);            // K as MN-major B of dQ
       const uint64_t dsm = smem_desc_sw128(smem_u32(sDS), kBoxBytes, 1024);           // dS as MN-major A of dQ
-      const uint64_t dsk = smem_desc_sw128(smem_u32(sDS), 16, 1024);                  // dS^T as K-major A of dK
       const uint64_t dq_base = smem_desc_sw128(smem_u32(sQ), 16, 1024);
       const uint64_t ddo_base = smem_desc_sw128(smem_u32(sDO), 16, 1024);
       const uint64_t dqm_base = smem_desc_sw128(smem_u32(sQ), kBoxBytes, 1024);      // Q / dO as MN-major B
@@ -689,6 +693,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         for (int kk = 0; kk < 8; ++kk)
           mma_ss(tmem + 384, dsm + ((kk * 2048) >> 4), dkm + ((kk * 2048) >> 4), idesc_dq, kk > 0);
         tc_commit(&bar->dq_full);
+        tc_commit(&bar->ds_free);
       };
       auto issue_dV = [&](int ds, bool first) {   // dV += P^T dO, P^T from the T columns
         const uint64_t dod = ddom_base + ds * kStageStep;
@@ -698,15 +703,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
                  (kk > 0 || !first) ? 1u : 0u);
         tc_commit(&bar->do_empty[ds]);
       };
-      auto issue_dK = [&](int qs, bool first) {   // dK += dS^T Q, dS^T from shared memory
+      auto issue_dK = [&](int qs, bool first) {   // dK += dS^T Q, dS^T from the U columns
         const uint64_t qd = dqm_base + qs * kStageStep;
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint32_t c = ((kk >> 2) * kBoxBytes + (kk & 3) * 32) >> 4;
-          mma_ss(tmem + D, dsk + c, qd + ((kk * 2048) >> 4), idesc_acc, (kk > 0 || !first) ? 1u : 0u);
-        }
+        for (int kk = 0; kk < 8; ++kk)
+          mma_ts(tmem + D, tmem + 384 + (kk >> 1) * 32 + (kk & 1) * 8, qd + ((kk * 2048) >> 4), idesc_acc,
+                 (kk > 0 || !first) ? 1u : 0u);
         tc_commit(&bar->q_empty[qs]);
-        tc_commit(&bar->ds_free);
       };
       bool ok = count > 0 && mbar_spin(&bar->kv_full, 0, abort_flag) && mbar_spin(&bar->q_full[0], 0, abort_flag) &&
                 mbar_spin(&bar->do_full[0], 0, abort_flag);
@@ -729,8 +732,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         }
         if (!mbar_spin(&bar->ds_full, i & 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        issue_dQ();
-        issue_dK(i & 1, i == 0);       // keeps the pipe busy while dQ(i) is read out
+        issue_dK(i & 1, i == 0);
+        issue_dQ();                    // over dS^T(i), which dK(i) ahead of it has read
         if (more) {
           const int sn = (i + 1) & 1;
           const uint32_t phn = ((i + 1) >> 1) & 1;
@@ -835,8 +838,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
           pd[e] = pack_bf16(ds.x, ds.y);
         }
       }
-      // dS goes to shared memory, [key][query] with the 128-byte swizzle of a TMA tile (two boxes of 64 queries); the
-      // tile of the previous item must have been consumed by dQ(i-1) and dK(i-1)
+      tmem_st16(dp_addr, pd);    // dS^T over the first half of this quarter's own dP^T columns
+      // dS also goes to shared memory, [key][query] with the 128-byte swizzle of a TMA tile (two boxes of 64 queries); the
+      // tile of the previous item must have been consumed by dQ(i-1)
       if (i > 0 && !__all_sync(0xffffffffu, mbar_wait(&bar->ds_free, (i - 1) & 1, abort_flag))) { ok = false; break; }
       {
         const uint32_t row = smem_u32(sDS) + (q >> 1) * kBoxBytes + kr * 128;
@@ -847,7 +851,8 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
                        "r"(pd[4 * c]), "r"(pd[4 * c + 1]), "r"(pd[4 * c + 2]), "r"(pd[4 * c + 3]) : "memory");
       }
       fence_async_smem();        // the MMA reads the tile through the async proxy
-      tc_fence_before();         // orders the dP^T read above before the dQ MMA that overwrites those columns
+      tmem_st_wait();
+      tc_fence_before();         // orders the TMEM accesses above before dK, and before dQ that overwrites the columns
       mbar_arrive(&bar->ds_full);
     }
     // epilogue: quarters 0,1 store the two column halves of dV, quarters 2,3 those of dK

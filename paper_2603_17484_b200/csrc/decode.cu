@@ -2,9 +2,9 @@
 // cache (Local Attention) and, only if its routing decision d = 1, to the whole cache (Global Attention);
 // o = s + d * a.  The work is one pass over the K/V cache: HBM-bound.  The cache of every KV head is cut at the window's
 // first key and split into chunks processed by independent CTAs; a chunk's partial soft-max (acc, max, sum) inside the
-// window serves both modules, those before it exist for routed tokens only.  The CTA of a (sequence, KV head) that
-// finishes last combines the chunks: o is one weighted sum of their accumulators.  A single chunk stores its result itself
-// (a window of 129 keys, 28/4 heads, not routed, calls back to back: 12.3 us through the combination, 8.3 without).
+// window serves both modules, those before it exist for routed tokens only.  decode_combine_kernel, whose CTAs (one per
+// sequence and query head) are resident when the last chunk ends, combines the chunks: o is one weighted sum of their
+// accumulators.  A single chunk stores its result itself.
 //
 // One CTA = one chunk of keys of one (batch entry, KV head), for all G query heads of the group:
 //   producer warp : streams 64-key K and V tiles through a ring of shared-memory stages with TMA (one 4-D copy
@@ -40,7 +40,7 @@ struct DecodeArgs {
   const bf16* q;           // [B, Hq, D]
   const uint8_t* d;        // [B] routing decision of the new token (NULL = never routed)
   float* part;             // [B, Hkv, n_win + n_out, G, D + 4]  (acc[D], m, l, 2 unused)
-  int* done;               // [B, Hkv] chunks finished so far; cleared by the caller
+  int* failed;             // [B, Hkv] a wait ran out in one of the chunks: nothing is stored
   bf16* O;                 // [B, Hq, D]
   int* status;             // workspace status word
 };
@@ -48,7 +48,6 @@ struct DecodeArgs {
 struct DecodeBars {
   uint64_t full[kDecStages], empty[kDecStages];
   int abort_flag;
-  int last;                // this CTA finished last of its (batch entry, KV head)
 };
 
 constexpr int kMaxWin = 64, kMaxOut = 512;   // chunks at most
@@ -56,8 +55,6 @@ template <int D>
 constexpr size_t decode_smem_bytes() {
   return (size_t)kDecStages * 2 * kDecKeys * D * 2 + sizeof(DecodeBars);
 }
-static_assert(kMaxGroup * (kMaxWin + kMaxOut) * sizeof(float2) <= kDecStages * 2 * kDecKeys * 64 * 2, "weights exceed the stages");
-
 __device__ __forceinline__ void chunk_range(int lo, int hi, int n, int i, int& c_lo, int& c_hi) {
   const int len = hi - lo + 1;
   int per = (len + n - 1) / n;
@@ -97,6 +94,11 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   constexpr int kTileBytes = kDecKeys * D * 2;
   constexpr int kStageBytes = 2 * kTileBytes;       // K tile, then V tile
   const int item = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
+  dependents_release();
+  if (item == 0 && threadIdx.x == 0) {       // (nothing sets them before a wait has run out, seconds from here)
+    a.failed[b * a.Hkv + g] = 0;
+    if (g == 0 && b == 0) *a.status = 0;
+  }
   const bool outside = item >= a.n_win;
   const bool routed = a.d != nullptr && a.d[b] != 0;
   if (outside && !routed) return;                              // Global Attention is skipped when d = 0
@@ -111,7 +113,7 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   DecodeBars* bar = reinterpret_cast<DecodeBars*>(smem + kDecStages * kStageBytes);
   volatile int* abort_flag = &bar->abort_flag;
   if ((smem_u32(smem) & 1023u) != 0) {       // the swizzled tile addressing needs a 1024-byte-aligned base
-    if (tid == 0) atomicExch(a.status, 2);
+    if (tid == 0) { atomicExch(a.status, 2); a.failed[b * a.Hkv + g] = 1; }
     return;
   }
   if (tid == 0) {
@@ -225,7 +227,7 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   // write the chunk's partial result
   __syncthreads();
   float* red_acc = reinterpret_cast<float*>(smem);                           // [warps][G][D]
-  float* red_m = red_acc + kDecComputeWarps * G * D;                         // [warps][G]
+  float* red_m = red_acc + kDecComputeWarps * G * D;                         // [warps][G], then the factors of the sums
   float* red_l = red_m + kDecComputeWarps * G;
   float ls = l_run;
   ls += __shfl_xor_sync(0xffffffffu, ls, 1);
@@ -242,113 +244,162 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   const int n_items = a.n_win + a.n_out;
   const bool single = (routed ? n_items : a.n_win) == 1;       // nothing to combine: the result goes straight out
   constexpr int kRow = D + 4;
-  float* base = a.part + ((int64_t)b * a.Hkv + g) * n_items * (G * kRow);
-  for (int i = tid; i < G * D; i += kDecThreads) {
-    const int h = i / D, col = i % D;
-    float M = -INFINITY;
-    for (int w = 0; w < kDecComputeWarps; ++w) M = fmaxf(M, red_m[w * G + h]);
-    float L = 0.f, A = 0.f;
+  float* base = a.part + (((int64_t)b * a.Hkv + g) * n_items + item) * (G * kRow);
+  // one thread per head takes the maximum and the sum; it leaves each warp's factor in place of its maximum
+  if (tid < G) {
+    float M = -INFINITY, L = 0.f;
+#pragma unroll
+    for (int w = 0; w < kDecComputeWarps; ++w) M = fmaxf(M, red_m[w * G + tid]);
+#pragma unroll
     for (int w = 0; w < kDecComputeWarps; ++w) {
-      const float mw = red_m[w * G + h];
+      const float mw = red_m[w * G + tid];
       const float f = (mw == -INFINITY) ? 0.f : exp2f(mw - M);
-      L += red_l[w * G + h] * f;
-      A += red_acc[(w * G + h) * D + col] * f;
+      L += red_l[w * G + tid] * f;
+      red_m[w * G + tid] = f;
     }
-    if (single) {
-      float w = 1.f / L;
-      if (routed) w += 1.f / L;        // window and whole cache are the same keys
-      if (bar->abort_flag == 0) a.O[((int64_t)b * a.Hq + g * G + h) * D + col] = __float2bfloat16(w * A);
-      continue;
-    }
-    float* dst = base + (item * G + h) * kRow;
-    dst[col] = A;
-    if (col == 0) { dst[D] = M; dst[D + 1] = L; }
+    if (single) red_l[tid] = routed ? 1.f / L + 1.f / L : 1.f / L;     // routed: window and whole cache are the same keys
+    else *reinterpret_cast<float2*>(base + tid * kRow + D) = make_float2(M, L);
   }
-  if (!single) {
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) bar->last = arrive_last(&a.done[b * a.Hkv + g], routed ? n_items : a.n_win, abort_flag);
-    __syncthreads();
-  }
-  if (!single && bar->last) {
-    // ---- the last CTA of the (batch entry, KV head): weight of chunk i in head h's result,
-    //   o = sum_win acc_i 2^(m_i - M_win) / L_win + d * sum_all acc_i 2^(m_i - M_all) / L_all
-    __threadfence();
-    const int n = routed ? n_items : a.n_win;
-    float2* ml = reinterpret_cast<float2*>(smem);            // [n][G] (m, l), then (weight, -)
-    for (int i = tid; i < n * G; i += kDecThreads)
-      ml[i] = __ldcg(reinterpret_cast<const float2*>(base + (int64_t)i * kRow + D));
-    __syncthreads();
-    for (int h = warp; h < G; h += kDecComputeWarps + 1) {
-      float M[2] = {-INFINITY, -INFINITY}, L[2] = {0.f, 0.f};   // window, everything
-      for (int i = lane; i < n; i += 32) {
-        const float m = ml[i * G + h].x;
-        M[1] = fmaxf(M[1], m);
-        if (i < a.n_win) M[0] = fmaxf(M[0], m);
-      }
+  __syncthreads();
+  for (int x = tid; x < G * (D / 4); x += kDecThreads) {
+    const int h = x / (D / 4), c4 = x % (D / 4);
+    float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        M[0] = fmaxf(M[0], __shfl_xor_sync(0xffffffffu, M[0], o));
-        M[1] = fmaxf(M[1], __shfl_xor_sync(0xffffffffu, M[1], o));
-      }
-      for (int i = lane; i < n; i += 32) {
-        const float2 v = ml[i * G + h];
-        if (v.x != -INFINITY) {                                 // (a chunk without keys wrote no maximum)
-          L[1] += v.y * exp2f(v.x - M[1]);
-          if (i < a.n_win) L[0] += v.y * exp2f(v.x - M[0]);
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        L[0] += __shfl_xor_sync(0xffffffffu, L[0], o);
-        L[1] += __shfl_xor_sync(0xffffffffu, L[1], o);
-      }
-      for (int i = lane; i < n; i += 32) {
-        const float m = ml[i * G + h].x;
-        float w = 0.f;
-        if (m != -INFINITY) {
-          if (i < a.n_win) w = exp2f(m - M[0]) / L[0];
-          if (routed) w += exp2f(m - M[1]) / L[1];
-        }
-        ml[i * G + h].x = w;
-      }
+    for (int w = 0; w < kDecComputeWarps; ++w) {
+      const float4 v = *reinterpret_cast<const float4*>(&red_acc[(w * G + h) * D + c4 * 4]);
+      const float f = red_m[w * G + h];
+      A.x += v.x * f; A.y += v.y * f; A.z += v.z * f; A.w += v.w * f;
     }
-    __syncthreads();
-    // four columns a thread, sixteen chunks in flight: what counts here is the latency of the rounds
-    for (int x = tid; x < G * (D / 4); x += kDecThreads) {
-      const int h = x / (D / 4), c4 = x % (D / 4);
-      const float* src = base + h * kRow + c4 * 4;
-      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int k0 = 0; k0 < n; k0 += 16) {
-        float4 v[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-          v[k] = k0 + k < n ? __ldcg(reinterpret_cast<const float4*>(src + (int64_t)(k0 + k) * (G * kRow)))
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          const float w = k0 + k < n ? ml[(k0 + k) * G + h].x : 0.f;
-          o.x = fmaf(w, v[k].x, o.x);
-          o.y = fmaf(w, v[k].y, o.y);
-          o.z = fmaf(w, v[k].z, o.z);
-          o.w = fmaf(w, v[k].w, o.w);
-        }
-      }
+    if (!single) {
+      *reinterpret_cast<float4*>(base + h * kRow + c4 * 4) = A;
+    } else if (bar->abort_flag == 0) {
+      const float w = red_l[h];
       reinterpret_cast<uint2*>(a.O + ((int64_t)b * a.Hq + g * G + h) * D)[c4] =
-          make_uint2(pack_bf16(o.x, o.y), pack_bf16(o.z, o.w));
+          make_uint2(pack_bf16(w * A.x, w * A.y), pack_bf16(w * A.z, w * A.w));
     }
   }
   if (bar->abort_flag) {
     // a bounded wait ran out: give copies still in flight time to land before shared memory is released
     const uint64_t t0 = globaltimer_ns();
     while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
-    if (tid == 0) atomicExch(a.status, 1);
+    if (tid == 0) { atomicExch(a.status, 1); a.failed[b * a.Hkv + g] = 1; }
     __syncthreads();
   }
 }
 
+// Combines the chunks of one query head of one sequence:
+//   o = sum_win acc_i 2^(m_i - M_win) / L_win + d * sum_all acc_i 2^(m_i - M_all) / L_all
+// Bound by latencies, not by the rows it reads: so every thread asks for its share of the first kCombineAhead * 128 / (D / 4)
+// chunks (48 for D = 128) before the weights are known, and the launch overlaps with the end of the chunks.  The CTA of a
+// (sequence, KV head) that finished last did this before, behind a counter that a memset ahead of the kernel cleared:
+// 6.7 of 12.7 us for one sequence of 9001 keys (28/4 heads, routed), and 2.3 us for the memset.
+constexpr int kCombineThreads = 128, kCombineAhead = 12;
+template <int D>
+__global__ void __launch_bounds__(kCombineThreads) decode_combine_kernel(const DecodeArgs a) {
+  constexpr int kLanes = D / 4, kGroups = kCombineThreads / kLanes, kRow = D + 4;
+  __shared__ float weight[kMaxWin + kMaxOut];
+  __shared__ float4 red[kGroups][kLanes];
+  __shared__ float2 red_win[kCombineThreads / 32], red_all[kCombineThreads / 32];    // (maximum, sum)
+  const int h = blockIdx.x, b = blockIdx.y, G = a.G, g = h / G;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c4 = tid % kLanes, grp = tid / kLanes;
+  const int n_items = a.n_win + a.n_out;
+  dependency_wait();
+  const bool routed = a.d != nullptr && a.d[b] != 0;
+  const int n = routed ? n_items : a.n_win;
+  if (n == 1) return;                                            // stored by its only chunk
+  const float* base = a.part + (((int64_t)b * a.Hkv + g) * n_items * G + h % G) * kRow;
+  const int64_t step = (int64_t)G * kRow;
+  float4 v[kCombineAhead];
+#pragma unroll
+  for (int i = 0; i < kCombineAhead; ++i) {
+    const int k = grp + i * kGroups;
+    v[i] = k < n ? __ldcg(reinterpret_cast<const float4*>(base + k * step + c4 * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  const int failed = __ldcg(&a.failed[b * a.Hkv + g]);
+  constexpr int kMine = (kMaxWin + kMaxOut + kCombineThreads - 1) / kCombineThreads;
+  float2 ml[kMine];
+  float m_win = -INFINITY, m_all = -INFINITY;
+#pragma unroll
+  for (int i = 0; i < kMine; ++i) {
+    const int k = tid + i * kCombineThreads;
+    ml[i] = k < n ? __ldcg(reinterpret_cast<const float2*>(base + k * step + D)) : make_float2(-INFINITY, 0.f);
+    m_all = fmaxf(m_all, ml[i].x);
+    if (k < a.n_win) m_win = fmaxf(m_win, ml[i].x);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    m_win = fmaxf(m_win, __shfl_xor_sync(0xffffffffu, m_win, o));
+    m_all = fmaxf(m_all, __shfl_xor_sync(0xffffffffu, m_all, o));
+  }
+  if (lane == 0) { red_win[warp].x = m_win; red_all[warp].x = m_all; }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kCombineThreads / 32; ++w) {
+    m_win = fmaxf(m_win, red_win[w].x);
+    m_all = fmaxf(m_all, red_all[w].x);
+  }
+  float l_win = 0.f, l_all = 0.f;
+#pragma unroll
+  for (int i = 0; i < kMine; ++i) {
+    if (ml[i].x == -INFINITY) continue;                          // (a chunk without keys wrote no maximum)
+    l_all += ml[i].y * exp2f(ml[i].x - m_all);
+    if (tid + i * kCombineThreads < a.n_win) l_win += ml[i].y * exp2f(ml[i].x - m_win);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    l_win += __shfl_xor_sync(0xffffffffu, l_win, o);
+    l_all += __shfl_xor_sync(0xffffffffu, l_all, o);
+  }
+  if (lane == 0) { red_win[warp].y = l_win; red_all[warp].y = l_all; }
+  __syncthreads();
+  l_win = 0.f;
+  l_all = 0.f;
+#pragma unroll
+  for (int w = 0; w < kCombineThreads / 32; ++w) {
+    l_win += red_win[w].y;
+    l_all += red_all[w].y;
+  }
+#pragma unroll
+  for (int i = 0; i < kMine; ++i) {
+    const int k = tid + i * kCombineThreads;
+    if (k >= n) continue;
+    float w = 0.f;
+    if (ml[i].x != -INFINITY) {
+      if (k < a.n_win) w = exp2f(ml[i].x - m_win) / l_win;
+      if (routed) w += exp2f(ml[i].x - m_all) / l_all;
+    }
+    weight[k] = w;
+  }
+  __syncthreads();
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [&](int k, const float4& x) {
+    const float w = weight[k];
+    o.x = fmaf(w, x.x, o.x);
+    o.y = fmaf(w, x.y, o.y);
+    o.z = fmaf(w, x.z, o.z);
+    o.w = fmaf(w, x.w, o.w);
+  };
+#pragma unroll
+  for (int i = 0; i < kCombineAhead; ++i)
+    if (grp + i * kGroups < n) add(grp + i * kGroups, v[i]);
+#pragma unroll 4
+  for (int k = grp + kCombineAhead * kGroups; k < n; k += kGroups)
+    add(k, __ldcg(reinterpret_cast<const float4*>(base + k * step + c4 * 4)));
+  red[grp][c4] = o;
+  __syncthreads();
+  if (grp == 0 && failed == 0) {
+#pragma unroll
+    for (int s = 1; s < kGroups; ++s) {
+      const float4 x = red[s][c4];
+      o.x += x.x; o.y += x.y; o.z += x.z; o.w += x.w;
+    }
+    reinterpret_cast<uint2*>(a.O + ((int64_t)b * a.Hq + h) * D)[c4] = make_uint2(pack_bf16(o.x, o.y), pack_bf16(o.z, o.w));
+  }
+}
+
 // Chunks as long as one resident wave of CTAs (two per SM, 148 SMs) allows, between 256 and 4096 keys: every chunk costs
-// its launch and a row per head that the last CTA reads back.  Measured against four times as many: one sequence of 128K
+// its launch and a row per head that the combination reads back.  Measured against four times as many: one sequence of 128K
 // keys (28/4 heads) 64 / 87 us, two of 40K 27 / 36, six of 100K with one KV head 63 / 84, 16 of 128K with four routed 342
 // (2048 keys at most: 353), 32 of 8000 not routed 90 / 92, one of 9001 16.4 with either.
 // Before the window only routed sequences have work, and the host does not know which are.  Chunks there are no longer than
@@ -356,6 +407,10 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
 // without this limit / with it (/ with 1024 / 2048 keys): one routed of 16 sequences of 32K (28/4 heads) 68 / 49 (47 / 52),
 // of 32 of 60K (8/1) 59 / 39 (37 / 43), of 16 of 128K (8/1) 50 / 37 (35 / 38); none of 32 of 8000 (32/8) 89 / 91 (102 / 90),
 // none of 16 of 128K (8/1) 18.7 / 21.6 (22.8 / 20.9); all of 16 of 128K (8/1) 170 / 179 (184 / 176).
+// (All of these with the combination by the CTA that finished last.  With decode_combine_kernel, captured calls back to
+// back: one sequence of 9001 keys (28/4 heads) routed 16.4 -> 7.6, not routed 14.4 -> 7.3; of 40000 30.4 -> 18.1; of 128K
+// (32/8) 96.6 -> 88.0; one routed of 16 of 32K (28/4) 45.7 -> 39.6, of 32 of 60K (8/1) 28.7 -> 19.7; none of 32 of 8000
+// (32/8) 92.1 -> 86.7; all of 16 of 128K (8/1) 180.1 -> 165.6; four routed of 16 of 128K (32/8) 346.8 -> 338.5.)
 constexpr int kChunkTarget = 2 * 148, kChunkMin = 256, kChunkMax = 4096;
 constexpr int kSoloTarget = 148, kSoloMin = 1536;
 void window_and_rest(const l2a_params* p, int* win, int* out) {
@@ -424,10 +479,10 @@ cudaError_t launch_split_d(const DecodeArgs& a, const CUtensorMap& mapK, const C
 
 using namespace l2a;
 
-static size_t done_bytes(const l2a_params* p) { return align_up((size_t)p->B * p->Hkv * sizeof(int), 256); }
+static size_t failed_bytes(const l2a_params* p) { return align_up((size_t)p->B * p->Hkv * sizeof(int), 256); }
 
 static size_t decode_ws_size(const l2a_params* p, int64_t chunks) {
-  return kWsHeaderBytes + done_bytes(p) + align_up((size_t)chunks * (p->Hq / p->Hkv) * (p->D + 4) * sizeof(float), 256);
+  return kWsHeaderBytes + failed_bytes(p) + align_up((size_t)chunks * (p->Hq / p->Hkv) * (p->D + 4) * sizeof(float), 256);
 }
 
 static l2a_status check_decode(const l2a_params* p) {
@@ -461,7 +516,6 @@ extern "C" l2a_status l2a_decode(const l2a_params* p, const void* q, const void*
       ws_bytes < decode_ws_size(p, (int64_t)p->B * p->Hkv * (a.n_win + a.n_out)))
     return L2A_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeaderBytes + done_bytes(p), s) != cudaSuccess) return L2A_ERR_CUDA;   // status, counters
   CUtensorMap mapK, mapV;
   if (!is_dense(p->q_stride, p->Lq, p->Hq * p->D) || !is_dense(p->o_stride, p->Lq, p->Hq * p->D)) return L2A_ERR_UNSUPPORTED;
   const RowStrides ks = resolve_strides(p->k_stride, p->Lk, p->Hkv * p->D);
@@ -476,10 +530,15 @@ extern "C" l2a_status l2a_decode(const l2a_params* p, const void* q, const void*
   a.q = static_cast<const bf16*>(q);
   a.d = d;
   a.status = static_cast<int*>(ws);
-  a.done = reinterpret_cast<int*>(static_cast<uint8_t*>(ws) + kWsHeaderBytes);
-  a.part = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + kWsHeaderBytes + done_bytes(p));
+  a.failed = reinterpret_cast<int*>(static_cast<uint8_t*>(ws) + kWsHeaderBytes);
+  a.part = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + kWsHeaderBytes + failed_bytes(p));
   a.O = static_cast<bf16*>(O);
   const dim3 grid(a.n_win + a.n_out, p->Hkv, p->B);
-  const cudaError_t e = p->D == 128 ? launch_split_d<128>(a, mapK, mapV, grid, s) : launch_split_d<64>(a, mapK, mapV, grid, s);
+  cudaError_t e = p->D == 128 ? launch_split_d<128>(a, mapK, mapV, grid, s) : launch_split_d<64>(a, mapK, mapV, grid, s);
+  if (e == cudaSuccess && grid.x > 1) {
+    const dim3 heads(p->Hq, p->B);
+    e = p->D == 128 ? launch_dependent(decode_combine_kernel<128>, heads, kCombineThreads, 0, s, true, a)
+                    : launch_dependent(decode_combine_kernel<64>, heads, kCombineThreads, 0, s, true, a);
+  }
   return e == cudaSuccess ? L2A_OK : L2A_ERR_CUDA;
 }

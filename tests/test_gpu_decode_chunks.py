@@ -1,5 +1,5 @@
-"""Decode: chunks cut at the window's first key, whose partial results serve both modules, combined by the CTA that
-finishes last.  Sizes around the cut and the chunk edges, against the fp64 oracle; repeated calls on one workspace."""
+"""Decode: chunks cut at the window's first key, whose partial results serve both modules, combined by a kernel behind
+them.  Sizes around the cut and the chunk edges, against the fp64 oracle; repeated calls on one workspace."""
 import numpy as np
 import pytest
 import torch
@@ -58,6 +58,27 @@ def test_error_is_that_of_rounding_the_result(B, Lk, Hq, Hkv, D, W):
     want = oracle.forward_full(sh, synth.as_u16(t["Q"]), synth.as_u16(t["K"]), synth.as_u16(t["V"]), d)["o"]
     rounded = torch.from_numpy(want).to(torch.bfloat16).double().numpy()
     assert np.linalg.norm(to_f64(O) - want) <= 1.02 * np.linalg.norm(rounded - want)
+
+
+@pytest.mark.parametrize("D,n", [(128, 2), (128, 47), (128, 48), (128, 49), (64, 95), (64, 96), (64, 97), (128, 128),
+                                 (128, 129), (64, 257)])
+def test_combination_of_n_chunks(D, n):
+    """Chunks of 256 keys around what a thread of the combination asks for ahead of the weights (48 or 96 chunks) and around
+    its 128 threads.  The bound is the one above: rounding the result, and 2 % for the fp32 sums."""
+    W, Lk = 255, 256 * n            # one chunk in the window, n - 1 before it
+    t = synth.qkv(1, 1, 3, 1, D, seed=n, Lk=Lk)
+    p = l2a.params(1, 1, Lk, 3, 1, D, W)
+    ws = torch.full((l2a.l2a_decode_workspace_bytes(p),), 0x5A, dtype=torch.uint8, device="cuda")
+    q, K, V = (t[k].cuda() for k in ("Q", "K", "V"))
+    sh = oracle.Shape(1, 1, Lk, 3, 1, D, W)
+    for routed in (1, 0):
+        d = np.full((1, 1), routed, np.uint8)
+        O = torch.full((1, 1, 3, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+        l2a.l2a_decode(p, q, K, V, torch.from_numpy(d[:, 0].copy()).cuda(), O, ws)
+        assert l2a.l2a_workspace_status(ws) == 0
+        want = oracle.forward_full(sh, synth.as_u16(t["Q"]), synth.as_u16(t["K"]), synth.as_u16(t["V"]), d)["o"]
+        rounded = torch.from_numpy(want).to(torch.bfloat16).double().numpy()
+        assert np.linalg.norm(to_f64(O) - want) <= 1.02 * np.linalg.norm(rounded - want), routed
 
 
 def test_infinite_values_stay_infinite():

@@ -31,7 +31,11 @@ constexpr float kLog2e = 1.4426950408889634f;
 // Delta / dgate preprocess.  The grid is one resident wave; the warps take the tokens round-robin, so that at any
 // moment the whole grid reads one contiguous stretch of each tensor (a contiguous range per warp, i.e. thousands of
 // separate streams, ran at 0.7 of this speed).  A token's Hq*D values are read with 16-byte loads: D/8 lanes per
-// head, 32/(D/8) heads per pass, several passes in flight.
+// head, 32/(D/8) heads per pass, four passes in flight: with the rows of two groups of passes in registers two CTAs fit an
+// SM (held to three or four they spill: 70 / 71 us instead of 59 beside a concurrent clearing, 2 x 4096 tokens).  The kernel
+// reads nothing that the gather ahead of it writes, so it waits for that at its end only.  From the gather to the end of the
+// clearing: 2 x 4096 tokens (28/4 heads) 90 -> 75 us, 16K tokens 121 -> 114, 64K packed (32/8) 546 -> 516.  Clearing
+// beside Delta instead of behind it: 69, 115 and 600 (DRAM turns between reads and writes).
 __device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
   const uint32_t a[4] = {x.x, x.y, x.z, x.w}, b[4] = {y.x, y.y, y.z, y.w};
   float acc = 0.f;
@@ -44,7 +48,7 @@ __device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(256) bwd_delta_kernel(const bf16* __restrict__ dO, const bf16* __restrict__ dO_loc,
+__global__ void __launch_bounds__(256, 2) bwd_delta_kernel(const bf16* __restrict__ dO, const bf16* __restrict__ dO_loc,
                                                         const bf16* __restrict__ S,
                                                         const bf16* __restrict__ A_c,
                                                         const uint8_t* __restrict__ d_mask,
@@ -60,16 +64,27 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(const bf16* __restrict__
   const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const bool split = dO_loc != dO;                     // separate gradient for the local output
-  dependency_wait();
-  dependents_release();
+  dependents_release();       // (reads nothing that the kernels ahead of it in the call write: it waits at its end)
   const int sub = lane / kLanesPerHead;                // head inside the pass
   const int n_pass = (Hq + kHeadsPerPass - 1) / kHeadsPerPass;
+  const bool global = d_mask != nullptr;               // NULL: the global part is skipped
+  bool next_routed = global && gw < n_tokens && d_mask[gw] != 0;
+  int next_c = global && gw < n_tokens ? prefix[gw / L * (L + 1) + gw % L] : 0;
   for (int64_t token = gw; token < n_tokens; token += n_warps) {
     const int b = (int)(token / L), t = (int)(token % L);
-    const bool routed = d_mask != nullptr && d_mask[token] != 0;     // NULL: the global part is skipped
-    const int c = routed ? prefix[(int64_t)b * (L + 1) + t] : 0;
+    const bool routed = next_routed;
+    const int c = next_c;
+    if (global && token + n_warps < n_tokens) {        // the next token's routing, ahead of this one's rows
+      const int64_t n = token + n_warps;
+      next_routed = d_mask[n] != 0;
+      next_c = prefix[n / L * (L + 1) + n % L];
+    }
     // a_by_row: the global output was computed for every token and A is indexed by row (forced-global iterations)
     const bool with_a = routed || a_by_row;
+    if (S == nullptr && !with_a) {                     // local part skipped, and no global part of this token
+      if (dgate != nullptr && lane == 0) dgate[token] = 0.f;
+      continue;
+    }
     const int64_t row = token * Hq * D;                          // S: dense
     const int64_t orow = b * do_bs + t * do_ts;                  // dO, dO_loc: the strides of O
     const int64_t crow = ((int64_t)b * L + (a_by_row ? t : c)) * Hq * D;
@@ -90,47 +105,66 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(const bf16* __restrict__
         }
       }
     }
-#pragma unroll 4
-    for (int p = 0; p < n_pass; ++p) {
-      const int h = p * kHeadsPerPass + sub;
-      float dl = 0.f, dg = 0.f;
-      if (h < Hq) {
-        const uint4 o = __ldg(po + p * 32);
-        if (S != nullptr) dl = dot8(split ? __ldg(pl + p * 32) : o, __ldg(ps + p * 32));   // NULL: local part skipped
-        if (with_a) dg = dot8(o, __ldg(pa + p * 32));
-      }
+    // The rows of one group of passes are asked for before those of the group ahead are reduced: the shuffles of a group
+    // otherwise stand between its loads and the next group's.
+    constexpr int kGroup = 2;
+    struct Rows { uint4 l[kGroup], s[kGroup], a[kGroup]; } cur, nxt;      // dO_loc, S, A
+    auto fetch = [&](int p0, Rows& x) {
 #pragma unroll
-      for (int off = kLanesPerHead / 2; off > 0; off >>= 1) {
-        dl += __shfl_xor_sync(0xffffffffu, dl, off);
-        dg += __shfl_xor_sync(0xffffffffu, dg, off);
-      }
-      // (every lane takes part in the shuffles; heads beyond 64 fall back to loads in place)
-      float pre_l = __shfl_sync(0xffffffffu, (h & 32) ? pre_loc[1] : pre_loc[0], h & 31);
-      float pre_g = __shfl_sync(0xffffffffu, (h & 32) ? pre_glb[1] : pre_glb[0], h & 31);
-      if (h < Hq && (lane % kLanesPerHead) == 0) {
-        const int64_t it = ((int64_t)b * Hq + h) * L + t, ic = ((int64_t)b * Hq + h) * L + c;
-        if (lse_eff != nullptr && h >= 64) {
-          pre_l = lse_loc[it];
-          pre_g = routed ? lse_glb[ic] : 0.f;
+      for (int i = 0; i < kGroup; ++i) {
+        const int p = p0 + i;
+        if (p < n_pass && p * kHeadsPerPass + sub < Hq) {
+          x.l[i] = __ldg(pl + p * 32);
+          if (S != nullptr) x.s[i] = __ldg(ps + p * 32);
+          if (with_a) x.a[i] = __ldg(pa + p * 32);
         }
-        float dl_out = dl;
-        if (lse_eff != nullptr) {
-          // Shared-window backward.  Inside the window of a routed row P_glb = beta * P_loc with
-          // beta = exp(lse_loc - lse_glb), and dP is the same product dO V^T for both modules, so the two
-          // contributions add up to P' (dP - Delta') with P' = (1 + beta) P_loc and
-          // Delta' = (Delta_loc + beta * Delta_glb) / (1 + beta): the local items carry them with these statistics.
-          float le = pre_l;
-          if (routed) {
-            const float beta = __expf(le - pre_g);
-            dl_out = (dl + beta * dg) / (1.0f + beta);
-            le -= log1pf(beta);
+      }
+    };
+    fetch(0, cur);
+    for (int p0 = 0; p0 < n_pass; p0 += kGroup) {
+      fetch(p0 + kGroup, nxt);
+#pragma unroll
+      for (int i = 0; i < kGroup; ++i) {
+        const int h = (p0 + i) * kHeadsPerPass + sub;
+        float dl = 0.f, dg = 0.f;
+        if (p0 + i < n_pass && h < Hq) {
+          if (S != nullptr) dl = dot8(cur.l[i], cur.s[i]);      // NULL: local part skipped
+          if (with_a) dg = dot8(split ? __ldg(po + (p0 + i) * 32) : cur.l[i], cur.a[i]);
+        }
+#pragma unroll
+        for (int off = kLanesPerHead / 2; off > 0; off >>= 1) {
+          dl += __shfl_xor_sync(0xffffffffu, dl, off);
+          dg += __shfl_xor_sync(0xffffffffu, dg, off);
+        }
+        // (every lane takes part in the shuffles; heads beyond 64 fall back to loads in place)
+        float pre_l = __shfl_sync(0xffffffffu, (h & 32) ? pre_loc[1] : pre_loc[0], h & 31);
+        float pre_g = __shfl_sync(0xffffffffu, (h & 32) ? pre_glb[1] : pre_glb[0], h & 31);
+        if (p0 + i < n_pass && h < Hq && (lane % kLanesPerHead) == 0) {
+          const int64_t it = ((int64_t)b * Hq + h) * L + t, ic = ((int64_t)b * Hq + h) * L + c;
+          if (lse_eff != nullptr && h >= 64) {
+            pre_l = lse_loc[it];
+            pre_g = routed ? lse_glb[ic] : 0.f;
           }
-          lse_eff[it] = le;
+          float dl_out = dl;
+          if (lse_eff != nullptr) {
+            // Shared-window backward.  Inside the window of a routed row P_glb = beta * P_loc with
+            // beta = exp(lse_loc - lse_glb), and dP is the same product dO V^T for both modules, so the two
+            // contributions add up to P' (dP - Delta') with P' = (1 + beta) P_loc and
+            // Delta' = (Delta_loc + beta * Delta_glb) / (1 + beta): the local items carry them with these statistics.
+            float le = pre_l;
+            if (routed) {
+              const float beta = __expf(le - pre_g);
+              dl_out = (dl + beta * dg) / (1.0f + beta);
+              le -= log1pf(beta);
+            }
+            lse_eff[it] = le;
+          }
+          if (S != nullptr) delta_loc[it] = dl_out;
+          if (routed) delta_glb[ic] = dg;
+          gate += dg;
         }
-        if (S != nullptr) delta_loc[it] = dl_out;
-        if (routed) delta_glb[ic] = dg;
-        gate += dg;
       }
+      cur = nxt;
     }
     if (dgate != nullptr) {
 #pragma unroll
@@ -138,6 +172,7 @@ __global__ void __launch_bounds__(256) bwd_delta_kernel(const bf16* __restrict__
       if (lane == 0) dgate[token] = with_a ? gate : 0.f;
     }
   }
+  dependency_wait();
 }
 
 // lse by row -> lse by compact row (forced-global iterations store the global log-sum-exp for every row)
@@ -1166,7 +1201,14 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
   if (!bwd_ws || (reinterpret_cast<uintptr_t>(bwd_ws) % 256) != 0 || bwd_ws_bytes < need) return L2A_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint8_t* ws = static_cast<uint8_t*>(bwd_ws);
-  if (clear_status && cudaMemsetAsync(ws, 0, kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
+  // the gather, first on the stream where there is one, clears the header (not in the debug build, whose index checks in the
+  // same kernel report through it)
+#ifdef L2A_DEBUG
+  const bool gather_clears = false;
+#else
+  const bool gather_clears = clear_status && !skip_global;
+#endif
+  if (clear_status && !gather_clears && cudaMemsetAsync(ws, 0, kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
   bf16* Qc = reinterpret_cast<bf16*>(ws + kWsHeaderBytes);
   bf16* dOc = reinterpret_cast<bf16*>(ws + kWsHeaderBytes + rows_bytes(p));
   float* delta_loc = reinterpret_cast<float*>(ws + kWsHeaderBytes + 2 * rows_bytes(p));
@@ -1198,10 +1240,9 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
   pe.mark(s);
   if (!skip_global) {
     if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s, nullptr, 0,
-                           0, qs, reinterpret_cast<int*>(ws)) != cudaSuccess)
-      return L2A_ERR_CUDA;
-    if (launch_gather_rows(static_cast<const bf16*>(dO), dOc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s, nullptr,
-                           0, 0, os, reinterpret_cast<int*>(ws), nullptr, 0, overlap) != cudaSuccess)
+                           0, qs, reinterpret_cast<int*>(ws), gather_clears ? reinterpret_cast<int32_t*>(ws) : nullptr,
+                           gather_clears ? (int)(kWsHeaderBytes / 4) : 0, false, static_cast<const bf16*>(dO), dOc, os) !=
+        cudaSuccess)
       return L2A_ERR_CUDA;
   }
   pe.mark(s);

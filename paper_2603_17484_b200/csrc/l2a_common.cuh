@@ -103,7 +103,9 @@ cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx,
                                int row_begin = 0, int row_end = 0, RowStrides src_strides = RowStrides{0, 0},
                                int* status = nullptr,    // status: workspace status word (debug-build index checks)
                                int32_t* zero = nullptr, int n_zero = 0,    // n_zero words to clear on the way
-                               bool overlap = false);    // may start under the end of the kernel before it
+                               bool overlap = false,     // may start under the end of the kernel before it
+                               const bf16* src2 = nullptr, bf16* dst2 = nullptr,    // a second tensor of the same shape
+                               RowStrides src2_strides = RowStrides{0, 0});
 
 // z[b,t] = w . S[b,t,:] + bias (fp32 accumulation); optional sum over t of sigmoid(z)^2 per batch entry
 cudaError_t launch_router_logits(const bf16* S, const float* w, float bias, float* logits, float* sum_sq, int B,

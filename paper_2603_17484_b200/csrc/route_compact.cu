@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kThreads) route_scan_kernel(RouteArgs a) {
   }
 }
 
-// One CTA per compact row (grid-stride); 16-byte chunks.  No input is __restrict__ or read with __ldg: the kernel may start
+// One CTA per compact row (grid-stride); 16-byte chunks; src2, if given, is gathered in the same way.  No input is __restrict__ or read with __ldg: the kernel may start
 // while the one before it (the routing, or whatever produced the queries) still writes them.
 __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16* dst, const int32_t* q_idx,
                                                           const int32_t* n_routed, int L,
@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16*
                                                           const int32_t* prefix, int row_begin,
                                                           int row_end, int64_t src_batch_chunks,
                                                           int64_t src_row_chunks, int* status, int32_t* zero,
-                                                          int n_zero) {
+                                                          int n_zero, const bf16* src2, bf16* dst2,
+                                                          int64_t src2_batch_chunks, int64_t src2_row_chunks) {
   const int b = blockIdx.y;
   dependency_wait();
   dependents_release();
@@ -143,15 +144,22 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16*
   }
   const uint4* s = reinterpret_cast<const uint4*>(src) + b * src_batch_chunks;   // source strides in 16-byte chunks
   uint4* d = reinterpret_cast<uint4*>(dst) + (int64_t)b * L * row_chunks;
+  const uint4* s2 = reinterpret_cast<const uint4*>(src2) + b * src2_batch_chunks;
+  uint4* d2 = reinterpret_cast<uint4*>(dst2) + (int64_t)b * L * row_chunks;
   for (int c = c_begin + blockIdx.x; c < n_pad; c += gridDim.x) {
     if (c < n_c) {
       const int t = q_idx[(int64_t)b * L + c];
       if (!dbg_in_range(t >= 0 && t < L, status)) continue;
-      for (int i = threadIdx.x; i < row_chunks; i += blockDim.x)
-        d[(int64_t)c * row_chunks + i] = __ldcg(&s[t * src_row_chunks + i]);
+      for (int i = threadIdx.x; i < row_chunks; i += blockDim.x) {
+        const uint4 x = __ldcg(&s[t * src_row_chunks + i]);
+        if (src2 != nullptr) d2[(int64_t)c * row_chunks + i] = __ldcg(&s2[t * src2_row_chunks + i]);
+        d[(int64_t)c * row_chunks + i] = x;
+      }
     } else {
-      for (int i = threadIdx.x; i < row_chunks; i += blockDim.x)
+      for (int i = threadIdx.x; i < row_chunks; i += blockDim.x) {
         d[(int64_t)c * row_chunks + i] = make_uint4(0, 0, 0, 0);
+        if (src2 != nullptr) d2[(int64_t)c * row_chunks + i] = make_uint4(0, 0, 0, 0);
+      }
     }
   }
 }
@@ -281,14 +289,17 @@ cudaError_t launch_route_compact(const RouteArgs& a, cudaStream_t stream) {
 
 cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx, const int32_t* n_routed, int B,
                                int L, int row_elems, cudaStream_t stream, const int32_t* prefix, int row_begin,
-                               int row_end, RowStrides src_strides, int* status, int32_t* zero, int n_zero, bool overlap) {
+                               int row_end, RowStrides src_strides, int* status, int32_t* zero, int n_zero, bool overlap,
+                               const bf16* src2, bf16* dst2, RowStrides src2_strides) {
   const int row_chunks = row_elems * 2 / 16;
   const int64_t ts = src_strides.t > 0 ? src_strides.t : row_elems;
   const int64_t bs = src_strides.b > 0 ? src_strides.b : (int64_t)L * ts;
+  const int64_t ts2 = src2_strides.t > 0 ? src2_strides.t : row_elems;
+  const int64_t bs2 = src2_strides.b > 0 ? src2_strides.b : (int64_t)L * ts2;
   int gx = L < 148 * 16 ? L : 148 * 16;
   dim3 grid(gx, B);
   return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, overlap, src, dst, q_idx, n_routed, L, row_chunks, prefix,
-                          row_begin, row_end, bs / 8, ts / 8, status, zero, n_zero);
+                          row_begin, row_end, bs / 8, ts / 8, status, zero, n_zero, src2, dst2, bs2 / 8, ts2 / 8);
 }
 
 }  // namespace l2a

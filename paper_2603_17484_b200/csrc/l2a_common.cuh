@@ -212,5 +212,9 @@ PhaseEvents& phase_events();  // defined with the backward
 // mapOut / mapOut2: out and out2 as store targets in 128-row tiles; used by the local mode only
 cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUtensorMap& mapK, const CUtensorMap& mapV,
                             const CUtensorMap& mapOut, const CUtensorMap& mapOut2, cudaStream_t stream);
+// the local mode with D = 128, for launches of more than one item per SM
+cudaError_t launch_attn_fwd_local(const FwdArgs& a, int64_t items, const CUtensorMap& mapQ, const CUtensorMap& mapK,
+                                  const CUtensorMap& mapV, const CUtensorMap& mapOut, const CUtensorMap& mapOut2,
+                                  cudaStream_t stream);
 
 }  // namespace l2a

@@ -214,6 +214,23 @@ __device__ __forceinline__ void named_barrier(int id, int threads) {
 __device__ __forceinline__ void dependents_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Cluster launch control: asks for a CTA of this grid that has not started yet; the answer, 16 bytes, arrives with the
+// barrier, for which 16 bytes are expected.  After an answer that none is left the CTA must not ask again.
+__device__ __forceinline__ void claim_cta(void* answer, uint64_t* bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+               ::"r"(smem_u32(answer)), "r"(smem_u32(bar)) : "memory");
+}
+// blockIdx.x of the CTA that the answer stands for (it will not run), -1: none was left
+__device__ __forceinline__ int claimed_cta(const void* answer) {
+  int x;
+  asm volatile(
+      "{\n .reg .b128 a;\n .reg .pred p;\n ld.shared.b128 a, [%1];\n"
+      " clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n mov.b32 %0, -1;\n"
+      " @p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, a;\n}"
+      : "=r"(x) : "r"(smem_u32(answer)) : "memory");
+  return x;
+}
+
 // ----------------------------------------------------------------------------------------------
 // TMA (tiled, no cluster features): global -> shared, completion counted on an mbarrier
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {

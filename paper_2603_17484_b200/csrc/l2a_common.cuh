@@ -31,7 +31,8 @@ __device__ __forceinline__ bool dbg_in_range(bool, int*) { return true; }
 #endif
 
 // Launch that may overlap with the end of the kernel before it on the stream (programmatic dependent launch): for kernels
-// that call dependency_wait() before they touch memory.  overlap = false: a plain launch.
+// that call dependency_wait() before they touch memory that the kernels ahead of them in the call write, and at their end at
+// the latest, so that whoever waits for them waits for those too.  overlap = false: a plain launch.
 template <class... P, class... A>
 cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, bool overlap,
                              A&&... args) {

@@ -55,8 +55,11 @@ struct Barriers {
   uint64_t s_full[kNumTiles];
   uint64_t p_half[kNumTiles], p_full[kNumTiles];   // P of the first 64 keys of a block / of all
   uint64_t o_final[kNumTiles];
-  uint64_t staged[kNumTiles];     // the tile's output rows are in the buffer
-  uint64_t stage_free;            // and have left it
+  // The tiles take turns on one output buffer.  The store warp gives a tile its turn when the rows staged before have left,
+  // so that each side waits for every phase of its barrier: a wait for every second phase of a common barrier returns at
+  // once, by the parity of the phase before, when the barrier is two phases behind.
+  uint64_t turn[kNumTiles];       // the buffer is the tile's
+  uint64_t staged[kNumTiles];     // the tile's output rows are in it
   uint64_t claim;
   uint64_t item_full, item_empty; // `next` holds the next item / every role has it
   Item next;
@@ -129,6 +132,7 @@ attn_fwd_local_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
       mbar_init(&bar->p_half[t], kTileM);
       mbar_init(&bar->p_full[t], kTileM);
       mbar_init(&bar->o_final[t], 1);
+      mbar_init(&bar->turn[t], 1);
       mbar_init(&bar->staged[t], kTileM);
     }
     for (int s = 0; s < kStages; ++s) {
@@ -137,7 +141,6 @@ attn_fwd_local_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
       mbar_init(&bar->v_full[s], 1);
       mbar_init(&bar->v_empty[s], 1);
     }
-    mbar_init(&bar->stage_free, 1);
     mbar_init(&bar->claim, 1);
     mbar_init(&bar->item_full, 1);
     mbar_init(&bar->item_empty, kSoftmaxWarps + 2);     // the soft-max warps, the MMA issuer, the store warp
@@ -318,6 +321,7 @@ attn_fwd_local_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
       int row0 = w.row0, hc = w.h * (D / 64), b = w.b, active1 = w.tr[1].active;
       uint32_t n1 = 0;
       bool ok = true;
+      mbar_arrive(&bar->turn[0]);
       for (uint32_t n_items = 0;; ++n_items) {
         for (int t = 0; t < 1 + active1; ++t) {
           ok = mbar_wait(&bar->staged[t], (t ? n1 : n_items) & 1, abort_flag);
@@ -326,7 +330,7 @@ attn_fwd_local_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
           if (a.out2) tma_store_4d(&mapOut2, sStage, 0, row0 + t * kTileM, hc, b);
           tma_store_commit();
           tma_store_wait_read();
-          mbar_arrive(&bar->stage_free);
+          mbar_arrive(&bar->turn[t < active1 ? 1 : 0]);     // tile 0 of the next item, if the tile was the item's last
         }
         n1 += active1;
         if (!ok || !mbar_wait(&bar->item_full, n_items & 1, abort_flag)) break;
@@ -348,8 +352,8 @@ attn_fwd_local_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
     const uint32_t s_addr = tmem + lane_base + t * kTileN;        // this row's 128 score columns
     const uint32_t o_addr = tmem + lane_base + kOCol0 + t * D;    // its D accumulator columns
     TileRange my = t ? w.tr[1] : w.tr[0];
-    int row0 = w.row0, h = w.h, b = w.b, active1 = w.tr[1].active;
-    uint32_t n_s = 0, n_o = 0, n_staged = 0;     // blocks and results of this tile, staged tiles of both, so far
+    int row0 = w.row0, h = w.h, b = w.b;
+    uint32_t n_s = 0, n_o = 0;     // blocks and results of this tile so far
     bool ok = true;
     for (uint32_t n_items = 0;; ++n_items) {
       if (my.active) {
@@ -437,15 +441,14 @@ attn_fwd_local_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
           mbar_arrive(&bar->p_full[t]);
         }
 
-        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bar->o_final[t], n_o++ & 1, abort_flag));
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bar->o_final[t], n_o & 1, abort_flag));
         tc_fence_after();
         // ---- epilogue: O / l through the buffer that the tiles use in turn, log-sum-exp
         if (ok) {
           const float inv_l = (l > 0.f) ? 1.0f / l : 0.f;
           if (valid && a.lse != nullptr)
             a.lse[((int64_t)b * a.Hq + h) * a.Lq + row] = (m_use + log2f(l)) * 0.6931471805599453f;
-          const uint32_t use = n_staged + t;
-          if (use > 0) ok = __all_sync(0xffffffffu, mbar_wait(&bar->stage_free, (use - 1) & 1, abort_flag));
+          ok = __all_sync(0xffffffffu, mbar_wait(&bar->turn[t], n_o & 1, abort_flag));
 #pragma unroll 1
           for (int c = 0; ok && c < D / 32; ++c) {
             uint32_t o[32];
@@ -467,14 +470,13 @@ attn_fwd_local_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
             mbar_arrive(&bar->staged[t]);
           }
         }
+        ++n_o;
       }
-      n_staged += 1 + active1;
       // the next item; its first scores are computed while this one's results leave
       if (!ok || !__all_sync(0xffffffffu, mbar_wait(&bar->item_full, n_items & 1, abort_flag))) break;
       const bool more = bar->next.exists != 0;
       my = bar->next.tr[t];
       row0 = bar->next.row0; h = bar->next.h; b = bar->next.b;
-      active1 = bar->next.tr[1].active;
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar->item_empty);
       if (!more) break;

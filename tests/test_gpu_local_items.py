@@ -49,3 +49,64 @@ def test_many_items_equal_few(B, L, Hq, Hkv, W, save):
             _, lse_part = call(Q[:, :, h], K[:, :, k], V[:, :, k], parts[:, :, h], h.stop - h.start, 1)
             assert torch.equal(lse_part, lse[:, h])
     assert torch.equal(whole.view(torch.int16), parts.view(torch.int16))
+
+
+def documents(L, lo, hi, seed):
+    """int32 [n + 1] boundaries of documents of lo to hi tokens that fill L."""
+    g = torch.Generator()
+    g.manual_seed(seed)
+    n = torch.randint(lo, hi + 1, (L // lo + 1,), generator=g)
+    cu = torch.cat([torch.zeros(1, dtype=torch.int64), torch.cumsum(n, 0)])
+    return torch.cat([cu[cu < L], torch.tensor([L])]).to(torch.int32)
+
+
+@pytest.mark.parametrize("L,Lk,W,save,docs", [
+    (32768, 32768, 0, True, None),            # items of one or two key blocks whose results, twice 268 MB, outlast them
+    (32768, 32768, 128, True, None),
+    (32768, 32768, 128, False, None),
+    (16384, 16384, 4096, True, (16, 200)),    # short documents: ranges of keys from the table
+    (16384, 16384, 4096, False, (16, 300)),
+    (16384, 16384, 100, True, (200, 3000)),
+    (3000, 5000, 64, True, None),             # queries behind cached keys; last group of a head with one tile
+])
+def test_short_items_hand_the_output_buffer_over(L, Lk, W, save, docs):
+    """Items that end sooner than the store of the results before them.  Every output is that of calls over so few heads that
+    each item has a CTA, bit for bit, time after time."""
+    Hq, Hkv, D = 32, 8, 128
+    g = torch.Generator(device="cuda")
+    g.manual_seed(L + W)
+    new = lambda *s: torch.empty(s, dtype=torch.bfloat16, device="cuda")
+    Q, K, V = (new(1, n, h, D).normal_(generator=g) for n, h in ((L, Hq), (Lk, Hkv), (Lk, Hkv)))
+    table = None if docs is None else l2a.l2a_pack_sequences(documents(L, *docs, seed=L + W).cuda(), L)
+    flags = l2a.FLAG_SKIP_GLOBAL | (l2a.FLAG_SAVE_FOR_BWD if save else 0)
+
+    def call(Q, K, V, O, S, lse, hq, hkv):
+        st = ((L * Hq * D, Hq * D), (Lk * Hkv * D, Hkv * D)) if hq < Hq else (None, None)
+        p = l2a.params(1, L, Lk, hq, hkv, D, W, flags=flags, q_stride=st[0], k_stride=st[1], v_stride=st[1], o_stride=st[0],
+                       seq_bounds=table)
+        ws = torch.empty(l2a.l2a_workspace_bytes(p)[1], dtype=torch.uint8, device="cuda")
+        l2a.l2a_forward(p, Q, K, V, None, None, None, None, O, S, S, lse, lse, ws)
+        return ws
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    groups = -(-L // 256)
+    assert groups * Hq > sms
+    want, want_lse = torch.full_like(Q, float("nan")), torch.empty((1, Hq, L), dtype=torch.float32, device="cuda")
+    step = next(h for h in (4, 2, 1) if groups * h <= sms)
+    for h0 in range(0, Hq, step):
+        h, k = slice(h0, h0 + step), slice(h0 * Hkv // Hq, h0 * Hkv // Hq + 1)
+        lse = torch.empty((1, step, L), dtype=torch.float32, device="cuda")
+        ws = call(Q[:, :, h], K[:, :, k], V[:, :, k], want[:, :, h], new(1, L, step, D) if save else None, lse, step, 1)
+        assert l2a.l2a_workspace_status(ws) == 0
+        want_lse[:, h] = lse
+    bits = want.view(torch.int16)
+    assert torch.isfinite(want.float()).all()
+    for _ in range(20):
+        O, S = torch.full_like(Q, float("nan")), torch.full_like(Q, float("nan")) if save else None
+        lse = torch.full_like(want_lse, float("nan"))
+        ws = call(Q, K, V, O, S, lse, Hq, Hkv)
+        assert l2a.l2a_workspace_status(ws) == 0
+        assert torch.equal(O.view(torch.int16), bits)
+        assert torch.equal(lse, want_lse)
+        if save:
+            assert torch.equal(S.view(torch.int16), bits)

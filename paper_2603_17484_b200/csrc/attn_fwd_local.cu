@@ -95,8 +95,10 @@ __device__ __forceinline__ void make_item(const FwdArgs& a, int index, Item& w) 
         lo_pos = max(lo_pos, a.seq_bounds[2 * first]);
         tr.max_lo = max(tr.max_lo, a.seq_bounds[2 * last]);
       }
-      tr.lo = lo_pos > 0 ? lo_pos / kTileN : 0;
+      // A tile takes at least one block, all of it masked if a table names a start behind the tile: every role counts on the
+      // barriers' phases of an active tile.
       tr.hi = max_pos / kTileN;
+      tr.lo = min(lo_pos > 0 ? lo_pos / kTileN : 0, tr.hi);
       w.jlo = min(w.jlo, tr.lo);
       w.jhi = max(w.jhi, tr.hi);
     }

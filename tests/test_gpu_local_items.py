@@ -110,3 +110,25 @@ def test_short_items_hand_the_output_buffer_over(L, Lk, W, save, docs):
         assert torch.equal(lse, want_lse)
         if save:
             assert torch.equal(S.view(torch.int16), bits)
+
+
+def test_rows_whose_sequence_starts_behind_them():
+    """A table that l2a_pack_sequences does not write: tiles of rows that see no key at all.  Their output is zero, the other
+    rows are those of the call without such starts, and no wait runs out."""
+    L, Hq, Hkv, D = 2048, 32, 8, 128
+    Q, K, V = (torch.randn((1, L, h, D), device="cuda").to(torch.bfloat16) for h in (Hq, Hkv, Hkv))
+    ws, out = None, []
+    for shift in (0, 300):
+        table = torch.tensor([[0, L]], dtype=torch.int32, device="cuda").repeat(L, 1)
+        if shift:
+            table[512:1024, 0] = torch.arange(512, 1024, dtype=torch.int32, device="cuda") + shift
+        p = l2a.params(1, L, L, Hq, Hkv, D, 4096, flags=l2a.FLAG_SKIP_GLOBAL, seq_bounds=table)
+        ws = torch.empty(l2a.l2a_workspace_bytes(p)[1], dtype=torch.uint8, device="cuda")
+        O = torch.full_like(Q, float("nan"))
+        l2a.l2a_forward(p, Q, K, V, None, None, None, None, O, None, None, None, None, ws)
+        assert l2a.l2a_workspace_status(ws) == 0
+        out.append(O)
+    whole, holes = out
+    assert not holes[:, 512:1024].any()
+    for rows in (slice(0, 512), slice(1024, L)):
+        assert torch.equal(holes[:, rows].view(torch.int16), whole[:, rows].view(torch.int16))

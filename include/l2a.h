@@ -307,8 +307,9 @@ l2a_status l2a_backward_sets(const l2a_params* p, const void* Q, const void* K, 
  * l2a_backward with a separate gradient for the local output.  o_t = s_t + d_t a_t, but s_t also feeds the
  * router (z_t = W s_t + bias, Eq. 3), so in a trained layer dL/ds_t = dL/do_t + dz_t W (Section 3.3, straight-
  * through estimator).  dS_loc (bf16 [B, Lq, Hq, D], e.g. written by l2a_router_backward) drives the Local
- * Attention backward; dO drives the Global Attention backward (da_t = d_t dO_t) and dgate.  Everything else is as
- * in l2a_backward, which is this call with dS_loc = dO.
+ * Attention backward; dO drives the Global Attention backward (da_t = d_t dO_t) and dgate.  With L2A_FLAG_SKIP_LOCAL
+ * dS_loc must be a 16-byte aligned address but is not read.  Everything else is as in l2a_backward, which is this call
+ * with dS_loc = dO.
  */
 l2a_status l2a_backward_split(const l2a_params* p, const void* Q, const void* K, const void* V,
                               const uint8_t* d_mask, const int32_t* q_idx, const int32_t* n_routed,

@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(256, 2) bwd_delta_kernel(const bf16* __restric
   const int64_t n_tokens = (int64_t)B * L;
   const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (S == nullptr) dO_loc = dO;                       // local part skipped: its gradient is not read
   const bool split = dO_loc != dO;                     // separate gradient for the local output
   dependents_release();       // (reads nothing that the kernels ahead of it in the call write: it waits at its end)
   const int sub = lane / kLanesPerHead;                // head inside the pass

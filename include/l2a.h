@@ -142,7 +142,7 @@ l2a_status l2a_workspace_bytes(const l2a_params* p, size_t* route_ws_bytes, size
                                size_t* bwd_ws_bytes);
 
 /*
- * Self-test of the bounded device-side wait (the mechanism behind L2A_ERR_DEVICE_TIMEOUT).  Launches one small
+ * Self-test of the bounded device-side wait (the mechanism behind L2A_ERR_DEVICE_TIMEOUT).  Launches a small
  * kernel in which a warp waits, with a limit of `limit_us` microseconds (1 .. 1000000), for an mbarrier arrival that
  * never comes, while the other warps wait for something else: the first wait runs out, raises the CTA's abort flag,
  * the other warps leave their waits on seeing it, and the CTA writes the status word of workspace `ws` (any 256-byte
@@ -150,8 +150,10 @@ l2a_status l2a_workspace_bytes(const l2a_params* p, size_t* route_ws_bytes, size
  * out.  Afterwards l2a_workspace_status(ws) returns L2A_ERR_DEVICE_TIMEOUT and the context stays usable.  The kernel runs
  * as two clusters of two CTAs with that wait in the first CTA only, and leaves int32 words behind the status word:
  * [1], [2] CTAs of each cluster that counted their part as done (1, 2), [3], [4] whether one of them would have combined
- * the parts (0, 1), [5] .. [8] whether each CTA would have stored results behind the exchange (0, 0, 1, 1).  Nothing
- * traps, faults or spins without a limit.  Returns L2A_ERR_INVALID_ARG for a limit outside the range.
+ * the parts (0, 1), [5] .. [8] whether each CTA would have stored results behind the exchange (0, 0, 1, 1), [9], [10]
+ * whether a CTA of each cluster marked its part as failed for a kernel behind it (1, 0), [11], [12] whether that kernel, a
+ * second small launch, would have stored a combination (0, 1).  Nothing traps, faults or spins without a limit.
+ * Returns L2A_ERR_INVALID_ARG for a limit outside the range.
  */
 l2a_status l2a_selftest_wait_timeout(void* ws, unsigned limit_us, void* stream);
 

@@ -95,7 +95,9 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   constexpr int kStageBytes = 2 * kTileBytes;       // K tile, then V tile
   const int item = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
   dependents_release();
-  if (item == 0 && threadIdx.x == 0) {       // (nothing sets them before a wait has run out, seconds from here)
+  // (Nobody else sets them so early: a wait runs out seconds from here, and a misaligned base below stops every CTA, this one
+  // included.)
+  if (item == 0 && threadIdx.x == 0) {
     a.failed[b * a.Hkv + g] = 0;
     if (g == 0 && b == 0) *a.status = 0;
   }
@@ -113,7 +115,7 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
   DecodeBars* bar = reinterpret_cast<DecodeBars*>(smem + kDecStages * kStageBytes);
   volatile int* abort_flag = &bar->abort_flag;
   if ((smem_u32(smem) & 1023u) != 0) {       // the swizzled tile addressing needs a 1024-byte-aligned base
-    if (tid == 0) { atomicExch(a.status, 2); a.failed[b * a.Hkv + g] = 1; }
+    if (tid == 0) mark_failed(a.status, 2, &a.failed[b * a.Hkv + g]);
     return;
   }
   if (tid == 0) {
@@ -282,7 +284,7 @@ decode_split_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap mapK
     // a bounded wait ran out: give copies still in flight time to land before shared memory is released
     const uint64_t t0 = globaltimer_ns();
     while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
-    if (tid == 0) { atomicExch(a.status, 1); a.failed[b * a.Hkv + g] = 1; }
+    if (tid == 0) mark_failed(a.status, 1, &a.failed[b * a.Hkv + g]);
     __syncthreads();
   }
 }
@@ -316,7 +318,7 @@ __global__ void __launch_bounds__(kCombineThreads) decode_combine_kernel(const D
     const int k = grp + i * kGroups;
     v[i] = k < n ? __ldcg(reinterpret_cast<const float4*>(base + k * step + c4 * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  const int failed = __ldcg(&a.failed[b * a.Hkv + g]);
+  const bool failed = has_failed(&a.failed[b * a.Hkv + g]);
   constexpr int kMine = (kMaxWin + kMaxOut + kCombineThreads - 1) / kCombineThreads;
   float2 ml[kMine];
   float m_win = -INFINITY, m_all = -INFINITY;
@@ -388,7 +390,7 @@ __global__ void __launch_bounds__(kCombineThreads) decode_combine_kernel(const D
     add(k, __ldcg(reinterpret_cast<const float4*>(base + k * step + c4 * 4)));
   red[grp][c4] = o;
   __syncthreads();
-  if (grp == 0 && failed == 0) {
+  if (grp == 0 && !failed) {
 #pragma unroll
     for (int s = 1; s < kGroups; ++s) {
       const float4 x = red[s][c4];

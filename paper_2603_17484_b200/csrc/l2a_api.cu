@@ -152,13 +152,16 @@ namespace {
 // arrival that never comes, the other warps wait for the first one's outcome through the same abort flag, and the
 // CTA records the failure in the status word -- what every kernel of this library does at its end.  Two clusters of two
 // CTAs: in the first CTA of the first one the wait runs out, the second cluster has no such wait.  The words behind the
-// status tell who counted and who went on to store results: see l2a_selftest_wait_timeout in l2a.h.
+// status tell who counted and who went on to store results: see l2a_selftest_wait_timeout in l2a.h.  A dependent launch
+// stands for the combination of the decode chunks.
 __global__ void __cluster_dims__(2) __launch_bounds__(128) wait_timeout_selftest_kernel(int* words, uint64_t limit_ns) {
   __shared__ uint64_t never_arrives;
   __shared__ uint64_t second;
   __shared__ int abort_flag;
   const int pair = blockIdx.x >> 1;
+  dependents_release();
   if (threadIdx.x == 0) {
+    if ((blockIdx.x & 1) == 0) words[9 + pair] = 0;
     mbar_init(&never_arrives, 1);
     mbar_init(&second, 1);
     abort_flag = 0;
@@ -173,6 +176,7 @@ __global__ void __cluster_dims__(2) __launch_bounds__(128) wait_timeout_selftest
   }
   __syncthreads();
   if (threadIdx.x == 0 && arrive_last(&words[1 + pair], 2, af)) words[3 + pair] = 1;
+  if (threadIdx.x == 0 && *af) mark_failed(&words[0], 1, &words[9 + pair]);
   __syncthreads();
   cluster_sync();
   if (threadIdx.x == 0) share_abort<2>(af);
@@ -183,6 +187,10 @@ __global__ void __cluster_dims__(2) __launch_bounds__(128) wait_timeout_selftest
     else words[5 + blockIdx.x] = 1;
   }
 }
+__global__ void wait_timeout_selftest_combine_kernel(int* words) {
+  dependency_wait();
+  if (!has_failed(&words[9 + blockIdx.x])) words[11 + blockIdx.x] = 1;
+}
 }  // namespace
 }  // namespace l2a
 
@@ -192,7 +200,9 @@ l2a_status l2a_selftest_wait_timeout(void* ws, unsigned limit_us, void* stream) 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(ws, 0, l2a::kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
   l2a::wait_timeout_selftest_kernel<<<4, 128, 0, s>>>(static_cast<int*>(ws), (uint64_t)limit_us * 1000ull);
-  return cudaGetLastError() == cudaSuccess ? L2A_OK : L2A_ERR_CUDA;
+  if (cudaGetLastError() != cudaSuccess) return L2A_ERR_CUDA;
+  return launch_dependent(wait_timeout_selftest_combine_kernel, dim3(2), 1, 0, s, true, static_cast<int*>(ws)) == cudaSuccess
+             ? L2A_OK : L2A_ERR_CUDA;
 }
 
 l2a_status l2a_workspace_status(const void* ws, void* stream) {

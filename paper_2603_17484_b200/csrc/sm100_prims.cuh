@@ -203,6 +203,14 @@ __device__ __forceinline__ bool arrive_last(int* counter, int n, const volatile 
   return *abort_flag == 0 && atomicAdd(counter, 1) == n - 1;
 }
 
+// A part that a kernel behind this one combines: one thread of a CTA whose wait ran out (code 1; 2: it cannot run at all) marks
+// the result as lost besides the status word, and that kernel stores nothing of it.
+__device__ __forceinline__ void mark_failed(int* status, int code, int* failed) {
+  atomicExch(status, code);
+  *failed = 1;
+}
+__device__ __forceinline__ bool has_failed(const int* failed) { return __ldcg(failed) != 0; }
+
 // barrier of `threads` threads of the CTA (id 1 .. 15)
 __device__ __forceinline__ void named_barrier(int id, int threads) {
   asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");

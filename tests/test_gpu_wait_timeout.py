@@ -35,9 +35,11 @@ def test_selftest_argument_checks():
 
 
 def test_nothing_is_stored_from_the_parts_of_a_cta_whose_wait_ran_out():
-    """Neither the CTA that would combine counted parts nor the other CTAs of a cluster go on to store results (the path of
-    the split key ranges, the decode chunks and the backward clusters); a cluster without such a wait does."""
+    """Neither the CTA that would combine counted parts (split key ranges) nor the other CTAs of a cluster (backward clusters)
+    go on to store results, nor does a kernel behind that finds its parts marked as failed (decode chunks); a cluster without
+    such a wait does."""
     ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
     l2a.l2a_selftest_wait_timeout(ws, 1000)
     assert l2a.l2a_workspace_status(ws) == -5
     assert ws.view(torch.int32)[:9].tolist() == [1, 1, 2, 0, 1, 0, 0, 1, 1]
+    assert ws.view(torch.int32)[9:13].tolist() == [1, 0, 0, 1]

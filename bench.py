@@ -34,7 +34,7 @@ sys.path.insert(0, ROOT)
 from paper_2603_17484_b200 import replicas, synth  # noqa: E402
 
 METRIC = "L2A fwd+bwd useful TFLOP/s at 128K (one layer, one GPU)"
-KERNELS_PER_STEP = 11  # route: count, scan | fwd: gather, local, global | bwd: gather x2, delta, zero, five-GEMM kernel, merge
+KERNELS_PER_STEP = 10  # route: count, scan | fwd: gather, local, global | bwd: gather, delta, zero, five-GEMM kernel, merge
 FWD_PHASES = ("gather_q", "attn_fwd_local", "attn_fwd_global")
 BWD_PHASES = ("gather_q_dO", "bwd_delta_zero", "bwd", "bwd_dq_merge")
 # DRAM read + write over algorithmic bytes of a launch, from the ncu capture of the 128K workload cut to two KV heads
@@ -278,7 +278,7 @@ def run_decode(args):
                      "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"],
                      "traffic": DECODE_TRAFFIC_RATIO * alg_bytes, "traffic_source": "scaled from the 4-sequence ncu capture",
                      "algorithmic_bytes_per_launch": alg_bytes},
-        "gpu_launches": args.steps}), flush=True)
+        "gpu_launches": 2 * args.steps}), flush=True)      # the chunks and their combination
 
 
 def run_router(args):

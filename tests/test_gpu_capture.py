@@ -11,7 +11,8 @@ from tests.gpu_util import Case, check_same_or_rounding, run_backward
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("L,Hq,Hkv,flags", [(700, 4, 2, 0), (4500, 2, 1, 0), (700, 4, 2, l2a.FLAG_SHARED_WINDOW)])
+@pytest.mark.parametrize("L,Hq,Hkv,flags", [(700, 4, 2, 0), (4500, 2, 1, 0), (700, 4, 2, l2a.FLAG_SHARED_WINDOW),
+                                             (4500, 12, 2, 0)])     # 216 local items: more than SMs
 def test_captured_step_equals_single_calls(L, Hq, Hkv, flags):
     D, W = 128, 200
     inputs = [Case(1, L, Hq, Hkv, D, W, synth.mask_bernoulli(1, L, rho, seed=3 + i), seed=20 + i, backward=True, flags=flags)

@@ -34,8 +34,10 @@ constexpr float kLog2e = 1.4426950408889634f;
 // head, 32/(D/8) heads per pass, four passes in flight: with the rows of two groups of passes in registers two CTAs fit an
 // SM (held to three or four they spill: 70 / 71 us instead of 59 beside a concurrent clearing, 2 x 4096 tokens).  The kernel
 // reads nothing that the gather ahead of it writes, so it waits for that at its end only.  From the gather to the end of the
-// clearing: 2 x 4096 tokens (28/4 heads) 90 -> 75 us, 16K tokens 121 -> 114, 64K packed (32/8) 546 -> 516.  Clearing
-// beside Delta instead of behind it: 69, 115 and 600 (DRAM turns between reads and writes).
+// clearing: 2 x 4096 tokens (28/4 heads) 90 -> 75 us, 16K tokens 121 -> 114, 64K packed (32/8) 546 -> 516; with a gradient of
+// its own for the local output, whose rows are those asked for ahead and not dO's, 92 -> 81, 140 -> 128 and (64K) 581 -> 545; of
+// the global part alone 50 -> 29, 68 -> 42 and 219 -> 115.  Clearing beside Delta instead of behind it (one gradient): 69, 115
+// and 600 (DRAM turns between reads and writes).
 __device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
   const uint32_t a[4] = {x.x, x.y, x.z, x.w}, b[4] = {y.x, y.y, y.z, y.w};
   float acc = 0.f;

@@ -630,8 +630,9 @@ cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUt
   if (a.pair_end <= a.pair_begin) return cudaSuccess;
   int64_t grid = (int64_t)(a.pair_end - a.pair_begin) * a.Hq * a.B;
   if (a.part != nullptr && grid < kSplitItems) grid = std::min<int64_t>(grid * kMaxKeySplit, kSplitItems);
-  // Local launches of more items than SMs take CTAs that process one item after the other.  Global ones do not: with the same
-  // loop 32K tokens took 1267 instead of 1256 us, 4001 tokens 66 instead of 62, 2000 tokens on 34K keys 328 instead of 303.
+  // Local launches of more items than SMs take CTAs that process one item after the other, at any window: attn_fwd_local.cu
+  // has both sides from W = 0 to 4096.  Global ones do not: with the same loop 32K tokens took 1267 instead of 1256 us, 4001
+  // tokens 66 instead of 62, 2000 tokens on 34K keys 328 instead of 303.
   const DeviceInfo* dev = device_info();
   if (dev == nullptr) return cudaErrorUnknown;
   if (!a.global_mode && a.D == 128 && grid > dev->sms)

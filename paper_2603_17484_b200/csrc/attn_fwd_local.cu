@@ -7,9 +7,11 @@
 // loads and exit, of 107000 at W = 4096 and fewer for short sequences.  What that takes beside attn_fwd_kernel: results leave
 // through a buffer of their own instead of the Q tiles, stored by a warp that does nothing else, and barriers whose
 // phases run on over the items.
-// Measured, local launch: 32K tokens (28 heads) 1467 -> 1417 us, 16K packed in documents of 2700 (32 heads) 463 -> 420, 4001
-// tokens (28 heads) 115 -> 110.  Launches of fewer items, and with D = 64 (where it gained nothing: 16K tokens 372 -> 382),
-// stay with a CTA per item.
+// Measured, local launch, a CTA per item -> this kernel: 32K tokens (28 heads) 1439 -> 1398 us, 16K packed in documents of 2700
+// (32 heads) 454 -> 404, 4001 tokens (28 heads) 119 -> 113.  Over windows, call with S_save of 32K tokens (32/8 heads): W = 0
+// 303 -> 170 us, 128 345 -> 248, 512 472 -> 375, 1000 679 -> 616, 4096 1963 -> 1890 (run to run 30); documents of 100 tokens
+// 441 -> 273; 4001 tokens (28/4) W = 0 49 -> 37, 4096 125 -> 118.  Without S_save the gains are the same or larger.
+// Launches of fewer items, and with D = 64 (where it gained nothing: 16K tokens 372 -> 382), stay with a CTA per item.
 #include "l2a_common.cuh"
 #include "sm100_prims.cuh"
 

@@ -117,8 +117,9 @@ __global__ void __launch_bounds__(kThreads) route_scan_kernel(RouteArgs a) {
   }
 }
 
-// One CTA per compact row (grid-stride); 16-byte chunks; src2, if given, is gathered in the same way.  No input is __restrict__ or read with __ldg: the kernel may start
-// while the one before it (the routing, or whatever produced the queries) still writes them.
+// One CTA per compact row (grid-stride); 16-byte chunks; src2, if given, is gathered in the same way.  No input is __restrict__
+// or read with __ldg: the kernel may start while the one before it (the routing, or whatever produced the queries) still
+// writes them.
 __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16* dst, const int32_t* q_idx,
                                                           const int32_t* n_routed, int L,
                                                           int row_chunks /* 16-byte chunks per row */,

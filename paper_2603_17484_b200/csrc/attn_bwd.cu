@@ -1242,8 +1242,8 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
   const bool overlap = pe.n == 0;
   pe.mark(s);
   if (!skip_global) {
-    if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s, nullptr, 0,
-                           0, qs, reinterpret_cast<int*>(ws), gather_clears ? reinterpret_cast<int32_t*>(ws) : nullptr,
+    if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D,
+                           1, p->Hq * p->D, s, nullptr, 0, 0, qs, reinterpret_cast<int*>(ws), gather_clears ? reinterpret_cast<int32_t*>(ws) : nullptr,
                            gather_clears ? (int)(kWsHeaderBytes / 4) : 0, false, static_cast<const bf16*>(dO), dOc, os) !=
         cudaSuccess)
       return L2A_ERR_CUDA;

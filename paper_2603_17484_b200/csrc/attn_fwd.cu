@@ -2,13 +2,18 @@
 //
 //   local  mode (Eq. 2, sliding-window mask of Section 2): query rows are sequence rows; key blocks
 //          wholly outside the band [p - W, p] are never loaded.
-//   global mode (Eq. 4; Algorithm 1): query rows are the compacted routed rows (Q_c); the causal
-//          mask uses the true position Q_idx of each compact row; the key loop of a tile stops at
+//   global mode (Eq. 4; Algorithm 1): query rows are the compacted routed rows (Q_c), the G query heads of a KV group
+//          packed into them (row c * G + i is head i of compact index c), so that the padding of the last group and the
+//          positions a group spans are those of one head in G; the causal
+//          mask uses the true position Q_idx of each compact index; the key loop of a tile stops at
 //          the block holding its largest position; the epilogue scatters the result to O by
 //          position and combines it with the local output already there (Eq. 5), and also stores
 //          the compact output O_c and log-sum-exp L_c.
 //
-// Structure (per CTA: two 128-row query tiles of one head, sharing the K/V stream):
+// Packed heads against a launch over the rows of each head, global pass: 64K tokens (28/4 heads, 8 % routed) 2333 -> 2057 us,
+// 64K in 24 documents (32/8, 20 %) 726 -> 607, 2 x 4096 tokens 104 -> 72; whole call of 2000 new tokens on 34K keys 421 -> 401.
+//
+// Structure (per CTA: two 128-row query tiles of one head or KV group, sharing the K/V stream):
 //   warps 0-7       : soft-max + correction + epilogue.  Warpgroup t (4 warps) owns tile t; one thread per query
 //                     row (= TMEM lane) holds the row's 128 scores of a key block in registers, so the row maximum
 //                     and the row sum need no exchange between threads.
@@ -81,7 +86,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   constexpr int kOCol0 = 2 * kTileN;   // first TMEM column of the O accumulators
 
   // ---- work item: heaviest first (largest row index first), heads fastest for K/V reuse in L2
-  const bool compact = a.global_mode && !a.all_rows;           // rows are compact indices into q_idx
+  const bool compact = a.global_mode && !a.all_rows;           // rows are (compact index into q_idx, head of the group)
+  const int G = a.Hq / a.Hkv;
   int item = blockIdx.x, split = 0, n_split = 1, pi;
   // (2: what is read up to the combination was complete before the local pass, a plain launch, started)
   if (a.overlap != 2) dependency_wait();
@@ -91,18 +97,20 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     int most = 0;
     for (int i = threadIdx.x & 31; i < a.B; i += 32) most = max(most, a.n_routed[i]);
     most = __reduce_max_sync(0xffffffffu, most);
-    const int64_t groups = (int64_t)((most + kRowsPerCta - 1) / kRowsPerCta) * a.Hq * a.B;
+    const int64_t groups = compact_groups(most, G) * a.Hkv * a.B;
     if (a.part != nullptr && groups > 0 && groups < kSplitGroups) n_split = min(kMaxKeySplit, kSplitItems / (int)groups);
     if (item >= groups * n_split) { dependency_wait(); return; }
     split = item % n_split;
     item /= n_split;
   }
   const int group = item;
-  const int h = item % a.Hq;
-  const int rest = item / a.Hq;
+  const int n_heads = compact ? a.Hkv : a.Hq;
+  const int hi = item % n_heads;                               // KV head, or head of the rows
+  const int rest = item / n_heads;
   const int b = rest % a.B;
-  const int g = h / (a.Hq / a.Hkv);
-  const int n_rows = compact ? a.n_routed[b] : a.Lq;           // valid (compact) rows of this batch entry
+  const int g = compact ? hi : hi / G;
+  const int pack = compact ? G : 1;                            // rows of one token
+  const int n_rows = compact ? a.n_routed[b] * G : a.Lq;       // valid rows of this batch entry
   pi = (compact ? (n_rows + kRowsPerCta - 1) / kRowsPerCta : a.pair_end) - 1 - rest / a.B;
   const int row0 = pi * kRowsPerCta;
   if (pi < 0 || row0 >= n_rows) { dependency_wait(); return; }
@@ -116,7 +124,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   if (a.global_mode) {
     // launches restricted to a row range take the groups whose last row falls into it: every group exactly once
     const int c_last = min(row0 + kRowsPerCta, n_rows) - 1;
-    const int t_last = compact ? q_idx_b[c_last] : c_last;
+    const int t_last = compact ? q_idx_b[c_last / pack] : c_last;
     if (t_last < a.row_begin || t_last >= a.row_end) { dependency_wait(); return; }
   }
 
@@ -129,7 +137,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     if (last > n_rows - 1) last = n_rows - 1;
     tr[t].active = first < n_rows;
     if (tr[t].active) {
-      const int first_seq = compact ? q_idx_b[first] : first, last_seq = compact ? q_idx_b[last] : last;
+      const int first_seq = compact ? q_idx_b[first / pack] : first, last_seq = compact ? q_idx_b[last / pack] : last;
       tr[t].min_pos = first_seq + a.q_pos_offset;
       tr[t].max_pos = last_seq + a.q_pos_offset;
       int lo_pos = tr[t].min_pos - w_eff;
@@ -224,7 +232,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       for (int t = 0; t < kNumTiles; ++t) {
         if (!tr[t].active || tr[t].lo > tr[t].hi) continue;
         mbar_expect_tx(&bar->q_full[t], SM::kQTileBytes);
-        tma_load_4d(sQ + t * SM::kQTileBytes, &mapQ, &bar->q_full[t], 0, row0 + t * kTileM, h * (D / 64), b);
+        tma_load_4d(sQ + t * SM::kQTileBytes, &mapQ, &bar->q_full[t], 0, row0 + t * kTileM, compact ? 0 : hi * (D / 64),
+                    compact ? b * a.Hkv + g : b);
       }
       for (int j = jlo; j <= jhi; ++j) {
         const int it = j - jlo, s = it % kStages;
@@ -346,7 +355,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     if (my.active) {
       const int row = row0 + t * kTileM + r;           // sequence row (local) or compact row (global)
       const bool valid = row < n_rows;
-      const int seq_row = valid ? (compact ? q_idx_b[row] : row) : -1;
+      const int seq_row = valid ? (compact ? q_idx_b[row / pack] : row) : -1;
       const int pos = valid ? seq_row + a.q_pos_offset - vis_shift : -1;   // largest visible key position
       int pos_lo = valid ? (pos - w_eff) : 0x7fffffff;                     // smallest visible key position
       if (valid && a.seq_bounds != nullptr) pos_lo = max(pos_lo, a.seq_bounds[2 * seq_row]);
@@ -476,8 +485,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     if (my.active) {
       // ---- epilogue: O / l, log-sum-exp, store (local) or scatter + combine (global)
       if (a.global_mode) dependency_wait();      // out2 and lse_loc are the local pass's results
-      const int row = row0 + t * kTileM + r;
-      const bool valid = row < n_rows;
+      const int tile_row = row0 + t * kTileM + r;
+      const bool valid = tile_row < n_rows;
+      const int row = compact ? tile_row / pack : tile_row;      // sequence row, or compact index
+      const int h = compact ? g * G + (tile_row - row * pack) : hi;
       const int seq_row = valid ? (compact ? q_idx_b[row] : row) : -1;
       if (ok) {
         float inv_l = (l > 0.f) ? 1.0f / l : 0.f;
@@ -522,8 +533,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
           fence_async_smem();
           mbar_arrive(&bar->staged[t]);
           if (r == 0 && mbar_wait(&bar->staged[t], 0, abort_flag)) {
-            tma_store_4d(&mapOut, sQ + t * SM::kQTileBytes, 0, row0 + t * kTileM, h * (D / 64), b);
-            if (a.out2) tma_store_4d(&mapOut2, sQ + t * SM::kQTileBytes, 0, row0 + t * kTileM, h * (D / 64), b);
+            tma_store_4d(&mapOut, sQ + t * SM::kQTileBytes, 0, row0 + t * kTileM, hi * (D / 64), b);
+            if (a.out2) tma_store_4d(&mapOut2, sQ + t * SM::kQTileBytes, 0, row0 + t * kTileM, hi * (D / 64), b);
             tma_store_commit();
             tma_store_wait_read();
           }
@@ -629,6 +640,7 @@ cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUt
                             cudaStream_t stream) {
   if (a.pair_end <= a.pair_begin) return cudaSuccess;
   int64_t grid = (int64_t)(a.pair_end - a.pair_begin) * a.Hq * a.B;
+  if (a.global_mode && !a.all_rows) grid = compact_groups(a.Lq, a.Hq / a.Hkv) * a.Hkv * a.B;
   if (a.part != nullptr && grid < kSplitItems) grid = std::min<int64_t>(grid * kMaxKeySplit, kSplitItems);
   // Local launches of more items than SMs take CTAs that process one item after the other, at any window: attn_fwd_local.cu
   // has both sides from W = 0 to 4096.  Global ones do not: with the same loop 32K tokens took 1267 instead of 1256 us, 4001

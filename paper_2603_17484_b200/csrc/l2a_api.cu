@@ -348,7 +348,7 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   if (!encode_rows_map(&mapQ, Q, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, qs.b, qs.t) ||
       !encode_rows_map(&mapK, K, p->B, p->Lk, p->Hkv * p->D, kTileN, p->D, ks.b, ks.t) ||
       !encode_rows_map(&mapV, V, p->B, p->Lk, p->Hkv * p->D, kTileN, p->D, vs.b, vs.t) ||
-      !encode_rows_map(&mapQc, Qc, p->B, p->Lq, p->Hq * p->D, kTileM, p->D))
+      !encode_rows_map(&mapQc, Qc, p->B * p->Hkv, p->Lq * (p->Hq / p->Hkv), p->D, kTileM, p->D))
     return L2A_ERR_CUDA;
 
   FwdArgs a;
@@ -381,8 +381,8 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   pe.mark(s);
   if (!skip_global && !force_all) {
     // consolidate routed query rows (Algorithm 1, step 1); independent of the local pass
-    if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D, s,
-                           row_range ? prefix : nullptr, row_begin, row_end, qs, status,
+    if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D,
+                           p->Hq / p->Hkv, p->D, s, row_range ? prefix : nullptr, row_begin, row_end, qs, status,
                            gather_clears ? status : part_count,
                            (int)((gather_clears ? kWsHeaderBytes + kPartCountBytes : kPartCountBytes) / 4), overlap) !=
         cudaSuccess)

@@ -50,6 +50,8 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned threads, 
 }
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
+// 256-row groups of n routed rows of one KV head: the rows of its G query heads lie packed, row c * G + i that of head i
+__host__ __device__ inline int64_t compact_groups(int n, int G) { return ((int64_t)n * G + kRowsPerCta - 1) / kRowsPerCta; }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Host-side: resolved driver entry point for cuTensorMapEncodeTiled, and a helper that encodes a
@@ -96,11 +98,12 @@ constexpr int kRouteBlockElems = 4096;  // positions per CTA of the route/compac
 cudaError_t launch_route_compact(const RouteArgs& a, cudaStream_t stream);
 cudaError_t launch_pack_sequences(const int32_t* cu_seqlens, int n_seq, int L, int32_t* seq_bounds, cudaStream_t stream);
 
-// Gathers rows src[b, q_idx[b][c], :] -> dst[b, c, :] for c < n_routed[b], and zero-fills rows up to
-// the next multiple of kRowsPerCta (bounded by L) so that padded MMA tiles read zeros.  With `prefix` given, only the
+// Gathers rows src[b, q_idx[b][c], :] -> dst[b, kv, c, :] (kv: KV head; its G heads of D elements together) for c <
+// n_routed[b], and zero-fills up to the next multiple of kRowsPerCta rows of a head (within c < L) so that padded MMA
+// tiles read zeros.  With `prefix` given, only the
 // routed rows t in [row_begin, row_end) are gathered (the padding with the range that ends at L).
 cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx, const int32_t* n_routed,
-                               int B, int L, int row_elems, cudaStream_t stream, const int32_t* prefix = nullptr,
+                               int B, int L, int row_elems, int G, int D, cudaStream_t stream, const int32_t* prefix = nullptr,
                                int row_begin = 0, int row_end = 0, RowStrides src_strides = RowStrides{0, 0},
                                int* status = nullptr,    // status: workspace status word (debug-build index checks)
                                int32_t* zero = nullptr, int n_zero = 0,    // n_zero words to clear on the way

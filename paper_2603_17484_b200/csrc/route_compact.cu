@@ -117,13 +117,14 @@ __global__ void __launch_bounds__(kThreads) route_scan_kernel(RouteArgs a) {
   }
 }
 
-// One CTA per compact row (grid-stride); 16-byte chunks; src2, if given, is gathered in the same way.  No input is __restrict__
-// or read with __ldg: the kernel may start while the one before it (the routing, or whatever produced the queries) still
-// writes them.
+// One CTA per routed row (grid-stride); 16-byte chunks; src2, if given, is gathered in the same way.  The heads of a KV group
+// (group_chunks chunks of a row) lie together in the result: [batch, KV head, compact row, group_chunks].  No input is
+// __restrict__ or read with __ldg: the kernel may start while the one before it (the routing, or whatever produced the queries)
+// still writes them.
 __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16* dst, const int32_t* q_idx,
                                                           const int32_t* n_routed, int L,
                                                           int row_chunks /* 16-byte chunks per row */,
-                                                          const int32_t* prefix, int row_begin,
+                                                          int group_chunks, int G, const int32_t* prefix, int row_begin,
                                                           int row_end, int64_t src_batch_chunks,
                                                           int64_t src_row_chunks, int* status, int32_t* zero,
                                                           int n_zero, const bf16* src2, bf16* dst2,
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16*
   if (blockIdx.x == 0 && b == 0)
     for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0;
   const int n_c = n_routed[b];
-  int n_pad = (n_c + kRowsPerCta - 1) / kRowsPerCta * kRowsPerCta;
+  int n_pad = (int)((compact_groups(n_c, G) * kRowsPerCta + G - 1) / G);
   if (n_pad > L) n_pad = L;
   // optional restriction to the routed rows t in [row_begin, row_end): they are the compact rows
   // [prefix[row_begin], prefix[row_end]); the zero padding belongs to the range that ends at L
@@ -147,19 +148,25 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16*
   uint4* d = reinterpret_cast<uint4*>(dst) + (int64_t)b * L * row_chunks;
   const uint4* s2 = reinterpret_cast<const uint4*>(src2) + b * src2_batch_chunks;
   uint4* d2 = reinterpret_cast<uint4*>(dst2) + (int64_t)b * L * row_chunks;
+  auto place = [&](int i, int c) {        // chunk i of compact row c
+    const int kv = i / group_chunks;
+    return ((int64_t)kv * L + c) * group_chunks + (i - kv * group_chunks);
+  };
   for (int c = c_begin + blockIdx.x; c < n_pad; c += gridDim.x) {
     if (c < n_c) {
       const int t = q_idx[(int64_t)b * L + c];
       if (!dbg_in_range(t >= 0 && t < L, status)) continue;
       for (int i = threadIdx.x; i < row_chunks; i += blockDim.x) {
         const uint4 x = __ldcg(&s[t * src_row_chunks + i]);
-        if (src2 != nullptr) d2[(int64_t)c * row_chunks + i] = __ldcg(&s2[t * src2_row_chunks + i]);
-        d[(int64_t)c * row_chunks + i] = x;
+        const int64_t o = place(i, c);
+        if (src2 != nullptr) d2[o] = __ldcg(&s2[t * src2_row_chunks + i]);
+        d[o] = x;
       }
     } else {
       for (int i = threadIdx.x; i < row_chunks; i += blockDim.x) {
-        d[(int64_t)c * row_chunks + i] = make_uint4(0, 0, 0, 0);
-        if (src2 != nullptr) d2[(int64_t)c * row_chunks + i] = make_uint4(0, 0, 0, 0);
+        const int64_t o = place(i, c);
+        d[o] = make_uint4(0, 0, 0, 0);
+        if (src2 != nullptr) d2[o] = make_uint4(0, 0, 0, 0);
       }
     }
   }
@@ -289,7 +296,7 @@ cudaError_t launch_route_compact(const RouteArgs& a, cudaStream_t stream) {
 }
 
 cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx, const int32_t* n_routed, int B,
-                               int L, int row_elems, cudaStream_t stream, const int32_t* prefix, int row_begin,
+                               int L, int row_elems, int G, int D, cudaStream_t stream, const int32_t* prefix, int row_begin,
                                int row_end, RowStrides src_strides, int* status, int32_t* zero, int n_zero, bool overlap,
                                const bf16* src2, bf16* dst2, RowStrides src2_strides) {
   const int row_chunks = row_elems * 2 / 16;
@@ -299,7 +306,7 @@ cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx,
   const int64_t bs2 = src2_strides.b > 0 ? src2_strides.b : (int64_t)L * ts2;
   int gx = L < 148 * 16 ? L : 148 * 16;
   dim3 grid(gx, B);
-  return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, overlap, src, dst, q_idx, n_routed, L, row_chunks, prefix,
+  return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, overlap, src, dst, q_idx, n_routed, L, row_chunks, G * D / 8, G, prefix,
                           row_begin, row_end, bs / 8, ts / 8, status, zero, n_zero, src2, dst2, bs2 / 8, ts2 / 8);
 }
 

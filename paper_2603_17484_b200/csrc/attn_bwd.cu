@@ -194,7 +194,8 @@ __global__ void __launch_bounds__(256) compact_stat_kernel(const float* __restri
 
 // ------------------------------------------------------------------------------------------------
 struct BwdArgs {
-  int B, Lq, Lk, Hq, Hkv, D;
+  int B, Lq, Lk, Hq, Hkv, D, G;      // G = Hq / Hkv
+  uint32_t g_inv;                    // ceil(2^31 / G)
   int window, q_pos_offset;
   float scale, scale_log2;
   int skip_local, skip_global;   // gradients of one module only (the other module has its own Q/K/V)
@@ -242,13 +243,13 @@ __device__ __forceinline__ float bf16hi_to_f32(uint32_t packed) { return __uint_
 
 struct ItemPlan {
   int loc_t0, loc_nt;   // first local query tile, number of local tiles
-  int glb_t0, glb_nt;   // first compact tile, number of compact tiles
-  int total;            // items of the key block: (loc_nt + glb_nt) * G
+  int glb_t0, glb_nt;   // first compact tile, number of compact tiles (the group's heads packed into their rows)
+  int total;            // items of the key block: loc_nt * G + glb_nt
 };
 
 // First tile at or after t0 that CTA `rank` of kSplit takes for head hg of the group: (tile + hg) % kSplit == rank.  By tile
 // and not by position in the item list, so that more query tiles behind a sequence (padding rows) leave the sums of dK
-// and dV as they are; shifted by the head, so that the shares are even.
+// and dV as they are; shifted by the head, so that the shares are even.  (Compact tiles: hg = 0.)
 template <int kSplit>
 __device__ __forceinline__ int first_tile(int t0, int hg, int rank) {
   return kSplit == 1 ? t0 : t0 + ((rank - t0 - hg) & (kSplit - 1));
@@ -256,15 +257,15 @@ __device__ __forceinline__ int first_tile(int t0, int hg, int rank) {
 template <int kSplit>
 __device__ __forceinline__ int share_count(const ItemPlan& p, int G, int rank) {
   if (kSplit == 1) return p.total;
-  int n = 0;
+  int n = (max(0, p.glb_t0 + p.glb_nt - first_tile<kSplit>(p.glb_t0, 0, rank)) + kSplit - 1) / kSplit;
   for (int hg = 0; hg < G; ++hg)
-    n += (max(0, p.loc_t0 + p.loc_nt - first_tile<kSplit>(p.loc_t0, hg, rank)) + kSplit - 1) / kSplit +
-         (max(0, p.glb_t0 + p.glb_nt - first_tile<kSplit>(p.glb_t0, hg, rank)) + kSplit - 1) / kSplit;
+    n += (max(0, p.loc_t0 + p.loc_nt - first_tile<kSplit>(p.loc_t0, hg, rank)) + kSplit - 1) / kSplit;
   return n;
 }
 
 __device__ __forceinline__ ItemPlan make_plan(const BwdArgs& a, int b, int k0, int span = kTileN) {
   ItemPlan p;
+  const int G = a.G;
   // packed sequences: no row at or after the end of the sequence that holds the block's last key sees any of its keys
   int row_end = a.Lq;
   if (a.seq_bounds != nullptr) {
@@ -284,45 +285,32 @@ __device__ __forceinline__ ItemPlan make_plan(const BwdArgs& a, int b, int k0, i
   if (tmin_g < 0) tmin_g = 0;
   if (tmin_g > row_end - 1 || n_c == 0) { p.glb_t0 = 0; p.glb_nt = 0; }
   else {
-    const int c_min = a.prefix[(int64_t)b * (a.Lq + 1) + (int)tmin_g];
-    const int c_end = row_end < a.Lq ? min(n_c, a.prefix[(int64_t)b * (a.Lq + 1) + row_end]) : n_c;
-    if (c_min >= c_end) { p.glb_t0 = 0; p.glb_nt = 0; }
-    else { p.glb_t0 = c_min / kTileM; p.glb_nt = (c_end - 1) / kTileM - p.glb_t0 + 1; }
+    const int r_min = a.prefix[(int64_t)b * (a.Lq + 1) + (int)tmin_g] * G;
+    const int r_end = (row_end < a.Lq ? min(n_c, a.prefix[(int64_t)b * (a.Lq + 1) + row_end]) : n_c) * G;
+    if (r_min >= r_end) { p.glb_t0 = 0; p.glb_nt = 0; }
+    else { p.glb_t0 = r_min / kTileM; p.glb_nt = (r_end - 1) / kTileM - p.glb_t0 + 1; }
   }
-  p.total = (p.loc_nt + p.glb_nt) * (a.Hq / a.Hkv);
+  p.total = p.loc_nt * G + p.glb_nt;
   return p;
 }
 
-// Walks the items of a CTA in order without divisions: (head, local/compact, tile).
+// Walks the items of a CTA in order without divisions: the local tiles of one head after the other, then the compact tiles.
+// The plan stays in shared memory and is looked at only where a head ends: the read-out warps have no registers to spare.
 template <int kSplit>
 struct ItemCursor {
-  int hg, t, glb_part, loc_end, glb_end, loc_t0, glb_t0, h0, rank;
-  __device__ __forceinline__ ItemCursor(const ItemPlan& p, int h0_, int rank_)
-      : hg(-1), t(0), glb_part(1), loc_end(p.loc_t0 + p.loc_nt), glb_end(p.glb_nt > 0 ? p.glb_t0 + p.glb_nt : 0),
-        loc_t0(p.loc_t0), glb_t0(p.glb_t0), h0(h0_), rank(rank_) {
-    t = glb_end;
-    settle();
-  }
-  __device__ __forceinline__ int h() const { return h0 + hg; }
-  __device__ __forceinline__ int glb() const { return glb_part; }
-  __device__ __forceinline__ int tile() const { return t; }
-  __device__ __forceinline__ void settle() {    // to the next tile of the share: a head may hold none, kSplit heads do not
-    for (int n = 0; n <= kSplit && t >= (glb_part ? glb_end : loc_end);) {
-      if (glb_part) { glb_part = 0; ++hg; t = first_tile<kSplit>(loc_t0, hg, rank); ++n; }
-      else { glb_part = 1; t = first_tile<kSplit>(glb_t0, hg, rank); }
+  int hg = -1, t = 0, left = 0;      // head of the group (G: compact tiles), tile, tiles of the share left in this head
+  __device__ __forceinline__ void settle(const ItemPlan& p, int G, int rank) {    // a head may hold no tile of the share
+    while (left <= 0 && hg < G) {
+      const bool glb = ++hg == G;
+      const int t0 = glb ? p.glb_t0 : p.loc_t0, nt = glb ? p.glb_nt : p.loc_nt;
+      t = first_tile<kSplit>(t0, glb ? 0 : hg, rank);
+      left = kSplit == 1 ? nt : (t0 + nt - t + kSplit - 1) / kSplit;
     }
   }
-  __device__ __forceinline__ void next() { t += kSplit; settle(); }
-};
-template <>
-struct ItemCursor<1> {
-  int head, r, per_head, loc_nt, loc_t0, glb_t0;
-  __device__ __forceinline__ ItemCursor(const ItemPlan& p, int h0, int)
-      : head(h0), r(0), per_head(p.loc_nt + p.glb_nt), loc_nt(p.loc_nt), loc_t0(p.loc_t0), glb_t0(p.glb_t0) {}
-  __device__ __forceinline__ int h() const { return head; }
-  __device__ __forceinline__ int glb() const { return r >= loc_nt; }
-  __device__ __forceinline__ int tile() const { return r < loc_nt ? loc_t0 + r : glb_t0 + (r - loc_nt); }
-  __device__ __forceinline__ void next() { if (++r == per_head) { r = 0; ++head; } }
+  __device__ __forceinline__ void next(const ItemPlan& p, int G, int rank) {
+    t += kSplit;
+    if (--left <= 0) settle(p, G, rank);
+  }
 };
 
 // ================================================================================================
@@ -356,9 +344,11 @@ __device__ __forceinline__ void red_add_v4(float* base, uint32_t a, uint32_t b, 
                "f"(__uint_as_float(b)), "f"(__uint_as_float(c)), "f"(__uint_as_float(d)), "n"(kBytes)
                : "memory");
 }
-// Least distance between two reductions of a read-out warp, in SM clocks (polled: a sleep is too coarse).  Sixteen
-// reductions then take about 1800 clocks of an item's 4000 or more; 96 to 128 measure the same, 64 and 160 are slower.
-constexpr int kRedSpacingClk = 112;
+// Least distance between two reductions of a read-out warp, in SM clocks (polled: a sleep is too coarse).  Two reads of the
+// clock and a comparison already take that long, and as little as that is needed: backward launch of 2 x 4096 tokens / of the
+// local module at 8155 tokens without it 830 / 1108 us, with 16 757 / 965, 40 766 / 974, 72 778 / 998, 112 781 / 1009, 140 818 /
+// 1067.  (The 64-bit clock, whose polling takes longer, at 96: 818 / 1057.)
+constexpr uint32_t kRedSpacingClk = 16;
 template <int D, int I>
 struct ReadOutReds {
   static constexpr int kCols = D / 4;                 // columns per quarter of the accumulator layout
@@ -367,7 +357,7 @@ struct ReadOutReds {
   __device__ __forceinline__ static void run(float* base, const uint32_t (&v)[D / 64][32]) {
     // spaced out: reductions issued back to back fill the queue of the memory pipe, and the compute warps' shared-memory
     // loads and stores (row statistics, dS) wait behind them; the read-out warps have most of an item's time to spare
-    { const long long t0 = clock64(); while (clock64() - t0 < kRedSpacingClk) { } }
+    { const uint32_t t0 = clock(); while ((uint32_t)clock() - t0 < kRedSpacingClk) { } }
     red_add_v4<kOff>(base, v[I / 8][4 * (I % 8)], v[I / 8][4 * (I % 8) + 1], v[I / 8][4 * (I % 8) + 2],
                      v[I / 8][4 * (I % 8) + 3]);
     ReadOutReds<D, I + 1>::run(base, v);
@@ -377,6 +367,13 @@ template <int D>
 struct ReadOutReds<D, D / 8> {
   __device__ __forceinline__ static void run(float*, const uint32_t (&)[D / 64][32]) {}
 };
+
+// threadIdx.x, read anew
+__device__ __forceinline__ uint32_t thread_index() {
+  uint32_t t;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+  return t;
+}
 
 template <int D>
 struct BwdSmem {
@@ -397,12 +394,14 @@ struct BwdBarriers {
   uint64_t do_full[2], do_empty[2];
   uint64_t st_full[2], st_empty[2];
   uint64_t s_full, dp_full, p_full, ds_full, ds_free, dq_full, u_free, final_bar;
+  ItemPlan plan;
+  int b, g, k0, n_c, count;   // batch entry, KV head, first key, routed rows, items of this CTA
   uint32_t tmem_base;
   int abort_flag;
 };
 static_assert(sizeof(BwdBarriers) <= 256, "barrier block");
 
-// Which of the 32 query rows col0 .. col0 + 31 (sequence rows, or compact rows of a global item) attend to key kp, as a
+// Which of the 32 query rows col0 .. col0 + 31 (sequence rows, or packed compact rows of a global item) attend to key kp, as a
 // bit mask.  The first row is the one at the key's own position -- for a global item the first routed row whose last
 // visible key is not before it, which the exclusive prefix gives -- and the last one ends the window or the sequence.
 __device__ __forceinline__ uint32_t visible_columns(const BwdArgs& a, int b, int n_c, int kp, int glb, int col0) {
@@ -413,7 +412,7 @@ __device__ __forceinline__ uint32_t visible_columns(const BwdArgs& a, int b, int
   if (glb) {
     const int32_t* prefix = a.prefix + (int64_t)b * (a.Lq + 1);
     const int c_end = row_end < a.Lq ? min(n_c, __ldg(&prefix[row_end])) : n_c;
-    return bit_range(__ldg(&prefix[(int)first]) - col0, c_end - col0);
+    return bit_range(__ldg(&prefix[(int)first]) * a.G - col0, c_end * a.G - col0);
   }
   const long long last = (long long)kp + a.window - a.q_pos_offset + 1;
   return bit_range((int)first - col0, (last < row_end ? (int)last : row_end) - col0);
@@ -508,10 +507,9 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   const int rest = a.kb_outermost ? work % heads : work / a.kb_count;
   const int b = rest % a.B;
   const int g = rest / a.B;
-  const int G = a.Hq / a.Hkv;
   const int k0 = j * kTileN;
   const ItemPlan plan = make_plan(a, b, k0);
-  const int count = share_count<kSplit>(plan, G, rank);      // this CTA's items
+  const int count = share_count<kSplit>(plan, a.G, rank);      // this CTA's items
   const int n_c = a.skip_global ? 0 : a.n_routed[b];   // the routing arrays may be NULL when the global part is skipped
 
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -557,6 +555,12 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     mbar_init(&bar->u_free, 8 * 32);     // dQ(i) has been read out: the columns may take dP^T(i+1)
     mbar_init(&bar->final_bar, 1);
     bar->abort_flag = 0;
+    bar->plan = plan;
+    bar->b = b;
+    bar->g = g;
+    bar->k0 = k0;
+    bar->n_c = n_c;
+    bar->count = count;
     fence_mbar_init();
   }
   if (warp == 17) { tmem_alloc(&bar->tmem_base, 512); tmem_relinquish(); }
@@ -585,34 +589,47 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     setmaxnreg_dec<72>();
     // lane == query row of the item's tile; this warp owns the 32 rows of its lane group and one half of the D columns,
     // read in one go: each 32 x 4 piece is then one 512-byte reduction (accumulator layout: see above)
-    const int grp = warp & 3, half = (warp - 20) >> 2;
-    const uint32_t lane_base = static_cast<uint32_t>(grp * 32) << 16;
-    const int n_tiles = (a.Lq + kTileM - 1) / kTileM;
     constexpr int kChunks = D / 32;     // 32-column TMEM loads of the whole tile; this warp takes half of them
-    ItemCursor<kSplit> cur(plan, g * G, rank);
-    for (int i = 0; i < count; ++i) {
-      const int h = cur.h(), glb = cur.glb(), tile = cur.tile();
-      cur.next();
-      float* acc = glb ? a.dq_acc_glb : a.dq_acc_loc;
-      const bool item_ok = dbg_in_range(tile >= 0 && tile < n_tiles && h >= 0 && h < a.Hq && acc != nullptr, a.status);
-      acc += (((int64_t)b * a.Hq + h) * n_tiles + tile) * (int64_t)(kTileM * D) + lane * 4;
-      if (!__all_sync(0xffffffffu, mbar_wait(&bar->dq_full, i & 1, abort_flag))) break;
+    // The tiles of a head follow one another in the accumulator: one pointer that advances, looked up where a head ends.  64
+    // of the 72 registers hold the tile, so next to nothing else lives across an item: the thread index is read anew, and
+    // head and phase share a register.
+    float* base = nullptr;
+    int left = 0, hg2 = -2;             // tiles left in this head; 2 * head (group's compact tiles: 2 * G) + phase of dq_full
+    bool item_ok = true;
+    while (true) {
+      if (left <= 0) {
+        ItemCursor<kSplit> cur;
+        cur.hg = hg2 >> 1;
+        cur.settle(bar->plan, a.G, rank);
+        if (cur.left <= 0) break;
+        const bool glb = cur.hg == a.G;
+        const int n = glb ? compact_tiles(a.Lq, a.G) : (a.Lq + kTileM - 1) / kTileM;
+        const int lane = thread_index() & 31, grp = (thread_index() >> 5) & 3, half = ((thread_index() >> 5) - 20) >> 2;
+        base = glb ? a.dq_acc_glb : a.dq_acc_loc;
+        item_ok = dbg_in_range(cur.t >= 0 && cur.t + (cur.left - 1) * kSplit < n && cur.hg <= a.G && base != nullptr, a.status);
+        // (this warp's columns start at (D / 2) * half, i.e. at quarter 2 * half of the layout)
+        base += ((glb ? (int64_t)bar->b * a.Hkv + bar->g : (int64_t)bar->b * a.Hq + bar->g * a.G + cur.hg) * n + cur.t) *
+                    (int64_t)(kTileM * D) + lane * 4 + ((2 * half) * 4 + grp) * (8 * D);
+        left = cur.left;
+        hg2 = 2 * cur.hg + (hg2 & 1);
+      }
+      if (!__all_sync(0xffffffffu, mbar_wait(&bar->dq_full, hg2 & 1, abort_flag))) break;
       tc_fence_after();
       // the warp's whole share (32 rows x D/2 columns) goes to registers first, so that the region is released before
       // the first reduction is issued: the reductions leave the SM at about 32 bytes per clock and must not hold up
       // dP^T(i+1)
       uint32_t v[kChunks / 2][32];
+      const uint32_t w = thread_index() >> 5, taddr = ((w & 3) << 21) + 384 + ((w - 20) >> 2) * (D / 2);   // (TMEM starts at 0)
 #pragma unroll
-      for (int cc = 0; cc < kChunks / 2; ++cc) tmem_ld32(tmem + lane_base + 384 + (half * (kChunks / 2) + cc) * 32, v[cc]);
+      for (int cc = 0; cc < kChunks / 2; ++cc) tmem_ld32(taddr + cc * 32, v[cc]);
       tmem_ld_wait();
       tc_fence_before();
       mbar_arrive(&bar->u_free);           // everything is in registers: dP^T(i+1) may overwrite the columns
-      if (item_ok) {
-        // this warp's columns start at (D / 2) * half, i.e. at quarter 2 * half of the accumulator layout; every further
-        // offset is a compile-time constant, so that the sixteen reductions share one address register pair
-        float* base = acc + ((2 * half) * 4 + grp) * (8 * D);
-        ReadOutReds<D, 0>::run(base, v);
-      }
+      // every offset from the base is a compile-time constant: the sixteen reductions share one address register pair
+      if (item_ok) ReadOutReds<D, 0>::run(base, v);
+      base += kSplit * kTileM * D;
+      --left;
+      hg2 ^= 1;
     }
   } else if (warp == 19) {
     setmaxnreg_dec<40>();     // idle
@@ -624,18 +641,20 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       mbar_expect_tx(&bar->kv_full, 2 * SM::kTileBytes);
       tma_load_4d(sK, &mapK, &bar->kv_full, 0, k0, g * (D / 64), b);
       tma_load_4d(sV, &mapV, &bar->kv_full, 0, k0, g * (D / 64), b);
-      ItemCursor<kSplit> cur(plan, g * G, rank);
+      ItemCursor<kSplit> cur;
+      cur.settle(bar->plan, a.G, rank);
       for (int i = 0; i < count; ++i) {
-        const int glb = cur.glb(), row0 = cur.tile() * kTileM, hc = cur.h() * (D / 64);
-        cur.next();
+        const int hg = cur.hg, glb = hg == a.G, row0 = cur.t * kTileM;
+        const int hc = glb ? 0 : (g * a.G + hg) * (D / 64), bc = glb ? b * a.Hkv + g : b;
+        cur.next(bar->plan, a.G, rank);
         const int st = i & 1;
         const uint32_t ph = ((i >> 1) & 1) ^ 1;
         if (!mbar_wait(&bar->q_empty[st], ph, abort_flag)) break;
         mbar_expect_tx(&bar->q_full[st], SM::kTileBytes);
-        tma_load_4d(sQ + st * SM::kTileBytes, glb ? &mapQc : &mapQ, &bar->q_full[st], 0, row0, hc, b);
+        tma_load_4d(sQ + st * SM::kTileBytes, glb ? &mapQc : &mapQ, &bar->q_full[st], 0, row0, hc, bc);
         if (!mbar_wait(&bar->do_empty[st], ph, abort_flag)) break;
         mbar_expect_tx(&bar->do_full[st], SM::kTileBytes);
-        tma_load_4d(sDO + st * SM::kTileBytes, glb ? &mapDOc : &mapDO, &bar->do_full[st], 0, row0, hc, b);
+        tma_load_4d(sDO + st * SM::kTileBytes, glb ? &mapDOc : &mapDO, &bar->do_full[st], 0, row0, hc, bc);
       }
     }
     __syncwarp();
@@ -646,19 +665,27 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
     // The global loads of item i+1 are issued before waiting for its slot, so their latency is hidden.
     float r_lse[4], r_delta[4];
     int r_pos[4], r_lo[4], r_glb = 0, r_row0 = 0;   // r_lo: first token of the row's sequence (packed batches)
-    ItemCursor<kSplit> cur(plan, g * G, rank);
+    ItemCursor<kSplit> cur;
+    cur.settle(bar->plan, a.G, rank);
     auto load_item = [&]() {
-      const int h = cur.h(), glb = cur.glb(), row0 = cur.tile() * kTileM;
-      cur.next();
-      const int n_rows = glb ? n_c : a.Lq;
+      const int hg = cur.hg, glb = hg == a.G, row0 = cur.t * kTileM;
+      cur.next(bar->plan, a.G, rank);
+      const int n_rows = glb ? n_c * a.G : a.Lq;
       const float* lse = glb ? a.lse_glb : a.lse_loc;
       const float* dl = glb ? a.delta_glb : a.delta_loc;
       r_glb = glb;
       r_row0 = row0;
+      // A packed row is (compact index, head of the group): one division a tile, and one by a reciprocal for each row, exact
+      // for what is left of it (x G < 2^31).
+      const int c0 = glb ? row0 / a.G : row0, rem0 = glb ? row0 - c0 * a.G : 0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int row = row0 + q * 32 + lane;
-        const bool valid = row < n_rows;
+        const int tile_row = row0 + q * 32 + lane;
+        const bool valid = tile_row < n_rows;
+        const int x = rem0 + q * 32 + lane;
+        const int dc = glb ? (int)__umulhi(2u * x, a.g_inv) : x;
+        const int row = c0 + dc;                               // sequence row, or compact index
+        const int h = g * a.G + (glb ? x - dc * a.G : hg);
         const int64_t si = ((int64_t)b * a.Hq + h) * a.Lq + (valid ? row : 0);
         // (written by launches of this call that this one may overlap with: not through the read-only path)
         r_lse[q] = valid ? __ldcg(&lse[si]) * kLog2e : 0.f;
@@ -788,13 +815,13 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   } else {
     // ------------------------------------------------------------------ P^T, dS and epilogue
     setmaxnreg_inc<80>();
+    bool ok = true;
+    {                                                  // (scope: nothing of the loop lives on into the epilogue)
     const int q = warp >> 2;                           // query-column quarter of this warp
     const int kr = (warp & 3) * 32 + lane;             // key inside the block == TMEM lane
-    const int kp = k0 + kr;
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const uint32_t s_addr = tmem + lane_base + 256 + q * 32;
     const uint32_t dp_addr = tmem + lane_base + 384 + q * 32;
-    bool ok = true;
     for (int i = 0; i < count; ++i) {
       const int s = i & 1;
       // this item's row statistics go to registers before the scores are waited for
@@ -812,7 +839,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       // bits within this warp's 32 columns.  (Reading position and sequence start of every column instead took an edge
       // tile's probabilities from 1100 to 5900 clk, for one tile in eight at 4K tokens.)
       uint32_t visible = 0;
-      if (masked) visible = visible_columns(a, b, n_c, kp, st_flags[4], st_flags[5] + q * 32);
+      if (masked) visible = visible_columns(a, bar->b, bar->n_c, k0 + kr, st_flags[4], st_flags[5] + q * 32);
       if (!__all_sync(0xffffffffu, mbar_wait(&bar->s_full, i & 1, abort_flag))) { ok = false; break; }
       tc_fence_after();
       uint32_t pp[16];
@@ -823,24 +850,20 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
           uint32_t sv[16];
           tmem_ld16(s_addr + hh * 16, sv);
           tmem_ld_wait();
-          // the element mask is needed only for the few tiles that straddle the causal diagonal or a window edge:
-          // two loop versions, so that the common one has no branches
-          if (!masked) {
+#pragma unroll
+          for (int e8 = 0; e8 < 8; ++e8) {
+            const int e = hh * 8 + e8;
+            const float2 x = __ffma2_rn(make_float2(__uint_as_float(sv[2 * e8]), __uint_as_float(sv[2 * e8 + 1])),
+                                        make_float2(a.scale_log2, a.scale_log2), make_float2(st[2 * e], st[2 * e + 1]));
+            pp[e] = pack_bf16(fast_exp2(x.x), fast_exp2(x.y));
+          }
+          // the element mask is needed only for the few tiles that straddle the causal diagonal or a window edge; it acts on
+          // the packed bits, whatever an invisible score's exponential is (a second loop version instead: 965 -> 985 us)
+          if (masked) {
 #pragma unroll
             for (int e8 = 0; e8 < 8; ++e8) {
               const int e = hh * 8 + e8;
-              const float2 x = __ffma2_rn(make_float2(__uint_as_float(sv[2 * e8]), __uint_as_float(sv[2 * e8 + 1])),
-                                          make_float2(a.scale_log2, a.scale_log2), make_float2(st[2 * e], st[2 * e + 1]));
-              pp[e] = pack_bf16(fast_exp2(x.x), fast_exp2(x.y));
-            }
-          } else {
-#pragma unroll
-            for (int e8 = 0; e8 < 8; ++e8) {
-              const int e = hh * 8 + e8;
-              const float2 x = __ffma2_rn(make_float2(__uint_as_float(sv[2 * e8]), __uint_as_float(sv[2 * e8 + 1])),
-                                          make_float2(a.scale_log2, a.scale_log2), make_float2(st[2 * e], st[2 * e + 1]));
-              pp[e] = pack_bf16((visible >> (2 * e)) & 1u ? fast_exp2(x.x) : 0.f,
-                                (visible >> (2 * e + 1)) & 1u ? fast_exp2(x.y) : 0.f);
+              pp[e] &= ((visible >> (2 * e)) & 1u ? 0xffffu : 0u) | ((visible >> (2 * e + 1)) & 1u ? 0xffff0000u : 0u);
             }
           }
         }
@@ -893,8 +916,12 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       tc_fence_before();         // orders the TMEM accesses above before dK, and before dQ that overwrites the columns
       mbar_arrive(&bar->ds_full);
     }
+    }
     // epilogue: quarters 0,1 store the two column halves of dV, quarters 2,3 those of dK
-    const bool own = count > 0;      // a CTA whose share is empty issued nothing and adds nothing
+    // (what it needs is read anew: in registers across the items it costs the loop spills)
+    const bool own = bar->count > 0; // a CTA whose share is empty issued nothing and adds nothing
+    const int q = thread_index() >> 7, kr = thread_index() & 127;
+    const uint32_t lane_base = (thread_index() & 96) << 16;
     if (own && ok) ok = __all_sync(0xffffffffu, mbar_wait(&bar->final_bar, 0, abort_flag));
     tc_fence_after();
     if (kSplit > 1) {
@@ -911,7 +938,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
       cluster_sync();
       ok = ok && owner == me && *abort_flag == 0;      // (all CTAs have left their waits: the flag is final)
     }
-    if (ok) store_dkv<D, kSplit>(a, smem, tmem + lane_base + q * (D / 2), own, b, g, k0 + kr, q, kr);
+    if (ok) store_dkv<D, kSplit>(a, smem, tmem + lane_base + q * (D / 2), own, bar->b, bar->g, bar->k0 + kr, q, kr);
   }
   if (kSplit > 1 && warp >= kComputeWarps) {   // the other warps' part in the two barriers
     __syncwarp();
@@ -929,18 +956,19 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   if (warp == 17) tmem_dealloc(tmem, 512);
 }
 
-// Zeroes the fp32 dQ accumulators: every row tile of the local one, the compact tiles below n_routed of the global one.
+// Zeroes the fp32 dQ accumulators: every row tile of the local one, the compact tiles in use of the global one.
 __global__ void __launch_bounds__(256) dq_zero_kernel(float* __restrict__ acc_loc, float* __restrict__ acc_glb,
-                                                      const int32_t* __restrict__ n_routed, int B, int Hq, int n_tiles,
+                                                      const int32_t* __restrict__ n_routed, int B, int Hq, int Hkv, int L,
                                                       int tile_floats) {
+  const int n_tiles = (L + kTileM - 1) / kTileM, n_ctiles = compact_tiles(L, Hq / Hkv);
   const int per = B * Hq * n_tiles;
   dependency_wait();
   dependents_release();
-  for (int item = blockIdx.x; item < 2 * per; item += gridDim.x) {
+  for (int item = blockIdx.x; item < per + B * Hkv * n_ctiles; item += gridDim.x) {
     const int which = item >= per, rem = which ? item - per : item;
     float* base = which ? acc_glb : acc_loc;
     if (base == nullptr) continue;
-    if (which && (rem % n_tiles) * kTileM >= n_routed[rem / (n_tiles * Hq)]) continue;
+    if (which && rem % n_ctiles >= compact_tiles(n_routed[rem / (n_ctiles * Hkv)], Hq / Hkv)) continue;
     float4* p = reinterpret_cast<float4*>(base + (int64_t)rem * tile_floats);
     for (int k = threadIdx.x; k < tile_floats / 4; k += blockDim.x) p[k] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
@@ -954,7 +982,7 @@ template <int D>
 __global__ void __launch_bounds__(256) dq_merge_kernel(const float* acc_loc, const float* acc_glb,
                                                        const uint8_t* __restrict__ d_mask,
                                                        const int32_t* __restrict__ prefix, bf16* __restrict__ dQ, int B,
-                                                       int L, int Hq, float scale, int64_t bs, int64_t ts,
+                                                       int L, int Hq, int Hkv, float scale, int64_t bs, int64_t ts,
                                                        int tile_begin, int tile_count, int* status) {
   constexpr int kChunks = D / 8;             // 16-byte chunks per bf16 row
   constexpr int kRowBytes = D * 2 + 16;      // padded: conflict-free 16-byte accesses down a column
@@ -965,6 +993,7 @@ __global__ void __launch_bounds__(256) dq_merge_kernel(const float* acc_loc, con
   const int tile = tile_begin + (blockIdx.x / Hq) % tile_count;
   const int b = blockIdx.x / (Hq * tile_count);
   const int64_t tile_floats = kTileM * D;
+  const int G = Hq / Hkv, kv = h / G, hg = h - kv * G, n_ctiles = compact_tiles(L, G);
   const float* loc = acc_loc ? acc_loc + (((int64_t)b * Hq + h) * n_tiles + tile) * tile_floats : nullptr;
   for (int idx = threadIdx.x; idx < kTileM * kChunks; idx += blockDim.x) {
     const int lane = idx & 31, rq = (idx >> 5) & 3, k = idx >> 7;
@@ -977,10 +1006,10 @@ __global__ void __launch_bounds__(256) dq_merge_kernel(const float* acc_loc, con
       x = __ldcg(p); y = __ldcg(p + 32);
     }
     if (acc_glb && d_mask[(int64_t)b * L + t]) {
-      const int cr = prefix[(int64_t)b * (L + 1) + t];
-      if (!dbg_in_range(cr >= 0 && cr < n_tiles * kTileM, status)) continue;
+      const int cr = prefix[(int64_t)b * (L + 1) + t] * G + hg;
+      if (!dbg_in_range(cr >= 0 && cr < n_ctiles * kTileM, status)) continue;
       const float4* p = reinterpret_cast<const float4*>(
-          acc_glb + (((int64_t)b * Hq + h) * n_tiles + (cr >> 7)) * tile_floats + (q * 4 + ((cr & 127) >> 5)) * (8 * D) +
+          acc_glb + (((int64_t)b * Hkv + kv) * n_ctiles + (cr >> 7)) * tile_floats + (q * 4 + ((cr & 127) >> 5)) * (8 * D) +
           c * 128 + (cr & 31) * 4);
       const float4 gx = __ldcg(p), gy = __ldcg(p + 32);
       x.x += gx.x; x.y += gx.y; x.z += gx.z; x.w += gx.w;
@@ -1091,7 +1120,7 @@ cudaError_t launch_bwd(const BwdArgs& base, const CUtensorMap& mapQ, const CUten
   const int n_tiles = (base.Lq + kTileM - 1) / kTileM;
   const bool overlap = phase_events().n == 0;    // (events between the launches ask for their times one after the other)
   cudaError_t err = launch_dependent(dq_zero_kernel, dim3(dev->sms * 8), 256, 0, s, overlap, base.dq_acc_loc, base.dq_acc_glb,
-                                     base.n_routed, base.B, base.Hq, n_tiles, kTileM * D);
+                                     base.n_routed, base.B, base.Hq, base.Hkv, base.Lq, kTileM * D);
   if (err != cudaSuccess) return err;
   phase_events().mark(s);
   const int n_kblocks = (base.Lk + kTileN - 1) / kTileN;
@@ -1111,7 +1140,7 @@ cudaError_t launch_bwd(const BwdArgs& base, const CUtensorMap& mapQ, const CUten
     const int t1 = part + 1 < n_ranges ? dq_final_tiles(kb_end, base.q_pos_offset, n_tiles) : n_tiles;
     if (t1 > t_done &&
         (err = launch_dependent(dq_merge_kernel<D>, dim3((unsigned)((t1 - t_done) * base.B * base.Hq)), 256, 0, s, overlap,
-                                base.dq_acc_loc, base.dq_acc_glb, d_mask, base.prefix, base.dQ, base.B, base.Lq, base.Hq,
+                                base.dq_acc_loc, base.dq_acc_glb, d_mask, base.prefix, base.dQ, base.B, base.Lq, base.Hq, base.Hkv,
                                 base.scale, base.dq_st.b, base.dq_st.t, t_done, t1 - t_done, base.status)) != cudaSuccess)
       return err;
     if (t1 > t_done) t_done = t1;
@@ -1231,8 +1260,8 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
   const RowStrides os = resolve_strides(p->o_stride, p->Lq, p->Hq * p->D);
   if (!encode_rows_map(&mapQ, Q, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, qs.b, qs.t) ||
       !encode_rows_map(&mapDO, dS_loc, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, os.b, os.t) ||   // local items: dL/ds_t
-      !encode_rows_map(&mapQc, Qc, p->B, p->Lq, p->Hq * p->D, kTileM, p->D) ||
-      !encode_rows_map(&mapDOc, dOc, p->B, p->Lq, p->Hq * p->D, kTileM, p->D) ||
+      !encode_rows_map(&mapQc, Qc, p->B * p->Hkv, p->Lq * (p->Hq / p->Hkv), p->D, kTileM, p->D) ||
+      !encode_rows_map(&mapDOc, dOc, p->B * p->Hkv, p->Lq * (p->Hq / p->Hkv), p->D, kTileM, p->D) ||
       !encode_rows_map(&mapK, K, p->B, p->Lk, p->Hkv * p->D, kTileN, p->D, ks.b, ks.t) ||
       !encode_rows_map(&mapV, V, p->B, p->Lk, p->Hkv * p->D, kTileN, p->D, vs.b, vs.t))
     return L2A_ERR_CUDA;
@@ -1243,7 +1272,7 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
   pe.mark(s);
   if (!skip_global) {
     if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D,
-                           1, p->Hq * p->D, s, nullptr, 0, 0, qs, reinterpret_cast<int*>(ws), gather_clears ? reinterpret_cast<int32_t*>(ws) : nullptr,
+                           p->Hq / p->Hkv, p->D, s, nullptr, 0, 0, qs, reinterpret_cast<int*>(ws), gather_clears ? reinterpret_cast<int32_t*>(ws) : nullptr,
                            gather_clears ? (int)(kWsHeaderBytes / 4) : 0, false, static_cast<const bf16*>(dO), dOc, os) !=
         cudaSuccess)
       return L2A_ERR_CUDA;
@@ -1272,6 +1301,8 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
   }
   BwdArgs a;
   a.B = p->B; a.Lq = p->Lq; a.Lk = p->Lk; a.Hq = p->Hq; a.Hkv = p->Hkv; a.D = p->D;
+  a.G = p->Hq / p->Hkv;
+  a.g_inv = (uint32_t)(((1ull << 31) + a.G - 1) / a.G);
   a.window = p->window < (1 << 30) ? p->window : (1 << 30);   // any window >= Lk is the same
   a.q_pos_offset = p->q_pos_offset;
   a.scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)p->D);

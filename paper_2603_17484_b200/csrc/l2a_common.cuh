@@ -52,6 +52,8 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned threads, 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 // 256-row groups of n routed rows of one KV head: the rows of its G query heads lie packed, row c * G + i that of head i
 __host__ __device__ inline int64_t compact_groups(int n, int G) { return ((int64_t)n * G + kRowsPerCta - 1) / kRowsPerCta; }
+// 128-row tiles of the same
+__host__ __device__ inline int compact_tiles(int n, int G) { return (int)(((int64_t)n * G + kTileM - 1) / kTileM); }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Host-side: resolved driver entry point for cuTensorMapEncodeTiled, and a helper that encodes a

@@ -34,8 +34,8 @@ sys.path.insert(0, ROOT)
 from paper_2603_17484_b200 import replicas, synth  # noqa: E402
 
 METRIC = "L2A fwd+bwd useful TFLOP/s at 128K (one layer, one GPU)"
-KERNELS_PER_STEP = 10  # route: count, scan | fwd: gather, local, global | bwd: gather, delta, zero, five-GEMM kernel, merge
-FWD_PHASES = ("gather_q", "attn_fwd_local", "attn_fwd_global")
+KERNELS_PER_STEP = 11  # route: count, scan | fwd: header, local, global, combination | bwd: gather, delta, zero, five-GEMM kernel, merge
+FWD_PHASES = ("fwd_start", "attn_fwd_local", "attn_fwd_global")
 BWD_PHASES = ("gather_q_dO", "bwd_delta_zero", "bwd", "bwd_dq_merge")
 # DRAM read + write over algorithmic bytes of a launch, from the ncu capture of the 128K workload cut to two KV heads
 # (profiles/bwd_kernel_l2_traffic_128k_one_kv_head.md): the launch order of the whole workload, small enough for counters
@@ -624,7 +624,7 @@ def main():
                    "useful_tflop_per_step": step_flops / 1e12, "pairs_per_head": pl + pg,
                    "tolerance": "max |err| <= 2e-2 + 2^-8 |want|, mean |err| <= 2e-3 + 2^-9 mean |want| against the "
                                 "fp64 oracle (tests/gpu_util.py)"},
-        "clocks": clocks, "e2e": e2e, "gpu_launches": KERNELS_PER_STEP * args.steps if backward else 5 * args.steps,
+        "clocks": clocks, "e2e": e2e, "gpu_launches": KERNELS_PER_STEP * args.steps if backward else 6 * args.steps,
         "roofline": roofline, "cpu_baseline": cpu,
         "phase_ms": phase_ms,
         "frac_of_peak": {"measured_burst_%.0f" % peaks["burst"]: value / world / peaks["burst"],

@@ -233,11 +233,11 @@ l2a_status l2a_router_logits(const l2a_params* p, const void* S, const float* w,
  *   lse_glb     out: fp32 [B, Hq, Lq], first n_routed[b] entries of each (b, h) row: natural-log
  *                    log-sum-exp of the global scores of compact row c (Algorithm 1's L_c).
  *                    Both lse outputs may be NULL unless L2A_FLAG_SAVE_FOR_BWD is set.
- *   fwd_ws         : workspace of at least fwd_ws_bytes (holds the compact query buffer Q_c, and the counters and
- *                    fp32 partial rows of split key ranges).
+ *   fwd_ws         : workspace of at least fwd_ws_bytes (holds the fp32 partial rows of split key ranges; the global
+ *                    kernel gathers the routed queries itself).
  * Scores and soft-max run in fp32, probabilities are rounded to bf16 for the second contraction,
  * accumulation is fp32.  Results are bit-reproducible; with few routed rows in the call the keys of a routed row
- * are split into parts (a function of Lq, Hq, B and the largest n_routed), each of which rounds its probabilities
+ * are split into parts (a function of Lq, Lk, Hq, Hkv, B and the largest n_routed), each of which rounds its probabilities
  * against its own running maximum, so that the routed rows of the same sequence in another batch can differ by
  * that rounding.  Returns L2A_ERR_UNSUPPORTED for D not in {64, 128}.
  */
@@ -469,8 +469,8 @@ l2a_status l2a_route_compact_static(const l2a_params* p, const void* router, int
  * `n_events` handles created by the caller with timing enabled; the array is copied).  The NEXT
  * l2a_forward or l2a_backward call made by this host thread records event k on its stream at its
  * k-th phase boundary and then clears the registration.  Phase boundaries:
- *   l2a_forward : 0 start | 1 after the query gather | 2 after the local kernel | 3 after the
- *                 global kernel
+ *   l2a_forward : 0 start | 1 the same (no kernel in between) | 2 after the local kernel | 3 after the
+ *                 global kernel and the combination of split key ranges
  *   l2a_backward: 0 start | 1 after the gathers | 2 after the Delta kernel and the clearing of the dQ accumulators |
  *                 3 after the five-GEMM kernel | 4 after the dQ merge (everything final).
  *                 With 7 (11) events the kernel runs as two (four) launches over key-block ranges -- keys below and

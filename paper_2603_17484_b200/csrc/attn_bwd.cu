@@ -1272,7 +1272,7 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
   pe.mark(s);
   if (!skip_global) {
     if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D,
-                           p->Hq / p->Hkv, p->D, s, nullptr, 0, 0, qs, reinterpret_cast<int*>(ws), gather_clears ? reinterpret_cast<int32_t*>(ws) : nullptr,
+                           p->Hq / p->Hkv, p->D, s, qs, reinterpret_cast<int*>(ws), gather_clears ? reinterpret_cast<int32_t*>(ws) : nullptr,
                            gather_clears ? (int)(kWsHeaderBytes / 4) : 0, false, static_cast<const bf16*>(dO), dOc, os) !=
         cudaSuccess)
       return L2A_ERR_CUDA;

@@ -10,6 +10,8 @@
 //          position and combines it with the local output already there (Eq. 5), and also stores
 //          the compact output O_c and log-sum-exp L_c.
 //
+//          The soft-max warps gather the routed rows of Q of their tile themselves, while barriers and tensor memory are set up
+//          (a kernel ahead of the local pass that wrote Q_c, 2 to 16 us, and its copy are gone).
 // Packed heads against a launch over the rows of each head, global pass: 64K tokens (28/4 heads, 8 % routed) 2333 -> 2057 us,
 // 64K in 24 documents (32/8, 20 %) 726 -> 607, 2 x 4096 tokens 104 -> 72; whole call of 2000 new tokens on 34K keys 421 -> 401.
 //
@@ -66,7 +68,6 @@ struct Barriers {
   uint64_t staged[kNumTiles];     // the tile's output rows are in shared memory
   uint32_t tmem_base;
   int abort_flag;
-  int last;       // this CTA finished last of its group's key splits
 };
 
 struct TileRange {
@@ -75,6 +76,61 @@ struct TileRange {
   int max_lo;    // largest "first visible key position" among the rows (the last row's)
   int lo, hi;    // first / last key block
 };
+
+// Key blocks of the last group of a launch over compact rows, if the last row is routed
+__host__ __device__ inline int longest_group(const FwdArgs& a) {
+  const int keys = a.Lq + a.q_pos_offset - (a.shared_window ? a.window + 1 : 0);
+  return keys > kTileN ? (keys + kTileN - 1) / kTileN : 1;
+}
+
+// Key-range splits of a launch over compact rows; every warp of a CTA calls it as a whole.  Each lane weighs one number of
+// parts, in key blocks' time (1.55 us for two tiles): an item's start, end and the gap to the next one cost kItemCost, the
+// combination kCombineCost and its data kPartCost a part.  Groups of about equal length (a chunk of new tokens) run in waves;
+// those of a whole prefill, whose lengths fall from the longest to nothing, fill the SMs, longest first, up to half a part.
+struct KeySplit {
+  int64_t groups;     // that exist (a batch entry of fewer routed rows has fewer)
+  int parts, blocks;  // most parts of a group, key blocks of a part
+};
+// Clock traces of the items of 4001 tokens: set-up 2.9 us, first scores 3.2, 1.54 a block, the end 0.5, the rows of a part 1.5,
+// to the next item 3.6.  Whole call, key ranges undivided below 32 key blocks and combined by the group's last CTA / this: one head
+// of 1024 tokens 32.8 / 26.7 us, 500 tokens (28/4 heads) 41.0 / 30.7, 2000 82.0 / 73.8, 4001 177 / 170, 100 new tokens on 60K keys 223
+// / 122, 500 (32/8, shared window) on 30K 193 / 140, 2000 on 33K 428 / 393.  (Twice as many parts: 2000 tokens 101, 4001 213: their
+// rows, 133 KB a part, take longer than the blocks they save.)  From kSplitGroups groups on nothing was gained by parts.
+constexpr float kItemCost = 7.f, kCombineCost = 4.f, kPartCost = 0.04f;
+constexpr int kShortGroup = 16, kFewGroups = 32;
+__device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
+  const int lane = threadIdx.x & 31;
+  int most = 0;
+  for (int i = lane; i < a.B; i += 32) most = max(most, a.n_routed[i]);
+  most = __reduce_max_sync(0xffffffffu, most);
+  KeySplit k;
+  k.groups = compact_groups(most, a.Hq / a.Hkv) * a.Hkv * a.B;
+  k.parts = 1;
+  const int longest = longest_group(a), shortest = max(0, longest - (a.Lq + kTileN - 1) / kTileN);
+  if (a.part != nullptr && k.groups > 0 && k.groups < kSplitGroups && longest > kMinSplitBlocks) {
+    const int p = lane + 1, items = (int)k.groups * p;      // (kMaxKeySplit = 32 candidates, one a lane)
+    const float part = (longest + p - 1) / p, sms = kSplitSms;
+    float cost;
+    if (2 * shortest >= longest) cost = ceilf(items / sms) * (part + kItemCost);
+    else cost = fmaxf(part + kItemCost, (items * kItemCost + k.groups * 0.5f * (longest + shortest)) / sms + 0.5f * part);
+    if (p > 1) cost += kCombineCost + kPartCost * items;
+    const bool possible = items <= kSplitItems && p <= longest;
+    const uint32_t key = possible ? ((uint32_t)fminf(cost * 16.f, 1e8f) << 5) + lane : 0xffffffffu;
+    const uint32_t best = __reduce_min_sync(0xffffffffu, key);
+    if (best != 0xffffffffu) k.parts = (int)(best & 31u) + 1;
+    // few short groups: two key blocks a part whatever their number, so that sequences and head shards of such a size give the
+    // same bits alone and together
+    if (longest <= kShortGroup && k.groups <= kFewGroups) k.parts = (longest + 1) / 2;
+  }
+  k.blocks = (longest + k.parts - 1) / k.parts;
+  return k;
+}
+
+// Row sum of row r of a slot
+template <int D>
+__device__ __forceinline__ void put_row_sum(const FwdArgs& a, int item, int r, float l) {
+  a.part[(size_t)item * (kRowsPerCta * (D + 2)) + (r / kTileM) * (kTileM * (D + 2)) + kTileM * (D + 1) + r % kTileM] = l;
+}
 
 template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 1)
@@ -91,17 +147,15 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   int item = blockIdx.x, split = 0, n_split = 1, pi;
   // (2: what is read up to the combination was complete before the local pass, a plain launch, started)
   if (a.overlap != 2) dependency_wait();
-  if (!a.global_mode) dependents_release();                    // the global pass may fill SMs as this one drains
+  // the global pass may fill SMs as the local one drains, the combination as the global one does
+  if (!a.global_mode || a.part != nullptr) dependents_release();
+  KeySplit ks;
   if (compact) {
     // the launch covers every row that could be routed; the groups that exist come first
-    int most = 0;
-    for (int i = threadIdx.x & 31; i < a.B; i += 32) most = max(most, a.n_routed[i]);
-    most = __reduce_max_sync(0xffffffffu, most);
-    const int64_t groups = compact_groups(most, G) * a.Hkv * a.B;
-    if (a.part != nullptr && groups > 0 && groups < kSplitGroups) n_split = min(kMaxKeySplit, kSplitItems / (int)groups);
-    if (item >= groups * n_split) { dependency_wait(); return; }
-    split = item % n_split;
-    item /= n_split;
+    ks = key_split(a);
+    if (item >= ks.groups * ks.parts) { dependency_wait(); return; }
+    split = item % ks.parts;
+    item /= ks.parts;
   }
   const int group = item;
   const int n_heads = compact ? a.Hkv : a.Hq;
@@ -121,7 +175,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   // local pass's share and enters in the epilogue)
   const bool shared = a.global_mode && a.shared_window;
   const int vis_shift = shared ? a.window + 1 : 0;
-  if (a.global_mode) {
+  if (a.global_mode && (a.row_begin > 0 || a.row_end < a.Lq)) {
     // launches restricted to a row range take the groups whose last row falls into it: every group exactly once
     const int c_last = min(row0 + kRowsPerCta, n_rows) - 1;
     const int t_last = compact ? q_idx_b[c_last / pack] : c_last;
@@ -163,8 +217,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   }
 
   // this item's part of the group's key blocks
-  n_split = max(1, min(n_split, (jhi - jlo + 1) / kMinSplitBlocks));
-  if (split >= n_split) { dependency_wait(); return; }
+  if (compact && ks.parts > 1) {
+    n_split = max(1, min(ks.parts, (jhi - jlo + ks.blocks) / ks.blocks));
+    if (split >= n_split) { dependency_wait(); return; }
+    if (split == 0 && threadIdx.x == 0) a.group_parts[group] = n_split;
+  }
   if (n_split > 1) {
     const int n = jhi - jlo + 1, first = jlo;
     jlo = first + n * split / n_split;
@@ -186,9 +243,31 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  if (tid == 0) {
+  if (compact && warp < kSoftmaxWarps) {
+    // Algorithm 1, step 1: each soft-max warp brings its 32 rows of Q, 16-byte pieces, into the layout a TMA copy would leave
+    constexpr int kPieces = D / 8, kRowsPerStep = 32 / kPieces;
+    const int row = row0 + warp * 32 + lane, c = row / pack;
+    const bf16* src = row < n_rows ? a.q + b * a.q_st.b + q_idx_b[c] * a.q_st.t + (int64_t)(g * G + row - c * pack) * D : nullptr;
+    const int piece = lane % kPieces;
+    uint4 x[kPieces];
+#pragma unroll
+    for (int k = 0; k < kPieces; ++k) {
+      const bf16* p = reinterpret_cast<const bf16*>(
+          __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(src), k * kRowsPerStep + lane / kPieces));
+      x[k] = p != nullptr ? __ldg(reinterpret_cast<const uint4*>(p) + piece) : make_uint4(0, 0, 0, 0);
+    }
+    const uint32_t dst = smem_u32(sQ + (warp >> 2) * SM::kQTileBytes) + (piece >> 3) * SM::kBoxBytes;
+#pragma unroll
+    for (int k = 0; k < kPieces; ++k) {
+      const int rr = (warp & 3) * 32 + k * kRowsPerStep + lane / kPieces;
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + rr * 128 + (((piece & 7) ^ (rr & 7)) << 4)),
+                   "r"(x[k].x), "r"(x[k].y), "r"(x[k].z), "r"(x[k].w) : "memory");
+    }
+    fence_async_smem();
+  }
+  if (tid == kTmaWarp * 32) {
     for (int t = 0; t < kNumTiles; ++t) {
-      mbar_init(&bar->q_full[t], 1);
+      mbar_init(&bar->q_full[t], compact ? kTileM : 1);
       mbar_init(&bar->s_full[t], 1);
       mbar_init(&bar->p_half[t], kTileM);
       mbar_init(&bar->p_full[t], kTileM);
@@ -218,6 +297,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     // keep its TMEM operand addresses compile-time constants
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tmem, 512);
+    if (n_split > 1 && tid < kRowsPerCta) put_row_sum<D>(a, blockIdx.x, tid, -1.f);
     if (tid == 0) atomicExch(a.status, 3);
     return;
   }
@@ -230,10 +310,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       tma_prefetch_desc(&mapK);
       tma_prefetch_desc(&mapV);
       for (int t = 0; t < kNumTiles; ++t) {
-        if (!tr[t].active || tr[t].lo > tr[t].hi) continue;
+        if (compact || !tr[t].active || tr[t].lo > tr[t].hi) continue;      // (compact rows: the soft-max warps gather them)
         mbar_expect_tx(&bar->q_full[t], SM::kQTileBytes);
-        tma_load_4d(sQ + t * SM::kQTileBytes, &mapQ, &bar->q_full[t], 0, row0 + t * kTileM, compact ? 0 : hi * (D / 64),
-                    compact ? b * a.Hkv + g : b);
+        tma_load_4d(sQ + t * SM::kQTileBytes, &mapQ, &bar->q_full[t], 0, row0 + t * kTileM, hi * (D / 64), b);
       }
       for (int j = jlo; j <= jhi; ++j) {
         const int it = j - jlo, s = it % kStages;
@@ -360,6 +439,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       int pos_lo = valid ? (pos - w_eff) : 0x7fffffff;                     // smallest visible key position
       if (valid && a.seq_bounds != nullptr) pos_lo = max(pos_lo, a.seq_bounds[2 * seq_row]);
 
+      if (compact && n_my > 0) mbar_arrive(&bar->q_full[t]);       // gathered ahead of the set-up
+
       for (int i = 0; i < n_my; ++i) {
         const int j = my.lo + i;
         // warp-uniform outcome: the TMEM loads/stores below are warp-collective
@@ -444,45 +525,24 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
       if (ok && n_my > 0) ok = __all_sync(0xffffffffu, mbar_wait(&bar->o_final[t], 0, abort_flag));
       tc_fence_after();
     }
-    const float* parts = nullptr;      // this row's slots, set in the CTA that combines them
-    if (n_split > 1) {
-      // Split key range: the rows go to this item's slot unnormalised, 16-byte pieces 128 rows apart; the CTA that
-      // finishes last combines the slots of the group.
-      constexpr size_t kSlot = kRowsPerCta * (D + 2);
-      float* slot = a.part + (size_t)blockIdx.x * kSlot + t * kTileM * (D + 2);
-      if (my.active) {
+    if (n_split > 1 && my.active) {
+      // Split key range: the rows go to this item's slot unnormalised, 16-byte pieces 128 rows apart; fwd_combine_kernel
+      // combines the slots of the group.  A negative sum marks a wait that ran out.
+      float* slot = a.part + (size_t)blockIdx.x * (kRowsPerCta * (D + 2)) + t * kTileM * (D + 2);
 #pragma unroll 1
-        for (int c = 0; n_my > 0 && c < D / 32; ++c) {
-          uint32_t o[32];
-          tmem_ld32(o_addr + c * 32, o);
-          tmem_ld_wait();
+      for (int c = 0; ok && n_my > 0 && c < D / 32; ++c) {
+        uint32_t o[32];
+        tmem_ld32(o_addr + c * 32, o);
+        tmem_ld_wait();
 #pragma unroll
-          for (int x = 0; x < 8; ++x)
-            *reinterpret_cast<uint4*>(slot + ((c * 8 + x) * kTileM + r) * 4) =
-                make_uint4(o[4 * x], o[4 * x + 1], o[4 * x + 2], o[4 * x + 3]);
-        }
-        slot[kTileM * D + r] = m_use;
-        slot[kTileM * (D + 1) + r] = n_my > 0 ? l : 0.f;
+        for (int x = 0; x < 8; ++x)
+          *reinterpret_cast<uint4*>(slot + ((c * 8 + x) * kTileM + r) * 4) =
+              make_uint4(o[4 * x], o[4 * x + 1], o[4 * x + 2], o[4 * x + 3]);
       }
-      __threadfence();
-      named_barrier(1, kSoftmaxWarps * 32);      // (reached by every soft-max warp, also after a wait that ran out)
-      if (tid == 0) bar->last = arrive_last(&a.part_count[group], n_split, abort_flag);
-      named_barrier(1, kSoftmaxWarps * 32);
-      ok = ok && bar->last;
-      __threadfence();
-      if (ok && my.active) {
-        parts = a.part + (size_t)(blockIdx.x - split) * kSlot + t * kTileM * (D + 2) + r;
-        m_use = -INFINITY;
-        for (int s = 0; s < n_split; ++s)
-          if (__ldcg(parts + s * kSlot + kTileM * (D + 1)) != 0.f) m_use = fmaxf(m_use, __ldcg(parts + s * kSlot + kTileM * D));
-        l = 0.f;
-        for (int s = 0; s < n_split; ++s) {
-          const float ls = __ldcg(parts + s * kSlot + kTileM * (D + 1));
-          if (ls != 0.f) l += ls * fast_exp2(__ldcg(parts + s * kSlot + kTileM * D) - m_use);
-        }
-      }
+      slot[kTileM * D + r] = m_use;
+      put_row_sum<D>(a, blockIdx.x, t * kTileM + r, !ok ? -1.f : n_my > 0 ? l : 0.f);
     }
-    if (my.active) {
+    if (my.active && n_split == 1) {
       // ---- epilogue: O / l, log-sum-exp, store (local) or scatter + combine (global)
       if (a.global_mode) dependency_wait();      // out2 and lse_loc are the local pass's results
       const int tile_row = row0 + t * kTileM + r;
@@ -550,28 +610,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 #pragma unroll 1
           for (int c = 0; c < D / 32; ++c) {
             uint32_t o[32];
-            if (n_my > 0 && parts == nullptr) {
+            if (n_my > 0) {
               tmem_ld32(o_addr + c * 32, o);
               tmem_ld_wait();
             } else {
 #pragma unroll
               for (int e = 0; e < 32; ++e) o[e] = 0u;    // no key before the window: the accumulator was never written
-            }
-            if (parts != nullptr) {
-              constexpr size_t kSlot = kRowsPerCta * (D + 2);
-              for (int s = 0; s < n_split; ++s) {
-                const float* p = parts + s * kSlot;
-                if (__ldcg(p + kTileM * (D + 1)) == 0.f) continue;      // no visible key in that part: nothing was written
-                const float w = fast_exp2(__ldcg(p + kTileM * D) - m_use);
-#pragma unroll
-                for (int x = 0; x < 8; ++x) {
-                  const float4 v = __ldcg(reinterpret_cast<const float4*>(p - r + ((c * 8 + x) * kTileM + r) * 4));
-                  o[4 * x] = __float_as_uint(fmaf(w, v.x, __uint_as_float(o[4 * x])));
-                  o[4 * x + 1] = __float_as_uint(fmaf(w, v.y, __uint_as_float(o[4 * x + 1])));
-                  o[4 * x + 2] = __float_as_uint(fmaf(w, v.z, __uint_as_float(o[4 * x + 2])));
-                  o[4 * x + 3] = __float_as_uint(fmaf(w, v.w, __uint_as_float(o[4 * x + 3])));
-                }
-              }
             }
             float f[32];
 #pragma unroll
@@ -633,6 +677,106 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   if (warp == kMmaWarp) tmem_dealloc(tmem, 512);
 }
 
+// Combines the parts of the groups whose key range was split, and does with their rows what the epilogue above does with
+// those of an undivided group.  A CTA takes 32 rows, a thread D / 8 columns of one: the parts of a group are read by eight CTAs
+// instead of the one that finished last (latency bound).
+template <int D>
+__global__ void __launch_bounds__(256) fwd_combine_kernel(const FwdArgs a) {
+  constexpr int kCols = D / 8, kSlot = kRowsPerCta * (D + 2);
+  dependency_wait();
+  const KeySplit ks = key_split(a);
+  const int group = blockIdx.x >> 3;
+  if (ks.parts <= 1 || group >= ks.groups) return;
+  const int G = a.Hq / a.Hkv, g = group % a.Hkv, b = group / a.Hkv % a.B, n_rows = a.n_routed[b] * G;
+  const int pi = (n_rows + kRowsPerCta - 1) / kRowsPerCta - 1 - group / a.Hkv / a.B, row0 = pi * kRowsPerCta;
+  if (pi < 0) return;
+  const int32_t* q_idx_b = a.q_idx + (int64_t)b * a.Lq;
+  const int t_last = q_idx_b[(min(row0 + kRowsPerCta, n_rows) - 1) / G];
+  if (t_last < a.row_begin || t_last >= a.row_end) return;
+  const int n_split = a.group_parts[group];
+  const int r = (blockIdx.x & 7) * 32 + (threadIdx.x & 31), col = (threadIdx.x >> 5) * kCols;
+  const int tile_row = row0 + r;
+  if (n_split <= 1 || tile_row >= n_rows) return;
+  const int row = tile_row / G, h = g * G + (tile_row - row * G), seq_row = q_idx_b[row];
+  if (!dbg_in_range(row < a.Lq && seq_row >= 0 && seq_row < a.Lq, a.status)) return;
+  const float* parts = a.part + (size_t)group * ks.parts * kSlot + (r / kTileM) * (kTileM * (D + 2)) + r % kTileM;
+  bf16* dst2 = a.out2 + b * a.out2_st.b + seq_row * a.out2_st.t + (int64_t)h * D + col;
+  uint4 old[kCols / 8];                // s_t
+#pragma unroll
+  for (int q = 0; q < kCols / 8; ++q)
+    old[q] = a.accumulate_into_out2 || a.shared_window ? reinterpret_cast<const uint4*>(dst2)[q] : make_uint4(0, 0, 0, 0);
+  float m = -INFINITY, least = 0.f, l = 0.f;
+#pragma unroll 4
+  for (int s = 0; s < n_split; ++s) {
+    const float ls = parts[s * kSlot + kTileM * (D + 1)], ms = parts[s * kSlot + kTileM * D];
+    least = fminf(least, ls);
+    if (ls != 0.f) m = fmaxf(m, ms);
+  }
+  if (least < 0.f) return;             // a wait ran out in a part: nothing of the group is stored
+  float f[kCols];
+#pragma unroll
+  for (int e = 0; e < kCols; ++e) f[e] = 0.f;
+  const float* p0 = parts - r % kTileM + (col / 4 * kTileM + r % kTileM) * 4;
+#pragma unroll 4
+  for (int s = 0; s < n_split; ++s) {
+    const float ls = parts[s * kSlot + kTileM * (D + 1)], ms = parts[s * kSlot + kTileM * D];
+    const bool any = ls != 0.f;        // else no key of that part is visible to the row, and perhaps nothing was written
+    const float w = any ? fast_exp2(ms - m) : 0.f;
+    l = fmaf(ls, w, l);
+#pragma unroll
+    for (int x = 0; x < kCols / 4; ++x) {
+      const float4 v = *reinterpret_cast<const float4*>(p0 + s * kSlot + x * (4 * kTileM));
+      f[4 * x] = any ? fmaf(w, v.x, f[4 * x]) : f[4 * x];
+      f[4 * x + 1] = any ? fmaf(w, v.y, f[4 * x + 1]) : f[4 * x + 1];
+      f[4 * x + 2] = any ? fmaf(w, v.z, f[4 * x + 2]) : f[4 * x + 2];
+      f[4 * x + 3] = any ? fmaf(w, v.w, f[4 * x + 3]) : f[4 * x + 3];
+    }
+  }
+  float inv_l = l > 0.f ? 1.0f / l : 0.f, lse2 = m + log2f(l), c_loc = 0.f;
+  if (a.shared_window) {             // (as in attn_fwd_kernel)
+    const float lse_out2 = l > 0.f ? lse2 : -INFINITY;
+    const float lse_loc2 = a.lse_loc[((int64_t)b * a.Hq + h) * a.Lq + seq_row] * 1.4426950408889634f;
+    const float mm = fmaxf(lse_out2, lse_loc2);
+    const float w_out = fast_exp2(lse_out2 - mm), w_loc = fast_exp2(lse_loc2 - mm);
+    const float inv = 1.0f / (w_out + w_loc);
+    inv_l *= w_out * inv;
+    c_loc = w_loc * inv;
+    lse2 = mm + log2f(w_out + w_loc);
+  }
+  if (col == 0 && a.lse != nullptr) a.lse[((int64_t)b * a.Hq + h) * a.Lq + row] = lse2 * 0.6931471805599453f;
+  bf16* dst1 = a.out ? a.out + b * a.out_st.b + row * a.out_st.t + (int64_t)h * D + col : nullptr;
+#pragma unroll
+  for (int q = 0; q < kCols / 8; ++q) {
+    const uint32_t ow[4] = {old[q].x, old[q].y, old[q].z, old[q].w};
+    uint32_t u[4], v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float s0 = __uint_as_float(ow[k] << 16), s1 = __uint_as_float(ow[k] & 0xffff0000u);       // s_t
+      float f0 = f[8 * q + 2 * k] * inv_l, f1 = f[8 * q + 2 * k + 1] * inv_l;
+      if (a.shared_window) { f0 = fmaf(c_loc, s0, f0); f1 = fmaf(c_loc, s1, f1); }
+      u[k] = pack_bf16(f0, f1);
+      v[k] = a.accumulate_into_out2 ? pack_bf16(f0 + s0, f1 + s1) : u[k];
+    }
+    if (dst1) reinterpret_cast<uint4*>(dst1)[q] = make_uint4(u[0], u[1], u[2], u[3]);
+    reinterpret_cast<uint4*>(dst2)[q] = make_uint4(v[0], v[1], v[2], v[3]);
+  }
+}
+
+template <int D>
+cudaError_t launch_fwd(const FwdArgs& a, int64_t grid, const CUtensorMap& mapQ, const CUtensorMap& mapK, const CUtensorMap& mapV,
+                       const CUtensorMap& mapOut, const CUtensorMap& mapOut2, int64_t groups, cudaStream_t stream) {
+  static PerDeviceOnce once;
+  cudaError_t e = once.run([] {
+    return cudaFuncSetAttribute(attn_fwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<D>::kTotal);
+  });
+  if (e != cudaSuccess) return e;
+  e = launch_dependent(attn_fwd_kernel<D>, dim3((unsigned)grid), kFwdThreads, FwdSmem<D>::kTotal, stream, a.overlap != 0, mapQ,
+                       mapK, mapV, mapOut, mapOut2, a);
+  if (e != cudaSuccess || a.part == nullptr || longest_group(a) <= kMinSplitBlocks) return e;     // nothing is split
+  return launch_dependent(fwd_combine_kernel<D>, dim3((unsigned)(8 * std::min<int64_t>(groups, kSplitGroups))), 256, 0, stream,
+                          a.overlap != 0, a);
+}
+
 }  // namespace
 
 cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUtensorMap& mapK,
@@ -641,7 +785,8 @@ cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUt
   if (a.pair_end <= a.pair_begin) return cudaSuccess;
   int64_t grid = (int64_t)(a.pair_end - a.pair_begin) * a.Hq * a.B;
   if (a.global_mode && !a.all_rows) grid = compact_groups(a.Lq, a.Hq / a.Hkv) * a.Hkv * a.B;
-  if (a.part != nullptr && grid < kSplitItems) grid = std::min<int64_t>(grid * kMaxKeySplit, kSplitItems);
+  const int64_t groups = grid;
+  if (a.part != nullptr) grid = std::max(grid, std::min<int64_t>(grid * kMaxKeySplit, kSplitItems));
   // Local launches of more items than SMs take CTAs that process one item after the other, at any window: attn_fwd_local.cu
   // has both sides from W = 0 to 4096.  Global ones do not: with the same loop 32K tokens took 1267 instead of 1256 us, 4001
   // tokens 66 instead of 62, 2000 tokens on 34K keys 328 instead of 303.
@@ -649,24 +794,8 @@ cudaError_t launch_attn_fwd(const FwdArgs& a, const CUtensorMap& mapQ, const CUt
   if (dev == nullptr) return cudaErrorUnknown;
   if (!a.global_mode && a.D == 128 && grid > dev->sms)
     return launch_attn_fwd_local(a, grid, mapQ, mapK, mapV, mapOut, mapOut2, stream);
-  cudaError_t e;
-  if (a.D == 128) {
-    static PerDeviceOnce once;
-    e = once.run([] {
-      return cudaFuncSetAttribute(attn_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::kTotal);
-    });
-    if (e != cudaSuccess) return e;
-    return launch_dependent(attn_fwd_kernel<128>, dim3((unsigned)grid), kFwdThreads, FwdSmem<128>::kTotal, stream, a.overlap != 0,
-                            mapQ, mapK, mapV, mapOut, mapOut2, a);
-  } else {
-    static PerDeviceOnce once;
-    e = once.run([] {
-      return cudaFuncSetAttribute(attn_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::kTotal);
-    });
-    if (e != cudaSuccess) return e;
-    return launch_dependent(attn_fwd_kernel<64>, dim3((unsigned)grid), kFwdThreads, FwdSmem<64>::kTotal, stream, a.overlap != 0,
-                            mapQ, mapK, mapV, mapOut, mapOut2, a);
-  }
+  return a.D == 128 ? launch_fwd<128>(a, grid, mapQ, mapK, mapV, mapOut, mapOut2, groups, stream)
+                    : launch_fwd<64>(a, grid, mapQ, mapK, mapV, mapOut, mapOut2, groups, stream);
 }
 
 }  // namespace l2a

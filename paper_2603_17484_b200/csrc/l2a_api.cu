@@ -52,8 +52,7 @@ size_t route_ws_size(const l2a_params* p) {
   const int nblocks = ceil_div(p->Lq, kRouteBlockElems);
   return kWsHeaderBytes + align_up((size_t)p->B * nblocks * sizeof(int32_t), 256);
 }
-size_t qrows_bytes(const l2a_params* p) { return align_up((size_t)p->B * p->Lq * p->Hq * p->D * sizeof(bf16), 256); }
-// forward workspace: header, counters of split key ranges, compacted queries, slots of split key ranges
+// forward workspace: header, numbers of parts of split key ranges, their slots
 constexpr size_t kPartCountBytes = (kSplitGroups * sizeof(int32_t) + 255) / 256 * 256;
 int group_count(const l2a_params* p) {
   const int64_t n = (int64_t)ceil_div(p->Lq, kRowsPerCta) * p->Hq * p->B;
@@ -63,7 +62,9 @@ size_t part_bytes(const l2a_params* p) {
   return align_up(split_slots(group_count(p)) * split_slot_floats(p->D) * sizeof(float), 256);
 }
 size_t fwd_ws_size(const l2a_params* p) {
-  return kWsHeaderBytes + kPartCountBytes + qrows_bytes(p) + part_bytes(p);
+  // (never less than one copy of Q)
+  const size_t q = align_up((size_t)p->B * p->Lq * p->Hq * p->D * sizeof(bf16), 256), parts = part_bytes(p);
+  return kWsHeaderBytes + kPartCountBytes + (q > parts ? q : parts);
 }
 
 bool ws_ok(const void* ws, size_t have, size_t need) { return ws && aligned(ws, 256) && have >= need; }
@@ -254,7 +255,7 @@ l2a_status l2a_route_compact(const l2a_params* p, const void* router, int router
 // is used by l2a_step_host to start Local Attention on the rows whose queries have already arrived; it is only
 // meaningful for the local module (L2A_FLAG_SKIP_GLOBAL), and only the first call of a step clears the status word.
 // [row_begin, row_end) restricts the global phase (L2A_FLAG_GLOBAL_PHASE) to the routed rows of that range: the
-// gather takes exactly those rows, the attention launch the compact groups whose last row lies in the range.
+// launch takes the compact groups whose last row lies in the range.
 static l2a_status forward_range(const l2a_params* p, const void* Q, const void* K, const void* V,
                                 const uint8_t* d_mask, const int32_t* q_idx, const int32_t* n_routed,
                                 const int32_t* prefix, void* O, void* S_save, void* A_c, float* lse_loc,
@@ -319,9 +320,8 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint8_t* ws = static_cast<uint8_t*>(fwd_ws);
   int* status = reinterpret_cast<int*>(ws);
-  int32_t* part_count = reinterpret_cast<int32_t*>(ws + kWsHeaderBytes);
-  bf16* Qc = reinterpret_cast<bf16*>(ws + kWsHeaderBytes + kPartCountBytes);
-  float* part = reinterpret_cast<float*>(ws + kWsHeaderBytes + kPartCountBytes + qrows_bytes(p));
+  int32_t* group_parts = reinterpret_cast<int32_t*>(ws + kWsHeaderBytes);
+  float* part = reinterpret_cast<float*>(ws + kWsHeaderBytes + kPartCountBytes);
   const int n_pairs = ceil_div(p->Lq, kRowsPerCta);
   const bool whole = pair_end < 0 || (pair_begin == 0 && pair_end == n_pairs);
   if (pair_end < 0) pair_end = n_pairs;
@@ -330,16 +330,11 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   const bool row_range = row_begin > 0 || row_end < p->Lq;
   if (row_range && (!global_phase || row_begin < 0 || row_begin > row_end)) return L2A_ERR_INVALID_ARG;
   if (row_end > p->Lq) row_end = p->Lq;
-  // the gather of the routed rows, first on the stream where there is one, clears the header and the counters behind it
-  // (not in the debug build, whose index checks in the same kernel report through the header)
-#ifdef L2A_DEBUG
-  const bool gather_clears = false;
-#else
-  const bool gather_clears = clear_status && !skip_global && !force_all;
-#endif
-  if (clear_status && !gather_clears && cudaMemsetAsync(ws, 0, kWsHeaderBytes, s) != cudaSuccess) return L2A_ERR_CUDA;
+  // (events between the launches ask for times of the passes one after the other)
+  const bool overlap = phase_events().n == 0;
+  if (clear_status && launch_clear_header(ws, overlap, s) != cudaSuccess) return L2A_ERR_CUDA;
 
-  CUtensorMap mapQ, mapK, mapV, mapQc;
+  CUtensorMap mapQ, mapK, mapV;
   const RowStrides qs = resolve_strides(p->q_stride, p->Lq, p->Hq * p->D);
   const RowStrides ks = resolve_strides(p->k_stride, p->Lk, p->Hkv * p->D);
   const RowStrides vs = resolve_strides(p->v_stride, p->Lk, p->Hkv * p->D);
@@ -347,8 +342,7 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   const RowStrides dense_q = {(int64_t)p->Lq * p->Hq * p->D, (int64_t)p->Hq * p->D};
   if (!encode_rows_map(&mapQ, Q, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, qs.b, qs.t) ||
       !encode_rows_map(&mapK, K, p->B, p->Lk, p->Hkv * p->D, kTileN, p->D, ks.b, ks.t) ||
-      !encode_rows_map(&mapV, V, p->B, p->Lk, p->Hkv * p->D, kTileN, p->D, vs.b, vs.t) ||
-      !encode_rows_map(&mapQc, Qc, p->B * p->Hkv, p->Lq * (p->Hq / p->Hkv), p->D, kTileM, p->D))
+      !encode_rows_map(&mapV, V, p->B, p->Lk, p->Hkv * p->D, kTileN, p->D, vs.b, vs.t))
     return L2A_ERR_CUDA;
 
   FwdArgs a;
@@ -369,26 +363,17 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   a.lse_loc = nullptr;
   a.seq_bounds = p->seq_bounds;
   a.part = nullptr;
-  a.part_count = nullptr;
+  a.group_parts = nullptr;
+  a.q = static_cast<const bf16*>(Q);
+  a.q_st = qs;
   a.overlap = 0;
   // split key ranges: launches over the compacted rows (those of a row range too, so that their results stay the same)
   const bool split = !skip_global && !force_all;
 
   PhaseEvents& pe = phase_events();
   struct ClearOnExit { PhaseEvents& p; ~ClearOnExit() { p.clear(); } } clear_on_exit{pe};
-  // (events between the launches ask for times of the passes one after the other)
-  const bool overlap = pe.n == 0;
   pe.mark(s);
-  if (!skip_global && !force_all) {
-    // consolidate routed query rows (Algorithm 1, step 1); independent of the local pass
-    if (launch_gather_rows(static_cast<const bf16*>(Q), Qc, q_idx, n_routed, p->B, p->Lq, p->Hq * p->D,
-                           p->Hq / p->Hkv, p->D, s, row_range ? prefix : nullptr, row_begin, row_end, qs, status,
-                           gather_clears ? status : part_count,
-                           (int)((gather_clears ? kWsHeaderBytes + kPartCountBytes : kPartCountBytes) / 4), overlap) !=
-        cudaSuccess)
-      return L2A_ERR_CUDA;
-  }
-  pe.mark(s);
+  pe.mark(s);      // (a gather of the routed rows once stood between the two)
   if (!skip_local && !global_phase) {
     a.global_mode = 0;
     a.accumulate_into_out2 = 0;
@@ -400,7 +385,7 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
     a.pair_begin = pair_begin;
     a.pair_end = pair_end;
     // Ahead of a global pass that starts under it the local pass is a plain launch: what the global pass reads before its
-    // own wait (routing, compacted queries) is then complete and visible before any kernel it can overlap with starts.
+    // own wait (routing, queries) is then complete and visible before any kernel it can overlap with starts.
     a.overlap = overlap && skip_global ? 1 : 0;
     CUtensorMap mapOut, mapOut2;
     if (!encode_rows_map(&mapOut, a.out, p->B, p->Lq, p->Hq * p->D, kTileM, p->D, a.out_st.b, a.out_st.t)) return L2A_ERR_CUDA;
@@ -430,10 +415,10 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
     a.lse_loc = lse_loc;
     if (split) {
       a.part = part;
-      a.part_count = part_count;
+      a.group_parts = group_parts;
     }
     // Behind the local pass the kernel waits only before it combines.  The local pass is the one kernel it can overlap
-    // with, and a plain launch: the gather and all before it are complete, and visible, before that starts.
+    // with, and a plain launch: all before it is complete, and visible, before that starts.
     a.overlap = !overlap ? 0 : !skip_local && !global_phase ? 2 : 1;
     if (force_all) {
       // Global Attention for every token (Section 3.3): same kernel over all rows in place; a_t is stored for
@@ -441,7 +426,7 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
       a.all_rows = 1;
       a.combine_mask = d_mask;
     }
-    if (launch_attn_fwd(a, force_all ? mapQ : mapQc, mapK, mapV, mapK, mapK, s) != cudaSuccess) return L2A_ERR_CUDA;
+    if (launch_attn_fwd(a, mapQ, mapK, mapV, mapK, mapK, s) != cudaSuccess) return L2A_ERR_CUDA;
   }
   pe.mark(s);
   return L2A_OK;

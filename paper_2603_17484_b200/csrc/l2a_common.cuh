@@ -98,15 +98,15 @@ struct RouteArgs {
 };
 constexpr int kRouteBlockElems = 4096;  // positions per CTA of the route/compact kernels
 cudaError_t launch_route_compact(const RouteArgs& a, cudaStream_t stream);
+cudaError_t launch_clear_header(void* ws, bool overlap, cudaStream_t stream);
 cudaError_t launch_pack_sequences(const int32_t* cu_seqlens, int n_seq, int L, int32_t* seq_bounds, cudaStream_t stream);
 
 // Gathers rows src[b, q_idx[b][c], :] -> dst[b, kv, c, :] (kv: KV head; its G heads of D elements together) for c <
 // n_routed[b], and zero-fills up to the next multiple of kRowsPerCta rows of a head (within c < L) so that padded MMA
-// tiles read zeros.  With `prefix` given, only the
-// routed rows t in [row_begin, row_end) are gathered (the padding with the range that ends at L).
+// tiles read zeros.
 cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx, const int32_t* n_routed,
-                               int B, int L, int row_elems, int G, int D, cudaStream_t stream, const int32_t* prefix = nullptr,
-                               int row_begin = 0, int row_end = 0, RowStrides src_strides = RowStrides{0, 0},
+                               int B, int L, int row_elems, int G, int D, cudaStream_t stream,
+                               RowStrides src_strides = RowStrides{0, 0},
                                int* status = nullptr,    // status: workspace status word (debug-build index checks)
                                int32_t* zero = nullptr, int n_zero = 0,    // n_zero words to clear on the way
                                bool overlap = false,     // may start under the end of the kernel before it
@@ -148,22 +148,21 @@ struct FwdArgs {
   // Packed variable-length batch (B == 1): per token {first token of its sequence, one past the last}; NULL otherwise
   const int32_t* seq_bounds;
   // Key-range splits of the compact groups (global mode; NULL: none): a slot of unnormalised rows with their maxima and
-  // sums for every work item of a split launch, and a zeroed counter per group, whose last CTA to finish combines them.
+  // sums for every work item of a split launch, and the number of parts of each group.
   float* part;
-  int32_t* part_count;
+  int32_t* group_parts;
+  const bf16* q;             // global mode over compact rows: Q, whose routed rows the kernel gathers
+  RowStrides q_st;
   int overlap;               // programmatic dependent launch; 1: the kernel waits for the one before it at its start, 2 (the
                              // global pass behind the plainly launched local one of the same call): only before it combines
 };
-// A global launch of so few groups (256 compact rows of a head) that they leave SMs idle splits their key ranges until it
-// has about two work items for each of the 148 SMs, at most kMaxKeySplit per group and not below kMinSplitBlocks key
-// blocks an item: an item's rows cost 3 us to store in fp32 and its group's last CTA reads them all back, about three key
-// blocks' time.  Measured, whole forward without / with: 2000 new tokens on 34K keys (64 groups) 525 / 369 us, 300 on 60K
-// (28 groups) 734 / 213, 4001 tokens (112 groups, 32 blocks at most) 178 / 169; but with 128 groups (8000 on 100K) 1686 /
-// 1707, and three items per SM there 1800, 196 groups (16K tokens) 901 / 945: no split from kSplitGroups on.
-constexpr int kSplitItems = 2 * 148;
+// A global launch of fewer than kSplitGroups groups may split their key ranges (key_split), from kMinSplitBlocks + 1 key blocks
+// on, into at most kMaxKeySplit parts of a group and kSplitItems in all.
+constexpr int kSplitSms = 148;
+constexpr int kSplitItems = 4 * kSplitSms;
 constexpr int kSplitGroups = 128;
-constexpr int kMaxKeySplit = 8;
-constexpr int kMinSplitBlocks = 16;
+constexpr int kMaxKeySplit = 32;
+constexpr int kMinSplitBlocks = 4;
 inline int split_slots(int n_groups) {       // slots a shape with that many groups (all rows routed) can need
   const int64_t n = (int64_t)n_groups * kMaxKeySplit;
   return n < kSplitItems ? (int)n : kSplitItems;

@@ -117,15 +117,14 @@ __global__ void __launch_bounds__(kThreads) route_scan_kernel(RouteArgs a) {
   }
 }
 
-// One CTA per routed row (grid-stride); 16-byte chunks; src2, if given, is gathered in the same way.  The heads of a KV group
+// For the backward (the forward's global pass gathers the rows of a tile itself).  One CTA per routed row (grid-stride); 16-byte chunks; src2, if given, is gathered in the same way.  The heads of a KV group
 // (group_chunks chunks of a row) lie together in the result: [batch, KV head, compact row, group_chunks].  No input is
 // __restrict__ or read with __ldg: the kernel may start while the one before it (the routing, or whatever produced the queries)
 // still writes them.
 __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16* dst, const int32_t* q_idx,
                                                           const int32_t* n_routed, int L,
                                                           int row_chunks /* 16-byte chunks per row */,
-                                                          int group_chunks, int G, const int32_t* prefix, int row_begin,
-                                                          int row_end, int64_t src_batch_chunks,
+                                                          int group_chunks, int G, int64_t src_batch_chunks,
                                                           int64_t src_row_chunks, int* status, int32_t* zero,
                                                           int n_zero, const bf16* src2, bf16* dst2,
                                                           int64_t src2_batch_chunks, int64_t src2_row_chunks) {
@@ -137,13 +136,6 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16*
   const int n_c = n_routed[b];
   int n_pad = (int)((compact_groups(n_c, G) * kRowsPerCta + G - 1) / G);
   if (n_pad > L) n_pad = L;
-  // optional restriction to the routed rows t in [row_begin, row_end): they are the compact rows
-  // [prefix[row_begin], prefix[row_end]); the zero padding belongs to the range that ends at L
-  int c_begin = 0;
-  if (prefix != nullptr) {
-    c_begin = prefix[(int64_t)b * (L + 1) + row_begin];
-    if (row_end < L) n_pad = prefix[(int64_t)b * (L + 1) + row_end];
-  }
   const uint4* s = reinterpret_cast<const uint4*>(src) + b * src_batch_chunks;   // source strides in 16-byte chunks
   uint4* d = reinterpret_cast<uint4*>(dst) + (int64_t)b * L * row_chunks;
   const uint4* s2 = reinterpret_cast<const uint4*>(src2) + b * src2_batch_chunks;
@@ -152,7 +144,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const bf16* src, bf16*
     const int kv = i / group_chunks;
     return ((int64_t)kv * L + c) * group_chunks + (i - kv * group_chunks);
   };
-  for (int c = c_begin + blockIdx.x; c < n_pad; c += gridDim.x) {
+  for (int c = blockIdx.x; c < n_pad; c += gridDim.x) {
     if (c < n_c) {
       const int t = q_idx[(int64_t)b * L + c];
       if (!dbg_in_range(t >= 0 && t < L, status)) continue;
@@ -240,6 +232,12 @@ __global__ void __launch_bounds__(256) router_logits_kernel(const bf16* __restri
   if (sum_sq != nullptr && lane == 0 && t_end > t_begin) atomicAdd(&sum_sq[reg_b], reg_sum);
 }
 
+// A kernel instead of a memset: it may start under the end of the kernel before it.
+__global__ void clear_header_kernel(int32_t* header) {
+  dependency_wait();
+  header[threadIdx.x] = 0;
+}
+
 // Packed variable-length batches: token t belongs to the sequence i with cu[i] <= t < cu[i + 1] (binary search over
 // the n_seq + 1 boundaries); tokens at or after cu[n_seq] are sequences of their own.
 __global__ void __launch_bounds__(256) pack_sequences_kernel(const int32_t* __restrict__ cu, int n_seq, int L,
@@ -278,6 +276,10 @@ cudaError_t launch_router_logits(const bf16* S, const float* w, float bias, floa
   return cudaGetLastError();
 }
 
+cudaError_t launch_clear_header(void* ws, bool overlap, cudaStream_t stream) {
+  return launch_dependent(clear_header_kernel, dim3(1), (unsigned)(kWsHeaderBytes / 4), 0, stream, overlap, static_cast<int32_t*>(ws));
+}
+
 cudaError_t launch_pack_sequences(const int32_t* cu_seqlens, int n_seq, int L, int32_t* seq_bounds, cudaStream_t stream) {
   pack_sequences_kernel<<<ceil_div(L, 256), 256, 0, stream>>>(cu_seqlens, n_seq, L, seq_bounds);
   return cudaGetLastError();
@@ -296,8 +298,7 @@ cudaError_t launch_route_compact(const RouteArgs& a, cudaStream_t stream) {
 }
 
 cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx, const int32_t* n_routed, int B,
-                               int L, int row_elems, int G, int D, cudaStream_t stream, const int32_t* prefix, int row_begin,
-                               int row_end, RowStrides src_strides, int* status, int32_t* zero, int n_zero, bool overlap,
+                               int L, int row_elems, int G, int D, cudaStream_t stream, RowStrides src_strides, int* status, int32_t* zero, int n_zero, bool overlap,
                                const bf16* src2, bf16* dst2, RowStrides src2_strides) {
   const int row_chunks = row_elems * 2 / 16;
   const int64_t ts = src_strides.t > 0 ? src_strides.t : row_elems;
@@ -306,8 +307,8 @@ cudaError_t launch_gather_rows(const bf16* src, bf16* dst, const int32_t* q_idx,
   const int64_t bs2 = src2_strides.b > 0 ? src2_strides.b : (int64_t)L * ts2;
   int gx = L < 148 * 16 ? L : 148 * 16;
   dim3 grid(gx, B);
-  return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, overlap, src, dst, q_idx, n_routed, L, row_chunks, G * D / 8, G, prefix,
-                          row_begin, row_end, bs / 8, ts / 8, status, zero, n_zero, src2, dst2, bs2 / 8, ts2 / 8);
+  return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, overlap, src, dst, q_idx, n_routed, L, row_chunks, G * D / 8, G,
+                          bs / 8, ts / 8, status, zero, n_zero, src2, dst2, bs2 / 8, ts2 / 8);
 }
 
 }  // namespace l2a

@@ -317,7 +317,8 @@ struct ItemCursor {
 // Five-GEMM backward kernel: the key/value-stationary kernel above plus the fifth GEMM, dQ(i) = dS(i) K, so that
 // S and dP are computed once per tile pair.  dQ(i) is a fresh 128 x D accumulator per item; the read-out warps take
 // it out (lane = query row) and add it into an fp32 accumulator in global memory whose layout is private to this
-// file: per (batch, head, 128-row tile) one block of 128 x D floats ordered [warp 16][piece D/16][lane 32][4], so
+// file: per (batch, head, 128-row tile) one block of 128 x D floats ordered [warp 16][piece D/16][lane 32][4] (the lanes of the
+// compact tiles ordered by head: head_slot), so
 // that every red.global.add.v4.f32 of a warp covers 512 contiguous bytes.  Local items add into the accumulator
 // indexed by row tile, global items into the one indexed by compact tile; dq_merge_kernel forms the bf16 dQ.
 // All key blocks meet in those accumulators in no fixed order: dQ is not bit-reproducible from run to run
@@ -336,6 +337,14 @@ struct ItemCursor {
 //   tokens (28/4 heads) 794 -> 758 us, of the local module at 8155 tokens 1037 -> 978; without the writes of dS it would
 //   take 685, without the TMA writes 694, without the statistics 732, without any of them and the reductions 560.
 
+// Where row `lane` of 32 packed rows lies in a piece of the compact accumulator: the rows of one head next to each other, so
+// that the merge, which reads the rows of one head, finds them in whole sectors.  (In the order of the rows the merge took, with
+// 32/8 heads, 1587 tokens 27 us instead of 17, 2 x 4096 tokens (28/4) 50 instead of 42.)
+__device__ __forceinline__ int head_slot(int lane, int G) {
+  const int q = lane % G, n = lane / G, per = 32 / G;
+  return q * per + min(q, 32 - per * G) + n;
+}
+
 // The reductions of one read-out warp: piece I of its 32 x D/2 share (4 columns each) goes to a byte offset from the
 // warp's base address that is a compile-time constant, so that all of them share one address register pair.
 template <int kBytes>
@@ -344,11 +353,11 @@ __device__ __forceinline__ void red_add_v4(float* base, uint32_t a, uint32_t b, 
                "f"(__uint_as_float(b)), "f"(__uint_as_float(c)), "f"(__uint_as_float(d)), "n"(kBytes)
                : "memory");
 }
-// Least distance between two reductions of a read-out warp, in SM clocks (polled: a sleep is too coarse).  Two reads of the
-// clock and a comparison already take that long, and as little as that is needed: backward launch of 2 x 4096 tokens / of the
-// local module at 8155 tokens without it 830 / 1108 us, with 16 757 / 965, 40 766 / 974, 72 778 / 998, 112 781 / 1009, 140 818 /
-// 1067.  (The 64-bit clock, whose polling takes longer, at 96: 818 / 1057.)
-constexpr uint32_t kRedSpacingClk = 16;
+// Least distance between two reductions of a read-out warp, in SM clocks (polled: a sleep has steps of 64 ns).  Passes one after
+// the other, at the board's power limit: 64K tokens / whole layer at 8155 tokens / 2 x 4096 tokens with 16 clk 22830 / 2074 us / -,
+// 56 22430 / 2055 / -, 96 22180 / 2020 / -, 112 22260 / 2027 / 1289, 128 22050 / 2000 / 1277, 144 21960 / 2011 / 1273, 168 22510 /
+// 2060 / 1299, 200 23310 / 2115 / 1341.
+constexpr uint32_t kRedSpacingClk = 136;
 template <int D, int I>
 struct ReadOutReds {
   static constexpr int kCols = D / 4;                 // columns per quarter of the accumulator layout
@@ -609,7 +618,7 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         item_ok = dbg_in_range(cur.t >= 0 && cur.t + (cur.left - 1) * kSplit < n && cur.hg <= a.G && base != nullptr, a.status);
         // (this warp's columns start at (D / 2) * half, i.e. at quarter 2 * half of the layout)
         base += ((glb ? (int64_t)bar->b * a.Hkv + bar->g : (int64_t)bar->b * a.Hq + bar->g * a.G + cur.hg) * n + cur.t) *
-                    (int64_t)(kTileM * D) + lane * 4 + ((2 * half) * 4 + grp) * (8 * D);
+                    (int64_t)(kTileM * D) + (glb ? head_slot(lane, a.G) : lane) * 4 + ((2 * half) * 4 + grp) * (8 * D);
         left = cur.left;
         hg2 = 2 * cur.hg + (hg2 & 1);
       }
@@ -987,7 +996,10 @@ __global__ void __launch_bounds__(256) dq_merge_kernel(const float* acc_loc, con
   constexpr int kChunks = D / 8;             // 16-byte chunks per bf16 row
   constexpr int kRowBytes = D * 2 + 16;      // padded: conflict-free 16-byte accesses down a column
   __shared__ __align__(16) uint8_t tile_s[kTileM * kRowBytes];
+  __shared__ int slot[32];
+  if (threadIdx.x < 32) slot[threadIdx.x] = head_slot(threadIdx.x, Hq / Hkv);
   dependency_wait();
+  __syncthreads();
   const int n_tiles = (L + kTileM - 1) / kTileM;
   const int h = blockIdx.x % Hq;
   const int tile = tile_begin + (blockIdx.x / Hq) % tile_count;
@@ -1010,7 +1022,7 @@ __global__ void __launch_bounds__(256) dq_merge_kernel(const float* acc_loc, con
       if (!dbg_in_range(cr >= 0 && cr < n_ctiles * kTileM, status)) continue;
       const float4* p = reinterpret_cast<const float4*>(
           acc_glb + (((int64_t)b * Hkv + kv) * n_ctiles + (cr >> 7)) * tile_floats + (q * 4 + ((cr & 127) >> 5)) * (8 * D) +
-          c * 128 + (cr & 31) * 4);
+          c * 128 + slot[cr & 31] * 4);
       const float4 gx = __ldcg(p), gy = __ldcg(p + 32);
       x.x += gx.x; x.y += gx.y; x.z += gx.z; x.w += gx.w;
       y.x += gy.x; y.y += gy.y; y.z += gy.z; y.w += gy.w;

@@ -218,7 +218,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 
   // this item's part of the group's key blocks
   if (compact && ks.parts > 1) {
-    n_split = max(1, min(ks.parts, (jhi - jlo + ks.blocks) / ks.blocks));
+    // (a group as short as those of a call without a combination stays whole: the same bits in both)
+    if (jhi - jlo >= kMinSplitBlocks) n_split = min(ks.parts, (jhi - jlo + ks.blocks) / ks.blocks);
     if (split >= n_split) { dependency_wait(); return; }
     if (split == 0 && threadIdx.x == 0) a.group_parts[group] = n_split;
   }

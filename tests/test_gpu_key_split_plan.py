@@ -1,4 +1,4 @@
-"""Into how many parts the key ranges of the routed groups are split: both sides of the lines of that rule (four and five key
+"""Into how many parts the key ranges of the routed groups are split: both sides of the lines of that rule (seven and eight key
 blocks; sixteen and seventeen; up to and beyond 32 groups; waves of equal groups), the most parts of a group, short prefills whose
 groups differ in length, against the fp64 oracle."""
 import numpy as np
@@ -12,13 +12,13 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,Lq,Lk,Hq,Hkv,D,W,n_routed,flags", [
-    (1, 30, 512, 2, 1, 128, 64, 9, 0),              # four key blocks: none
-    (1, 30, 513, 2, 1, 128, 64, 9, 0),              # five: parts of two, the last one of a single key
+    (1, 30, 896, 2, 1, 128, 64, 9, 0),              # seven key blocks: none
+    (1, 30, 897, 2, 1, 128, 64, 9, 0),              # eight: parts of two, the last block of a single key
     (1, 30, 2048, 2, 1, 64, 64, 9, 0),              # sixteen
     (1, 30, 2049, 2, 1, 64, 64, 9, 0),              # seventeen: by cost
-    (1, 640, 640, 6, 1, 128, 100, 640, 0),          # 15 groups of one to five blocks, every token
-    (33, 20, 900, 1, 1, 64, 30, 11, 0),             # 33 groups: by cost
-    (2, 300, 700, 14, 2, 128, 50, 150, l2a.FLAG_SHARED_WINDOW),
+    (1, 1100, 1100, 6, 1, 128, 100, 1100, 0),       # 26 groups of one to nine blocks, every token
+    (33, 20, 1300, 1, 1, 64, 30, 11, 0),             # 33 groups: by cost
+    (2, 300, 1100, 14, 2, 128, 50, 150, l2a.FLAG_SHARED_WINDOW),
     (1, 9, 20000, 1, 1, 128, 64, 5, 0),             # one group, the most parts
     (3, 64, 9000, 8, 8, 64, 200, 20, 0),            # 24 equal groups: one or two waves
 ])

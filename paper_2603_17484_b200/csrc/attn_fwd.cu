@@ -95,7 +95,9 @@ struct KeySplit {
 // to the next item 3.6.  Whole call, key ranges undivided below 32 key blocks and combined by the group's last CTA / this: one head
 // of 1024 tokens 32.8 / 26.7 us, 500 tokens (28/4 heads) 41.0 / 30.7, 2000 82.0 / 73.8, 4001 177 / 170, 100 new tokens on 60K keys 223
 // / 122, 500 (32/8, shared window) on 30K 193 / 140, 2000 on 33K 428 / 393.  (Twice as many parts: 2000 tokens 101, 4001 213: their
-// rows, 133 KB a part, take longer than the blocks they save.)  From kSplitGroups groups on nothing was gained by parts.
+// rows, 133 KB a part, take longer than the blocks they save.)
+// With the SMs of a small local pass taken as busy until it ends, against all SMs as free: 100 new tokens on 60K keys 123.5 -> 88, 500
+// on 30K 138 -> 110, 64 on 40K 111 -> 78; of 1000 tokens and more the same.  From kSplitGroups groups on nothing was gained by parts.
 constexpr float kItemCost = 7.f, kCombineCost = 4.f, kPartCost = 0.04f;
 constexpr int kShortGroup = 16, kFewGroups = 32;
 __device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
@@ -111,8 +113,22 @@ __device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
     const int p = lane + 1, items = (int)k.groups * p;      // (kMaxKeySplit = 32 candidates, one a lane)
     const float part = (longest + p - 1) / p, sms = kSplitSms;
     float cost;
-    if (2 * shortest >= longest) cost = ceilf(items / sms) * (part + kItemCost);
-    else cost = fmaxf(part + kItemCost, (items * kItemCost + k.groups * 0.5f * (longest + shortest)) / sms + 0.5f * part);
+    if (2 * shortest >= longest) {
+      // Waves of equal items, on the SMs that the local pass leaves and on its own from its end on: from the time at which the
+      // SMs could have done them without waves up to a wave's end on either side.
+      const float c = part + kItemCost, inv = __fdividef(1.f, c);
+      if (a.local_items == 0) {
+        cost = ceilf(items * (1.f / kSplitSms)) * c;
+      } else {
+        const float busy = (float)a.local_items, until = a.local_blocks + kItemCost;
+        const float even = (items * c + busy * until) * (1.f / kSplitSms);
+        const float k = ceilf(even * inv - 1e-3f), n = fmaxf(1.f, ceilf((even - until) * inv - 1e-3f));
+        float t0 = k * c, t1 = until + n * c;
+        if ((sms - busy) * k + busy * floorf(fmaxf(t0 - until, 0.f) * inv + 1e-3f) < items) t0 += c;
+        if ((sms - busy) * floorf(t1 * inv + 1e-3f) + busy * n < items) t1 += c;
+        cost = fmaxf(fminf(t0, t1), until);
+      }
+    } else cost = fmaxf(part + kItemCost, (items * kItemCost + k.groups * 0.5f * (longest + shortest)) / sms + 0.5f * part);
     if (p > 1) cost += kCombineCost + kPartCost * items;
     const bool possible = items <= kSplitItems && p <= longest;
     const uint32_t key = possible ? ((uint32_t)fminf(cost * 16.f, 1e8f) << 5) + lane : 0xffffffffu;

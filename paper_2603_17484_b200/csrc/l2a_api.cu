@@ -364,6 +364,14 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   a.seq_bounds = p->seq_bounds;
   a.part = nullptr;
   a.group_parts = nullptr;
+  // SMs that a local pass of this shape leaves to the global one (from the shape alone, also where the global phase is a call of
+  // its own: either way the same plan, so the same bits)
+  a.local_items = a.local_blocks = 0;
+  if (!skip_local && (int64_t)n_pairs * p->Hq * p->B < kSplitSms) {
+    const int64_t keys = (int64_t)a.window + kRowsPerCta, all = (int64_t)p->Lq + p->q_pos_offset;
+    a.local_items = n_pairs * p->Hq * p->B;
+    a.local_blocks = (int)(((keys < all ? keys : all) + kTileN - 1) / kTileN);
+  }
   a.q = static_cast<const bf16*>(Q);
   a.q_st = qs;
   a.overlap = 0;

@@ -151,6 +151,7 @@ struct FwdArgs {
   // sums for every work item of a split launch, and the number of parts of each group.
   float* part;
   int32_t* group_parts;
+  int local_items, local_blocks;   // items of the local pass if they leave SMs idle (else 0), key blocks of each
   const bf16* q;             // global mode over compact rows: Q, whose routed rows the kernel gathers
   RowStrides q_st;
   int overlap;               // programmatic dependent launch; 1: the kernel waits for the one before it at its start, 2 (the

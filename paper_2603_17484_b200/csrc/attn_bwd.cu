@@ -9,7 +9,7 @@
 //
 // Kernels
 //   bwd_delta_kernel : Delta_loc (all rows), Delta_glb (compact rows), optional dgate.  HBM bound.
-//   dq_zero_kernel   : clears the fp32 dQ accumulators.
+//   dq_zero_kernel   : clears the fp32 dQ accumulators (where they are small CTAs of bwd_delta_kernel do).
 //   bwd_kernel       : key/value-stationary, five GEMMs per (query tile, key block) pair.  One CTA owns a block of
 //                      128 keys of one KV head and walks every query tile that can see it -- local band tiles of
 //                      the G query heads, then the compact routed tiles from the first one at or after the block.
@@ -49,6 +49,30 @@ __device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
   return acc;
 }
 
+// CTA `cta` of n_ctas zeroes its share of the fp32 dQ accumulators: every row tile of the local one, the compact tiles in use of
+// the global one.
+__device__ __forceinline__ void zero_accumulators(float* acc_loc, float* acc_glb, const int32_t* n_routed, int B, int Hq, int Hkv,
+                                                  int L, int tile_floats, int cta, int n_ctas) {
+  const int n_tiles = (L + kTileM - 1) / kTileM, n_ctiles = compact_tiles(L, Hq / Hkv);
+  const int per = B * Hq * n_tiles;
+  for (int item = cta; item < per + B * Hkv * n_ctiles; item += n_ctas) {
+    const int which = item >= per, rem = which ? item - per : item;
+    float* base = which ? acc_glb : acc_loc;
+    if (base == nullptr) continue;
+    if (which && rem % n_ctiles >= compact_tiles(n_routed[rem / (n_ctiles * Hkv)], Hq / Hkv)) continue;
+    float4* p = reinterpret_cast<float4*>(base + (int64_t)rem * tile_floats);
+    for (int k = threadIdx.x; k < tile_floats / 4; k += blockDim.x) p[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
+// What the CTAs behind the first n_delta do: the accumulators are cleared by the Delta kernel itself where they are small.
+struct ZeroArgs {
+  int n_delta;
+  float *acc_loc, *acc_glb;
+  const int32_t* n_routed;
+  int Hkv;
+};
+
 template <int D>
 __global__ void __launch_bounds__(256, 2) bwd_delta_kernel(const bf16* __restrict__ dO, const bf16* __restrict__ dO_loc,
                                                         const bf16* __restrict__ S,
@@ -58,16 +82,23 @@ __global__ void __launch_bounds__(256, 2) bwd_delta_kernel(const bf16* __restric
                                                         float* __restrict__ delta_glb, float* __restrict__ dgate, int B,
                                                         int L, int Hq, int a_by_row, int64_t do_bs, int64_t do_ts,
                                                         const float* __restrict__ lse_loc,
-                                                        const float* __restrict__ lse_glb, float* __restrict__ lse_eff) {
+                                                        const float* __restrict__ lse_glb, float* __restrict__ lse_eff,
+                                                        const ZeroArgs z) {
   constexpr int kLanesPerHead = D / 8;                 // 16-byte chunks per head row
   constexpr int kHeadsPerPass = 32 / kLanesPerHead;
   const int lane = threadIdx.x & 31;
   const int64_t n_tokens = (int64_t)B * L;
-  const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const int64_t n_warps = (int64_t)z.n_delta * (blockDim.x >> 5);
   const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (S == nullptr) dO_loc = dO;                       // local part skipped: its gradient is not read
   const bool split = dO_loc != dO;                     // separate gradient for the local output
   dependents_release();       // (reads nothing that the kernels ahead of it in the call write: it waits at its end)
+  if ((int)blockIdx.x >= z.n_delta) {
+    zero_accumulators(z.acc_loc, z.acc_glb, z.n_routed, B, Hq, z.Hkv, L, kTileM * D, blockIdx.x - z.n_delta,
+                      gridDim.x - z.n_delta);
+    dependency_wait();
+    return;
+  }
   const int sub = lane / kLanesPerHead;                // head inside the pass
   const int n_pass = (Hq + kHeadsPerPass - 1) / kHeadsPerPass;
   const bool global = d_mask != nullptr;               // NULL: the global part is skipped
@@ -965,22 +996,12 @@ bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
   if (warp == 17) tmem_dealloc(tmem, 512);
 }
 
-// Zeroes the fp32 dQ accumulators: every row tile of the local one, the compact tiles in use of the global one.
 __global__ void __launch_bounds__(256) dq_zero_kernel(float* __restrict__ acc_loc, float* __restrict__ acc_glb,
                                                       const int32_t* __restrict__ n_routed, int B, int Hq, int Hkv, int L,
                                                       int tile_floats) {
-  const int n_tiles = (L + kTileM - 1) / kTileM, n_ctiles = compact_tiles(L, Hq / Hkv);
-  const int per = B * Hq * n_tiles;
   dependency_wait();
   dependents_release();
-  for (int item = blockIdx.x; item < per + B * Hkv * n_ctiles; item += gridDim.x) {
-    const int which = item >= per, rem = which ? item - per : item;
-    float* base = which ? acc_glb : acc_loc;
-    if (base == nullptr) continue;
-    if (which && rem % n_ctiles >= compact_tiles(n_routed[rem / (n_ctiles * Hkv)], Hq / Hkv)) continue;
-    float4* p = reinterpret_cast<float4*>(base + (int64_t)rem * tile_floats);
-    for (int k = threadIdx.x; k < tile_floats / 4; k += blockDim.x) p[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+  zero_accumulators(acc_loc, acc_glb, n_routed, B, Hq, Hkv, L, tile_floats, blockIdx.x, gridDim.x);
 }
 
 // fp32 dQ accumulators -> bf16 dQ: dQ_t = scale * (local(t) + d_t * global(prefix[t])), for the row tiles
@@ -1126,13 +1147,15 @@ cudaError_t launch_bwd_kernel(BwdArgs a, const CUtensorMap& mapQ, const CUtensor
 template <int D>
 cudaError_t launch_bwd(const BwdArgs& base, const CUtensorMap& mapQ, const CUtensorMap& mapDO,
                        const CUtensorMap& mapQc, const CUtensorMap& mapDOc, const CUtensorMap& mapK,
-                       const CUtensorMap& mapV, const uint8_t* d_mask, cudaStream_t s) {
+                       const CUtensorMap& mapV, const uint8_t* d_mask, bool zeroed, cudaStream_t s) {
   const DeviceInfo* dev = device_info();
   if (dev == nullptr) return cudaErrorUnknown;
   const int n_tiles = (base.Lq + kTileM - 1) / kTileM;
   const bool overlap = phase_events().n == 0;    // (events between the launches ask for their times one after the other)
-  cudaError_t err = launch_dependent(dq_zero_kernel, dim3(dev->sms * 8), 256, 0, s, overlap, base.dq_acc_loc, base.dq_acc_glb,
-                                     base.n_routed, base.B, base.Hq, base.Hkv, base.Lq, kTileM * D);
+  cudaError_t err = cudaSuccess;
+  if (!zeroed)
+    err = launch_dependent(dq_zero_kernel, dim3(dev->sms * 8), 256, 0, s, overlap, base.dq_acc_loc, base.dq_acc_glb, base.n_routed,
+                           base.B, base.Hq, base.Hkv, base.Lq, kTileM * D);
   if (err != cudaSuccess) return err;
   phase_events().mark(s);
   const int n_kblocks = (base.Lk + kTileN - 1) / kTileN;
@@ -1160,6 +1183,11 @@ cudaError_t launch_bwd(const BwdArgs& base, const CUtensorMap& mapQ, const CUten
   }
   return cudaGetLastError();
 }
+
+// Up to this size of an accumulator further CTAs of the Delta kernel clear it, beside Delta where that leaves SMs idle; beyond it a
+// kernel behind does (DRAM turns between reads and writes: see Delta).  A step of 706 tokens (4 heads) 55.3 -> 53.2 us, of 2 x 793
+// (32/8) 144.6 -> 138.1, 1587 205 -> 198.4, 3000 (28/4) 432 -> 422, layer of 8155 2005 -> 1981, 2 x 4096 the same.
+constexpr size_t kZeroByDelta = 128u << 20;
 
 // one fp32 dQ accumulator: whole 128-row tiles
 size_t acc_bytes(const l2a_params* p) {
@@ -1278,6 +1306,7 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
       !encode_rows_map(&mapV, V, p->B, p->Lk, p->Hkv * p->D, kTileN, p->D, vs.b, vs.t))
     return L2A_ERR_CUDA;
 
+  const bool zeroed = (size_t)p->B * p->Hq * p->Lq * p->D * sizeof(float) <= kZeroByDelta;
   PhaseEvents& pe = phase_events();
   struct ClearOnExit { PhaseEvents& p; ~ClearOnExit() { p.clear(); } } clear_on_exit{pe};
   const bool overlap = pe.n == 0;
@@ -1298,10 +1327,11 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
     int64_t blocks = (int64_t)dev->sms * (p->D == 128 ? dev->delta_ctas_128 : dev->delta_ctas_64);
     const int64_t max_blocks = ((int64_t)p->B * p->Lq + 7) / 8;
     if (blocks > max_blocks) blocks = max_blocks;
-    if (launch_dependent(kern, dim3((unsigned)blocks), 256, 0, s, overlap && !skip_global, static_cast<const bf16*>(dO),
+    const ZeroArgs z = {(int)blocks, skip_local ? nullptr : dq_acc_loc, skip_global ? nullptr : dq_acc_glb, n_routed, p->Hkv};
+    if (launch_dependent(kern, dim3((unsigned)(blocks + (zeroed ? 2 * dev->sms : 0))), 256, 0, s, overlap && !skip_global, static_cast<const bf16*>(dO),
                          static_cast<const bf16*>(dS_loc), static_cast<const bf16*>(skip_local ? nullptr : S_save),
                          static_cast<const bf16*>(A_c), skip_global ? nullptr : d_mask, prefix, delta_loc, delta_glb, dgate,
-                         p->B, p->Lq, p->Hq, force_all ? 1 : 0, os.b, os.t, lse_loc, lse_glb, share ? lse_c : nullptr) !=
+                         p->B, p->Lq, p->Hq, force_all ? 1 : 0, os.b, os.t, lse_loc, lse_glb, share ? lse_c : nullptr, z) !=
         cudaSuccess)
       return L2A_ERR_CUDA;
     if (force_all) {
@@ -1331,7 +1361,7 @@ static l2a_status backward_impl(const l2a_params* p, const void* Q, const void* 
   a.dq_acc_glb = !skip_global ? dq_acc_glb : nullptr;
   a.status = reinterpret_cast<int*>(ws);
   const cudaError_t e =
-      p->D == 128 ? launch_bwd<128>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, skip_global ? nullptr : d_mask, s)
-                  : launch_bwd<64>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, skip_global ? nullptr : d_mask, s);
+      p->D == 128 ? launch_bwd<128>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, skip_global ? nullptr : d_mask, zeroed, s)
+                  : launch_bwd<64>(a, mapQ, mapDO, mapQc, mapDOc, mapK, mapV, skip_global ? nullptr : d_mask, zeroed, s);
   return e == cudaSuccess ? L2A_OK : L2A_ERR_CUDA;
 }

@@ -11,7 +11,7 @@
 //          the compact output O_c and log-sum-exp L_c.
 //
 //          The soft-max warps gather the routed rows of Q of their tile themselves, while barriers and tensor memory are set up
-//          (a kernel ahead of the local pass that wrote Q_c, 2 to 16 us, and its copy are gone).
+//          (instead of a kernel ahead of the local pass that writes Q_c, 2 to 16 us).
 // Packed heads against a launch over the rows of each head, global pass: 64K tokens (28/4 heads, 8 % routed) 2333 -> 2057 us,
 // 64K in 24 documents (32/8, 20 %) 726 -> 607, 2 x 4096 tokens 104 -> 72; whole call of 2000 new tokens on 34K keys 421 -> 401.
 //

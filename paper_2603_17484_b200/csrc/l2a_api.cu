@@ -53,7 +53,7 @@ size_t route_ws_size(const l2a_params* p) {
   return kWsHeaderBytes + align_up((size_t)p->B * nblocks * sizeof(int32_t), 256);
 }
 // forward workspace: header, numbers of parts of split key ranges, their slots
-constexpr size_t kPartCountBytes = (kSplitGroups * sizeof(int32_t) + 255) / 256 * 256;
+constexpr size_t kGroupPartsBytes = (kSplitGroups * sizeof(int32_t) + 255) / 256 * 256;
 int group_count(const l2a_params* p) {
   const int64_t n = (int64_t)ceil_div(p->Lq, kRowsPerCta) * p->Hq * p->B;
   return n < kSplitGroups ? (int)n : kSplitGroups;     // launches with more groups are not split
@@ -64,7 +64,7 @@ size_t part_bytes(const l2a_params* p) {
 size_t fwd_ws_size(const l2a_params* p) {
   // (never less than one copy of Q)
   const size_t q = align_up((size_t)p->B * p->Lq * p->Hq * p->D * sizeof(bf16), 256), parts = part_bytes(p);
-  return kWsHeaderBytes + kPartCountBytes + (q > parts ? q : parts);
+  return kWsHeaderBytes + kGroupPartsBytes + (q > parts ? q : parts);
 }
 
 bool ws_ok(const void* ws, size_t have, size_t need) { return ws && aligned(ws, 256) && have >= need; }
@@ -321,7 +321,7 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   uint8_t* ws = static_cast<uint8_t*>(fwd_ws);
   int* status = reinterpret_cast<int*>(ws);
   int32_t* group_parts = reinterpret_cast<int32_t*>(ws + kWsHeaderBytes);
-  float* part = reinterpret_cast<float*>(ws + kWsHeaderBytes + kPartCountBytes);
+  float* part = reinterpret_cast<float*>(ws + kWsHeaderBytes + kGroupPartsBytes);
   const int n_pairs = ceil_div(p->Lq, kRowsPerCta);
   const bool whole = pair_end < 0 || (pair_begin == 0 && pair_end == n_pairs);
   if (pair_end < 0) pair_end = n_pairs;
@@ -381,7 +381,7 @@ static l2a_status forward_range(const l2a_params* p, const void* Q, const void* 
   PhaseEvents& pe = phase_events();
   struct ClearOnExit { PhaseEvents& p; ~ClearOnExit() { p.clear(); } } clear_on_exit{pe};
   pe.mark(s);
-  pe.mark(s);      // (a gather of the routed rows once stood between the two)
+  pe.mark(s);      // (two boundaries in one place: the global pass gathers its rows itself)
   if (!skip_local && !global_phase) {
     a.global_mode = 0;
     a.accumulate_into_out2 = 0;

@@ -118,23 +118,24 @@ def make_workload(args, seed_offset=0):
     return cfg, rho, seed, d, logits
 
 
-def issued_tile_pairs(mask, L, W, shared=False, tile=128):
+def issued_tile_pairs(mask, L, W, shared=False, tile=128, pack=1):
     """Score elements the tensor cores really compute, (local, global): every (128-row tile, 128-key block) pair a launch
     issues MMAs for counts whole (edge blocks are masked after the product, ragged tiles are padded with zero rows).
     Local: the blocks between the first row's window start and the last row's diagonal; global: the blocks up to the
-    last row of each compact tile of 128 routed rows (up to its position - W - 1 with the shared-window flag)."""
+    last row of each compact tile of 128 routed rows (up to its position - W - 1 with the shared-window flag).  pack: query
+    heads packed into the compact rows; the result is that of one of them."""
     T = tile
     loc = glb = 0
     for b in range(mask.shape[0]):
         r0 = np.arange(0, L, T, dtype=np.int64)
         r1 = np.minimum(r0 + T, L) - 1
         loc += int((r1 // T - np.maximum(r0 - W, 0) // T + 1).sum())
-        t = np.nonzero(mask[b])[0].astype(np.int64)
+        t = np.repeat(np.nonzero(mask[b])[0].astype(np.int64), pack)
         if len(t):
             last = t[np.minimum(np.arange(T - 1, len(t) + T - 1, T), len(t) - 1)]      # last row of each compact tile
             bound = last - (W + 1 if shared else 0)
             glb += int((bound[bound >= 0] // T + 1).sum())
-    return loc * T * T, glb * T * T
+    return loc * T * T, glb * T * T // pack
 
 
 def cpu_oracle_sample(cfg, seed, d, rows_per_head=96, key_span=2500, n_keys=8, backward=True, host=None):
@@ -428,7 +429,7 @@ def main():
         return pl, pg, pw
 
     def issued_pairs(mask, shared):
-        return issued_tile_pairs(mask, cfg.L, cfg.W, shared)
+        return issued_tile_pairs(mask, cfg.L, cfg.W, shared, pack=cfg.Hq // cfg.Hkv)
 
     def step(profile=None):
         buf.route(kind, 0.0)

@@ -233,11 +233,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
   }
 
   // this item's part of the group's key blocks
-  if (compact && ks.parts > 1) {
+  if (compact && a.part != nullptr) {
     // (a group as short as those of a call without a combination stays whole: the same bits in both)
-    if (jhi - jlo >= kMinSplitBlocks) n_split = min(ks.parts, (jhi - jlo + ks.blocks) / ks.blocks);
+    if (ks.parts > 1 && jhi - jlo >= kMinSplitBlocks) n_split = min(ks.parts, (jhi - jlo + ks.blocks) / ks.blocks);
     if (split >= n_split) { dependency_wait(); return; }
-    if (split == 0 && threadIdx.x == 0) a.group_parts[group] = n_split;
+    // the plan for fwd_combine_kernel, undivided groups included: slots of a group, parts in use
+    if (split == 0 && threadIdx.x == 0 && group < kSplitGroups) a.group_parts[group] = (ks.parts << 16) | n_split;
   }
   if (n_split > 1) {
     const int n = jhi - jlo + 1, first = jlo;
@@ -696,27 +697,28 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 
 // Combines the parts of the groups whose key range was split, and does with their rows what the epilogue above does with
 // those of an undivided group.  A CTA takes 32 rows, a thread D / 8 columns of one: the parts of a group are read by eight CTAs
-// instead of the one that finished last (latency bound).
+// instead of the one that finished last (latency bound).  The plan comes from the workspace, where attn_fwd_kernel left it: a second
+// evaluation of key_split, compiled into another kernel, could round a cost differently and look for the parts in other slots.
 template <int D>
 __global__ void __launch_bounds__(256) fwd_combine_kernel(const FwdArgs a) {
   constexpr int kCols = D / 8, kSlot = kRowsPerCta * (D + 2);
   dependency_wait();
-  const KeySplit ks = key_split(a);
   const int group = blockIdx.x >> 3;
-  if (ks.parts <= 1 || group >= ks.groups) return;
   const int G = a.Hq / a.Hkv, g = group % a.Hkv, b = group / a.Hkv % a.B, n_rows = a.n_routed[b] * G;
   const int pi = (n_rows + kRowsPerCta - 1) / kRowsPerCta - 1 - group / a.Hkv / a.B, row0 = pi * kRowsPerCta;
-  if (pi < 0) return;
+  if (pi < 0) return;                  // no such group
   const int32_t* q_idx_b = a.q_idx + (int64_t)b * a.Lq;
-  const int t_last = q_idx_b[(min(row0 + kRowsPerCta, n_rows) - 1) / G];
-  if (t_last < a.row_begin || t_last >= a.row_end) return;
-  const int n_split = a.group_parts[group];
+  if (a.row_begin > 0 || a.row_end < a.Lq) {       // (as in attn_fwd_kernel, which then has written the group's word)
+    const int t_last = q_idx_b[(min(row0 + kRowsPerCta, n_rows) - 1) / G];
+    if (t_last < a.row_begin || t_last >= a.row_end) return;
+  }
+  const int plan = a.group_parts[group], n_split = plan & 0xffff, n_slots = plan >> 16;
   const int r = (blockIdx.x & 7) * 32 + (threadIdx.x & 31), col = (threadIdx.x >> 5) * kCols;
   const int tile_row = row0 + r;
   if (n_split <= 1 || tile_row >= n_rows) return;
   const int row = tile_row / G, h = g * G + (tile_row - row * G), seq_row = q_idx_b[row];
   if (!dbg_in_range(row < a.Lq && seq_row >= 0 && seq_row < a.Lq, a.status)) return;
-  const float* parts = a.part + (size_t)group * ks.parts * kSlot + (r / kTileM) * (kTileM * (D + 2)) + r % kTileM;
+  const float* parts = a.part + (size_t)group * n_slots * kSlot + (r / kTileM) * (kTileM * (D + 2)) + r % kTileM;
   bf16* dst2 = a.out2 + b * a.out2_st.b + seq_row * a.out2_st.t + (int64_t)h * D + col;
   uint4 old[kCols / 8];                // s_t
 #pragma unroll

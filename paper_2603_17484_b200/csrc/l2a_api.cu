@@ -52,7 +52,7 @@ size_t route_ws_size(const l2a_params* p) {
   const int nblocks = ceil_div(p->Lq, kRouteBlockElems);
   return kWsHeaderBytes + align_up((size_t)p->B * nblocks * sizeof(int32_t), 256);
 }
-// forward workspace: header, numbers of parts of split key ranges, their slots
+// forward workspace: header, plan of each group whose key range may be split, slots of the parts
 constexpr size_t kGroupPartsBytes = (kSplitGroups * sizeof(int32_t) + 255) / 256 * 256;
 int group_count(const l2a_params* p) {
   const int64_t n = (int64_t)ceil_div(p->Lq, kRowsPerCta) * p->Hq * p->B;

@@ -148,7 +148,7 @@ struct FwdArgs {
   // Packed variable-length batch (B == 1): per token {first token of its sequence, one past the last}; NULL otherwise
   const int32_t* seq_bounds;
   // Key-range splits of the compact groups (global mode; NULL: none): a slot of unnormalised rows with their maxima and
-  // sums for every work item of a split launch, and the number of parts of each group.
+  // sums for every work item of a split launch, and for each of the first kSplitGroups groups its slots << 16 | parts in use.
   float* part;
   int32_t* group_parts;
   int local_items, local_blocks;   // items of the local pass if they leave SMs idle (else 0), key blocks of each

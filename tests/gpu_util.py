@@ -189,3 +189,10 @@ def check_same_split(a: torch.Tensor, b: torch.Tensor, V: torch.Tensor, what: st
     bound = 2.0 ** -8 * float(V.float().abs().max()) + 2.0 ** -7 * torch.maximum(x.abs(), y.abs())
     assert bool(((x - y).abs() <= bound).all()), (what, float(((x - y).abs() / bound).max()))
     assert float((x - y).norm()) <= 2.0 ** -8 * float(y.norm()), (what, float((x - y).norm() / y.norm()))
+
+
+def split_plan(case: "Case", n_groups: int):
+    """(slots, parts in use) of the first n_groups groups of routed rows (256 packed rows of a KV head; last rows first, heads and
+    batch entries fastest), as the global pass leaves them behind the header of the forward workspace."""
+    words = case.buf.fwd_ws[256:256 + 4 * n_groups].view(torch.int32).cpu().tolist()
+    return [(w >> 16, w & 0xffff) for w in words]

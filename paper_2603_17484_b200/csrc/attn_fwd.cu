@@ -92,14 +92,12 @@ struct KeySplit {
   int parts, blocks;  // most parts of a group, key blocks of a part
 };
 // Clock traces of the items of 4001 tokens: set-up 2.9 us, first scores 3.2, 1.54 a block, the end 0.5, the rows of a part 1.5,
-// to the next item 3.6.  Whole call, key ranges undivided below 32 key blocks and combined by the group's last CTA / this: one head
-// of 1024 tokens 32.8 / 26.7 us, 500 tokens (28/4 heads) 41.0 / 30.7, 2000 82.0 / 73.8, 4001 177 / 170, 100 new tokens on 60K keys 223
-// / 122, 500 (32/8, shared window) on 30K 193 / 140, 2000 on 33K 428 / 393.  (Twice as many parts: 2000 tokens 101, 4001 213: their
-// rows, 133 KB a part, take longer than the blocks they save.)
+// to the next item 3.6.  Whole call, key ranges undivided below 32 key blocks and combined by the group's last CTA / this: 4001
+// tokens (28/4 heads) 177 / 170 us, 100 new tokens on 60K keys 223 / 122, 500 (32/8, shared window) on 30K 193 / 140, 2000 on 33K
+// 428 / 393.  (Twice as many parts: 4001 tokens 213: their rows, 133 KB a part, take longer than the blocks they save.)
 // With the SMs of a small local pass taken as busy until it ends, against all SMs as free: 100 new tokens on 60K keys 123.5 -> 88, 500
 // on 30K 138 -> 110, 64 on 40K 111 -> 78; of 1000 tokens and more the same.  From kSplitGroups groups on nothing was gained by parts.
 constexpr float kItemCost = 7.f, kCombineCost = 4.f, kPartCost = 0.04f;
-constexpr int kShortGroup = 16, kFewGroups = 32;
 __device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
   const int lane = threadIdx.x & 31;
   int most = 0;
@@ -109,7 +107,7 @@ __device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
   k.groups = compact_groups(most, a.Hq / a.Hkv) * a.Hkv * a.B;
   k.parts = 1;
   const int longest = longest_group(a), shortest = max(0, longest - (a.Lq + kTileN - 1) / kTileN);
-  if (a.part != nullptr && k.groups > 0 && k.groups < kSplitGroups && longest > kMinSplitBlocks) {
+  if (a.part != nullptr && k.groups > 0 && k.groups < kSplitGroups && longest >= kMinSplitBlocks) {
     const int p = lane + 1, items = (int)k.groups * p;      // (kMaxKeySplit = 32 candidates, one a lane)
     const float part = (longest + p - 1) / p, sms = kSplitSms;
     float cost;
@@ -134,9 +132,6 @@ __device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
     const uint32_t key = possible ? ((uint32_t)fminf(cost * 16.f, 1e8f) << 5) + lane : 0xffffffffu;
     const uint32_t best = __reduce_min_sync(0xffffffffu, key);
     if (best != 0xffffffffu) k.parts = (int)(best & 31u) + 1;
-    // few short groups: two key blocks a part whatever their number, so that sequences and head shards of such a size give the
-    // same bits alone and together
-    if (longest <= kShortGroup && k.groups <= kFewGroups) k.parts = (longest + 1) / 2;
   }
   k.blocks = (longest + k.parts - 1) / k.parts;
   return k;
@@ -234,8 +229,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 
   // this item's part of the group's key blocks
   if (compact && a.part != nullptr) {
-    // (a group as short as those of a call without a combination stays whole: the same bits in both)
-    if (ks.parts > 1 && jhi - jlo >= kMinSplitBlocks) n_split = min(ks.parts, (jhi - jlo + ks.blocks) / ks.blocks);
+    if (ks.parts > 1 && jhi - jlo + 1 >= kMinSplitGroup) n_split = min(ks.parts, (jhi - jlo + ks.blocks) / ks.blocks);
     if (split >= n_split) { dependency_wait(); return; }
     // the plan for fwd_combine_kernel, undivided groups included: slots of a group, parts in use
     if (split == 0 && threadIdx.x == 0 && group < kSplitGroups) a.group_parts[group] = (ks.parts << 16) | n_split;
@@ -791,7 +785,7 @@ cudaError_t launch_fwd(const FwdArgs& a, int64_t grid, const CUtensorMap& mapQ, 
   if (e != cudaSuccess) return e;
   e = launch_dependent(attn_fwd_kernel<D>, dim3((unsigned)grid), kFwdThreads, FwdSmem<D>::kTotal, stream, a.overlap != 0, mapQ,
                        mapK, mapV, mapOut, mapOut2, a);
-  if (e != cudaSuccess || a.part == nullptr || longest_group(a) <= kMinSplitBlocks) return e;     // nothing is split
+  if (e != cudaSuccess || a.part == nullptr || longest_group(a) < kMinSplitBlocks) return e;     // nothing is split
   return launch_dependent(fwd_combine_kernel<D>, dim3((unsigned)(8 * std::min<int64_t>(groups, kSplitGroups))), 256, 0, stream,
                           a.overlap != 0, a);
 }

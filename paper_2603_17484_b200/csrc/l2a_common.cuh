@@ -157,14 +157,19 @@ struct FwdArgs {
   int overlap;               // programmatic dependent launch; 1: the kernel waits for the one before it at its start, 2 (the
                              // global pass behind the plainly launched local one of the same call): only before it combines
 };
-// A global launch of fewer than kSplitGroups groups may split their key ranges (key_split), from kMinSplitBlocks + 1 key blocks
-// on, into at most kMaxKeySplit parts of a group and kSplitItems in all.  Up to kMinSplitBlocks the host, which knows the
-// length of the longest group, leaves out the launch that combines the parts: it costs a step of 706 tokens (4 heads) 55 -> 61 us.
+// A global launch of fewer than kSplitGroups groups whose last one may see kMinSplitBlocks key blocks or more splits key ranges
+// (key_split), those of kMinSplitGroup blocks and more, into at most kMaxKeySplit parts of a group and kSplitItems in all.  In
+// shorter calls none is split, whatever their batch and heads: the routed rows of up to 31 blocks of keys then have the same bits
+// alone, in a batch and as a head shard, and the launch that combines parts is left out.  Whole call undivided / with the parts
+// that the cost estimate favours (from 8 blocks on, two blocks a part up to 16): 1024 tokens (28/4 heads, window 4096, 20 % routed)
+// 37 / 49 us, 2000 (8/1) 48 / 57, 1500 (12/2, D = 64) 37 / 45, 3000 (28/4) 118 / 113, 64 new tokens on 3900 keys 65 / 66; but with a
+// window of 128 and few heads, where the local pass is over early, one head of 1024 tokens 33 / 26, 64 on 3900 66 / 34.
 constexpr int kSplitSms = 148;
 constexpr int kSplitItems = 4 * kSplitSms;
 constexpr int kSplitGroups = 128;
 constexpr int kMaxKeySplit = 32;
-constexpr int kMinSplitBlocks = 7;
+constexpr int kMinSplitBlocks = 32;
+constexpr int kMinSplitGroup = 8;
 inline int split_slots(int n_groups) {       // slots a shape with that many groups (all rows routed) can need
   const int64_t n = (int64_t)n_groups * kMaxKeySplit;
   return n < kSplitItems ? (int)n : kSplitItems;

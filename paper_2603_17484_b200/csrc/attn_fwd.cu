@@ -86,7 +86,8 @@ __host__ __device__ inline int longest_group(const FwdArgs& a) {
 // Key-range splits of a launch over compact rows; every warp of a CTA calls it as a whole.  Each lane weighs one number of
 // parts, in key blocks' time (1.55 us for two tiles): an item's start, end and the gap to the next one cost kItemCost, the
 // combination kCombineCost and its data kPartCost a part.  Groups of about equal length (a chunk of new tokens) run in waves;
-// those of a whole prefill, whose lengths fall from the longest to nothing, fill the SMs, longest first, up to half a part.
+// those of a whole prefill, whose lengths fall from the longest to nothing, fill the SMs, longest first, up to half a part.  Nothing
+// is gained by ending ahead of a local pass of fewer items than SMs.
 struct KeySplit {
   int64_t groups;     // that exist (a batch entry of fewer routed rows has fewer)
   int parts, blocks;  // most parts of a group, key blocks of a part
@@ -97,7 +98,11 @@ struct KeySplit {
 // 428 / 393.  (Twice as many parts: 4001 tokens 213: their rows, 133 KB a part, take longer than the blocks they save.)
 // With the SMs of a small local pass taken as busy until it ends, against all SMs as free: 100 new tokens on 60K keys 123.5 -> 88, 500
 // on 30K 138 -> 110, 64 on 40K 111 -> 78; of 1000 tokens and more the same.  From kSplitGroups groups on nothing was gained by parts.
-constexpr float kItemCost = 7.f, kCombineCost = 4.f, kPartCost = 0.04f;
+// The same for a prefill, and a last wave behind a local pass that fills the SMs counted half (they come free one after the other):
+// over 634 calls of 32 to 940 blocks and 1 to 127 groups the plan is on average 3.7 % off the best number of parts instead of 5.2 %,
+// and 33 instead of 57 of them are more than 2.5 % slower than with at most eight parts of 16 blocks or more (20000 tokens, one head,
+// window 4096: 102 -> 78 us, 81 with those).
+constexpr float kItemCost = 7.f, kCombineCost = 3.f, kPartCost = 0.04f;
 __device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
   const int lane = threadIdx.x & 31;
   int most = 0;
@@ -116,7 +121,8 @@ __device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
       // SMs could have done them without waves up to a wave's end on either side.
       const float c = part + kItemCost, inv = __fdividef(1.f, c);
       if (a.local_items == 0) {
-        cost = ceilf(items * (1.f / kSplitSms)) * c;
+        const float waves = items * (1.f / kSplitSms);
+        cost = fmaxf(1.f, 0.5f * (waves + ceilf(waves))) * c;
       } else {
         const float busy = (float)a.local_items, until = a.local_blocks + kItemCost;
         const float even = (items * c + busy * until) * (1.f / kSplitSms);
@@ -126,7 +132,10 @@ __device__ __forceinline__ KeySplit key_split(const FwdArgs& a) {
         if ((sms - busy) * floorf(t1 * inv + 1e-3f) + busy * n < items) t1 += c;
         cost = fmaxf(fminf(t0, t1), until);
       }
-    } else cost = fmaxf(part + kItemCost, (items * kItemCost + k.groups * 0.5f * (longest + shortest)) / sms + 0.5f * part);
+    } else {
+      cost = fmaxf(part + kItemCost, (items * kItemCost + k.groups * 0.5f * (longest + shortest)) / sms + 0.5f * part);
+      if (a.local_items > 0) cost = fmaxf(cost, a.local_blocks + kItemCost);
+    }
     if (p > 1) cost += kCombineCost + kPartCost * items;
     const bool possible = items <= kSplitItems && p <= longest;
     const uint32_t key = possible ? ((uint32_t)fminf(cost * 16.f, 1e8f) << 5) + lane : 0xffffffffu;

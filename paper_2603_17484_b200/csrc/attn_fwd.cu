@@ -268,7 +268,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     // Algorithm 1, step 1: each soft-max warp brings its 32 rows of Q, 16-byte pieces, into the layout a TMA copy would leave
     constexpr int kPieces = D / 8, kRowsPerStep = 32 / kPieces;
     const int row = row0 + warp * 32 + lane, c = row / pack;
-    const bf16* src = row < n_rows ? a.q + b * a.q_st.b + q_idx_b[c] * a.q_st.t + (int64_t)(g * G + row - c * pack) * D : nullptr;
+    const int t = row < n_rows ? q_idx_b[c] : -1;
+    // (debug build: an index outside of Q is reported and its row read as zeros)
+    const bool inside = row < n_rows && dbg_in_range(t >= 0 && t < a.Lq, a.status);
+    const bf16* src = inside ? a.q + b * a.q_st.b + t * a.q_st.t + (int64_t)(g * G + row - c * pack) * D : nullptr;
     const int piece = lane % kPieces;
     uint4 x[kPieces];
 #pragma unroll

@@ -278,7 +278,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     for (int k = 0; k < kPieces; ++k) {
       const bf16* p = reinterpret_cast<const bf16*>(
           __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(src), k * kRowsPerStep + lane / kPieces));
-      x[k] = p != nullptr ? __ldg(reinterpret_cast<const uint4*>(p) + piece) : make_uint4(0, 0, 0, 0);
+      x[k] = p != nullptr ? __ldcg(reinterpret_cast<const uint4*>(p) + piece) : make_uint4(0, 0, 0, 0);
     }
     const uint32_t dst = smem_u32(sQ + (warp >> 2) * SM::kQTileBytes) + (piece >> 3) * SM::kBoxBytes;
 #pragma unroll

@@ -55,14 +55,16 @@ size_t route_ws_size(const l2a_params* p) {
 // forward workspace: header, plan of each group whose key range may be split, slots of the parts
 constexpr size_t kGroupPartsBytes = (kSplitGroups * sizeof(int32_t) + 255) / 256 * 256;
 int group_count(const l2a_params* p) {
-  const int64_t n = (int64_t)ceil_div(p->Lq, kRowsPerCta) * p->Hq * p->B;
+  const int64_t n = compact_groups(p->Lq, p->Hq / p->Hkv) * p->Hkv * p->B;
   return n < kSplitGroups ? (int)n : kSplitGroups;     // launches with more groups are not split
 }
+// (from queries, heads and batch alone: a workspace serves every number of keys before them)
 size_t part_bytes(const l2a_params* p) {
   return align_up(split_slots(group_count(p)) * split_slot_floats(p->D) * sizeof(float), 256);
 }
 size_t fwd_ws_size(const l2a_params* p) {
-  // (never less than one copy of Q)
+  // Never less than one copy of Q, although no kernel keeps one any more: the size has always had room for the compact queries, and
+  // tests/test_abi.py holds it to that.
   const size_t q = align_up((size_t)p->B * p->Lq * p->Hq * p->D * sizeof(bf16), 256), parts = part_bytes(p);
   return kWsHeaderBytes + kGroupPartsBytes + (q > parts ? q : parts);
 }

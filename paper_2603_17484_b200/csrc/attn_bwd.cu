@@ -384,11 +384,14 @@ __device__ __forceinline__ void red_add_v4(float* base, uint32_t a, uint32_t b, 
                "f"(__uint_as_float(b)), "f"(__uint_as_float(c)), "f"(__uint_as_float(d)), "n"(kBytes)
                : "memory");
 }
-// Least distance between two reductions of a read-out warp, in SM clocks (polled: a sleep has steps of 64 ns).  Passes one after
-// the other, at the board's power limit: 64K tokens / whole layer at 8155 tokens / 2 x 4096 tokens with 16 clk 22830 / 2074 us / -,
-// 56 22430 / 2055 / -, 96 22180 / 2020 / -, 112 22260 / 2027 / 1289, 128 22050 / 2000 / 1277, 144 21960 / 2011 / 1273, 168 22510 /
-// 2060 / 1299, 200 23310 / 2115 / 1341.
-constexpr uint32_t kRedSpacingClk = 136;
+// Least distance between two reductions of a read-out warp, in SM clocks (polled: a sleep has steps of 64 ns), sixteen an item with
+// D = 128, eight with D = 64.  Passes one after the other, at the board's power limit:
+//   D = 128: 64K tokens / whole layer at 8155 tokens / 2 x 4096 tokens: 16 clk 22830 / 2074 us / -, 56 22430 / 2055 / -, 96 22180 /
+//   2020 / -, 112 22260 / 2027 / 1289, 128 22050 / 2000 / 1277, 144 21960 / 2011 / 1273, 168 22510 / 2060 / 1299, 200 23310 / 2115 /
+//   1341; on another day 112 22560 / 2055 / 1307, 128 22420 / 2035 / 1293, 136 22380 / 2038 / 1291, 144 22340 / 2034 / 1294.
+//   D = 64, 16384 tokens with 4/4 / 12/2 heads: 16 clk 514 / 1480 us, 64 515 / 1483, 88 516 / 1484, 112 518 / 1498, 136 522 / 1503.
+template <int D>
+constexpr uint32_t kRedSpacingClk = D == 128 ? 136 : 64;
 template <int D, int I>
 struct ReadOutReds {
   static constexpr int kCols = D / 4;                 // columns per quarter of the accumulator layout
@@ -397,7 +400,7 @@ struct ReadOutReds {
   __device__ __forceinline__ static void run(float* base, const uint32_t (&v)[D / 64][32]) {
     // spaced out: reductions issued back to back fill the queue of the memory pipe, and the compute warps' shared-memory
     // loads and stores (row statistics, dS) wait behind them; the read-out warps have most of an item's time to spare
-    { const uint32_t t0 = clock(); while ((uint32_t)clock() - t0 < kRedSpacingClk) { } }
+    { const uint32_t t0 = clock(); while ((uint32_t)clock() - t0 < kRedSpacingClk<D>) { } }
     red_add_v4<kOff>(base, v[I / 8][4 * (I % 8)], v[I / 8][4 * (I % 8) + 1], v[I / 8][4 * (I % 8) + 2],
                      v[I / 8][4 * (I % 8) + 3]);
     ReadOutReds<D, I + 1>::run(base, v);

@@ -1,7 +1,8 @@
 """Head-parallel sharding needs no exchange on the attention path: a rank that owns the KV heads [g0, g1) and their
 query heads calls the same entry points on slices of the tensors (the head stride stays D, the token stride is the
 full row), and gets the columns the whole call writes: exactly where both calls share key blocks among as many CTAs and
-split key ranges alike (which follows from their numbers of key blocks and of groups of routed rows, so from the heads),
+split key ranges alike (which follows from their numbers of key blocks and of groups of routed rows, so from the heads;
+none below 32 key blocks),
 up to rounding elsewhere.  Run here as two shards on one GPU."""
 import numpy as np
 import pytest
@@ -20,7 +21,7 @@ def test_two_head_shards_equal_the_whole_layer(extra):
 
 @pytest.mark.parametrize("B,L,Hq,Hkv,D,rho,differs", [
     (1, 1500, 8, 8, 64, 0.3, "backward"),     # 96 key blocks: two CTAs each; 48 in a shard: four
-    (1, 4500, 32, 2, 64, 0.2, "forward"),     # 128 groups of routed rows: no split; 64 in a shard: two parts from 32 key blocks on
+    (1, 4500, 32, 2, 64, 0.2, "forward"),     # 114 groups of routed rows, 36 key blocks: no split; 57 in a shard: three parts
 ])
 def test_two_head_shards_across_the_lines_of_the_plan(B, L, Hq, Hkv, D, rho, differs):
     _two_shards(B, L, Hq, Hkv, D, 160, rho, 0, differs)

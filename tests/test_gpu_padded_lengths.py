@@ -52,7 +52,7 @@ def test_right_padded_batch_matches_single_sequences():
 
 @pytest.mark.parametrize("lens,Hq,Hkv,D,split", [
     ((1100, 517, 1024), 8, 4, 128, "backward"),          # key blocks 36 (20, 32) alone: four CTAs each; 108 in the batch: two
-    ((4500,) + (300,) * 8, 4, 1, 64, "forward"),         # 16 groups of routed rows alone: two parts from 32 key blocks on; 144: none
+    ((4500,) + (300,) * 8, 4, 1, 64, "forward"),         # 15 groups of routed rows alone, 36 key blocks: nine parts; 135: none
 ])
 def test_padded_batch_across_the_lines_of_the_plan(lens, Hq, Hkv, D, split):
     """A batch in which another number of CTAs shares a key block, or key ranges are not split, than in the single calls."""

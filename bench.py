@@ -39,7 +39,7 @@ FWD_PHASES = ("fwd_start", "attn_fwd_local", "attn_fwd_global")
 BWD_PHASES = ("gather_q_dO", "bwd_delta_zero", "bwd", "bwd_dq_merge")
 # DRAM read + write over algorithmic bytes of a launch, from the ncu capture of the 128K workload cut to two KV heads
 # (profiles/bwd_kernel_l2_traffic_128k_one_kv_head.md): the launch order of the whole workload, small enough for counters
-TRAFFIC_RATIO = {"bwd": 1.55, "attn_fwd_local": 0.95, "attn_fwd_global": 1.74}
+TRAFFIC_RATIO = {"bwd": 1.52, "attn_fwd_local": 0.95, "attn_fwd_global": 1.73}
 # the same of a decode launch with every sequence routed (profiles/decode_split_kernel_decode_128k.md)
 DECODE_TRAFFIC_RATIO = 1.004
 

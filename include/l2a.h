@@ -234,12 +234,14 @@ l2a_status l2a_router_logits(const l2a_params* p, const void* S, const float* w,
  *                    log-sum-exp of the global scores of compact row c (Algorithm 1's L_c).
  *                    Both lse outputs may be NULL unless L2A_FLAG_SAVE_FOR_BWD is set.
  *   fwd_ws         : workspace of at least fwd_ws_bytes (holds the fp32 partial rows of split key ranges; the global
- *                    kernel gathers the routed queries itself).
+ *                    kernel gathers the routed queries itself).  The size follows from Lq, Hq, Hkv, D and B alone.
  * Scores and soft-max run in fp32, probabilities are rounded to bf16 for the second contraction,
- * accumulation is fp32.  Results are bit-reproducible; with few routed rows in the call the keys of a routed row
- * are split into parts (a function of Lq, Lk, Hq, Hkv, B and the largest n_routed), each of which rounds its probabilities
- * against its own running maximum, so that the routed rows of the same sequence in another batch can differ by
- * that rounding.  Returns L2A_ERR_UNSUPPORTED for D not in {64, 128}.
+ * accumulation is fp32.  Results are bit-reproducible; with few routed rows in a call whose keys before the last row
+ * (before its window with L2A_FLAG_SHARED_WINDOW) fill 32 blocks of 128 or more, the keys of a routed row are split
+ * into parts (a function of Lq, q_pos_offset, window, Hq, Hkv, B, the largest n_routed, L2A_FLAG_SKIP_LOCAL and
+ * L2A_FLAG_SHARED_WINDOW), each of which rounds its probabilities against its own running maximum, so that the routed
+ * rows of the same sequence in another batch, as a head shard or beside another window can differ by that rounding.
+ * In shorter calls none is split, and routed rows have the same bits in all of them.  Returns L2A_ERR_UNSUPPORTED for D not in {64, 128}.
  */
 l2a_status l2a_forward(const l2a_params* p, const void* Q, const void* K, const void* V,
                        const uint8_t* d_mask, const int32_t* q_idx, const int32_t* n_routed,

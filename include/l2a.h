@@ -241,7 +241,8 @@ l2a_status l2a_router_logits(const l2a_params* p, const void* S, const float* w,
  * into parts (a function of Lq, q_pos_offset, window, Hq, Hkv, B, the largest n_routed, L2A_FLAG_SKIP_LOCAL and
  * L2A_FLAG_SHARED_WINDOW), each of which rounds its probabilities against its own running maximum, so that the routed
  * rows of the same sequence in another batch, as a head shard or beside another window can differ by that rounding.
- * In shorter calls none is split, and routed rows have the same bits in all of them.  Returns L2A_ERR_UNSUPPORTED for D not in {64, 128}.
+ * In shorter calls none is split, and routed rows have the same bits in all of them.  Returns L2A_ERR_UNSUPPORTED for
+ * D not in {64, 128}.
  */
 l2a_status l2a_forward(const l2a_params* p, const void* Q, const void* K, const void* V,
                        const uint8_t* d_mask, const int32_t* q_idx, const int32_t* n_routed,

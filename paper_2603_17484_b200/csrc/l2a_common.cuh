@@ -158,8 +158,8 @@ struct FwdArgs {
                              // global pass behind the plainly launched local one of the same call): only before it combines
 };
 // A global launch of fewer than kSplitGroups groups whose last one may see kMinSplitBlocks key blocks or more splits key ranges
-// (key_split), those of kMinSplitGroup blocks and more, into at most kMaxKeySplit parts of a group and kSplitItems in all.  In
-// shorter calls none is split, whatever their batch and heads: the routed rows of up to 31 blocks of keys then have the same bits
+// (key_split), those of kMinSplitGroup blocks and more (an item costs seven blocks' time besides its own), into at most kMaxKeySplit
+// parts of a group and kSplitItems in all.  In shorter calls none is split, whatever their batch and heads: the routed rows of up to 31 blocks of keys then have the same bits
 // alone, in a batch and as a head shard, and the launch that combines parts is left out.  Whole call undivided / with the parts
 // that the cost estimate favours (from 8 blocks on, two blocks a part up to 16): 1024 tokens (28/4 heads, window 4096, 20 % routed)
 // 37 / 49 us, 2000 (8/1) 48 / 57, 1500 (12/2, D = 64) 37 / 45, 3000 (28/4) 118 / 113, 64 new tokens on 3900 keys 65 / 66; but with a
